@@ -2,7 +2,8 @@
 
 The module-level ``ubep_*`` functions have the names and argument order of the C entry
 points and only marshal arguments (torch tensors -> device pointers, the current torch
-stream -> ``void*``).  ``Buffer`` is a small convenience holder for an arena tensor and its
+stream -> ``void*``); the calls of every step go through the CPython module ``_native``
+instead of ctypes.  ``Buffer`` is a small convenience holder for an arena tensor and its
 views.  PyTorch supplies device memory and streams; every step of dispatch / combine runs
 in the library's kernels.  There is no fallback: if the library is missing, loading raises.
 """
@@ -110,8 +111,27 @@ def load() -> ctypes.CDLL:
     lib.ubep_wait_arrivals.restype, lib.ubep_wait_arrivals.argtypes = ctypes.c_int, [vp, vp]
     lib.ubep_combine_sharded.restype = ctypes.c_int
     lib.ubep_combine_sharded.argtypes = [vp, vp, vp, i32, vp, vp]
+    native = _load_native()
+    native.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in
+                  (lib.ubep_dispatch, lib.ubep_combine, lib.ubep_get_dispatch_layout, lib.ubep_dispatch_sync)))
     _lib = lib
     return lib
+
+
+_native = None
+
+
+def _load_native():
+    """The CPython module built beside the library (ubep_py.cpp); no ctypes fallback exists for its calls."""
+    global _native
+    if _native is None:
+        try:
+            from . import _native as mod
+        except ImportError as e:
+            raise RuntimeError(f"{_HERE}/_native.so is missing or does not load: build it with "
+                               f"`python -m paper_2607_06202_b200.build` ({e})") from e
+        _native = mod
+    return _native
 
 
 class UbepError(RuntimeError):
@@ -134,9 +154,14 @@ def _ptr(t: Optional[torch.Tensor]):
     return ctypes.c_void_p(t.data_ptr())
 
 
+def _handle(buf):
+    """Buffer handle as an integer (what `_native` takes)."""
+    return buf.value if isinstance(buf, ctypes.c_void_p) else buf
+
+
 def _stream(stream) -> ctypes.c_void_p:
     if stream is None:
-        stream = torch.cuda.current_stream()
+        return ctypes.c_void_p(_load_native().current_stream())
     return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
 
 
@@ -180,9 +205,9 @@ def ubep_set_dest_order(buf, order) -> None:
 
 def ubep_get_dispatch_layout(buf, topk_idx: torch.Tensor, T: int, num_tokens_per_rank, num_tokens_per_expert,
                              is_token_in_rank, stream=None) -> None:
-    _check(load().ubep_get_dispatch_layout(buf, _ptr(topk_idx), T, _ptr(num_tokens_per_rank),
-                                           _ptr(num_tokens_per_expert), _ptr(is_token_in_rank), _stream(stream)),
-           "ubep_get_dispatch_layout", buf)
+    load()
+    _check(_native.layout(_handle(buf), topk_idx, T, num_tokens_per_rank, num_tokens_per_expert, is_token_in_rank,
+                          stream), "ubep_get_dispatch_layout", buf)
 
 
 def ubep_get_dispatch_layout_static(topk_idx: torch.Tensor, T: int, topk: int, num_experts: int, num_ranks: int,
@@ -196,12 +221,13 @@ def ubep_get_dispatch_layout_static(topk_idx: torch.Tensor, T: int, topk: int, n
 
 
 def ubep_dispatch(buf, x: torch.Tensor, topk_idx: torch.Tensor, topk_w: torch.Tensor, T: int, stream=None) -> None:
-    _check(load().ubep_dispatch(buf, _ptr(x), _ptr(topk_idx), _ptr(topk_w), T, _stream(stream)),
-           "ubep_dispatch", buf)
+    load()
+    _check(_native.dispatch(_handle(buf), x, topk_idx, topk_w, T, stream), "ubep_dispatch", buf)
 
 
 def ubep_combine(buf, y: torch.Tensor, topk_w: torch.Tensor, T: int, out: torch.Tensor, stream=None) -> None:
-    _check(load().ubep_combine(buf, _ptr(y), _ptr(topk_w), T, _ptr(out), _stream(stream)), "ubep_combine", buf)
+    load()
+    _check(_native.combine(_handle(buf), y, topk_w, T, out, stream), "ubep_combine", buf)
 
 
 def ubep_map_workers(order: torch.Tensor, counts: torch.Tensor, n_workers: int, start_pos: torch.Tensor,
@@ -269,8 +295,8 @@ def ubep_sync_attach(buf, wire: torch.Tensor, stream=None) -> None:
 
 def ubep_dispatch_sync(buf, protocol: int, x: torch.Tensor, topk_idx: torch.Tensor, topk_w: torch.Tensor, T: int,
                        stream=None) -> None:
-    _check(load().ubep_dispatch_sync(buf, protocol, _ptr(x), _ptr(topk_idx), _ptr(topk_w), T, _stream(stream)),
-           "ubep_dispatch_sync", buf)
+    load()
+    _check(_native.dispatch_sync(_handle(buf), protocol, x, topk_idx, topk_w, T, stream), "ubep_dispatch_sync", buf)
 
 
 def ubep_sync_view(buf, which: int):
@@ -331,6 +357,10 @@ class Buffer:
         if fill is not None:
             self.arena.fill_(fill)
         self.handle = ubep_buffer_create(self.cfg, self.arena)
+        # what the calls of every step need, as plain integers (reading ctypes fields costs more than the call)
+        self._h = self.handle.value
+        self._ranks, self._experts, self._hidden = int(num_ranks), int(num_experts), int(hidden)
+        self._device = self.arena.device.index
         self.views = {}
         base = self.arena.data_ptr()
         for which, (name, dt) in enumerate(zip(VIEW_NAMES, _VIEW_DTYPES)):
@@ -364,23 +394,25 @@ class Buffer:
         ubep_set_dest_order(self.handle, order)
 
     def get_dispatch_layout(self, topk_idx, stream=None):
-        T = topk_idx.shape[0]
-        R, E = self.cfg.num_ranks, self.cfg.num_experts
-        dev = self.arena.device
-        npr = torch.empty(R, dtype=torch.int32, device=dev)
-        npe = torch.empty(E, dtype=torch.int32, device=dev)
-        itr = torch.empty((T, R), dtype=torch.uint8, device=dev)
-        ubep_get_dispatch_layout(self.handle, topk_idx, T, npr, npe, itr, stream)
-        return npr, npe, itr
+        out = _native.layout_new(self._h, topk_idx, self._ranks, self._experts, self._device, stream)
+        if type(out) is int:
+            _check(out, "ubep_get_dispatch_layout", self.handle)
+        return out
 
     def dispatch(self, x, topk_idx, topk_w, stream=None):
-        ubep_dispatch(self.handle, x, topk_idx, topk_w, x.shape[0], stream)
+        rc = _native.dispatch(self._h, x, topk_idx, topk_w, None, stream)
+        if rc:
+            _check(rc, "ubep_dispatch", self.handle)
 
     def combine(self, y, topk_w, out=None, stream=None):
-        T = topk_w.shape[0]
         if out is None:
-            out = torch.empty((T, self.cfg.hidden), dtype=torch.bfloat16, device=self.arena.device)
-        ubep_combine(self.handle, y, topk_w, T, out, stream)
+            out = _native.combine_new(self._h, y, topk_w, self._hidden, self._device, stream)
+            if type(out) is int:
+                _check(out, "ubep_combine", self.handle)
+            return out
+        rc = _native.combine(self._h, y, topk_w, None, out, stream)
+        if rc:
+            _check(rc, "ubep_combine", self.handle)
         return out
 
     def status(self) -> int:
@@ -410,7 +442,9 @@ class Buffer:
     def dispatch_sync(self, protocol, x, topk_idx, topk_w, stream=None):
         if isinstance(protocol, str):
             protocol = SYNC_NAMES[protocol]
-        ubep_dispatch_sync(self.handle, protocol, x, topk_idx, topk_w, x.shape[0], stream)
+        rc = _native.dispatch_sync(self._h, protocol, x, topk_idx, topk_w, None, stream)
+        if rc:
+            _check(rc, "ubep_dispatch_sync", self.handle)
 
     def scan_sentinel(self, x, stream=None) -> int:
         return ubep_sync_scan_sentinel(self.handle, x, x.shape[0], stream)
@@ -418,7 +452,7 @@ class Buffer:
     def close(self):
         if getattr(self, "handle", None):
             ubep_buffer_destroy(self.handle)
-            self.handle = None
+            self.handle = self._h = None
 
     def __del__(self):
         try:
