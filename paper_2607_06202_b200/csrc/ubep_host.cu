@@ -273,14 +273,18 @@ int ubep_buffer_create(const ubep_config_t* cfg, void* dev_arena, size_t bytes, 
     if (bytes < make_layout(*cfg, cfg->num_ctas).total) return UBEP_ERR_ARENA;
     DeviceGuard guard(cfg->device);
     if (guard.err != cudaSuccess) return UBEP_ERR_CUDA;
-    cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, cfg->device) != cudaSuccess) return UBEP_ERR_CUDA;
+    // (single attributes: cudaGetDeviceProperties fills in everything there is to know, and the clock rate alone
+    // takes milliseconds to ask for)
+    int sms = 0, smem = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, cfg->device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, cfg->device) != cudaSuccess)
+        return UBEP_ERR_CUDA;
     ubep_buffer* b = new (std::nothrow) ubep_buffer();
     if (!b) return UBEP_ERR_ARG;
     b->cfg = *cfg;
-    b->num_sms = prop.multiProcessorCount;
-    b->max_smem = (int)prop.sharedMemPerBlockOptin;
-    b->sm_khz = prop.clockRate > 0 ? prop.clockRate : 1965000;
+    b->num_sms = sms;
+    b->max_smem = smem;
+    b->sm_khz = 1965000;
     int n = cfg->num_ctas > 0 ? cfg->num_ctas : b->num_sms;
     if (n > b->num_sms) n = b->num_sms;  // all CTAs of the persistent kernel must be resident
     if (n > ubep::kMaxChunks) n = ubep::kMaxChunks;
@@ -779,6 +783,12 @@ int ubep_debug_withhold_flag(ubep_buffer_t* buf, int32_t chunk) {
 int ubep_debug_trace(ubep_buffer_t* buf, int32_t enable) {
     if (!buf) return UBEP_ERR_ARG;
     buf->tracing = enable != 0;
+    if (buf->tracing) {   // the stamps are derived with the SM clock
+        int khz = 0;
+        const cudaError_t e = cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, buf->cfg.device);
+        if (e != cudaSuccess) return cuda_fail(buf, e);
+        if (khz > 0) buf->sm_khz = khz;
+    }
     return UBEP_OK;
 }
 
