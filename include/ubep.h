@@ -179,8 +179,8 @@ int ubep_get_dispatch_layout(ubep_buffer_t *buf, const int32_t *topk_idx /*[dev]
  * ubep_get_dispatch_layout, but it needs no buffer handle and no arena: a caller that
  * runs inside somebody else's memory plan -- a plugin handed fixed input and output
  * tensors, code running while allocation is forbidden -- cannot reserve an arena, so the
- * chunk histograms live in a fixed array of UBEP_STATIC_MAX_BINS x 64 32-bit words
- * (about 257 KB) inside the library's device image.  Every GPU that loads the library holds
+ * totals being added up live in a fixed array of UBEP_STATIC_MAX_BINS 32-bit words
+ * (about 4 KB) inside the library's device image.  Every GPU that loads the library holds
  * that array until the process exits.
  *
  * Limits: num_experts + num_ranks <= UBEP_STATIC_MAX_BINS, topk <= 32, num_experts %
@@ -192,8 +192,8 @@ int ubep_get_dispatch_layout(ubep_buffer_t *buf, const int32_t *topk_idx /*[dev]
  * current) and keeps it; make that first call before any stream capture begins.  The call
  * itself calls no cudaMalloc, cudaFree or other allocating routine.  All calls on a device
  * share the one array: calls whose kernels may overlap on the GPU (different streams) race
- * on it -- keep them on one stream or otherwise ordered.  The array keeps the previous
- * call's contents; the kernel overwrites what it reads and re-arms its own counter.
+ * on it -- keep them on one stream or otherwise ordered.  The array is zero between calls;
+ * the kernel leaves it so.
  */
 #define UBEP_STATIC_MAX_BINS 1024
 int ubep_get_dispatch_layout_static(const int32_t *topk_idx /*[dev]*/, int32_t T, int32_t topk,

@@ -39,7 +39,7 @@ struct ArenaLayout {
     size_t off[UBEP_VIEW_COUNT_];
     size_t slot_pos, copy_pos, chunk_hist, partial, chunk_base, trace;
     size_t flags_begin, hist_flag, scan_flag, status, ticket, epoch_ctr, done_ticket, cursor, pos_flag, claimed,
-        order_pos, flags_end, peer_delta;
+        layout_acc, order_pos, flags_end, peer_delta;
     size_t total;
     int er_cap, nchunks, S, rowB, G, B;
 };
@@ -100,6 +100,7 @@ ArenaLayout make_layout(const ubep_config_t& c, int nchunks) {
     a.off[UBEP_VIEW_ARRIVAL] = take(2 * R * 4);
     a.status = take(4);
     a.ticket = take(4);
+    a.layout_acc = take(B * 4);
     a.off[UBEP_VIEW_EPOCH] = a.epoch_ctr = take(4);
     a.done_ticket = take(4);
     a.cursor = take(n * 4);
@@ -368,7 +369,7 @@ int ubep_get_dispatch_layout(ubep_buffer_t* buf, const int32_t* topk_idx, int32_
     Params p = make_params(buf, T);
     p.topk_idx = topk_idx;
     cudaError_t e = ubep::launch_layout(p, num_tokens_per_rank, num_tokens_per_expert, is_token_in_rank,
-                                        p.chunk_hist, at<unsigned>(buf, buf->lay.ticket), st);
+                                        at<int32_t>(buf, buf->lay.layout_acc), at<unsigned>(buf, buf->lay.ticket), st);
     if (e != cudaSuccess) return cuda_fail(buf, e);
     g_launches += 1;
     return UBEP_OK;

@@ -1,7 +1,6 @@
 // ubep_get_dispatch_layout_static: the counts-only step for callers that cannot give the
 // library any device memory of their own beyond inputs and outputs -- no arena, no buffer
-// handle.  The per-chunk histograms and the completion ticket of the counting kernel live
-// in a fixed array inside this library's device image instead.
+// handle.  The totals that the counting kernel adds up and its completion ticket live in a fixed array inside this library's device image instead.
 #include <cstdint>
 
 #include "../../include/ubep.h"
@@ -10,10 +9,9 @@
 namespace {
 
 // Scratch held by every GPU that loads the library, until the process exits:
-// kStaticChunks * kStaticBins histogram words, one ticket word, one status word (~257 KB).
-constexpr int kStaticChunks = 64;
+// kStaticBins words of totals, one ticket word, one status word (~4 KB).
 constexpr int kStaticBins = UBEP_STATIC_MAX_BINS;
-constexpr int kStaticWords = kStaticChunks * kStaticBins + 64;
+constexpr int kStaticWords = kStaticBins + 64;
 static __device__ __align__(256) int32_t g_static_scratch[kStaticWords];
 
 // Device address of g_static_scratch per device ordinal.  In host code the array's name is
@@ -51,12 +49,11 @@ extern "C" int ubep_get_dispatch_layout_static(const int32_t* topk_idx, int32_t 
     ubep::Params p{};
     p.T = T; p.k = topk; p.E = num_experts; p.R = num_ranks; p.L = num_experts / num_ranks;
     p.B = num_experts + num_ranks;
-    p.nchunks = kStaticChunks;
+    p.L_magic = p.L == 1 ? 0xffffffffu : (unsigned)((0x100000000ull + (uint64_t)p.L - 1) / (uint64_t)p.L);
     p.topk_idx = topk_idx;
-    p.status = scratch + kStaticChunks * kStaticBins + 32;   // ids out of range are skipped; code kept here
-    unsigned* ticket = reinterpret_cast<unsigned*>(scratch + kStaticChunks * kStaticBins);
-    // The kernel writes every histogram word it later reads and re-arms the ticket (back to
-    // zero) when its last CTA finishes, so nothing has to be cleared between calls.
+    p.status = scratch + kStaticBins + 32;   // ids out of range are skipped; code kept here
+    unsigned* ticket = reinterpret_cast<unsigned*>(scratch + kStaticBins);
+    // The kernel's last CTA leaves the totals and the ticket at zero, so nothing has to be cleared between calls.
     const cudaError_t e = ubep::launch_layout(p, num_tokens_per_rank, num_tokens_per_expert, is_token_in_rank, scratch,
                                               ticket, static_cast<cudaStream_t>(cuda_stream));
     return e == cudaSuccess ? UBEP_OK : UBEP_ERR_CUDA;

@@ -1,0 +1,41 @@
+"""The counts entry point at the edges of its work split: 32 tokens per warp, four warps per CTA, at most 296
+CTAs; rank masks of one word, of four words and the slot-by-slot variant beyond 128 ranks; slots per token with
+a variant of their own (2, 4, 8) and without.  Integers: exact against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2607_06202_b200 import binding as B
+from paper_2607_06202_b200 import workload as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("T", [1, 31, 33, 129, 40001])
+@pytest.mark.parametrize("E,R,k", [(4, 1, 3), (15, 5, 2), (64, 32, 4), (128, 16, 8), (66, 33, 4), (288, 72, 8),
+                                   (256, 128, 16), (390, 130, 8), (200, 200, 2)])
+def test_counts_match_the_oracle(T, E, R, k):
+    rng = np.random.Generator(np.random.PCG64(T * 1000 + E))
+    idx = np.argsort(rng.random((T, E)), axis=1)[:, :k].astype(np.int32)
+    idx[rng.random(idx.shape) < 0.1] = -1
+    lay = oracle.layout(idx, E, R, R, 0)
+    dup = idx.copy()      # the last slot repeats the first one: reported, counted as if it were empty
+    if k > 2:
+        dup[:, -1] = dup[:, 0]
+    clean = dup.copy()
+    if k > 2:
+        clean[:, -1] = -1
+    lay_dup = oracle.layout(clean, E, R, R, 0)
+    buf = B.Buffer(num_ranks=R, num_experts=E, hidden=8, topk=k, max_tokens=T, rows_per_rank_cap=1)
+    for table, want, code in ((idx, lay, 0), (dup, lay_dup, B.UBEP_ERR_BAD_INDEX if (k > 2 and (dup[:, 0] >= 0).any()) else 0),
+                              (idx, lay, 0)):
+        npr, npe, itr = buf.get_dispatch_layout(torch.from_numpy(table).cuda())
+        assert buf.status() == code
+        assert np.array_equal(npr.cpu().numpy(), want.num_tokens_per_rank)
+        assert np.array_equal(npe.cpu().numpy(), want.num_tokens_per_expert)
+        assert np.array_equal(itr.cpu().numpy(), want.is_token_in_rank)
+    # through the C entry point with some of the outputs left out
+    only = torch.full((E,), -1, dtype=torch.int32, device="cuda")
+    B.ubep_get_dispatch_layout(buf.handle, torch.from_numpy(idx).cuda(), T, None, only, None)
+    assert np.array_equal(only.cpu().numpy(), lay.num_tokens_per_expert)
