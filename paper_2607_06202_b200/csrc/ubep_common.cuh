@@ -25,7 +25,7 @@ constexpr int kFastQuantWarps = 5;     // FP8 in the flag-free kernel with rank-
                                        // 512 / 1024 tokens: 15.5 / 24.3 us with 4, 15.5 / 25.3 with 6, 15.7 / 30.7 with 8, 18.0 / 38.2 with 10)
 constexpr int kStorePending = 3;       // FP8: rows whose bulk stores may still be reading shared memory
 constexpr int kTraceSlots = 16;        // per-CTA phase time stamps (optional tracing)
-constexpr int kModePhased = 1, kModeFused = 2, kModeLocal = 3;
+constexpr int kModePhased = 1, kModeFused = 2, kModeLocal = 3, kModeCluster = 4;
 // Every wait in the kernels gives up after this many nanoseconds of wall time.
 constexpr unsigned long long kWaitLimitNs = 1500000000ull;
 
@@ -37,6 +37,7 @@ struct Params {
     int G;           // H / 128 scale groups (FP8)
     int B;           // histogram bins: E expert bins followed by R rank bins
     int nchunks;     // token chunks (contiguous, equal to +-1 token)
+    int cluster;     // CTAs per thread-block cluster (layout by clusters; else 1)
     int parts;       // column parts per row: CTA c moves part c % parts of chunk c / parts
     int grid;        // CTAs of the dispatch kernel = nchunks * parts
     unsigned L_magic;  // ceil(2^32 / L): e / L == umulhi(e, L_magic) for e < 65536
@@ -309,6 +310,7 @@ struct SmemPlan {
     int map_groups, map_wb, map_bp;   // bin bitmaps: 32-token groups, words of bins, padded bins
     int off_out, off_ids, off_mask, off_bm, off_pos, off_key, off_ord, off_w, off_hist, off_arr, off_order;
     int off_item;                     // per ring stage: where its token comes from, positions of stolen tokens
+    int off_cnt;                      // layout by clusters: three arrays of counts
     int total;
 };
 

@@ -31,8 +31,13 @@ constexpr int64_t kLocalMaxSlots = 8192;        // small-T limit of the combine 
 constexpr int64_t kLocalFastMaxSlots = 16384;     // one row per (token, rank), bf16 rows: the rank-level fast path
                                                   // (2048 tokens: 50.4 against 58.4 us; larger tables do not fit in shared memory)
 constexpr int64_t kLocalFastFp8MaxSlots = 8192;   // the same with FP8 rows (1024 tokens: 25.3 against 31.5 us, 1536: 39.4 against 38.4)
-constexpr int64_t kLocalAllBinsMaxSlots = 3072;   // every bin's bitmaps have to be built, bf16 rows
-constexpr int64_t kLocalAllBinsFp8MaxSlots = 1536;   // ... FP8 rows
+// One row per (token, expert), bf16 rows: every CTA derives the layout alone where the table has at most 512 slots
+// and slots * bins are at most 32 K (8 tokens of top-8, 288 bins: 7.5 us against 7.9 by clusters, 32 tokens: 7.7 and
+// 7.4; 128 tokens of top-4, 40 bins: 7.3 and 7.6, 512 tokens: 12.7 and 9.0).  FP8 rows: by clusters throughout.
+constexpr int64_t kLocalAllBinsMaxSlots = 512, kLocalAllBinsMaxSlotBins = 32768;
+// Cluster sizes: two up to 32 K slots, eight from 64 K on (dispatch + combine, sizes 2 / 4 / 8: 24576 slots 88.2 / 88.8 /
+// 90.2 us, 32768 slots 150 / 151 / 152, 65536 slots 213 / 212 / 209, 131072 slots 555 / 555 / 544).
+constexpr int64_t kCluster2MaxSlots = 32768, kCluster8MinSlots = 65536;
 inline size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
 struct ArenaLayout {
@@ -192,7 +197,7 @@ Params make_params(ubep_buffer* b, int T) {
     p.T = T; p.H = c.hidden; p.E = c.num_experts; p.R = c.num_ranks; p.L = p.E / p.R; p.k = c.topk;
     p.S = a.S; p.cap = c.rows_per_rank_cap; p.payload = c.payload; p.dedup = c.dedup;
     p.rowB = a.rowB; p.G = a.G; p.B = a.B; p.nchunks = a.nchunks; p.er_cap = a.er_cap;
-    p.parts = 1; p.grid = a.nchunks;
+    p.cluster = 1; p.parts = 1; p.grid = a.nchunks;
     p.L_magic = p.L == 1 ? 0xffffffffu : (unsigned)((0x100000000ull + (uint64_t)p.L - 1) / (uint64_t)p.L);
     p.local_fast = (c.dedup && p.L < 32 && p.L > 1 && p.R <= 32 * ubep::kRankWordsHost) ? 1 : 0;
     p.epoch_ctr = at<unsigned>(b, a.epoch_ctr);
@@ -239,6 +244,37 @@ Params make_params(ubep_buffer* b, int T) {
     p.peer_delta = at<long long>(b, a.peer_delta);
     p.shard_arrival = at<unsigned>(b, a.off[UBEP_VIEW_SHARD_ARRIVAL]);
     return p;
+}
+
+// Cuts the work of a flag-free kernel over `ctas` CTAs: token chunks, and column parts of a row so that the slices
+// are balanced to about 5 %.  The CTA with the most work sets the pace: ceil(T / chunks) tokens of 1 / parts of a
+// row each.  Smaller pieces cost more per byte (measured on the decode shape, layout by every CTA alone: 4 parts
+// + 8 %, 8 parts + 60 %).  With the layout by clusters pieces are cut for balance only where they keep 4 KB (512
+// tokens of 1024 bf16 channels: 9.0 us whole, 10.4 in halves; 7168 channels: 16.3 and 15.3), FP8 rows not at all
+// (512 tokens of 7168 channels: 13.3 and 16.4 us); a CTA that has one token at most takes any piece.
+void split_work(Params& p, int ctas) {
+    int best = 1;
+    double best_cost = 0.0;
+    const bool by_cluster = p.cluster > 1;
+    const double piece_penalty[4] = {1.0, by_cluster ? 1.05 : 1.0, by_cluster ? 1.1 : 1.08, by_cluster ? 1.15 : 1.6};
+    for (int parts = 1, i = 0; parts <= 8; parts *= 2, ++i) {
+        const int chunks = ctas / parts;
+        if (chunks < 1 || (p.H * 2 / parts) % 16 != 0 || (p.H * 2) % parts != 0) break;
+        if (p.payload && ((p.H / parts) % 128 != 0 || p.H % parts != 0)) break;
+        // FP8 rows: a piece's scales must still be a bulk copy (a multiple of 16 bytes); with plain stores for
+        // the scales and payload pieces under 2 KB a dispatch of 384 tokens took 33 us against 21 us for 512
+        if (p.payload && parts > 1 && ((p.G / parts) * 4) % 16 != 0) break;
+        const int most = (p.T + chunks - 1) / chunks;
+        if (by_cluster && parts > 1 && most > 1 && (p.payload || p.H * 2 / parts < 4096)) break;
+        const double cost = (double)most / parts * piece_penalty[i];
+        if (parts == 1 || cost < best_cost * 0.999) {
+            best = parts;
+            best_cost = cost;
+        }
+    }
+    p.parts = best;
+    p.nchunks = ctas / best;
+    p.grid = p.nchunks * best;
 }
 
 // Makes the buffer's device current for the scope of one call.
@@ -397,62 +433,54 @@ int ubep_dispatch(ubep_buffer_t* buf, const void* x, const int32_t* topk_idx, co
     p.topk_w = topk_w;
     p.withhold = buf->withhold;
     buf->withhold = -1;
-    // AUTO: a routing table that fits in shared memory is cheaper to recount in every CTA
-    // than to exchange through flags; larger ones use the decomposed kernel.
     int mode = buf->cfg.pipeline;
-    if (mode == UBEP_PIPELINE_AUTO) {
-        // With the rank-level fast path the flag-free kernel wins up to about 1800 tokens of top-8 (bf16 rows);
-        // when every CTA has to build the bitmaps of every bin it wins only for a few hundred tokens, and
-        // with FP8 rows (whose quantising warps are the layout warps there, so nothing moves before the
-        // layout and its outputs are done) for fewer still.
-        const int64_t slots = (int64_t)T * p.k;
-        const int64_t limit = p.local_fast ? (p.payload ? kLocalFastFp8MaxSlots : kLocalFastMaxSlots)
-                                           : (p.payload ? kLocalAllBinsFp8MaxSlots : kLocalAllBinsMaxSlots);
-        const bool local = slots <= limit;
-        mode = local ? UBEP_PIPELINE_LOCAL : UBEP_PIPELINE_FUSED;
-    }
     ubep::SmemPlan pl{};
     int launches = 0;
     p.parts = 1;
     p.grid = p.nchunks;
-    if (mode == UBEP_PIPELINE_LOCAL) {
-        // split rows into column parts until the slices of work are balanced to ~5 %
-        const int n = buf->lay.nchunks;
-        // The CTA with the most work sets the pace: ceil(T / chunks) tokens of 1 / parts of a row each.
-        // Smaller pieces cost more per byte (measured on the decode shape: 4 parts + 8 %, 8 parts + 60 %).
-        int best = 1;
-        double best_cost = 0.0;
-        static const double kPiecePenalty[4] = {1.0, 1.0, 1.08, 1.6};
-        for (int parts = 1, i = 0; parts <= 8; parts *= 2, ++i) {
-            const int chunks = n / parts;
-            if (chunks < 1 || (p.H * 2 / parts) % 16 != 0 || (p.H * 2) % parts != 0) break;
-            if (p.payload && ((p.H / parts) % 128 != 0 || p.H % parts != 0)) break;
-            // FP8 rows: a piece's scales must still be a bulk copy (a multiple of 16 bytes); with plain stores for
-            // the scales and payload pieces under 2 KB a dispatch of 384 tokens took 33 us against 21 us for 512
-            if (p.payload && parts > 1 && ((p.G / parts) * 4) % 16 != 0) break;
-            const double cost = (double)((T + chunks - 1) / chunks) / parts * kPiecePenalty[i];
-            if (parts == 1 || cost < best_cost * 0.999) {
-                best = parts;
-                best_cost = cost;
+    const int n = buf->lay.nchunks;
+    const int64_t slots = (int64_t)T * p.k;
+    if (mode == UBEP_PIPELINE_AUTO) {
+        // With the rank-level fast path, and for the smallest tables, every CTA derives what it needs alone; beyond
+        // that clusters of CTAs count the table between them (larger clusters cost CTAs: of a B200's 148 SMs 132
+        // can be used in clusters of four, 120 in clusters of eight).
+        mode = UBEP_PIPELINE_FUSED;
+        const bool alone = p.local_fast ? slots <= (p.payload ? kLocalFastFp8MaxSlots : kLocalFastMaxSlots)
+                                        : !p.payload && slots <= kLocalAllBinsMaxSlots && slots * p.B <= kLocalAllBinsMaxSlotBins;
+        if (alone) {
+            mode = UBEP_PIPELINE_LOCAL;
+        } else {
+            const int cs = slots <= kCluster2MaxSlots ? 2 : slots < kCluster8MinSlots ? 4 : 8;
+            int ctas = ubep::cluster_ctas(cs, buf->max_smem);
+            ctas = (ctas < n ? ctas : n) / cs * cs;
+            if (ctas > 0 && T <= 65535) {   // (counts are 16 bits wide)
+                p.cluster = cs;
+                p.steal = T >= kStealMinTokensPerChunk * ctas ? 1 : 0;
+                if (p.steal) p.nchunks = p.grid = ctas;   // whole rows are handed out
+                else split_work(p, ctas);
+                if (ubep::plan_dispatch(p, ubep::kModeCluster, buf->max_smem, &pl) == 0) mode = ubep::kModeCluster;
+                else p.cluster = 1;
             }
         }
-        p.parts = best;
-        p.nchunks = n / best;
-        p.grid = p.nchunks * best;
+    }
+    if (mode == UBEP_PIPELINE_LOCAL) {
+        split_work(p, n);
         if (ubep::plan_dispatch(p, mode, buf->max_smem, &pl) != 0) {
             if (buf->cfg.pipeline == UBEP_PIPELINE_LOCAL) return UBEP_ERR_ARG;
             mode = UBEP_PIPELINE_FUSED;   // table too large for shared memory
-            p.parts = 1;
-            p.nchunks = n;
-            p.grid = n;
         }
     }
-    // slices that are long enough are handed out in blocks so that faster SMs can take over the tail of slower ones
-    if (mode != UBEP_PIPELINE_LOCAL) p.steal = T >= kStealMinTokensPerChunk * p.nchunks ? 1 : 0;
-    // With token stealing the count group is not used unless asked for: measured equal at top-8 and slower at
-    // top-4 (16384 tokens: 161 against 174 us) -- every hand-out is a round trip that idle quantising warps do not hide.
-    if (p.steal && buf->count_warps < 0) p.count_warps = 0;
-    if (mode != UBEP_PIPELINE_LOCAL && ubep::plan_dispatch(p, mode, buf->max_smem, &pl) != 0) return UBEP_ERR_ARG;
+    if (mode == UBEP_PIPELINE_FUSED || mode == UBEP_PIPELINE_PHASED) {
+        p.parts = 1;
+        p.nchunks = n;
+        p.grid = n;
+        // slices that are long enough are handed out in blocks so that faster SMs can take over the tail of slower ones
+        p.steal = T >= kStealMinTokensPerChunk * p.nchunks ? 1 : 0;
+        // With token stealing the count group is not used unless asked for: measured equal at top-8 and slower at
+        // top-4 (16384 tokens: 161 against 174 us) -- every hand-out is a round trip that idle quantising warps do not hide.
+        if (p.steal && buf->count_warps < 0) p.count_warps = 0;
+        if (ubep::plan_dispatch(p, mode, buf->max_smem, &pl) != 0) return UBEP_ERR_ARG;
+    }
     cudaError_t e = ubep::launch_dispatch(p, mode, pl, st, &launches);
     if (e != cudaSuccess) return cuda_fail(buf, e);
     g_launches += launches;

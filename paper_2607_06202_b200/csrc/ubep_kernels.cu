@@ -12,6 +12,7 @@
 //   layout_kernel<K, W>               counts only (ubep_get_dispatch_layout)
 #include <atomic>
 
+#include "ubep_cluster.cuh"
 #include "ubep_kernels.h"
 #include "ubep_layout.cuh"
 #include "ubep_quant.cuh"
@@ -105,6 +106,7 @@ struct Cta {
 // so the k copies of a row are issued side by side; for FP8 rows the warp only loads.
 template <int kMode, bool kFp8, bool kSteal>
 __device__ __forceinline__ void mover_warp(Cta& x) {
+    if (kMode == kModeCluster) cluster_arrive();   // (this warp counts nothing)
     if (kMode != kModeLocal) {
         // The epoch: one acquire load and one ticket, two round trips to L2.  This warp has nothing
         // urgent to do yet, so it fetches it while the layout group already stages the routing table.
@@ -223,7 +225,7 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
     // meanwhile fills the memory system's queues in front of them.  Three rows start the copies, the
     // rest follows once the movers are released.  (Not with stealing: there every block of rows costs a
     // claim, a round trip each, and those are best paid while the layout runs.)
-    const int early = (kMode == kModeLocal || kSteal) ? kMaxStages : 3;
+    const int early = (kMode == kModeLocal || kMode == kModeCluster || kSteal) ? kMaxStages : 3;
     if (!kFp8) {
         // loads run (stages - 3) rows ahead; up to 3 rows' stores stay in flight
         int tl = 0;
@@ -242,6 +244,19 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
             }
             local_stage_and_rank_maps(p, ids_sm, rm, rm.groups, 0, kWarps, lane);
             group_sync(2, kThreads);
+        } else if (kMode == kModeCluster) {
+            // Two rows at once, the rest of the ring when the counts have been exchanged: a ring-full of rows per
+            // CTA in flight slows the reads of the other CTAs' shared memory down (by 2 us at 1537 tokens).
+            if (kSteal) {
+                while (head < 2 && next_token(tl, false) == 1) issue_item(tl);
+            } else {
+                issue_first(max(min(2, min(stages - 3, ntok)), 0));
+            }
+            issued = head;
+            cluster_wait();
+            cluster_arrive();    // (this warp reads nothing of the others)
+            ok = mbar_wait(x.staged_bar, 0, abortp);
+            ok = __all_sync(0xffffffffu, ok);
         } else if (kMode == kModeLocal) {
             ok = mbar_wait(x.staged_bar, 0, abortp);
             ok = __all_sync(0xffffffffu, ok);
@@ -255,7 +270,7 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
         issued = head;
         ok = mbar_wait(&ready_bar, 0, abortp) && !*abortp;  // no rows without a layout
         ok = __all_sync(0xffffffffu, ok);
-        if (kMode != kModeLocal && ok) {   // the rest of the ring
+        if (kMode != kModeLocal && kMode != kModeCluster && ok) {   // the rest of the ring
             if (kSteal) {
                 while (head < stages - 3 && next_token(tl, false) == 1) issue_item(tl);
             } else {
@@ -323,6 +338,15 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
             const RankMaps rm{bmaps.bm, bmaps.mask_t, (p.R + 31) / 32, ((p.R + 31) / 32) * 32, (p.T + 31) / 32};
             local_stage_and_rank_maps(p, ids_sm, rm, rm.groups, 0, kWarps, lane);   // the table first, the rows after it
             group_sync(2, kThreads);
+        } else if (kMode == kModeCluster) {
+            if (!kSteal) {   // (see above)
+                for (int n = 0; n < min(2, min(stages, ntok)); ++n) issue_item(n);
+                issued = head;
+            }
+            cluster_wait();
+            cluster_arrive();
+            ok = mbar_wait(x.staged_bar, 0, abortp);
+            ok = __all_sync(0xffffffffu, ok);
         } else if (kMode == kModeLocal || x.beside) {
             // the routing table first: it is the one load the layout waits for
             ok = mbar_wait(x.staged_bar, 0, abortp);
@@ -412,6 +436,191 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
     if (lane == 0) trace(p, c, kTrStored);
 }
 
+// ------------------------------------------------------------- layout by clusters
+// (see ubep_cluster.cuh)  Every CTA counts its slice of the routing table and its own tokens; after a barrier of
+// the cluster it reads, per bin, what the others counted and has all totals and the rows before its own tokens.
+// Ends with the movers released.  FP8 rows: once the counting is done the warps behind the first five quantise.
+constexpr int kClusterCountWarps = 5;
+template <bool kFp8, bool kSteal>
+__device__ __forceinline__ void cluster_layout(Cta& x) {
+    UBEP_CTA_LOCALS(x, !kFp8);
+    int* tot = hist;
+    int* base = hist + p.B;    // rows before the CTA's tokens in the bin's segment
+    int* eo = hist + 2 * p.B;
+    int* row_sm = reinterpret_cast<int*>(w_sm);
+    unsigned* cnt = reinterpret_cast<unsigned*>(smem + pl.off_cnt);   // per bin: counts of the slice,
+    unsigned* own = cnt + p.B + 1;                                    // counts of the own tokens
+    const int cs = p.cluster, me = (int)cluster_ctarank(), c0 = c - me;
+    const int first = (int)chunk_begin(c0 / p.parts, p.T, p.nchunks);   // first token of the cluster
+    // tokens per rank are an output of their own with one row per (token, expert); the first cluster counts them
+    const bool ranks = p.dedup || c0 == 0;
+    const int nb = p.E + (ranks ? p.R : 0);
+    const int per = (p.T + cs - 1) / cs;
+    const int lo = min(p.T, me * per), hi = min(p.T, lo + per);
+    constexpr int an = kThreads - 32;   // all warps but the mover count
+    // (the own tokens from the last thread on: the first ones may have a token more to count)
+    const bool twice = stage_own(p, t0, t1, ids_sm, bmaps.bm, bmaps.bp, own, an - 1 - gtid, an);
+    count_tokens(count_args(p), lo, hi, first, ranks, cnt, gtid, an);
+    if (p.ordered)
+        for (int r = gtid; r < p.R; r += an) order_sm[r] = __ldg(p.order_pos + r);
+    if (group_or(1, an, twice)) {
+        local_clean_own_duplicates(p, 0, ntok, ids_sm, gtid, an);
+        group_sync(1, an);
+    }
+    if (gtid == 0) trace(p, c, kTrCounted);
+    cluster_arrive();          // this CTA's counts are there
+    cluster_wait();            // ... and so are the others'
+    if (kFp8 && gw >= nw) {    // FP8 rows: the warps behind the count group go on to quantise
+        cluster_arrive();
+        return;
+    }
+    if (gtid == 0) trace(p, c, kTrHistSeen);
+    constexpr int bid = kFp8 ? 4 : 1;   // barrier of the count group
+#pragma unroll 1
+    for (int b = gtid; b < nb; b += gn) {
+        unsigned below = 0u, all = 0u;
+#pragma unroll 2
+        for (int q = 0; q < cs; ++q) {
+            const unsigned v = ld_cluster(cnt + b, (unsigned)q);
+            below += v & 0xffffu;
+            all += v >> 16;
+            // its own tokens come earlier than this CTA's (the column parts of a chunk count them once)
+            if (c0 + q < c - part && ((c0 + q) & (p.parts - 1)) == 0) below += ld_cluster(own + b, (unsigned)q);
+        }
+        tot[b] = (int)all;
+        base[b] = (int)below;
+    }
+    cluster_arrive();   // the others' counts have been read: they may leave
+    group_sync(bid, gn);
+    if (gtid == 0) mbar_arrive(x.staged_bar);   // the mover may fetch the rest of the ring's rows now
+#pragma unroll 1
+    for (int e = gtid; e < p.E; e += gn) {
+        int o = 0;
+        for (int q = (e / p.L) * p.L; q < e; ++q) o += tot[q];
+        eo[e] = o;
+        base[e] += o;
+    }
+    group_sync(bid, gn);
+    if (gtid == 0) trace(p, c, kTrScanSeen);
+    bool full = false;
+#pragma unroll 1
+    for (int li = gtid; li < ntok * p.k; li += gn) {
+        const int tl = li / p.k, packed = ids_sm[li];
+        const bool have = packed >= 0;
+        const int r = have ? slot_rank(packed) : 0;
+        bool first_of_rank = have;
+        int bin = have ? slot_expert(packed) : 0;
+        if (p.dedup) {
+            for (int i = tl * p.k; i < li; ++i) first_of_rank = first_of_rank && slot_rank(ids_sm[i]) != r;   // (-1 >> 16 is no rank)
+            bin = p.E + r;
+        }
+        const int row = base[bin] + own_below(bmaps, bin, tl);
+        const bool fits = row < p.cap, send = first_of_rank && fits;
+        full = full || (have && !fits);
+        if (send && !kSteal) atomicAdd(&arr[r], 1);   // rows this CTA will copy to rank r (stealing: counted at copy time)
+        pos_raw[li] = send ? r * p.cap + row : -1;
+        row_sm[li] = have ? row : -1;
+        if (p.ordered) key[li] = send ? rotated_key(order_sm, r, c, p.R) : p.R;
+    }
+    if (full) report(p.status, kErrCapacity);
+    group_sync(bid, gn);
+    if (gtid == 0) trace(p, c, kTrFinalized);
+    if (p.ordered) {   // a destination table is set: the copies of a token in its order (else pos_raw is pos)
+        order_destinations(p, pos_raw, key, pos, ntok * p.k, gtid, gn);
+        group_sync(bid, gn);
+    }
+    if (gtid == 0) {
+        mbar_arrive(&ready_bar);
+        trace(p, c, kTrReady);
+    }
+    if (kSteal) {
+        // this chunk's destinations, for CTAs that run out of work and take over some of its tokens
+        for (int i = gtid; i < ntok * p.k; i += gn) p.copy_pos[(size_t)t0 * p.k + i] = pos[i];
+        if (gtid == 0) (void)mbar_wait(x.epoch_bar, 0, abortp);
+        group_sync(bid, gn);
+        if (gtid == 0) st_release(p.pos_flag + ch, *reinterpret_cast<volatile unsigned*>(x.epoch_late));
+    }
+}
+
+// What nobody inside the kernel waits for: the metadata of the own tokens, the totals (one CTA) and the counts and
+// offsets of the source ranks whose tokens begin among the CTA's own.  Tokens of such a rank beyond the CTA's own
+// are counted from the table.
+template <bool kFp8>
+__device__ __forceinline__ void cluster_duty(Cta& x, int dtid, int dn, int bar) {
+    UBEP_CTA_LOCALS(x, !kFp8);
+    const int* tot = hist;
+    const int* base = hist + p.B;
+    const int* eo = hist + 2 * p.B;
+    const int* row_sm = reinterpret_cast<const int*>(w_sm);
+    unsigned* cnt = reinterpret_cast<unsigned*>(smem + pl.off_cnt) + 2 * (p.B + 1);   // (those in front are read by the cluster)
+    if (c == 0) write_totals(p, tot, eo, dtid, dn);
+    if (part != 0 || ntok == 0) return;
+#pragma unroll 1
+    for (int li = dtid; li < ntok * p.k; li += dn) {
+        const int tl = li / p.k, packed = ids_sm[li], row = row_sm[li], where = pos_raw[li];
+        const size_t i = (size_t)t0 * p.k + li;
+        const bool have = packed >= 0;
+        const int r = have ? slot_rank(packed) : 0;
+        p.slot_row[i] = row;
+        p.slot_pos[i] = have && row < p.cap ? r * p.cap + row : -1;
+        if (p.dedup && have) {
+            const int e = slot_expert(packed), at = base[e] + own_below(bmaps, e, tl);
+            if (at < p.er_cap) p.expert_rows[(size_t)r * p.er_cap + at] = row;
+            else report(p.status, kErrCapacity);
+        }
+        if (where < 0) continue;
+        p.recv_src_idx[where] = t0 + tl;
+        if (!p.dedup) {
+            p.recv_weight[where] = __ldg(p.topk_w + i);
+        } else if ((p.k & 3) == 0) {   // rows of the two arrays start on 16-byte boundaries: four slots per store
+#pragma unroll 1
+            for (int j = 0; j < p.k; j += 4) {
+                const float4 w = __ldg(reinterpret_cast<const float4*>(p.topk_w + (size_t)(t0 + tl) * p.k + j));
+                const float wv[4] = {w.x, w.y, w.z, w.w};
+                int e4[4];
+                float w4[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int v = ids_sm[tl * p.k + j + u];
+                    const bool here = v >= 0 && slot_rank(v) == r;
+                    e4[u] = here ? slot_expert(v) - r * p.L : -1;
+                    w4[u] = here ? wv[u] : 0.0f;
+                }
+                *reinterpret_cast<int4*>(p.recv_topk_idx + (size_t)where * p.k + j) = make_int4(e4[0], e4[1], e4[2], e4[3]);
+                *reinterpret_cast<float4*>(p.recv_topk_w + (size_t)where * p.k + j) = make_float4(w4[0], w4[1], w4[2], w4[3]);
+            }
+        } else {
+#pragma unroll 1
+            for (int j = 0; j < p.k; ++j) {
+                const int v = ids_sm[tl * p.k + j];
+                const bool here = v >= 0 && slot_rank(v) == r;
+                p.recv_topk_idx[(size_t)where * p.k + j] = here ? slot_expert(v) - r * p.L : -1;
+                p.recv_topk_w[(size_t)where * p.k + j] = here ? __ldg(p.topk_w + (size_t)(t0 + tl) * p.k + j) : 0.0f;
+            }
+        }
+    }
+    const int s_lo = (int)(((int64_t)t0 * p.S + p.T - 1) / p.T);  // smallest s with src_begin(s) >= t0
+#pragma unroll 1
+    for (int s = s_lo; s < p.S; ++s) {
+        const int b0 = src_begin(s, p.T, p.S);
+        if (b0 >= t1) break;
+        const int b1 = src_begin(s + 1, p.T, p.S);
+        const bool beyond = b1 > t1;   // (only the last of them)
+        if (beyond) {
+            for (int e = dtid; e < p.E; e += dn) cnt[e] = 0u;
+            group_sync(bar, dn);
+            count_tokens(count_args(p), t1, b1, 0, false, cnt, dtid, dn);
+            group_sync(bar, dn);
+        }
+#pragma unroll 1
+        for (int e = dtid; e < p.E; e += dn) {
+            const int before = own_below(bmaps, e, b0 - t0);
+            p.cnt[(size_t)s * p.E + e] = own_below(bmaps, e, min(b1, t1) - t0) - before + (beyond ? (int)(cnt[e] >> 16) : 0);
+            p.src_offset[(size_t)s * p.E + e] = base[e] + before;
+        }
+    }
+}
+
 // ---------------------------------------------------------------------- layout group
 // Warps 1..15: TokenCnt, CalCumSum (by exchange or alone), slot -> row assignment; releases
 // the movers and then writes what nobody inside the kernel waits for.  Returns 1, 0 if a wait ran
@@ -423,8 +632,8 @@ __device__ __forceinline__ int layout_group(Cta& x) {
     const int* ids = ids_sm;  // staged slots of this CTA's tokens
     // Small global reads whose values are needed only after the first barriers: issue the
     // loads now (first trip of each loop), store to shared memory after the ids are staged.
-    const int order_r = gtid < p.R ? __ldg(p.order_pos + gtid) : 0;
-    const bool stage_w = !(kMode == kModeLocal && p.local_fast);
+    const int order_r = kMode != kModeCluster && gtid < p.R ? __ldg(p.order_pos + gtid) : 0;
+    const bool stage_w = kMode != kModeCluster && !(kMode == kModeLocal && p.local_fast);
     const float w_first = (stage_w && gtid < ntok * p.k) ? __ldg(p.topk_w + (size_t)t0 * p.k + gtid) : 0.0f;
     auto stage_small = [&](int n) {   // by n threads
         if (gtid < p.R) order_sm[gtid] = order_r;
@@ -554,6 +763,13 @@ __device__ __forceinline__ int layout_group(Cta& x) {
         if (c == 0) write_totals(p, tot, eo, gtid, gn);
         if (part == 0)
             for (int s = ch; s < p.S; s += p.nchunks) write_source_from_maps(p, s, bmaps, eo, gtid, gn);   // source ranks this CTA reports
+    } else if (kMode == kModeCluster) {
+        cluster_layout<kFp8, kSteal>(x);
+        if (kFp8 && gw >= nw) return 2;   // off to quantise
+        if (kFp8 && gw == 0) return 1;    // off to issue the copies
+        // the others write what nobody waits for
+        cluster_duty<kFp8>(x, gtid - (kFp8 ? 32 : 0), gn - (kFp8 ? 32 : 0), kFp8 ? 3 : 1);
+        return kFp8 ? 3 : 1;
     } else {
         // FP8 rows with a count group: TokenCnt itself -- staging the ids, the bitmaps, publishing the
         // chunk's counts -- is pure computation and is done by all 15 warps; then the warps behind the
@@ -840,8 +1056,8 @@ __global__ void __launch_bounds__(kThreads, 1) dispatch_kernel(const Params p, c
     const int part = c % p.parts, ch = c / p.parts;
     const int t0 = (int)chunk_begin(ch, p.T, p.nchunks), t1 = (int)chunk_begin(ch + 1, p.T, p.nchunks);
     const int stages = pl.stages;
-    const bool beside = kFp8 && kMode != kModeLocal && p.count_warps > 0;
-    const int nw = beside ? p.count_warps : kWarps - 1;      // layout group: warps 1 .. nw
+    const bool beside = kFp8 && (kMode == kModeCluster || (kMode != kModeLocal && p.count_warps > 0));
+    const int nw = kFp8 && kMode == kModeCluster ? kClusterCountWarps : beside ? p.count_warps : kWarps - 1;      // layout group: warps 1 .. nw
     const int qwarp0 = beside ? nw + 1 : 2;                    // FP8: warps qwarp0 .. qwarp0 + nq - 1 quantise
     // (flag-free kernel with rank-level rows: a CTA has few rows, and the warps that do not quantise write
     // the expert-level outputs meanwhile)
@@ -867,7 +1083,13 @@ __global__ void __launch_bounds__(kThreads, 1) dispatch_kernel(const Params p, c
         mbar_fence_init();
     }
     for (int r = tid; r < p.R; r += kThreads) arr[r] = 0;
-    if (kMode == kModeLocal) {
+    if (kMode == kModeCluster) {
+        unsigned* cnt = reinterpret_cast<unsigned*>(smem + pl.off_cnt);
+        unsigned* bm = reinterpret_cast<unsigned*>(smem + pl.off_bm);
+        for (int b = tid; b < 2 * (p.B + 1); b += kThreads) cnt[b] = 0u;
+        for (int b = tid; b < pl.map_groups * pl.map_bp; b += kThreads) bm[b] = 0u;
+    }
+    if (kMode == kModeLocal || kMode == kModeCluster) {
         // The routing table is the first thing every CTA of the flag-free kernel needs, and it comes cold
         // from HBM.  A prefetch into L2 reads no value, so it may run ahead of the wait below: L2 is where
         // an earlier kernel's stores to the table land too, so the line cannot go stale.
@@ -880,7 +1102,7 @@ __global__ void __launch_bounds__(kThreads, 1) dispatch_kernel(const Params p, c
         const unsigned piece = (unsigned)(p.H * 2 / p.parts);
         const int lines = (int)((piece + 127u) / 128u);
         const char* xs = reinterpret_cast<const char*>(p.x) + (size_t)t0 * p.H * 2 + (size_t)part * piece;
-        for (int i = tid; i < (t1 - t0) * lines; i += kThreads) {
+        for (int i = tid; kMode == kModeLocal && i < (t1 - t0) * lines; i += kThreads) {
             const int tl = i / lines, l = i - tl * lines;
             asm volatile("prefetch.global.L2 [%0];" ::"l"(xs + (size_t)tl * p.H * 2 + (size_t)l * 128));
         }
@@ -926,6 +1148,7 @@ __global__ void __launch_bounds__(kThreads, 1) dispatch_kernel(const Params p, c
             else if (!beside && x.warp - 2 < nq) fp8_quantiser<kSteal>(x, x.warp - 2);
         }
     }
+    if (kMode == kModeCluster) cluster_wait();   // the others have read what this CTA counted
     __syncthreads();
     const unsigned half = epoch_sm & 1u;
     if (abort_flag) {
@@ -1160,9 +1383,9 @@ int plan_dispatch(const Params& p, int mode, int max_smem, SmemPlan* out) {
     const int chunk_slots = chunk_tokens * p.k;
     const int map_tokens = mode == kModeLocal ? p.T : chunk_tokens;   // tokens the bitmaps cover
     const int64_t ids_ints = (int64_t)map_tokens * p.k;
-    int hist_ints = mode == kModeLocal ? 2 * p.B + p.E : 2 * p.B;
+    int hist_ints = mode == kModeLocal || mode == kModeCluster ? 2 * p.B + p.E : 2 * p.B;
     if (hist_ints < 64) hist_ints = 64;   // the per-rank duty of the flag-free kernel keeps 2 x 32 ints here
-    pl.map_groups = (map_tokens + 31) / 32;
+    pl.map_groups = map_tokens / 32 + (mode == kModeCluster || map_tokens % 32 != 0 ? 1 : 0);   // (own_below may look at one more)
     pl.map_wb = (p.B + 31) / 32;
     pl.map_bp = pl.map_wb * 32;
     pl.stage_bytes = round_up_i(p.H * 2 / p.parts, 128);
@@ -1170,11 +1393,13 @@ int plan_dispatch(const Params& p, int mode, int max_smem, SmemPlan* out) {
     const int64_t mask_ints = (int64_t)pl.map_groups * 32;
     const int64_t bm_ints = (int64_t)pl.map_groups * pl.map_bp;
     const int item_ints = (kMaxStages + kMaxOutStages) * (p.k + 1);
-    const int64_t ints = ids_ints + mask_ints + bm_ints + 4 * (int64_t)chunk_slots + hist_ints + 2 * p.R + item_ints;
+    const int64_t cnt_ints = mode == kModeCluster ? 3 * ((int64_t)p.B + 1) : 0;
+    const int64_t ints = ids_ints + mask_ints + bm_ints + 4 * (int64_t)chunk_slots + hist_ints + 2 * p.R + item_ints +
+                         cnt_ints;
     const int64_t fixed = ints * 4 + 128 + 1536;  // 1.5 KB: static shared memory
     // no more stages than rows this CTA will ever hold at once
     const int want = chunk_tokens + 3 < 4 ? 4 : chunk_tokens + 3;
-    const bool beside = p.payload && mode != kModeLocal && p.count_warps > 0;
+    const bool beside = p.payload && (mode == kModeCluster || (mode != kModeLocal && p.count_warps > 0));
     if (!beside) {
         // the quantising warps (if any) start after the layout: a deep input ring that the loader fills
         // meanwhile, a short ring of quantised rows
@@ -1212,6 +1437,7 @@ int plan_dispatch(const Params& p, int mode, int max_smem, SmemPlan* out) {
     pl.off_arr = at; at += p.R * 4;
     pl.off_order = at; at += p.R * 4;
     pl.off_item = at; at += item_ints * 4;
+    pl.off_cnt = at; at += (int)cnt_ints * 4;
     pl.total = round_up_i(at, 128);
     *out = pl;
     return 0;
@@ -1225,13 +1451,13 @@ int plan_dispatch(const Params& p, int mode, int max_smem, SmemPlan* out) {
 // when every CTA has a place.  Such a kernel is not launched ahead of its predecessor's end.
 template <typename... KArgs, typename... Args>
 static cudaError_t launch_overlapped(void (*kern)(KArgs...), int grid, int block, size_t smem, cudaStream_t st,
-                                     bool together, Args... args) {
+                                     bool together, int cluster, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     if (together) {
         attr[0].id = cudaLaunchAttributeCooperative;
         attr[0].val.cooperative = 1;
@@ -1241,6 +1467,12 @@ static cudaError_t launch_overlapped(void (*kern)(KArgs...), int grid, int block
     }
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    if (cluster > 1) {
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = (unsigned)cluster;
+        attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+        cfg.numAttrs = 2;
+    }
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
@@ -1260,12 +1492,18 @@ static cudaError_t allow_dynamic_smem(const void* kern, int bytes, std::atomic<i
 }
 
 template <int kMode, bool kFp8, bool kSteal>
+static cudaError_t allow_dispatch_smem(int bytes) {
+    static std::atomic<int> granted[kAttrDevices];
+    return allow_dynamic_smem(reinterpret_cast<const void*>(dispatch_kernel<kMode, kFp8, kSteal>), bytes, granted);
+}
+
+template <int kMode, bool kFp8, bool kSteal>
 static cudaError_t launch_dispatch_s(const Params& p, const SmemPlan& pl, cudaStream_t st) {
     auto kern = dispatch_kernel<kMode, kFp8, kSteal>;
-    static std::atomic<int> granted[kAttrDevices];
-    cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void*>(kern), pl.total, granted);
+    cudaError_t e = allow_dispatch_smem<kMode, kFp8, kSteal>(pl.total);
     if (e != cudaSuccess) return e;
-    return launch_overlapped(kern, p.grid, kThreads, (size_t)pl.total, st, kMode == kModeFused, p, pl);
+    return launch_overlapped(kern, p.grid, kThreads, (size_t)pl.total, st, kMode == kModeFused,
+                             kMode == kModeCluster ? p.cluster : 1, p, pl);
 }
 
 template <int kMode, bool kFp8>
@@ -1288,6 +1526,38 @@ cudaError_t launch_count_scan(const Params& p, const SmemPlan& pl, cudaStream_t 
     return cudaGetLastError();
 }
 
+// CTAs of the dispatch kernel, one per SM, that can run at once in clusters of `cluster` on the current device (SMs are
+// grouped, and a group's size need not be a multiple of the cluster's: on a B200 148, 132, 120 for 2, 4, 8).
+int cluster_ctas(int cluster, int max_smem) {
+    static std::atomic<int> known[kAttrDevices][4];
+    const int slot = cluster == 2 ? 1 : cluster == 4 ? 2 : cluster == 8 ? 3 : 0;
+    int dev = 0;
+    if (slot == 0 || cudaGetDevice(&dev) != cudaSuccess) return 0;
+    const bool cached = dev >= 0 && dev < kAttrDevices;
+    if (cached) {
+        const int v = known[dev][slot].load(std::memory_order_relaxed);
+        if (v) return v - 1;
+    }
+    const int smem = max_smem - 2048;   // (more than half of an SM's: one CTA per SM)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)cluster);
+    cfg.blockDim = dim3((unsigned)kThreads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)cluster;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (allow_dispatch_smem<kModeCluster, false, false>(smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, reinterpret_cast<const void*>(dispatch_kernel<kModeCluster, false, false>), &cfg) != cudaSuccess)
+        n = 0;
+    (void)cudaGetLastError();
+    if (cached) known[dev][slot].store(n * cluster + 1, std::memory_order_relaxed);
+    return n * cluster;
+}
+
 cudaError_t launch_dispatch(const Params& p, int mode, const SmemPlan& pl, cudaStream_t st, int* launches) {
     cudaError_t e;
     *launches = 1;
@@ -1297,6 +1567,9 @@ cudaError_t launch_dispatch(const Params& p, int mode, const SmemPlan& pl, cudaS
         return p.payload ? launch_dispatch_t<kModePhased, true>(p, pl, st)
                          : launch_dispatch_t<kModePhased, false>(p, pl, st);
     }
+    if (mode == kModeCluster)
+        return p.payload ? launch_dispatch_t<kModeCluster, true>(p, pl, st)
+                         : launch_dispatch_t<kModeCluster, false>(p, pl, st);
     if (mode == kModeLocal)
         return p.payload ? launch_dispatch_t<kModeLocal, true>(p, pl, st)
                          : launch_dispatch_t<kModeLocal, false>(p, pl, st);
@@ -1307,7 +1580,7 @@ cudaError_t launch_dispatch(const Params& p, int mode, const SmemPlan& pl, cudaS
 template <int K>
 static cudaError_t launch_combine_k(bool ahead, int g, cudaStream_t st, const uint16_t* y, const int32_t* slot_pos,
                                     const float* topk_w, int T, int H, int k, uint16_t* out) {
-    if (ahead) return launch_overlapped(combine_kernel<K>, g, 256, 0, st, false, y, slot_pos, topk_w, T, H, k, out);
+    if (ahead) return launch_overlapped(combine_kernel<K>, g, 256, 0, st, false, 1, y, slot_pos, topk_w, T, H, k, out);
     combine_kernel<K><<<g, 256, 0, st>>>(y, slot_pos, topk_w, T, H, k, out);
     return cudaGetLastError();
 }
@@ -1340,7 +1613,7 @@ __global__ void __launch_bounds__(32) empty_kernel(int) {
 }
 
 cudaError_t launch_empty(int num_sms, bool ahead, cudaStream_t st) {
-    if (ahead) return launch_overlapped(empty_kernel, num_sms, 32, 0, st, false, 0);
+    if (ahead) return launch_overlapped(empty_kernel, num_sms, 32, 0, st, false, 1, 0);
     empty_kernel<<<num_sms, 32, 0, st>>>(0);
     return cudaGetLastError();
 }
@@ -1354,7 +1627,7 @@ cudaError_t launch_layout(const Params& p, int32_t* num_tokens_per_rank, int32_t
     if (blocks < 1) blocks = 1;
     const size_t smem = sizeof(int) * (size_t)p.B;
     auto go = [&](auto kern) {
-        return launch_overlapped(kern, (int)blocks, kLayoutThreads, smem, st, false, p, num_tokens_per_rank,
+        return launch_overlapped(kern, (int)blocks, kLayoutThreads, smem, st, false, 1, p, num_tokens_per_rank,
                                  num_tokens_per_expert, is_token_in_rank, acc, ticket);
     };
     if (p.R > 32 * kLayoutMaskWords) return go(layout_kernel<0, 0>);

@@ -1,0 +1,71 @@
+"""AUTO where the layout is computed by thread-block clusters: token counts at the edges of the slices, groups of
+32 tokens and chunks (fewer tokens than CTAs, than ranks, than a cluster's slices; the cluster sizes' boundaries;
+token stealing), rank counts, slots per token, column parts, source ranks whose tokens span many CTAs or
+share one, few CTAs, an expert named twice.  Dispatch bit by bit against the oracle, combine within its tolerance."""
+import numpy as np
+import pytest
+
+from paper_2607_06202_b200 import binding as B
+from paper_2607_06202_b200 import workload as W
+from tests import harness as Hn
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(cfg, empty=0.0, **kw):
+    wl = W.make_workload(cfg)
+    if empty:
+        wl = W.with_empty_slots(wl, empty, seed=cfg.seed + 1)
+    Hn.run_case(wl, threads=8, **kw)
+
+
+@pytest.mark.parametrize("payload,dedup", [(0, 0), (1, 0), (0, 1), (1, 1)])
+@pytest.mark.parametrize("T", [1, 31, 65, 300, 2049, 4096, 4097, 8192])
+def test_token_counts(T, payload, dedup):
+    # (L = 32 experts per rank keeps the one-row-per-rank cases off the rank-level fast path)
+    _run(W.Config("t", T=T, H=256, E=128, R=4, k=8, payload=payload, dedup=dedup, seed=T, num_src_ranks=7))
+
+
+@pytest.mark.parametrize("E,R,k", [(1, 1, 1), (31, 1, 3), (160, 5, 8), (161, 7, 5), (288, 72, 8), (289, 17, 8),
+                                   (512, 128, 8), (512, 2, 12), (256, 64, 16), (513, 27, 8), (258, 129, 8)])
+@pytest.mark.parametrize("dedup", [0, 1])
+def test_bins(E, R, k, dedup):
+    _run(W.Config("b", T=777, H=128, E=E, R=R, k=k, dedup=dedup, seed=E + R), empty=0.1)
+    _run(W.Config("b", T=4097, H=128, E=E, R=R, k=k, dedup=dedup, payload=1, seed=E + R))
+
+
+@pytest.mark.parametrize("S", [1, 2, 40, 900])
+def test_source_ranks(S):
+    for T in (200, 1500):
+        _run(W.Config("s", T=T, H=128, E=64, R=8, k=4, seed=S + T, num_src_ranks=S))
+
+
+@pytest.mark.parametrize("num_ctas", [1, 2, 3, 5, 34])
+def test_few_ctas(num_ctas):
+    _run(W.Config("c", T=400, H=128, E=64, R=8, k=4, seed=num_ctas), num_ctas=num_ctas)
+
+
+@pytest.mark.parametrize("payload", [0, 1])
+def test_replicas_and_wide_rows(payload):
+    cfg = W.Config("r", T=1000, H=7168, E=72, R=8, k=8, payload=payload, seed=5, E_logical=64)
+    _run(cfg, dest_order=np.arange(8)[::-1].copy())
+    for T in (20, 40, 70):   # eight, two and two column parts
+        _run(W.Config("p", T=T, H=7168, E=256, R=8, k=8, payload=payload, seed=6))
+
+
+@pytest.mark.parametrize("k", [4, 7, 8, 11])
+@pytest.mark.parametrize("dedup", [0, 1])
+def test_an_expert_named_twice(k, dedup):
+    cfg = W.Config("d", T=1200, H=128, E=128, R=4, k=k, dedup=dedup, seed=k)
+    wl = W.make_workload(cfg)
+    clean = wl.topk_idx.copy()
+    clean[::3, k - 1] = -1
+    wl_clean = W.Workload(cfg, wl.x, clean, wl.topk_w)
+    _, lay, cap, recv = Hn.oracle_reference(wl_clean)
+    buf = Hn.make_buffer(cfg, cap)
+    x, _, w, _, _ = Hn.device_inputs(wl)
+    dup = wl.topk_idx.copy()
+    dup[::3, k - 1] = dup[::3, 0]
+    buf.dispatch(x, Hn.to_dev(dup), w)
+    assert buf.status() == B.UBEP_ERR_BAD_INDEX
+    Hn.check_dispatch(buf, wl_clean, lay, cap, recv)
