@@ -769,6 +769,7 @@ __device__ __forceinline__ int layout_group(Cta& x) {
         if (kFp8 && gw == 0) return 1;    // off to issue the copies
         // the others write what nobody waits for
         cluster_duty<kFp8>(x, gtid - (kFp8 ? 32 : 0), gn - (kFp8 ? 32 : 0), kFp8 ? 3 : 1);
+        if (gtid == (kFp8 ? 32 : 0)) trace(p, c, kTrScanned);   // deferred outputs written
         return kFp8 ? 3 : 1;
     } else {
         // FP8 rows with a count group: TokenCnt itself -- staging the ids, the bitmaps, publishing the
