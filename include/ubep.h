@@ -444,14 +444,14 @@ int ubep_debug_trace(ubep_buffer_t *buf, int32_t enable);
 /*
  * Warp-role split of the FP8 dispatch kernel (the paper's core-allocation question, Sec. 3.2
  * "most cores send tokens, a few compute token counts", and App. A / C: how many cores count and
- * how many send).  Of the CTA's 16 warps one loads rows and one issues the stores.
+ * how many send).  Of the CTA's 16 warps one loads rows and, for long rows, one issues the stores.
  *
- * ubep_debug_set_count_warps: n warps (the store issuer among them) form the count group that
+ * ubep_debug_set_count_warps: n warps (the store issuer of long rows among them) form the count group that
  * computes the layout -- TokenCnt, the flag exchange, CalCumSum, row assignment -- while the
  * remaining 15 - n warps already quantise the rows the loader has fetched into a ring of
  * quantised rows that waits for the layout (1 <= n <= 13).  TokenCnt itself is done by all 15
  * warps first; the count group is what goes on through the flag exchange.  n = 0: all 15 warps
- * compute the layout and 14 of them quantise afterwards.  n = -1 (default): 8, or 0 when slices
+ * compute the layout and up to 14 of them quantise afterwards.  n = -1 (default): 8, or 0 when slices
  * are long enough for token stealing.  Applies to the PHASED and FUSED schedules; the flag-free
  * LOCAL schedule, whose layout waits for nobody, always runs as n = 0.
  * ubep_debug_set_quant_warps: at most n warps quantise (1 <= n <= 14, default 14), the rest idle.

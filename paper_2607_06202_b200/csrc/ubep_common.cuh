@@ -16,14 +16,15 @@ constexpr int kThreads = 512;          // threads per persistent CTA
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxTopk = 32;
 constexpr int kMaxChunks = 320;        // scan keeps chunks/32 values per lane in registers
-constexpr int kMaxStages = 16;         // rows in the shared-memory ring
+constexpr int kMaxStages = 40;         // rows in the shared-memory ring
+constexpr int kStealStages = 16;       // ... with token stealing
 constexpr int kRankWordsHost = 4;      // the rank-level fast path handles up to 128 ranks
 constexpr int kStealBlock = 2;         // tokens handed out per claim
-constexpr int kOutStages = 4;          // FP8, quantising after the layout: quantised rows waiting for their stores
-constexpr int kMaxOutStages = 24;      // FP8, quantising beside the layout: at most this many quantised rows wait
-constexpr int kFastQuantWarps = 5;     // FP8 in the flag-free kernel with rank-level rows: quantising warps (measured per dispatch of
+constexpr int kOutStages = 4;          // FP8, long rows, quantising after the layout: quantised rows waiting for their stores
+constexpr int kMaxOutStages = 24;      // FP8, long rows, quantising beside the layout: at most this many quantised rows wait
+constexpr int kFastQuantWarps = 5;     // FP8, long rows, in the flag-free kernel with rank-level rows: quantising warps (measured per dispatch of
                                        // 512 / 1024 tokens: 15.5 / 24.3 us with 4, 15.5 / 25.3 with 6, 15.7 / 30.7 with 8, 18.0 / 38.2 with 10)
-constexpr int kStorePending = 3;       // FP8: rows whose bulk stores may still be reading shared memory
+constexpr int kStorePending = 3;       // FP8, long rows: rows whose bulk stores may still be reading shared memory
 constexpr int kTraceSlots = 16;        // per-CTA phase time stamps (optional tracing)
 constexpr int kModePhased = 1, kModeFused = 2, kModeLocal = 3, kModeCluster = 4;
 // Every wait in the kernels gives up after this many nanoseconds of wall time.
@@ -306,7 +307,10 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 // Where the dispatch kernel keeps things in dynamic shared memory (byte offsets).
 struct SmemPlan {
     int stages, stage_bytes;          // input row ring
-    int out_stages, out_stage_bytes;  // FP8: ring of quantised rows
+    int out_stages, out_stage_bytes;  // FP8: quantised rows in shared memory (long rows: a ring; short ones: two per team)
+    int q_long;                       // ... 1 = long rows
+    int q_warps, q_warp0;             // ... quantising warps, the first of them
+    int q_teams, q_team_warps;        // ... short rows: teams of them, warps per team
     int map_groups, map_wb, map_bp;   // bin bitmaps: 32-token groups, words of bins, padded bins
     int off_out, off_ids, off_mask, off_bm, off_pos, off_key, off_ord, off_w, off_hist, off_arr, off_order;
     int off_item;                     // per ring stage: where its token comes from, positions of stolen tokens

@@ -479,7 +479,8 @@ int ubep_dispatch(ubep_buffer_t* buf, const void* x, const int32_t* topk_idx, co
         // With token stealing the count group is not used unless asked for: measured equal at top-8 and slower at
         // top-4 (16384 tokens: 161 against 174 us) -- every hand-out is a round trip that idle quantising warps do not hide.
         if (p.steal && buf->count_warps < 0) p.count_warps = 0;
-        if (ubep::plan_dispatch(p, mode, buf->max_smem, &pl) != 0) return UBEP_ERR_ARG;
+        if (p.steal && ubep::plan_dispatch(p, mode, buf->max_smem, &pl) != 0) p.steal = 0;   // (rows too long for the ring it needs)
+        if (!p.steal && ubep::plan_dispatch(p, mode, buf->max_smem, &pl) != 0) return UBEP_ERR_ARG;
     }
     cudaError_t e = ubep::launch_dispatch(p, mode, pl, st, &launches);
     if (e != cudaSuccess) return cuda_fail(buf, e);

@@ -50,10 +50,8 @@ struct Cta {
     uint8_t* smem;
     uint64_t *full_bar, *empty_bar, *out_full, *out_empty, *ready_bar, *epoch_bar, *staged_bar;
     int* abort_flag;
-    int tid, lane, warp, c, part, ch, t0, t1, ntok, stages, nq;
+    int tid, lane, warp, c, part, ch, t0, t1, ntok, stages;
     int gn, nw;        // layout (count) group: warps 1 .. nw, gn = 32 * nw threads
-    int out_stages;    // FP8: depth of the ring of quantised rows
-    int qwarp0;        // FP8: first quantising warp (warps qwarp0 .. qwarp0 + nq - 1 quantise)
     bool beside;       // FP8: the quantising warps are not layout warps and run beside the layout
     int *ids_sm, *pos, *pos_raw, *key;
     float* w_sm;
@@ -81,7 +79,7 @@ struct Cta {
     [[maybe_unused]] volatile int* const abortp = (x).abort_flag;                                            \
     [[maybe_unused]] const int tid = (x).tid, lane = (x).lane, warp = (x).warp, c = (x).c;                   \
     [[maybe_unused]] const int part = (x).part, ch = (x).ch, t0 = (x).t0, t1 = (x).t1, ntok = (x).ntok;     \
-    [[maybe_unused]] const int stages = (x).stages, nq = (x).nq;                                             \
+    [[maybe_unused]] const int stages = (x).stages, nq = (x).pl.q_warps;                                       \
     [[maybe_unused]] int* const ids_sm = (x).ids_sm;                                                         \
     [[maybe_unused]] int* const pos = (x).pos;                                                               \
     [[maybe_unused]] int* const pos_raw = (x).pos_raw;                                                       \
@@ -98,7 +96,7 @@ struct Cta {
     /* layout group: warps 1 .. nw; a compile-time constant where it is always all 15 */                    \
     [[maybe_unused]] const int nw = (all15) ? kWarps - 1 : (x).nw;                                           \
     [[maybe_unused]] const int gn = nw * 32;                                                                 \
-    [[maybe_unused]] const int out_stages = (x).out_stages;                                                  \
+    [[maybe_unused]] const int out_stages = (x).pl.out_stages;                                               \
     [[maybe_unused]] const int gtid = (x).tid - 32, gw = (x).warp - 1
 
 // ------------------------------------------------------------------------ mover warp
@@ -186,7 +184,7 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
         return 1;
     };
     int* item_src = reinterpret_cast<int*>(smem + pl.off_item);           // [stages] (chunk << 16 | index), -1 = end
-    int* item_pos = item_src + kMaxStages + kMaxOutStages;                // [stages, k] destinations of stolen tokens
+    int* item_pos = item_src + kStealStages;                              // [stages, k] destinations of stolen tokens
     int head = 0, tail = 0;   // rows whose load was issued / whose copies were issued
     // load of the feeder's next token into ring stage head % stages
     auto issue_item = [&](int tl) {
@@ -227,7 +225,8 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
     // claim, a round trip each, and those are best paid while the layout runs.)
     const int early = (kMode == kModeLocal || kMode == kModeCluster || kSteal) ? kMaxStages : 3;
     if (!kFp8) {
-        // loads run (stages - 3) rows ahead; up to 3 rows' stores stay in flight
+        // loads run (stages - 3) rows ahead; up to 3 rows' stores stay in flight (all rows at once where they fit)
+        const int ahead = !kSteal && ntok <= stages ? ntok : stages - 3;
         int tl = 0;
         // Flag-free kernel: the routing table first, the rows after it.  The table is the one load the
         // whole layout waits for; the rows of 148 CTAs queued in front of it cost about a microsecond.
@@ -239,7 +238,7 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
             // queue in front of the one load the layout waits for: measured per layer 25.6 us with one or two
             // rows first, 25.9 with four or with none, 26.5 with the whole ring.)
             if (!kSteal) {
-                issue_first(max(min(2, min(stages - 3, ntok)), 0));
+                issue_first(max(min(2, min(ahead, ntok)), 0));
                 issued = head;
             }
             local_stage_and_rank_maps(p, ids_sm, rm, rm.groups, 0, kWarps, lane);
@@ -250,7 +249,7 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
             if (kSteal) {
                 while (head < 2 && next_token(tl, false) == 1) issue_item(tl);
             } else {
-                issue_first(max(min(2, min(stages - 3, ntok)), 0));
+                issue_first(max(min(2, min(ahead, ntok)), 0));
             }
             issued = head;
             cluster_wait();
@@ -262,26 +261,46 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
             ok = __all_sync(0xffffffffu, ok);
         }
         if (kSteal) {
-            while (head < min(stages - 3, early) && next_token(tl, false) == 1) issue_item(tl);
+            while (head < min(ahead, early) && next_token(tl, false) == 1) issue_item(tl);
         } else {
-            issue_first(max(min(min(min(stages - 3, early), ntok), 32) - head, 0));
-            while (head < min(min(stages - 3, early), ntok)) issue_item(head);
+            issue_first(max(min(min(min(ahead, early), ntok), 32) - head, 0));
+            while (head < min(min(ahead, early), ntok)) issue_item(head);
         }
         issued = head;
         ok = mbar_wait(&ready_bar, 0, abortp) && !*abortp;  // no rows without a layout
         ok = __all_sync(0xffffffffu, ok);
         if (kMode != kModeLocal && kMode != kModeCluster && ok) {   // the rest of the ring
             if (kSteal) {
-                while (head < stages - 3 && next_token(tl, false) == 1) issue_item(tl);
+                while (head < ahead && next_token(tl, false) == 1) issue_item(tl);
             } else {
-                while (head < min(stages - 3, ntok)) issue_item(head);
+                while (head < min(ahead, ntok)) issue_item(head);
             }
             issued = head;
         }
         if (!kSteal) {
             // the CTA's own rows, in order: row n sits in stage n % stages
             const int n0 = x.early0 ? 1 : 0;   // (the first row's copies may have been issued by the row group)
-            for (int n = n0; ok && n < ntok; ++n) {
+            // Short rows, all of them in the ring: several at once, a lane per copy.  (A trip costs 0.4 us however few
+            // bytes it sends; rows with 32 KB of copies take longer than that by themselves.  Dispatch of 1536 tokens,
+            // 1024 channels, top-4: 11.4 us, one row at a time 14.3.)
+            const int copies = p.k * (int)out_bytes;
+            const int m = p.k <= 16 && ntok <= stages && copies <= 16384 ? min(32 / p.k, 32768 / copies) : 1;
+            if (m > 1) {
+                const int sub = lane / p.k, j = lane - sub * p.k;
+                for (int n = n0; ok && n < ntok; n += m) {
+                    const int row = n + sub;
+                    const bool mine = sub < m && row < ntok;
+                    if (mine) ok = mbar_wait(&full_bar[row], 0, abortp);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    if (n == n0 && lane == 0) trace(p, c, kTrFirstRow);
+                    const int where = mine ? pos[row * p.k + j] : -1;
+                    if (where >= 0)
+                        bulk_store(p.recv_x + (size_t)where * p.rowB + out_off, smem + (size_t)row * pl.stage_bytes, out_bytes);
+                    bulk_commit();
+                }
+            }
+            for (int n = n0; m == 1 && ok && n < ntok; ++n) {
                 const int s = n % stages;
                 ok = mbar_wait(&full_bar[s], (n / stages) & 1, abortp);
                 ok = __all_sync(0xffffffffu, ok);
@@ -340,7 +359,7 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
             group_sync(2, kThreads);
         } else if (kMode == kModeCluster) {
             if (!kSteal) {   // (see above)
-                for (int n = 0; n < min(2, min(stages, ntok)); ++n) issue_item(n);
+                issue_first(min(min(2, p.prefetch_rows), min(stages, ntok)));
                 issued = head;
             }
             cluster_wait();
@@ -353,7 +372,7 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
             ok = __all_sync(0xffffffffu, ok);
         }
         // loader only; the quantising warps free the stages.  A closing item with no row
-        // tells them (and through them the store issuer) that nothing follows.  Rows are fetched as
+        // tells them that nothing follows.  Rows are fetched as
         // far ahead as the rings allow, at most prefetch_rows of them before the layout is done.
         int tl = 0;
         bool ready_seen = kMode == kModeLocal;   // (the flag-free kernel: its quantisers start after the layout)
@@ -365,7 +384,9 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
             return __shfl_sync(0xffffffffu, (int)r, 0) != 0;
         };
         if (!kSteal) {
-            // the CTA's own rows only: one thread, as far ahead as the ring allows
+            // the CTA's own rows only, as far ahead as the ring allows
+            issue_first(max(min(min(p.prefetch_rows, 32), min(stages, ntok)) - head, 0));
+            issued = head;
             while (ok && head < ntok) {
                 ok = wait_ready_at(head);
                 if (!ok) break;
@@ -406,9 +427,17 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
                 issue_item(tl);
                 issued = head;
             } else {
-                if (lane == 0) {   // (without stealing the consumers know the row count)
-                    item_src[s] = -1;
-                    mbar_arrive(&full_bar[s]);
+                // closing items, one for each team of quantising warps (without stealing they know the row count)
+                for (int q = 0; ok && q < (pl.q_long ? 1 : pl.q_teams); ++q) {
+                    const int cs = (head + q) % stages;
+                    if (head + q >= stages) {
+                        ok = mbar_wait(&empty_bar[cs], (((head + q) / stages) - 1) & 1, abortp);
+                        ok = __all_sync(0xffffffffu, ok);
+                    }
+                    if (ok && lane == 0) {
+                        item_src[cs] = -1;
+                        mbar_arrive(&full_bar[cs]);
+                    }
                 }
                 break;
             }
@@ -713,11 +742,11 @@ __device__ __forceinline__ int layout_group(Cta& x) {
                 epoch_finish_check_in(p, ticket, ep_mine);
                 if (p.trace) p.trace[(size_t)c * kTraceSlots + 12] = trace_ns(p);
             }
-        } else if (kFp8 && warp - x.qwarp0 < x.nq) {
+        } else if (kFp8 && warp - pl.q_warp0 < nq) {
             return 1;   // FP8 rows: the first warps behind the row group quantise as well
         } else {
             // expert-level outputs of rank r: shared by Q CTAs so that no CTA trails the others
-            const int dgw0 = kFp8 ? max(kRowWarps, x.qwarp0 + x.nq - 1) : kRowWarps;   // first warp of the duty group
+            const int dgw0 = kFp8 ? max(kRowWarps, pl.q_warp0 + nq - 1) : kRowWarps;   // first warp of the duty group
             const int dn = gn - dgw0 * 32, dw = nw - dgw0;
             const int Q = p.grid / p.R > 1 ? p.grid / p.R : 1;
             // ... once the movers are released: started earlier, these warps take issue slots and
@@ -766,10 +795,11 @@ __device__ __forceinline__ int layout_group(Cta& x) {
     } else if (kMode == kModeCluster) {
         cluster_layout<kFp8, kSteal>(x);
         if (kFp8 && gw >= nw) return 2;   // off to quantise
-        if (kFp8 && gw == 0) return 1;    // off to issue the copies
+        const int d0 = kFp8 && pl.q_long ? 1 : 0;
+        if (gw < d0) return 1;            // off to issue the copies
         // the others write what nobody waits for
-        cluster_duty<kFp8>(x, gtid - (kFp8 ? 32 : 0), gn - (kFp8 ? 32 : 0), kFp8 ? 3 : 1);
-        if (gtid == (kFp8 ? 32 : 0)) trace(p, c, kTrScanned);   // deferred outputs written
+        cluster_duty<kFp8>(x, gtid - d0 * 32, gn - d0 * 32, kFp8 ? 3 : 1);
+        if (gtid == d0 * 32) trace(p, c, kTrScanned);   // deferred outputs written
         return kFp8 ? 3 : 1;
     } else {
         // FP8 rows with a count group: TokenCnt itself -- staging the ids, the bitmaps, publishing the
@@ -877,20 +907,28 @@ __device__ __forceinline__ int layout_group(Cta& x) {
 }
 
 // ------------------------------------------------------------ FP8: quantise and store
-// Two roles around a ring of quantised rows (payload + scales).  The quantising warps turn the
-// rows the loader has fetched into FP8 and know nothing about destinations (own rows) -- so they
-// can run beside the layout; the store issuer sends every quantised row to its destinations
-// with bulk copies once the layout is done.
+// Long rows (40 KB of copies and more).  Two roles around a ring of quantised rows (payload + scales): the quantising
+// warps turn one row after the other into FP8 and know nothing about destinations (own rows) -- so they can run
+// beside the layout; the store issuer sends every quantised row to its destinations with bulk copies once the
+// layout is done, at most three rows at a time.
+//
+// Short rows.  The quantising warps work in teams (fp8_worker).  A team takes every teams-th row the loader has fetched,
+// quantises it into one of its two slots and sends it itself once the layout is done; the next row is quantised
+// meanwhile.  A team is one warp, so that a row costs no barrier and as many rows are on their way as there are
+// warps; only where a CTA has fewer rows than warps do several of them share one.  (In the arrangement for long rows
+// each row costs a CTA 1.1 us, however short.  Dispatch of 1536 tokens, 1024 channels, top-4: 24.0 us that way, 11.6 this
+// way; 2048 channels: 21.6 and 13.5; 4096 channels, top-8: 21.8 and 18.9.  So many long rows on their way at once run at
+// less bandwidth: 7168 channels, top-8, 1024 / 4096 tokens 18.0 / 62 and 20.3 / 67 us.)
 //
 // Shared-memory bookkeeping behind the input ring's items: out_src[os] = where the row of
 // output stage os comes from (chunk << 16 | index, -1 = nothing follows), out_pos[os] = the
 // destinations of a row taken over from another chunk.
 struct Fp8Ring {
     uint8_t* out_ring;
-    const int* item_src;   // [kMaxStages]
-    const int* item_pos;   // [kMaxStages, k]
-    int* out_src;          // [kMaxOutStages]
-    int* out_pos;          // [kMaxOutStages, k]
+    const int* item_src;   // [kStealStages]
+    const int* item_pos;   // [kStealStages, k]
+    int* out_src;          // [out_stages]
+    int* out_pos;          // [out_stages, k]
     int g0;                // first scale group of this CTA's piece
     unsigned scale_bytes;  // its scales travel with the payload
     bool scale_bulk;       // ... by a bulk copy when their size allows it
@@ -901,16 +939,42 @@ __device__ __forceinline__ Fp8Ring fp8_ring(const Cta& x) {
     Fp8Ring q;
     q.out_ring = x.smem + x.pl.off_out;
     q.item_src = item;
-    q.out_src = item + kMaxStages;
-    q.item_pos = item + kMaxStages + kMaxOutStages;
-    q.out_pos = item + kMaxStages + kMaxOutStages + kMaxStages * p.k;
+    q.item_pos = item + kStealStages;
+    q.out_src = item + kStealStages * (p.k + 1);
+    q.out_pos = q.out_src + x.pl.out_stages;
     q.g0 = x.part * (p.G / p.parts);
     q.scale_bytes = (unsigned)(p.G / p.parts) * 4u;
     q.scale_bulk = (q.scale_bytes & 15u) == 0;
     return q;
 }
 
-// Quantising warp qw of nq.
+// The copies of the quantised row in stage `os`; lanes 0 .. k - 1 the payload, k .. 2k - 1 the scales.
+template <bool kSteal>
+__device__ __forceinline__ void fp8_issue(Cta& x, const Fp8Ring& q, const uint8_t* src, int from, int os) {
+    UBEP_CTA_LOCALS(x, false);
+    const int* wpos = (from >> 16) == ch ? pos + (from & 0xffff) * p.k : q.out_pos + os * p.k;
+    for (int j = lane; j < (q.scale_bulk ? 2 * p.k : p.k); j += 32) {
+        const bool payload = j < p.k;
+        const int where = wpos[payload ? j : j - p.k];
+        if (where < 0) continue;
+        uint8_t* dst = payload ? p.recv_x + (size_t)where * p.rowB + out_off
+                               : reinterpret_cast<uint8_t*>(p.recv_scale + (size_t)where * p.G + q.g0);
+        bulk_store(dst, payload ? src : src + out_bytes, payload ? out_bytes : q.scale_bytes);
+        if (kSteal && payload) atomicAdd(&arr[where / p.cap], 1);
+    }
+    if (!q.scale_bulk) {   // a piece of scales that no bulk copy can carry: plain stores
+        const int Gp = p.G / p.parts;   // scale groups of this CTA's piece
+        const float* sc = reinterpret_cast<const float*>(src + out_bytes);
+        for (int i = lane; i < p.k * Gp; i += 32) {
+            const int jj = i / Gp, g = i - jj * Gp;
+            const int where = wpos[jj];
+            if (where >= 0) p.recv_scale[(size_t)where * p.G + q.g0 + g] = sc[g];
+        }
+    }
+    bulk_commit();
+}
+
+// Long rows: quantising warp qw of nq.
 template <bool kSteal>
 __device__ __forceinline__ void fp8_quantiser(Cta& x, int qw) {
     UBEP_CTA_LOCALS(x, false);
@@ -973,12 +1037,11 @@ __device__ __forceinline__ void fp8_quantiser(Cta& x, int qw) {
     }
 }
 
-// Store issuer (one warp, after the layout): lane j issues the copy of slot j.
+// Long rows: the store issuer (one warp, after the layout).
 template <bool kSteal>
 __device__ __forceinline__ void fp8_store_issuer(Cta& x) {
     UBEP_CTA_LOCALS(x, false);
     const Fp8Ring q = fp8_ring(x);
-    const int Gp = p.G / p.parts;   // scale groups of this CTA's piece
     bool sok = true;
     unsigned long long w_full = 0, w_read = 0, tq = 0;
     for (int n = 0; kSteal || n < ntok; ++n) {
@@ -990,29 +1053,7 @@ __device__ __forceinline__ void fp8_store_issuer(Cta& x) {
         const int from = kSteal ? q.out_src[os] : ((ch << 16) | n);
         if (!sok || from < 0) break;
         if (n == 0 && lane == 0) trace(p, c, kTrFirstRow);
-        const int* wpos = (from >> 16) == ch ? pos + (from & 0xffff) * p.k : q.out_pos + os * p.k;
-        const uint8_t* src = q.out_ring + (size_t)os * pl.out_stage_bytes;
-        // lanes 0..k-1: payload of slot j; lanes k..2k-1: its scales (when bulk-storable)
-        for (int j = lane; j < (q.scale_bulk ? 2 * p.k : p.k); j += 32) {
-            const int jj = j < p.k ? j : j - p.k;
-            const int where = wpos[jj];
-            if (where < 0) continue;
-            if (j < p.k) {
-                bulk_store(p.recv_x + (size_t)where * p.rowB + out_off, src, out_bytes);
-                if (kSteal) atomicAdd(&arr[where / p.cap], 1);
-            } else {
-                bulk_store(p.recv_scale + (size_t)where * p.G + q.g0, src + out_bytes, q.scale_bytes);
-            }
-        }
-        if (!q.scale_bulk) {   // a piece of scales that no bulk copy can carry: plain stores
-            const float* sc = reinterpret_cast<const float*>(src + out_bytes);
-            for (int i = lane; i < p.k * Gp; i += 32) {
-                const int jj = i / Gp, g = i - jj * Gp;
-                const int where = wpos[jj];
-                if (where >= 0) p.recv_scale[(size_t)where * p.G + q.g0 + g] = sc[g];
-            }
-        }
-        bulk_commit();
+        fp8_issue<kSteal>(x, q, q.out_ring + (size_t)os * pl.out_stage_bytes, from, os);
         if (n + 1 >= kStorePending) {
             if (p.trace) tq = trace_ns(p);
             bulk_wait_read<kStorePending - 1>();   // every lane: the copies of the row kStorePending - 1 back have read it
@@ -1032,12 +1073,111 @@ __device__ __forceinline__ void fp8_store_issuer(Cta& x) {
     }
 }
 
+// Short rows (see Fp8Ring): quantising warp qw, in teams that send what they have quantised themselves.
+template <bool kSteal>
+__device__ __forceinline__ void fp8_worker(Cta& x, int qw) {
+    UBEP_CTA_LOCALS(x, false);
+    const Fp8Ring q = fp8_ring(x);
+    const int teams = pl.q_teams, tw = pl.q_team_warps, team = qw / tw, m = qw - team * tw;
+    if (team >= teams) return;
+    auto team_sync = [&]() {
+        if (tw > 1) group_sync(5 + team, tw * 32);
+        else __syncwarp();
+    };
+    const int nvec = (int)in_bytes / 16;   // 8-channel vectors in this CTA's piece
+    bool ready = false, good = true;
+    int sent = 0, from0 = 0, from1 = 0;    // rows of this team on their way; origins of the rows in its two slots
+    auto layout_done = [&]() {
+        if (!ready) {
+            good = __all_sync(0xffffffffu, mbar_wait_idle(&ready_bar, 0, abortp) && !*abortp);   // no rows without a layout
+            ready = true;
+        }
+    };
+    auto send = [&]() {
+        const int os = team * 2 + (sent & 1);
+        fp8_issue<kSteal>(x, q, q.out_ring + (size_t)os * pl.out_stage_bytes, (sent & 1) ? from1 : from0, os);
+        ++sent;
+    };
+    int i = 0;
+    for (;; ++i) {
+        const int n = team + i * teams;
+        if (!kSteal && n >= ntok) break;
+        const int s = n % stages;
+        const unsigned par = (n / stages) & 1;
+        if (tw == 1 && sent < i) {   // the first row still waits for the layout: whichever comes first
+            const unsigned long long t_end = global_ns() + kWaitLimitNs;
+            for (;;) {
+                if (__any_sync(0xffffffffu, mbar_test_wait(&ready_bar, 0))) {
+                    layout_done();
+                    if (good) send();
+                    break;
+                }
+                if (__any_sync(0xffffffffu, mbar_try_wait(&full_bar[s], par, 200u))) break;
+                if (__any_sync(0xffffffffu, *abortp || global_ns() > t_end)) break;   // (the wait below gives up)
+            }
+        }
+        good = good && __all_sync(0xffffffffu, mbar_wait_idle(&full_bar[s], par, abortp));
+        if (tw > 1) good = !group_or(5 + team, tw * 32, !good);   // (the warps of a team leave together)
+        if (!good) break;
+        const int from = kSteal ? q.item_src[s] : ((ch << 16) | n);
+        if (from < 0) break;   // the loader's closing item
+        if (i >= 2) {          // the copies of the row before the last one have read its slot
+            if (m == 0) bulk_wait_read<1>();
+            team_sync();
+        }
+        const int os = team * 2 + (i & 1);
+        if (i & 1) from1 = from;
+        else from0 = from;
+        if (kSteal && m == 0 && (from >> 16) != ch)   // a row of another chunk: its destinations travel with it
+            for (int j = lane; j < p.k; j += 32) q.out_pos[os * p.k + j] = q.item_pos[s * p.k + j];
+        const uint8_t* src = smem + (size_t)s * pl.stage_bytes;
+        uint8_t* dst = q.out_ring + (size_t)os * pl.out_stage_bytes;
+        float* dst_scale = reinterpret_cast<float*>(dst + out_bytes);
+        // four vectors per thread and trip, independent of each other
+        for (int vb = m * 32; vb < nvec; vb += 4 * tw * 32) {
+            uint4 in[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int v = vb + u * tw * 32 + lane;
+                in[u] = v < nvec ? *reinterpret_cast<const uint4*>(src + (size_t)v * 16) : make_uint4(0, 0, 0, 0);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int v = vb + u * tw * 32 + lane;
+                uint2 o;
+                float sc;
+                quantize8(in[u], v < nvec, o, sc);
+                if (v < nvec) {
+                    *reinterpret_cast<uint2*>(dst + (size_t)v * 8) = o;
+                    if ((lane & 15) == 0) dst_scale[v >> 4] = sc;
+                }
+            }
+        }
+        fence_proxy_async_smem();   // the bulk stores read what we just wrote
+        team_sync();
+        if (lane == 0) mbar_arrive(&empty_bar[s]);
+        if (m != 0) continue;
+        if (tw == 1 && i == 0 && !ready && !__any_sync(0xffffffffu, mbar_test_wait(&ready_bar, 0))) continue;
+        layout_done();
+        while (good && sent <= i) send();
+    }
+    if (m == 0) {
+        if (good && sent < i) layout_done();
+        if (good && sent < i) send();
+        if (!good && lane == 0) {
+            report(p.status, kErrTimeout);
+            *abortp = 1;
+        }
+        bulk_wait_all<0>();
+    }
+}
+
 // --------------------------------------------------------------------- dispatch kernel
 // Warp roles: warp 0 = mover; warps 1..15 = layout group (count, prefix sums, row
 // assignment).  FP8 rows: warp 0 only loads; either the layout group is warps 1 .. count_warps and
 // the warps behind them quantise beside it (the kernels whose layout waits for other CTAs or was
 // computed by earlier launches), or all 15 warps compute the layout and warps 2..15 quantise
-// afterwards (the flag-free kernel, whose layout is pure computation); warp 1 issues the stores
+// afterwards (the flag-free kernel, whose layout is pure computation); warp 1 issues the copies of long rows
 // once the layout is done.
 template <int kMode, bool kFp8, bool kSteal>
 __global__ void __launch_bounds__(kThreads, 1) dispatch_kernel(const Params p, const SmemPlan pl) {
@@ -1059,21 +1199,16 @@ __global__ void __launch_bounds__(kThreads, 1) dispatch_kernel(const Params p, c
     const int stages = pl.stages;
     const bool beside = kFp8 && (kMode == kModeCluster || (kMode != kModeLocal && p.count_warps > 0));
     const int nw = kFp8 && kMode == kModeCluster ? kClusterCountWarps : beside ? p.count_warps : kWarps - 1;      // layout group: warps 1 .. nw
-    const int qwarp0 = beside ? nw + 1 : 2;                    // FP8: warps qwarp0 .. qwarp0 + nq - 1 quantise
-    // (flag-free kernel with rank-level rows: a CTA has few rows, and the warps that do not quantise write
-    // the expert-level outputs meanwhile)
-    const int nq = kFp8 ? min(kMode == kModeLocal && p.local_fast ? min(p.quant_warps, kFastQuantWarps) : p.quant_warps, kWarps - qwarp0)
-                        : kWarps - 2;
     int* arr = reinterpret_cast<int*>(smem + pl.off_arr);
     griddep_launch();   // the next kernel in the stream may be placed as soon as SMs have room
 
     if (tid == 0) {
         for (int s = 0; s < stages; ++s) {
             mbar_init(&full_bar[s], 1);
-            mbar_init(&empty_bar[s], nq);
+            mbar_init(&empty_bar[s], !kFp8 ? 1 : pl.q_long ? pl.q_warps : pl.q_team_warps);
         }
-        for (int s = 0; s < pl.out_stages; ++s) {
-            mbar_init(&out_full[s], nq);
+        for (int s = 0; kFp8 && pl.q_long && s < pl.out_stages; ++s) {
+            mbar_init(&out_full[s], pl.q_warps);
             mbar_init(&out_empty[s], 1);
         }
         mbar_init(&ready_bar, 1);
@@ -1119,8 +1254,8 @@ __global__ void __launch_bounds__(kThreads, 1) dispatch_kernel(const Params p, c
     const unsigned in_bytes = (unsigned)(p.H * 2 / p.parts);   // this CTA's piece of a bf16 row
     const unsigned out_bytes = (unsigned)(p.rowB / p.parts);   // and of a payload row
     Cta x{p, pl, smem, full_bar, empty_bar, out_full, out_empty, &ready_bar, &epoch_bar, &staged_bar, &abort_flag,
-          tid, tid & 31, tid >> 5, c, part, ch, t0, t1, t1 - t0, stages, nq,
-          nw * 32, nw, pl.out_stages, qwarp0, beside,
+          tid, tid & 31, tid >> 5, c, part, ch, t0, t1, t1 - t0, stages,
+          nw * 32, nw, beside,
           reinterpret_cast<int*>(smem + pl.off_ids),
           reinterpret_cast<int*>(smem + pl.off_ord),    // destinations in issue order
           reinterpret_cast<int*>(smem + (p.ordered ? pl.off_pos : pl.off_ord)),   // in slot order (the same array
@@ -1142,11 +1277,13 @@ __global__ void __launch_bounds__(kThreads, 1) dispatch_kernel(const Params p, c
     } else {
         const int lg = layout_group<kMode, kFp8, kSteal>(x);   // 0 = a wait ran out, 1 = done, 2 = left to quantise
         if (!kFp8 && x.early0 && x.warp == 1) bulk_wait_all<0>();   // the first row's copies (issued by this warp)
-        if (kFp8 && lg == 2) {
-            if (x.warp - qwarp0 < nq) fp8_quantiser<kSteal>(x, x.warp - qwarp0);   // beside the rest of the layout
-        } else if (kFp8 && lg == 1) {
-            if (x.warp == 1) fp8_store_issuer<kSteal>(x);
-            else if (!beside && x.warp - 2 < nq) fp8_quantiser<kSteal>(x, x.warp - 2);
+        // (2: beside the rest of the layout; 1: after it, unless the quantising warps are others)
+        const int qw = x.warp - pl.q_warp0;
+        if (kFp8 && pl.q_long && lg == 1 && x.warp == 1) {
+            fp8_store_issuer<kSteal>(x);
+        } else if (kFp8 && (lg == 2 || (lg == 1 && !beside)) && qw >= 0 && qw < pl.q_warps) {
+            if (pl.q_long) fp8_quantiser<kSteal>(x, qw);
+            else fp8_worker<kSteal>(x, qw);
         }
     }
     if (kMode == kModeCluster) cluster_wait();   // the others have read what this CTA counted
@@ -1393,38 +1530,50 @@ int plan_dispatch(const Params& p, int mode, int max_smem, SmemPlan* out) {
     pl.out_stage_bytes = p.payload ? round_up_i(p.rowB / p.parts + (p.G / p.parts) * 4, 128) : 0;
     const int64_t mask_ints = (int64_t)pl.map_groups * 32;
     const int64_t bm_ints = (int64_t)pl.map_groups * pl.map_bp;
-    const int item_ints = (kMaxStages + kMaxOutStages) * (p.k + 1);
+    const bool beside = p.payload && (mode == kModeCluster || (mode != kModeLocal && p.count_warps > 0));
+    if (p.payload) {   // who quantises, and how (see Fp8Ring)
+        const bool fast = mode == kModeLocal && p.local_fast;
+        pl.q_long = (int64_t)p.k * (p.rowB / p.parts) >= 40 * 1024 ? 1 : 0;
+        pl.q_warp0 = beside ? (mode == kModeCluster ? kClusterCountWarps : p.count_warps) + 1 : pl.q_long ? 2 : 1;
+        const int most = fast ? kFastQuantWarps + (pl.q_long ? 0 : 1) : kWarps - pl.q_warp0;
+        pl.q_warps = p.quant_warps < most ? p.quant_warps : most;
+        pl.q_teams = pl.q_warps;
+        if (!p.steal && pl.q_teams > chunk_tokens) pl.q_teams = chunk_tokens < 1 ? 1 : chunk_tokens;
+        pl.out_stages = !pl.q_long ? 2 * pl.q_teams : beside ? kMaxOutStages : kOutStages;   // at most
+    }
+    const int item_ints = p.steal ? (kStealStages + pl.out_stages) * (p.k + 1) : 0;
+    const int max_stages = p.steal ? kStealStages : kMaxStages;
     const int64_t cnt_ints = mode == kModeCluster ? 3 * ((int64_t)p.B + 1) : 0;
     const int64_t ints = ids_ints + mask_ints + bm_ints + 4 * (int64_t)chunk_slots + hist_ints + 2 * p.R + item_ints +
                          cnt_ints;
     const int64_t fixed = ints * 4 + 128 + 1536;  // 1.5 KB: static shared memory
     // no more stages than rows this CTA will ever hold at once
     const int want = chunk_tokens + 3 < 4 ? 4 : chunk_tokens + 3;
-    const bool beside = p.payload && (mode == kModeCluster || (mode != kModeLocal && p.count_warps > 0));
-    if (!beside) {
-        // the quantising warps (if any) start after the layout: a deep input ring that the loader fills
-        // meanwhile, a short ring of quantised rows
-        pl.out_stages = p.payload ? kOutStages : 0;
-        const int64_t rest = max_smem - fixed - (int64_t)pl.out_stages * pl.out_stage_bytes;
-        if (rest < 4 * (int64_t)pl.stage_bytes) return -1;
-        pl.stages = (int)(rest / pl.stage_bytes);
-        if (pl.stages > kMaxStages) pl.stages = kMaxStages;
-        if (pl.stages > want) pl.stages = want;
-    } else {
-        // the quantising warps run beside the layout: a short input ring (enough loads in flight to keep
-        // them busy) and as many quantised rows as fit, which wait for the layout
-        const int64_t room = max_smem - fixed;
-        if (room < 2 * (int64_t)pl.stage_bytes + 4 * (int64_t)pl.out_stage_bytes) return -1;
-        pl.stages = 4;
-        while (pl.stages > 2 && room < (int64_t)pl.stages * pl.stage_bytes + 4 * (int64_t)pl.out_stage_bytes) --pl.stages;
-        pl.out_stages = (int)((room - (int64_t)pl.stages * pl.stage_bytes) / pl.out_stage_bytes);
-        if (pl.out_stages > kMaxOutStages) pl.out_stages = kMaxOutStages;
-        if (pl.out_stages > want) pl.out_stages = want < 4 ? 4 : want;
-        // what is left over goes to the input ring
-        const int more = (int)((room - (int64_t)pl.out_stages * pl.out_stage_bytes) / pl.stage_bytes);
-        pl.stages = more > kMaxStages ? kMaxStages : more;
-        if (pl.stages > want) pl.stages = want;
+    int64_t room = max_smem - fixed;
+    const int64_t in = pl.stage_bytes, out_b = pl.out_stage_bytes;
+    if (p.payload && !pl.q_long) {
+        // Two quantised rows per team, the rest for rows that have been fetched: as many as there are teams at least.
+        // (Then the row a team waits for is at most one round of the ring behind the row it had before, and the
+        // parity of the stage's barrier tells them apart.)
+        while (pl.q_teams > 1 && room < pl.q_teams * (in + 2 * out_b)) --pl.q_teams;
+        pl.q_team_warps = pl.q_warps / pl.q_teams;
+        pl.out_stages = 2 * pl.q_teams;
+    } else if (beside) {
+        // the quantising warps run beside the layout: a short input ring (enough loads in flight to keep them busy) and
+        // as many quantised rows as fit, which wait for the layout.  (Otherwise they start after the layout: a deep
+        // input ring that the loader fills meanwhile, a short ring of quantised rows.)
+        int st = 4;
+        while (st > 2 && room < st * in + 4 * out_b) --st;
+        if (room < st * in + 4 * out_b) return -1;
+        const int64_t fit = (room - st * in) / out_b;
+        if (pl.out_stages > fit) pl.out_stages = (int)fit;
+        if (pl.out_stages > want) pl.out_stages = want;
     }
+    room -= pl.out_stages * out_b;
+    const int least = p.payload && !p.steal ? 2 : 4;   // (stealing looks at the row three back)
+    if (room < least * in) return -1;
+    pl.stages = room / in > max_stages ? max_stages : (int)(room / in);
+    if (pl.stages > want) pl.stages = want;
     int at = pl.stages * pl.stage_bytes;
     pl.off_out = at; at += pl.out_stages * pl.out_stage_bytes;
     pl.off_ids = at; at += (int)ids_ints * 4;
