@@ -25,16 +25,22 @@ constexpr int kStealMinTokensPerChunk = 40;  // shorter slices: the hand-out cos
 constexpr int kDefaultCountWarps = 8;            // FP8: warps of the count group while the others quantise (measured sweep;
                                                  // -1 in the buffer = this default, and none with token stealing)
 constexpr int64_t kLocalMaxSlots = 8192;        // small-T limit of the combine launch mode and of the protocol / sharded paths
-// AUTO's crossovers between the flag-free and the flag-exchanging schedule, in routing-table slots (T * k);
-// measured over three shape families (H / E / R = 7168 / 256 / 32, 4096 / 128 / 16, 7168 / 288 / 72), top-8,
-// 64 .. 2048 tokens: the crossover follows the slots, not the number of bins.
-constexpr int64_t kLocalFastMaxSlots = 16384;     // one row per (token, rank), bf16 rows: the rank-level fast path
-                                                  // (2048 tokens: 50.4 against 58.4 us; larger tables do not fit in shared memory)
-constexpr int64_t kLocalFastFp8MaxSlots = 8192;   // the same with FP8 rows (1024 tokens: 25.3 against 31.5 us, 1536: 39.4 against 38.4)
-// One row per (token, expert), bf16 rows: every CTA derives the layout alone where the table has at most 512 slots
-// and slots * bins are at most 32 K (8 tokens of top-8, 288 bins: 7.5 us against 7.9 by clusters, 32 tokens: 7.7 and
-// 7.4; 128 tokens of top-4, 40 bins: 7.3 and 7.6, 512 tokens: 12.7 and 9.0).  FP8 rows: by clusters throughout.
-constexpr int64_t kLocalAllBinsMaxSlots = 512, kLocalAllBinsMaxSlotBins = 32768;
+// AUTO: up to which size every CTA derives the layout alone; larger tables are counted by clusters of CTAs.  Measured on
+// seven shape families; the figures are dispatches alone, every CTA alone against clusters of two.
+// One row per (token, rank): the work per CTA grows with the tokens; the more bytes a token has, the more of it is
+// hidden behind the copies (7168 channels: 1536 tokens 34.5 and 35.8 us, 2048 tokens 48.8 and 47.0; 4096 channels: 512
+// tokens 11.1 and 11.6, 1024 tokens 16.7 and 16.1; 1024 channels: 512 tokens 9.2 and 9.4, 1024 tokens 12.2 and 10.7).
+// FP8 rows have fewer (7168 channels: 512 tokens 13.1 and 13.4, 768 tokens 18.2 and 16.2).  More than 32 ranks take
+// more words per token (72 ranks, bf16 512 tokens 15.8 and 15.6, FP8 128 tokens 9.7 and 10.1, 512 tokens 16.5 and 14.0).
+int local_fast_max_tokens(const Params& p) {
+    if (p.payload) return p.R > 32 ? 224 : 544;
+    const int by_bytes = p.H * 2 / 9;
+    return p.R > 32 || by_bytes < 448 ? 448 : by_bytes;
+}
+// One row per (token, expert), bf16 rows, in tokens * bins (8 tokens, 288 bins: 7.5 and 7.9 us, 32 tokens: 7.7 and 7.4;
+// 64 tokens, 136 bins: 7.2 and 7.6, 256 tokens: 10.1 and 8.2; 512 tokens, 20 bins: 7.9 and 8.2, 1024 tokens: 10.5
+// and 8.5).  FP8 rows: by clusters throughout.
+constexpr int64_t kLocalAllBinsMax = 9000;
 // Cluster sizes: two up to 32 K slots, eight from 64 K on (dispatch + combine, sizes 2 / 4 / 8: 24576 slots 88.2 / 88.8 /
 // 90.2 us, 32768 slots 150 / 151 / 152, 65536 slots 213 / 212 / 209, 131072 slots 555 / 555 / 544).
 constexpr int64_t kCluster2MaxSlots = 32768, kCluster8MinSlots = 65536;
@@ -248,15 +254,16 @@ Params make_params(ubep_buffer* b, int T) {
 
 // Cuts the work of a flag-free kernel over `ctas` CTAs: token chunks, and column parts of a row so that the slices
 // are balanced to about 5 %.  The CTA with the most work sets the pace: ceil(T / chunks) tokens of 1 / parts of a
-// row each.  Smaller pieces cost more per byte (measured on the decode shape, layout by every CTA alone: 4 parts
-// + 8 %, 8 parts + 60 %).  With the layout by clusters pieces are cut for balance only where they keep 4 KB (512
-// tokens of 1024 bf16 channels: 9.0 us whole, 10.4 in halves; 7168 channels: 16.3 and 15.3), FP8 rows not at all
-// (512 tokens of 7168 channels: 13.3 and 16.4 us); a CTA that has one token at most takes any piece.
+// row each.  Smaller pieces cost more per byte (measured on the decode shape, layout by every CTA alone: 4 parts + 8 to
+// 15 %, 8 parts + 60 %).  A CTA that has one token at most takes pieces down to 2 KB (16 tokens of 2048 bf16 channels:
+// 6.8 us whole, 7.1 in eight pieces; 7168 channels: 7.3 and 6.8).  Otherwise pieces are cut for balance only where
+// they keep 4 KB (512 tokens of 1024 channels, by clusters: 9.0 us whole, 10.4 in halves; 7168 channels: 16.3 and 15.3),
+// FP8 rows not at all (512 tokens of 7168 channels, by clusters: 13.3 and 16.4 us, every CTA alone: 13.1 and 14.9).
 void split_work(Params& p, int ctas) {
     int best = 1;
     double best_cost = 0.0;
     const bool by_cluster = p.cluster > 1;
-    const double piece_penalty[4] = {1.0, by_cluster ? 1.05 : 1.0, by_cluster ? 1.1 : 1.08, by_cluster ? 1.15 : 1.6};
+    const double piece_penalty[4] = {1.0, by_cluster ? 1.05 : 1.0, by_cluster ? 1.1 : 1.15, by_cluster ? 1.15 : 1.6};
     for (int parts = 1, i = 0; parts <= 8; parts *= 2, ++i) {
         const int chunks = ctas / parts;
         if (chunks < 1 || (p.H * 2 / parts) % 16 != 0 || (p.H * 2) % parts != 0) break;
@@ -264,8 +271,8 @@ void split_work(Params& p, int ctas) {
         // FP8 rows: a piece's scales must still be a bulk copy (a multiple of 16 bytes); with plain stores for
         // the scales and payload pieces under 2 KB a dispatch of 384 tokens took 33 us against 21 us for 512
         if (p.payload && parts > 1 && ((p.G / parts) * 4) % 16 != 0) break;
-        const int most = (p.T + chunks - 1) / chunks;
-        if (by_cluster && parts > 1 && most > 1 && (p.payload || p.H * 2 / parts < 4096)) break;
+        const int most = (p.T + chunks - 1) / chunks, piece = p.H * 2 / parts;
+        if (parts > 1 && (piece < (most > 1 ? 4096 : 2048) || (most > 1 && p.payload))) break;
         const double cost = (double)most / parts * piece_penalty[i];
         if (parts == 1 || cost < best_cost * 0.999) {
             best = parts;
@@ -445,8 +452,7 @@ int ubep_dispatch(ubep_buffer_t* buf, const void* x, const int32_t* topk_idx, co
         // that clusters of CTAs count the table between them (larger clusters cost CTAs: of a B200's 148 SMs 132
         // can be used in clusters of four, 120 in clusters of eight).
         mode = UBEP_PIPELINE_FUSED;
-        const bool alone = p.local_fast ? slots <= (p.payload ? kLocalFastFp8MaxSlots : kLocalFastMaxSlots)
-                                        : !p.payload && slots <= kLocalAllBinsMaxSlots && slots * p.B <= kLocalAllBinsMaxSlotBins;
+        const bool alone = p.local_fast ? T <= local_fast_max_tokens(p) : !p.payload && (int64_t)T * p.B <= kLocalAllBinsMax;
         if (alone) {
             mode = UBEP_PIPELINE_LOCAL;
         } else {
