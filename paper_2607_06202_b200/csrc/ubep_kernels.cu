@@ -99,6 +99,24 @@ struct Cta {
     [[maybe_unused]] const int out_stages = (x).pl.out_stages;                                               \
     [[maybe_unused]] const int gtid = (x).tid - 32, gw = (x).warp - 1
 
+// Short rows, all of them in the ring (row n in stage n): `rows` of them at once, a lane per copy.  (A trip costs 0.4 us
+// however few bytes it sends; rows with 32 KB of copies take longer than that by themselves.  Dispatch of 1536
+// tokens, 1024 channels, top-4: 11.4 us, one row at a time 14.3.)  Out of line: the code of long rows stays short.
+static __device__ __noinline__ bool send_short_rows(int n0, int ntok, int rows, int k, uint64_t* full_bar, const int* pos,
+                                                    const uint8_t* smem, int stage_bytes, uint8_t* dst, int rowB,
+                                                    unsigned bytes, volatile int* abort) {
+    const int lane = threadIdx.x & 31, sub = lane / k, j = lane - sub * k;
+    for (int n = n0; n < ntok; n += rows) {
+        const int row = n + sub;
+        const bool mine = sub < rows && row < ntok;
+        if (!__all_sync(0xffffffffu, !mine || mbar_wait(&full_bar[mine ? row : 0], 0, abort))) return false;
+        const int where = mine ? pos[row * k + j] : -1;
+        if (where >= 0) bulk_store(dst + (size_t)where * rowB, smem + (size_t)row * stage_bytes, bytes);
+        bulk_commit();
+    }
+    return true;
+}
+
 // ------------------------------------------------------------------------ mover warp
 // Warp 0.  Lane 0 issues the TMA loads; for bf16 rows lane j issues the TMA store of slot j,
 // so the k copies of a row are issued side by side; for FP8 rows the warp only loads.
@@ -280,27 +298,12 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
         if (!kSteal) {
             // the CTA's own rows, in order: row n sits in stage n % stages
             const int n0 = x.early0 ? 1 : 0;   // (the first row's copies may have been issued by the row group)
-            // Short rows, all of them in the ring: several at once, a lane per copy.  (A trip costs 0.4 us however few
-            // bytes it sends; rows with 32 KB of copies take longer than that by themselves.  Dispatch of 1536 tokens,
-            // 1024 channels, top-4: 11.4 us, one row at a time 14.3.)
-            const int copies = p.k * (int)out_bytes;
-            const int m = p.k <= 16 && ntok <= stages && copies <= 16384 ? min(32 / p.k, 32768 / copies) : 1;
-            if (m > 1) {
-                const int sub = lane / p.k, j = lane - sub * p.k;
-                for (int n = n0; ok && n < ntok; n += m) {
-                    const int row = n + sub;
-                    const bool mine = sub < m && row < ntok;
-                    if (mine) ok = mbar_wait(&full_bar[row], 0, abortp);
-                    ok = __all_sync(0xffffffffu, ok);
-                    if (!ok) break;
-                    if (n == n0 && lane == 0) trace(p, c, kTrFirstRow);
-                    const int where = mine ? pos[row * p.k + j] : -1;
-                    if (where >= 0)
-                        bulk_store(p.recv_x + (size_t)where * p.rowB + out_off, smem + (size_t)row * pl.stage_bytes, out_bytes);
-                    bulk_commit();
-                }
-            }
-            for (int n = n0; m == 1 && ok && n < ntok; ++n) {
+            if (pl.trip_rows > 1) {
+                if (lane == 0) trace(p, c, kTrFirstRow);
+                ok = send_short_rows(n0, ntok, pl.trip_rows, p.k, full_bar, pos, smem, pl.stage_bytes, p.recv_x + out_off, p.rowB,
+                                     out_bytes, x.abort_flag);
+            } else
+            for (int n = n0; ok && n < ntok; ++n) {
                 const int s = n % stages;
                 ok = mbar_wait(&full_bar[s], (n / stages) & 1, abortp);
                 ok = __all_sync(0xffffffffu, ok);
@@ -1575,6 +1578,10 @@ int plan_dispatch(const Params& p, int mode, int max_smem, SmemPlan* out) {
     pl.stages = room / in > max_stages ? max_stages : (int)(room / in);
     if (pl.stages > want) pl.stages = want;
     int at = pl.stages * pl.stage_bytes;
+    const int copies = p.k * (p.rowB / p.parts);
+    pl.trip_rows = 1;
+    if (!p.payload && !p.steal && p.k <= 16 && chunk_tokens <= pl.stages && copies <= 16384)
+        pl.trip_rows = 32 / p.k < 32768 / copies ? 32 / p.k : 32768 / copies;
     pl.off_out = at; at += pl.out_stages * pl.out_stage_bytes;
     pl.off_ids = at; at += (int)ids_ints * 4;
     pl.off_mask = at; at += (int)mask_ints * 4;
