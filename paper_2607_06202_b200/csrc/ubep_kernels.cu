@@ -43,6 +43,8 @@ __global__ void __launch_bounds__(256) scan_kernel(const Params p) {
     scan_rank_sources(p, blockIdx.x, sm_i, threadIdx.x, 256);
 }
 
+constexpr int kRowWarps = 4;   // flag-free kernel, rank-level rows: warps 1 .. 4 assign the rows of the CTA's tokens
+
 // Everything the roles of one dispatch CTA share.
 struct Cta {
     const Params& p;
@@ -63,6 +65,13 @@ struct Cta {
     bool fast_local;
     bool early0;  // flag-free kernel: the copies of the CTA's first row are issued by the warp that assigns the rows
     int issued;   // rows whose load the mover has started (thread 0's copy is used when leaving early)
+    bool early_arrival;   // the mover warp publishes the arrival counters
+    int landed_warps;     // ... once these warps (itself among them) have met: they issue copies or write row metadata
+    // Every one of those warps calls this once, whatever happened to it; only the mover (wait = 1) stays.
+    __device__ __forceinline__ void rows_landed(int wait) const {
+        if (wait) asm volatile("bar.sync 14, %0;" ::"r"(landed_warps * 32) : "memory");
+        else asm volatile("bar.arrive 14, %0;" ::"r"(landed_warps * 32) : "memory");
+    }
 };
 
 // The role functions below keep the names the kernel uses for these.
@@ -98,6 +107,14 @@ struct Cta {
     [[maybe_unused]] const int gn = nw * 32;                                                                 \
     [[maybe_unused]] const int out_stages = (x).pl.out_stages;                                               \
     [[maybe_unused]] const int gtid = (x).tid - 32, gw = (x).warp - 1
+
+// Pieces of this CTA's rows have landed: add them to the per-region arrival counters (unit: eighths of a row, so that
+// the total does not depend on the column split); thread i of n.
+__device__ __forceinline__ void publish_arrivals(const Params& p, const int* arr, unsigned half, int i, int n) {
+    fence_proxy_async();   // rows written through the async proxy, counters through the generic one
+    for (int r = i; r < p.R; r += n)
+        if (arr[r]) red_release_add(p.arrival + half * p.R + r, (unsigned)(arr[r] * (8 / p.parts)));
+}
 
 // Short rows, all of them in the ring (row n in stage n): `rows` of them at once, a lane per copy.  (A trip costs 0.4 us
 // however few bytes it sends; rows with 32 KB of copies take longer than that by themselves.  Dispatch of 1536
@@ -300,7 +317,7 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
             const int n0 = x.early0 ? 1 : 0;   // (the first row's copies may have been issued by the row group)
             if (pl.trip_rows > 1) {
                 if (lane == 0) trace(p, c, kTrFirstRow);
-                ok = send_short_rows(n0, ntok, pl.trip_rows, p.k, full_bar, pos, smem, pl.stage_bytes, p.recv_x + out_off, p.rowB,
+                if (ok) ok = send_short_rows(n0, ntok, pl.trip_rows, p.k, full_bar, pos, smem, pl.stage_bytes, p.recv_x + out_off, p.rowB,
                                      out_bytes, x.abort_flag);
             } else
             for (int n = n0; ok && n < ntok; ++n) {
@@ -464,6 +481,13 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
     if (lane == 0) trace(p, c, kTrIssued);
     bulk_wait_all<0>();
     if (lane == 0) trace(p, c, kTrStored);
+    if (x.early_arrival) {
+        // The arrival counters, as soon as the rows have landed and their metadata is written, while other warps still
+        // write what belongs to no row.  (At the kernel's end the release waited for those stores as well: 1.6 us of
+        // a dispatch of 128 tokens.)
+        x.rows_landed(1);
+        if (!*abortp) publish_arrivals(p, arr, *reinterpret_cast<volatile unsigned*>(x.epoch_late) & 1u, lane, 32);
+    }
 }
 
 // ------------------------------------------------------------- layout by clusters
@@ -575,6 +599,7 @@ __device__ __forceinline__ void cluster_layout(Cta& x) {
 // What nobody inside the kernel waits for: the metadata of the own tokens, the totals (one CTA) and the counts and
 // offsets of the source ranks whose tokens begin among the CTA's own.  Tokens of such a rank beyond the CTA's own
 // are counted from the table.
+constexpr int kEarlyDutyTokens = 256;   // flag-free kernel, rank-level rows: the expert-level outputs do not wait for the movers
 template <bool kFp8>
 __device__ __forceinline__ void cluster_duty(Cta& x, int dtid, int dn, int bar) {
     UBEP_CTA_LOCALS(x, !kFp8);
@@ -583,10 +608,8 @@ __device__ __forceinline__ void cluster_duty(Cta& x, int dtid, int dn, int bar) 
     const int* eo = hist + 2 * p.B;
     const int* row_sm = reinterpret_cast<const int*>(w_sm);
     unsigned* cnt = reinterpret_cast<unsigned*>(smem + pl.off_cnt) + 2 * (p.B + 1);   // (those in front are read by the cluster)
-    if (c == 0) write_totals(p, tot, eo, dtid, dn);
-    if (part != 0 || ntok == 0) return;
 #pragma unroll 1
-    for (int li = dtid; li < ntok * p.k; li += dn) {
+    for (int li = dtid; part == 0 && li < ntok * p.k; li += dn) {
         const int tl = li / p.k, packed = ids_sm[li], row = row_sm[li], where = pos_raw[li];
         const size_t i = (size_t)t0 * p.k + li;
         const bool have = packed >= 0;
@@ -629,25 +652,28 @@ __device__ __forceinline__ void cluster_duty(Cta& x, int dtid, int dn, int bar) 
             }
         }
     }
-    const int s_lo = (int)(((int64_t)t0 * p.S + p.T - 1) / p.T);  // smallest s with src_begin(s) >= t0
+    x.rows_landed(0);
+    if (c == 0) write_totals(p, tot, eo, dtid, dn);
+    if (part != 0 || ntok == 0) return;
+    // source ranks s_lo .. s_hi - 1 begin among the own tokens
+    const int s_lo = (int)(((int64_t)t0 * p.S + p.T - 1) / p.T);
+    const int s_hi = min(p.S, (int)(((int64_t)t1 * p.S + p.T - 1) / p.T));
+    if (s_hi <= s_lo) return;
+    const int last_end = src_begin(s_hi, p.T, p.S);
+    const bool beyond = last_end > t1;   // (only the last of them reaches beyond the own tokens)
+    if (beyond) {
+        for (int e = dtid; e < p.E; e += dn) cnt[e] = 0u;
+        group_sync(bar, dn);
+        count_tokens(count_args(p), t1, last_end, 0, false, cnt, dtid, dn);
+        group_sync(bar, dn);
+    }
 #pragma unroll 1
-    for (int s = s_lo; s < p.S; ++s) {
-        const int b0 = src_begin(s, p.T, p.S);
-        if (b0 >= t1) break;
-        const int b1 = src_begin(s + 1, p.T, p.S);
-        const bool beyond = b1 > t1;   // (only the last of them)
-        if (beyond) {
-            for (int e = dtid; e < p.E; e += dn) cnt[e] = 0u;
-            group_sync(bar, dn);
-            count_tokens(count_args(p), t1, b1, 0, false, cnt, dtid, dn);
-            group_sync(bar, dn);
-        }
-#pragma unroll 1
-        for (int e = dtid; e < p.E; e += dn) {
-            const int before = own_below(bmaps, e, b0 - t0);
-            p.cnt[(size_t)s * p.E + e] = own_below(bmaps, e, min(b1, t1) - t0) - before + (beyond ? (int)(cnt[e] >> 16) : 0);
-            p.src_offset[(size_t)s * p.E + e] = base[e] + before;
-        }
+    for (int i = dtid; i < (s_hi - s_lo) * p.E; i += dn) {
+        const int d = i / p.E, e = i - d * p.E, s = s_lo + d;
+        const int b0 = src_begin(s, p.T, p.S), b1 = src_begin(s + 1, p.T, p.S);
+        const int before = own_below(bmaps, e, b0 - t0);
+        p.cnt[(size_t)s * p.E + e] = own_below(bmaps, e, min(b1, t1) - t0) - before + (b1 > t1 ? (int)(cnt[e] >> 16) : 0);
+        p.src_offset[(size_t)s * p.E + e] = base[e] + before;
     }
 }
 
@@ -686,7 +712,7 @@ __device__ __forceinline__ int layout_group(Cta& x) {
         // rows, release the movers and write the metadata of the own tokens, while the other warps
         // (the duty group) already derive the expert-level outputs from the staged table.  (One after
         // the other, the expert-level outputs ended after the last copy and set the kernel's duration.)
-        constexpr int kRowWarps = 4, kRowThreads = kRowWarps * 32;
+        constexpr int kRowThreads = kRowWarps * 32;
         if (gw < kRowWarps) {
             const int rn = kRowThreads;
             local_rows_dedup(p, t0, t1, ids_sm, rm, c, order_sm, pos_raw, key, row_sm, arr, gtid, rn);
@@ -743,6 +769,8 @@ __device__ __forceinline__ int layout_group(Cta& x) {
                 epoch_finish_check_in(p, ticket, ep_mine);
                 if (p.trace) p.trace[(size_t)c * kTraceSlots + 12] = trace_ns(p);
             }
+            if (x.early0 && gw == 0) bulk_wait_all<0>();   // the first row's copies (issued by this warp)
+            x.rows_landed(0);
         } else if (kFp8 && warp - pl.q_warp0 < nq) {
             return 1;   // FP8 rows: the first warps behind the row group quantise as well
         } else {
@@ -751,8 +779,9 @@ __device__ __forceinline__ int layout_group(Cta& x) {
             const int dn = gn - dgw0 * 32, dw = nw - dgw0;
             const int Q = p.grid / p.R > 1 ? p.grid / p.R : 1;
             // ... once the movers are released: started earlier, these warps take issue slots and
-            // shared-memory bandwidth from the few threads every copy of this CTA is waiting for
-            const bool go = mbar_wait_idle(&ready_bar, 0, abortp);
+            // shared-memory bandwidth from the few threads every copy of this CTA is waiting for.  (Small tables: the
+            // copies end long before these outputs, which start at once.)
+            const bool go = p.T <= kEarlyDutyTokens || mbar_wait_idle(&ready_bar, 0, abortp);
             for (int u = c; go && u < p.R * Q; u += p.grid)
                 local_rank_duty(p, u / Q, u % Q, Q, ids_sm, rm, hist, gw - dgw0, dw, lane, gtid - dgw0 * 32, dn, 3);
             if (gtid == dgw0 * 32) trace(p, c, kTrScanned);   // deferred outputs written
@@ -1273,20 +1302,24 @@ __global__ void __launch_bounds__(kThreads, 1) dispatch_kernel(const Params p, c
           // (its stage is never loaded a second time, no order of destinations is asked for, a lane per copy)
           kMode == kModeLocal && p.local_fast != 0 && !kFp8 && !kSteal && !p.ordered && p.k <= 32 && t1 > t0 &&
               t1 - t0 <= stages,
-          0};
+          0, kMode == kModeCluster || (kMode == kModeLocal && p.local_fast != 0),
+          // the mover; the row group (rank-level rows, bf16) or the duty group (clusters); who issues FP8 copies
+          1 + (kMode == kModeCluster ? nw - (kFp8 && pl.q_long ? 1 : 0) : kFp8 ? 0 : kRowWarps) +
+              (kFp8 ? (pl.q_long ? 1 : pl.q_warps) : 0)};
 
     if (x.warp == 0) {
         mover_warp<kMode, kFp8, kSteal>(x);
     } else {
         const int lg = layout_group<kMode, kFp8, kSteal>(x);   // 0 = a wait ran out, 1 = done, 2 = left to quantise
-        if (!kFp8 && x.early0 && x.warp == 1) bulk_wait_all<0>();   // the first row's copies (issued by this warp)
         // (2: beside the rest of the layout; 1: after it, unless the quantising warps are others)
         const int qw = x.warp - pl.q_warp0;
         if (kFp8 && pl.q_long && lg == 1 && x.warp == 1) {
             fp8_store_issuer<kSteal>(x);
+            if (x.early_arrival) x.rows_landed(0);
         } else if (kFp8 && (lg == 2 || (lg == 1 && !beside)) && qw >= 0 && qw < pl.q_warps) {
             if (pl.q_long) fp8_quantiser<kSteal>(x, qw);
             else fp8_worker<kSteal>(x, qw);
+            if (x.early_arrival && !pl.q_long) x.rows_landed(0);
         }
     }
     if (kMode == kModeCluster) cluster_wait();   // the others have read what this CTA counted
@@ -1307,11 +1340,7 @@ __global__ void __launch_bounds__(kThreads, 1) dispatch_kernel(const Params p, c
         }
         return;
     }
-    // pieces of this CTA's rows have landed: add them to the per-region arrival counters
-    // (unit: eighths of a row, so that the total does not depend on the column split)
-    fence_proxy_async();   // rows written through the async proxy, counters through the generic one
-    for (int r = tid; r < p.R; r += kThreads)
-        if (arr[r]) red_release_add(p.arrival + half * p.R + r, (unsigned)(arr[r] * (8 / p.parts)));
+    if (!x.early_arrival) publish_arrivals(p, arr, half, tid, kThreads);
     // the arrival counters of the next call live in the other half; clear them now
     if (c == 0) {
         for (int r = tid; r < p.R; r += kThreads) p.arrival[(half ^ 1u) * p.R + r] = 0;

@@ -471,7 +471,8 @@ static __device__ void write_totals(const Params& p, const int* tot, const int* 
     }
     for (int r = gtid; r < p.R; r += gn) {
         p.num_tokens_per_rank[r] = tot[p.E + r];
-        p.num_rows_per_rank[r] = rows_of_rank(p, tot, r);
+        const int e1 = (r + 1) * p.L - 1;   // (eo: offset inside the region, so the last expert's end is its row count)
+        p.num_rows_per_rank[r] = p.dedup ? tot[p.E + r] : eo[e1] + tot[e1];
     }
 }
 
@@ -762,22 +763,18 @@ static __device__ void local_rank_duty(const Params& p, int r, int q, int Q, con
         }
         return c;
     };
-    int* tot = sm;
-    int* eo = sm + 32;
-    if (gtid <= L) tot[gtid] = bits(gtid, 0, T);
-    group_sync(bar_id, gn);
-    if (gtid <= L) {
-        int o = 0;
-#pragma unroll 1
-        for (int i = 0; i < gtid; ++i) o += tot[i];
-        eo[gtid] = o;
+    int* eo = sm;
+    if (gw == 0) {
+        const int tot = lane <= L ? bits(lane, 0, T) : 0;
+        const int o = warp_incl_scan(tot, lane) - tot;
+        eo[lane] = o;
         if (q == 0) {
-            if (gtid < L) {
-                p.expert_offset[r * L + gtid] = o;
-                p.num_tokens_per_expert[r * L + gtid] = tot[gtid];
-            } else {
-                p.num_tokens_per_rank[r] = tot[L];
-                p.num_rows_per_rank[r] = tot[L];
+            if (lane < L) {
+                p.expert_offset[r * L + lane] = o;
+                p.num_tokens_per_expert[r * L + lane] = tot;
+            } else if (lane == L) {
+                p.num_tokens_per_rank[r] = tot;
+                p.num_rows_per_rank[r] = tot;
             }
         }
     }
