@@ -255,8 +255,8 @@ Params make_params(ubep_buffer* b, int T) {
 // Cuts the work of a flag-free kernel over `ctas` CTAs: token chunks, and column parts of a row so that the slices
 // are balanced to about 5 %.  The CTA with the most work sets the pace: ceil(T / chunks) tokens of 1 / parts of a
 // row each.  Smaller pieces cost more per byte (measured on the decode shape, layout by every CTA alone: 4 parts + 8 to
-// 15 %, 8 parts + 60 %).  A CTA that has one token at most takes pieces down to 2 KB (16 tokens of 2048 bf16 channels:
-// 6.8 us whole, 7.1 in eight pieces; 7168 channels: 7.3 and 6.8).  Otherwise pieces are cut for balance only where
+// 15 %, 8 parts + 60 %).  A CTA that has one token at most takes pieces down to 1.5 KB (16 tokens of 2048 bf16
+// channels: 6.8 us whole, 7.1 in eight pieces; 7168 channels: 7.3 and 6.8).  Otherwise pieces are cut for balance only where
 // they keep 4 KB (512 tokens of 1024 channels, by clusters: 9.0 us whole, 10.4 in halves; 7168 channels: 16.3 and 15.3),
 // FP8 rows not at all (512 tokens of 7168 channels, by clusters: 13.3 and 16.4 us, every CTA alone: 13.1 and 14.9).
 void split_work(Params& p, int ctas) {
@@ -272,7 +272,7 @@ void split_work(Params& p, int ctas) {
         // the scales and payload pieces under 2 KB a dispatch of 384 tokens took 33 us against 21 us for 512
         if (p.payload && parts > 1 && ((p.G / parts) * 4) % 16 != 0) break;
         const int most = (p.T + chunks - 1) / chunks, piece = p.H * 2 / parts;
-        if (parts > 1 && (piece < (most > 1 ? 4096 : 2048) || (most > 1 && p.payload))) break;
+        if (parts > 1 && (piece < (most > 1 ? 4096 : 1536) || (most > 1 && p.payload))) break;
         const double cost = (double)most / parts * piece_penalty[i];
         if (parts == 1 || cost < best_cost * 0.999) {
             best = parts;

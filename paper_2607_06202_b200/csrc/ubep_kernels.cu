@@ -703,6 +703,8 @@ __device__ __forceinline__ int layout_group(Cta& x) {
         // rank-level rows first, movers released, expert-level outputs afterwards
         const RankMaps rm{bmaps.bm, bmaps.mask_t, (p.R + 31) / 32, ((p.R + 31) / 32) * 32, (p.T + 31) / 32};
         int* row_sm = reinterpret_cast<int*>(w_sm);
+        // (the own tokens' gate weights, asked for while the table is on its way; needed for the metadata)
+        const float w_row = !kFp8 && part == 0 && gw < kRowWarps && gtid < ntok * p.k ? __ldg(p.topk_w + (size_t)t0 * p.k + gtid) : 0.0f;
         local_stage_and_rank_maps(p, ids_sm, rm, rm.groups, warp, kWarps, lane);   // with the mover warp
         stage_small(gn);
         group_sync(2, kThreads);
@@ -759,7 +761,8 @@ __device__ __forceinline__ int layout_group(Cta& x) {
             }
             if (part == 0) {
                 float* w_own = reinterpret_cast<float*>(key);   // the ordering keys are no longer needed
-                for (int i = gtid; i < ntok * p.k; i += rn) w_own[i] = __ldg(p.topk_w + (size_t)t0 * p.k + i);
+                if (gtid < ntok * p.k) w_own[gtid] = w_row;
+                for (int i = gtid + rn; i < ntok * p.k; i += rn) w_own[i] = __ldg(p.topk_w + (size_t)t0 * p.k + i);
             }
             local_clean_own_duplicates(p, t0, t1, ids_sm, gtid, rn);   // (rank-level rows do not depend on them)
             group_sync(1, rn);
@@ -1560,11 +1563,11 @@ int plan_dispatch(const Params& p, int mode, int max_smem, SmemPlan* out) {
     pl.map_bp = pl.map_wb * 32;
     pl.stage_bytes = round_up_i(p.H * 2 / p.parts, 128);
     pl.out_stage_bytes = p.payload ? round_up_i(p.rowB / p.parts + (p.G / p.parts) * 4, 128) : 0;
-    const int64_t mask_ints = (int64_t)pl.map_groups * 32;
+    const bool fast = mode == kModeLocal && p.local_fast;
+    const int64_t mask_ints = (int64_t)(fast ? 2 * pl.map_groups + 1 : pl.map_groups) * 32;   // (fast: local_rank_duty)
     const int64_t bm_ints = (int64_t)pl.map_groups * pl.map_bp;
     const bool beside = p.payload && (mode == kModeCluster || (mode != kModeLocal && p.count_warps > 0));
     if (p.payload) {   // who quantises, and how (see Fp8Ring)
-        const bool fast = mode == kModeLocal && p.local_fast;
         pl.q_long = (int64_t)p.k * (p.rowB / p.parts) >= 40 * 1024 ? 1 : 0;
         pl.q_warp0 = beside ? (mode == kModeCluster ? kClusterCountWarps : p.count_warps) + 1 : pl.q_long ? 2 : 1;
         const int most = fast ? kFastQuantWarps + (pl.q_long ? 0 : 1) : kWarps - pl.q_warp0;
@@ -1609,7 +1612,7 @@ int plan_dispatch(const Params& p, int mode, int max_smem, SmemPlan* out) {
     int at = pl.stages * pl.stage_bytes;
     const int copies = p.k * (p.rowB / p.parts);
     pl.trip_rows = 1;
-    if (!p.payload && !p.steal && p.k <= 16 && chunk_tokens <= pl.stages && copies <= 16384)
+    if (!p.payload && !p.steal && p.k <= 16 && chunk_tokens > 2 && chunk_tokens <= pl.stages && copies <= 16384)
         pl.trip_rows = 32 / p.k < 32768 / copies ? 32 / p.k : 32768 / copies;
     pl.off_out = at; at += pl.out_stages * pl.out_stage_bytes;
     pl.off_ids = at; at += (int)ids_ints * 4;

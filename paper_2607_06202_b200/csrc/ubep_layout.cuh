@@ -654,27 +654,28 @@ static __device__ void local_rows_dedup(const Params& p, int t0, int t1, const i
     else rows_dedup_pass<0>(p, t0, t1, ids_all, rm, worker, order_sm, pos_raw, dst_key, row_sm, arr, gtid, gn);
 }
 
-// The ids of a token must be distinct: the later of two slots naming one expert is reported
-// (kErrBadIndex) and emptied.  In the flag-free kernel every CTA holds the whole table, but only two
-// things read expert ids from it: the metadata of the CTA's own tokens, for which this empties the
-// repeated slots of tokens [t0, t1) in the CTA's copy, and the per-rank duty, whose bitmaps take a
-// repeated expert once by construction (it reports it) and whose row lists write the same entry twice.
+// The later of two slots of a token that name one expert is reported (kErrBadIndex) and emptied, tokens [t0, t1); a
+// thread per slot.  (A slot beside it that still reads the old value is not misled: an expert's first slot stays.)
 static __device__ void local_clean_own_duplicates(const Params& p, int t0, int t1, int* ids_all, int gtid, int gn) {
-    const int k = p.k;
+    const int k = p.k, nslots = (t1 - t0) * k;
 #pragma unroll 1
-    for (int t = t0 + gtid; t < t1; t += gn) {
-        int* row = ids_all + (size_t)t * k;
+    for (int li = gtid; li < nslots; li += gn) {
+        const int tl = li / k, j = li - tl * k;
+        int* tok = ids_all + (size_t)(t0 + tl) * k;
+        const int v = tok[j];
+        bool dup = false;
+        if (k == 8) {
+            const int4 a = *reinterpret_cast<const int4*>(tok), b = *reinterpret_cast<const int4*>(tok + 4);
+            const int w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+            for (int jj = 0; jj < 7; ++jj) dup = dup || (jj < j && w[jj] == v);   // same expert => same packed word
+        } else {
 #pragma unroll 1
-        for (int j = 1; j < k; ++j) {
-            const int v = row[j];
-            if (v < 0) continue;
-            bool dup = false;
-#pragma unroll 1
-            for (int jj = 0; jj < j; ++jj) dup = dup || row[jj] == v;   // same expert => same packed word
-            if (dup) {
-                report(p.status, kErrBadIndex);
-                row[j] = -1;
-            }
+            for (int jj = 0; jj < j; ++jj) dup = dup || tok[jj] == v;
+        }
+        if (dup && v >= 0) {
+            report(p.status, kErrBadIndex);
+            tok[j] = -1;
         }
     }
 }
@@ -726,52 +727,61 @@ static __device__ void local_meta_dedup(const Params& p, int t0, int t1, const i
 
 // Everything about rank r that nobody inside the kernel waits for: expert totals and
 // offsets, tokens per rank, counts and offsets per source rank, the per-expert row lists.
-// Needs L < 32.  `sm` holds 2 * 32 ints.  Run by the whole layout group (barrier bar_id).
+// Needs L < 32.  `eo` holds 32 ints.  Run by the duty group (barrier bar_id).
 // The rank's share is cut into Q parts handled by Q different CTAs: part q writes every
 // Q-th entry of the per-source tables and of the row lists; part 0 also writes the totals.
+// For small tables this is what the kernel's end waits for: the counts below a token come from a table of counts per
+// group of 32 tokens instead of a walk over the groups (128 tokens: 2.8 us with the walk, 512 tokens 6.6).
 static __device__ void local_rank_duty(const Params& p, int r, int q, int Q, const int* ids_all, const RankMaps& rm,
-                                int* sm, int gw, int nw, int lane, int gtid, int gn, int bar_id) {
-    const int k = p.k, L = p.L, T = p.T, S = p.S, E = p.E;
+                                int* eo, int gw, int nw, int lane, int gtid, int gn, int bar_id) {
+    const int k = p.k, L = p.L, T = p.T, S = p.S, E = p.E, e0 = r * L;
+    unsigned* const dbm = rm.dbm;                                        // [groups, 32]
+    int* const pre = reinterpret_cast<int*>(rm.dbm + rm.groups * 32);    // [groups + 1, 32] tokens of earlier groups
+    bool twice = false;
 #pragma unroll 1
     for (int g = gw; g < rm.groups; g += nw) {
         const int t = g * 32 + lane;
         unsigned m = 0u;
-        if (t < T)
-#pragma unroll 1
-            for (int j = 0; j < k; ++j) {
-                const int v = ids_all[(size_t)t * k + j];
-                if (v >= 0 && slot_rank(v) == r) {
-                    const unsigned bit = 1u << (slot_expert(v) - r * L);
-                    if (m & bit) report(p.status, kErrBadIndex);   // an expert named twice by this token
-                    m |= bit | (1u << L);
+        auto add = [&](int v) {
+            if (slot_rank(v) != r) return;   // (-1 >> 16 is no rank)
+            const unsigned bit = 1u << (slot_expert(v) - e0);
+            twice = twice || (m & bit) != 0u;   // an expert named twice by this token
+            m |= bit;
+        };
+        if (t < T) {
+            const int* tok = ids_all + (size_t)t * k;
+            if ((k & 3) == 0) {
+#pragma unroll 2
+                for (int j = 0; j < k; j += 4) {
+                    const int4 v = *reinterpret_cast<const int4*>(tok + j);
+                    add(v.x); add(v.y); add(v.z); add(v.w);
                 }
+            } else {
+#pragma unroll 1
+                for (int j = 0; j < k; ++j) add(tok[j]);
             }
-        rm.dbm[(size_t)g * 32 + lane] = transpose32(m, lane);
+            if (m) m |= 1u << L;
+        }
+        dbm[g * 32 + lane] = transpose32(m, lane);
     }
+    if (twice) report(p.status, kErrBadIndex);
     group_sync(bar_id, gn);
     if (p.trace && gtid == 0) p.trace[(size_t)blockIdx.x * kTraceSlots + 13] = trace_ns(p);
-    auto bits = [&](int l, int lo, int hi) {   // tokens in [lo, hi) with bit l
-        if (hi <= lo) return 0;
-        const int g0 = lo >> 5, g1 = (hi - 1) >> 5;
-        int c = 0;
-#pragma unroll 1
-        for (int g = g0; g <= g1; ++g) {
-            unsigned w = rm.dbm[(size_t)g * 32 + l];
-            if (g == g0) w &= 0xffffffffu << (lo & 31);
-            if (g == g1 && (hi & 31) != 0) w &= (1u << (hi & 31)) - 1u;
-            c += __popc(w);
-        }
-        return c;
-    };
-    int* eo = sm;
     if (gw == 0) {
-        const int tot = lane <= L ? bits(lane, 0, T) : 0;
+        int tot = 0;
+#pragma unroll 8
+        for (int g = 0; g < rm.groups; ++g) {
+            const int c = __popc(dbm[g * 32 + lane]);
+            pre[g * 32 + lane] = tot;
+            tot += c;
+        }
+        pre[rm.groups * 32 + lane] = tot;
         const int o = warp_incl_scan(tot, lane) - tot;
         eo[lane] = o;
         if (q == 0) {
             if (lane < L) {
-                p.expert_offset[r * L + lane] = o;
-                p.num_tokens_per_expert[r * L + lane] = tot;
+                p.expert_offset[e0 + lane] = o;
+                p.num_tokens_per_expert[e0 + lane] = tot;
             } else if (lane == L) {
                 p.num_tokens_per_rank[r] = tot;
                 p.num_rows_per_rank[r] = tot;
@@ -779,24 +789,31 @@ static __device__ void local_rank_duty(const Params& p, int r, int q, int Q, con
         }
     }
     group_sync(bar_id, gn);
+    // tokens below t with bit l (t = T on a group's edge reads a word of pre[], of which no bit is taken)
+    auto below = [&](int l, int t) {
+        const int i = (t >> 5) * 32 + l;
+        return pre[i] + __popc(dbm[i] & ((1u << (t & 31)) - 1u));
+    };
 #pragma unroll 1
     for (int i = q + Q * gtid; i < S * L; i += Q * gn) {
         const int s = i / L, l = i - s * L;
-        const int b0 = src_begin(s, T, S), b1 = src_begin(s + 1, T, S);
-        p.cnt[(size_t)s * E + r * L + l] = bits(l, b0, b1);
-        p.src_offset[(size_t)s * E + r * L + l] = eo[l] + bits(l, 0, b0);
+        const int before = below(l, src_begin(s, T, S));
+        p.cnt[(size_t)s * E + e0 + l] = below(l, src_begin(s + 1, T, S)) - before;
+        p.src_offset[(size_t)s * E + e0 + l] = eo[l] + before;
     }
     if (p.trace && gtid == 0) p.trace[(size_t)blockIdx.x * kTraceSlots + 14] = trace_ns(p);
+    bool full = false;
 #pragma unroll 1
     for (int i = q + Q * gtid; i < T * k; i += Q * gn) {
         const int v = ids_all[i];
-        if (v < 0 || slot_rank(v) != r) continue;
-        const int t = i / k, l = slot_expert(v) - r * L;
-        const int at = eo[l] + bits(l, 0, t);
-        if (at < p.er_cap) p.expert_rows[(size_t)r * p.er_cap + at] = bits(L, 0, t);
-        else report(p.status, kErrCapacity);
+        if (slot_rank(v) != r) continue;
+        const int t = i / k, l = slot_expert(v) - e0;
+        const int at = eo[l] + below(l, t);
+        if (at < p.er_cap) p.expert_rows[(size_t)r * p.er_cap + at] = below(L, t);
+        else full = true;
     }
-    group_sync(bar_id, gn);   // sm and dbm are reused by the next rank
+    if (full) report(p.status, kErrCapacity);
+    group_sync(bar_id, gn);   // eo and the maps are reused by the next rank
 }
 
 // Per token, put the destinations into the order of the destination-ordering table rotated
