@@ -187,4 +187,30 @@ __device__ __forceinline__ int own_below(const BinMaps& m, int bin, int tl) {
     return c;
 }
 
+// What the source ranks whose tokens begin among [t0, t1) report (cnt, src_offset).  base[e]: rows before the CTA's
+// tokens in expert e's segment.  Tokens of the last such rank beyond the CTA's own are counted from the table into
+// cnt (E + R + 1 words).  Run by n threads that share barrier `bar`.
+static __device__ void write_own_sources(const Params& p, int t0, int t1, const BinMaps& bmaps, const int* base, unsigned* cnt,
+                                         int tid, int n, int bar) {
+    // source ranks s_lo .. s_hi - 1
+    const int s_lo = (int)(((int64_t)t0 * p.S + p.T - 1) / p.T);
+    const int s_hi = min(p.S, (int)(((int64_t)t1 * p.S + p.T - 1) / p.T));
+    if (s_hi <= s_lo) return;
+    const int last_end = src_begin(s_hi, p.T, p.S);
+    if (last_end > t1) {
+        for (int e = tid; e < p.E; e += n) cnt[e] = 0u;
+        group_sync(bar, n);
+        count_tokens(count_args(p), t1, last_end, 0, false, cnt, tid, n);
+        group_sync(bar, n);
+    }
+#pragma unroll 1
+    for (int i = tid; i < (s_hi - s_lo) * p.E; i += n) {
+        const int d = i / p.E, e = i - d * p.E, s = s_lo + d;
+        const int b0 = src_begin(s, p.T, p.S), b1 = src_begin(s + 1, p.T, p.S);
+        const int before = own_below(bmaps, e, b0 - t0);
+        p.cnt[(size_t)s * p.E + e] = own_below(bmaps, e, min(b1, t1) - t0) - before + (b1 > t1 ? (int)(cnt[e] >> 16) : 0);
+        p.src_offset[(size_t)s * p.E + e] = base[e] + before;
+    }
+}
+
 }  // namespace ubep

@@ -566,7 +566,7 @@ int ubep_dispatch_sync(ubep_buffer_t* buf, int protocol, const void* x, const in
     // Small tables are recounted by every CTA; for larger ones TokenCnt and CalCumSum run as launches of their
     // own in front of the kernel, over the same chunks (as the phased schedule of ubep_dispatch does).
     const bool whole_table = (int64_t)T * buf->cfg.topk <= kLocalMaxSlots &&
-                             ubep::plan_dispatch(p, UBEP_PIPELINE_LOCAL, buf->max_smem - extra, &pl) == 0;
+                             ubep::plan_dispatch(p, ubep::kModeCluster, buf->max_smem - extra, &pl) == 0;   // (a cluster of one)
     if (!whole_table && ubep::plan_dispatch(p, UBEP_PIPELINE_PHASED, buf->max_smem - extra, &pl) != 0)
         return UBEP_ERR_ARG;
     const WireLayout& w = buf->wlay;

@@ -655,26 +655,7 @@ __device__ __forceinline__ void cluster_duty(Cta& x, int dtid, int dn, int bar) 
     x.rows_landed(0);
     if (c == 0) write_totals(p, tot, eo, dtid, dn);
     if (part != 0 || ntok == 0) return;
-    // source ranks s_lo .. s_hi - 1 begin among the own tokens
-    const int s_lo = (int)(((int64_t)t0 * p.S + p.T - 1) / p.T);
-    const int s_hi = min(p.S, (int)(((int64_t)t1 * p.S + p.T - 1) / p.T));
-    if (s_hi <= s_lo) return;
-    const int last_end = src_begin(s_hi, p.T, p.S);
-    const bool beyond = last_end > t1;   // (only the last of them reaches beyond the own tokens)
-    if (beyond) {
-        for (int e = dtid; e < p.E; e += dn) cnt[e] = 0u;
-        group_sync(bar, dn);
-        count_tokens(count_args(p), t1, last_end, 0, false, cnt, dtid, dn);
-        group_sync(bar, dn);
-    }
-#pragma unroll 1
-    for (int i = dtid; i < (s_hi - s_lo) * p.E; i += dn) {
-        const int d = i / p.E, e = i - d * p.E, s = s_lo + d;
-        const int b0 = src_begin(s, p.T, p.S), b1 = src_begin(s + 1, p.T, p.S);
-        const int before = own_below(bmaps, e, b0 - t0);
-        p.cnt[(size_t)s * p.E + e] = own_below(bmaps, e, min(b1, t1) - t0) - before + (b1 > t1 ? (int)(cnt[e] >> 16) : 0);
-        p.src_offset[(size_t)s * p.E + e] = base[e] + before;
-    }
+    write_own_sources(p, t0, t1, bmaps, base, cnt, dtid, dn, bar);
 }
 
 // ---------------------------------------------------------------------- layout group

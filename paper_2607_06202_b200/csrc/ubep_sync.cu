@@ -6,12 +6,12 @@
 // (grid <= number of SMs, one CTA per SM).
 //
 // The layout (TokenCnt, CalCumSum, slot -> row) is derived by every CTA alone from the
-// whole routing table, with the same device functions and in the same order as the
-// flag-free instance of the main dispatch kernel, so the two paths leave identical
-// metadata in the arena.
+// whole routing table, by the counting functions of the layout by clusters (a cluster of one), so the two
+// paths leave identical metadata in the arena.  (From bitmaps of every bin over the whole table it took 7.4 us at
+// 128 tokens and 21.7 us at 900; this way MEASURED_LAYOUT.)
 //
 // A DataBlock is the 16 bytes one thread stores with a single 128-bit access.
-#include "ubep_layout.cuh"
+#include "ubep_cluster.cuh"
 #include "ubep_quant.cuh"
 #include "ubep_sync.h"
 
@@ -22,6 +22,8 @@ namespace {
 constexpr int kSW = 0, kTFF = 1, kDC = 2, kSP = 3;
 constexpr int kDcBlockVecs = 32;    // 512-byte checksum block = 32 vectors of 16 bytes
 constexpr int kDcMarkerVecs = 2;    // its leading 32 bytes are the marker
+constexpr int kStrip = 256;         // DataBlocks a warp of a receiver looks at together: eight loads in flight per lane
+constexpr int kStripWords = kStrip * 3;   // payload words of a Token-Flag strip
 
 __device__ __forceinline__ uint4 ld_relaxed_v4(const void* ptr) {
     uint4 v;
@@ -92,6 +94,11 @@ __device__ __forceinline__ bool wait_count(const unsigned* ctr, unsigned want, W
     return true;
 }
 
+__host__ __device__ inline int qrow_bytes(const Params& p) { return p.payload ? ((p.H + 4 * p.G + 15) / 16) * 16 : 0; }
+__host__ __device__ inline bool strips_in_ring(const Params& p) {   // (a plan has four rows at least, two for FP8 rows)
+    return (p.payload ? 2 : 4) * 2 * p.H >= kWarps * kStripWords * 4;
+}
+
 // kFp8: rows travel quantised (e4m3 payload, then the fp32 scales of the row's 128-channel groups, as one
 // wire row of H + 4 * H / 128 bytes); the sender quantises a row once into shared memory and sends from
 // there; what arrives goes to the payload and the scale array of the receive region.  The checksum
@@ -120,6 +127,9 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
     int* order_sm = reinterpret_cast<int*>(smem + pl.off_order);
     unsigned long long* chk_sm = reinterpret_cast<unsigned long long*>(smem + pl.total);   // DC: [R]
     uint8_t* qrow = smem + pl.total + (((size_t)p.R * 8 + 15) & ~(size_t)15);              // FP8: the quantised row
+    // TFF: [kWarps, kStripWords]; in the ring of rows, which the receiver no longer needs, where that is large enough
+    uint32_t* strips = reinterpret_cast<uint32_t*>(strips_in_ring(p) ? smem : qrow + qrow_bytes(p));
+    __shared__ __align__(8) uint64_t row_bar[2];   // the row of an even / odd token has landed in ring stage 0 / 1
     const BinMaps bmaps{reinterpret_cast<unsigned*>(smem + pl.off_mask), reinterpret_cast<unsigned*>(smem + pl.off_bm),
                         pl.map_wb, pl.map_bp, pl.map_groups};
     const int t0 = (int)chunk_begin(c, p.T, p.nchunks), t1 = (int)chunk_begin(c + 1, p.T, p.nchunks);
@@ -138,26 +148,63 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
     }
     if (kProto == kDC)
         for (int r = tid; r < R; r += kThreads) chk_sm[r] = 0ull;
+    auto fetch_row = [&](int tl) {   // one thread; the row before the last one has been sent
+        mbar_arrive_expect_tx(&row_bar[tl & 1], (unsigned)p.H * 2u);
+        bulk_load(smem + (size_t)(tl & 1) * pl.stage_bytes, p.x + (size_t)(t0 + tl) * p.H, (unsigned)p.H * 2u, &row_bar[tl & 1]);
+    };
+    if (tid == 32) {
+        mbar_init(&row_bar[0], 1);
+        mbar_init(&row_bar[1], 1);
+        mbar_fence_init();
+        if (ntok > 0) fetch_row(0);   // on its way while the layout is computed
+        if (ntok > 1) fetch_row(1);
+    }
 
-    // ---- layout: bitmaps of every bin over the whole routing table -> totals, the rows
-    // before this CTA's tokens, expert offsets, rows of this CTA's slots
+    // ---- layout: counts of every bin over the whole routing table -> totals, the rows before this CTA's tokens,
+    // expert offsets, rows of this CTA's slots
     int* tot = hist;
-    int* pre = hist + p.B;
+    int* base = hist + p.B;   // rows before the CTA's tokens in the bin's segment
     int* eo = hist + 2 * p.B;
-    if (kTable) stage_ids(p, 0, p.T, ids_sm, tid, kThreads);
-    else stage_ids(p, t0, t1, ids_sm, tid, kThreads);
+    unsigned* cnt = reinterpret_cast<unsigned*>(smem + pl.off_cnt);   // (kTable)
+    unsigned* own = cnt + p.B + 1;
+    bool twice = false;
+    if (kTable) {
+        for (int b = tid; b < 2 * (p.B + 1); b += kThreads) cnt[b] = 0u;
+        for (int b = tid; b < pl.map_groups * pl.map_bp; b += kThreads) bmaps.bm[b] = 0u;
+        __syncthreads();
+        twice = stage_own(p, t0, t1, ids_sm, bmaps.bm, bmaps.bp, own, kThreads - 1 - tid, kThreads);
+        count_tokens(count_args(p), 0, p.T, t0, true, cnt, tid, kThreads);
+    } else {
+        stage_ids(p, t0, t1, ids_sm, tid, kThreads);
+    }
     for (int r = tid; r < R; r += kThreads) order_sm[r] = __ldg(p.order_pos + r);
     for (int i = tid; i < ntok * k; i += kThreads) w_sm[i] = __ldg(p.topk_w + (size_t)t0 * k + i);
-    __syncthreads();
+    if (__syncthreads_or(twice)) {
+        local_clean_own_duplicates(p, 0, ntok, ids_sm, tid, kThreads);
+        __syncthreads();
+    }
     const unsigned seq = seq_sm;
     const int par = (int)(seq & 1u);
     if (kTable) {
-        local_counts_all_bins(p, ids_sm, bmaps, t0, tot, pre, eo, tid, kThreads, warp, kWarps, lane, 0);
-        for (int r = tid; r < R; r += kThreads) nrows[r] = rows_of_rank(p, tot, r);
+        for (int b = tid; b < p.B; b += kThreads) {
+            tot[b] = (int)(cnt[b] >> 16);
+            base[b] = (int)(cnt[b] & 0xffffu);
+        }
         __syncthreads();
-        finalize_chunk(p, t0, t1, ids_sm + (size_t)t0 * k, w_sm,
-                       [&](int e, int tl) { return eo[e] + pre[e] + bits_in_range(bmaps, e, t0, t0 + tl); },
-                       [&](int r, int tl) { return pre[p.E + r] + bits_in_range(bmaps, p.E + r, t0, t0 + tl); },
+        for (int e = tid; e < p.E; e += kThreads) {
+            int o = 0;
+            for (int q = (e / p.L) * p.L; q < e; ++q) o += tot[q];
+            eo[e] = o;
+            base[e] += o;
+        }
+        __syncthreads();
+        for (int r = tid; r < R; r += kThreads) {
+            const int e1 = (r + 1) * p.L - 1;
+            nrows[r] = p.dedup ? tot[p.E + r] : eo[e1] + tot[e1];
+        }
+        finalize_chunk(p, t0, t1, ids_sm, w_sm,
+                       [&](int e, int tl) { return base[e] + own_below(bmaps, e, tl); },
+                       [&](int r, int tl) { return base[p.E + r] + own_below(bmaps, p.E + r, tl); },
                        true, c, order_sm, pos, key, nullptr, tid, kThreads);
     } else {
         build_bin_maps(p, ids_sm, ntok, bmaps, warp, kWarps, lane);
@@ -173,12 +220,6 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
     }
     __syncthreads();
     if (tid == 0) times[1] = global_ns();
-    if (kTable) {
-        // counts and offsets nobody inside this kernel waits for (the launches before wrote them otherwise)
-        if (c == 0) write_totals(p, tot, eo, tid, kThreads);
-        for (int s = c; s < p.S; s += p.grid) write_source_from_maps(p, s, bmaps, eo, tid, kThreads);
-    }
-
     // ---- sender: the rows of tokens [t0, t1), one token at a time, all threads on a row
     const int wbytes = kFp8 ? p.H + 4 * p.G : p.rowB;   // bytes of one row on the wire
     const int nvec = (wbytes + 15) / 16;                // its 16-byte blocks (FP8: the last may be cut short)
@@ -193,16 +234,20 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
         if (!kFp8 || w < pwords) reinterpret_cast<uint32_t*>(p.recv_x + where * p.rowB)[w] = val;
         else reinterpret_cast<uint32_t*>(p.recv_scale + where * p.G)[w - pwords] = val;
     };
+    bool lost = false;   // a row did not come: what is sent is not it, and the call reports the timeout
+    if (wire_unusable)
+        for (int tl = 0; tl < min(2, ntok); ++tl) (void)mbar_wait(&row_bar[tl], 0, nullptr);
     for (int tl = 0; tl < ntok && !wire_unusable; ++tl) {
         const int* ps = pos + tl * k;
-        const uint4* xrow = reinterpret_cast<const uint4*>(p.x + (size_t)(t0 + tl) * p.H);
+        const uint4* xrow = reinterpret_cast<const uint4*>(smem + (size_t)(tl & 1) * pl.stage_bytes);
+        lost = !mbar_wait(&row_bar[tl & 1], (tl >> 1) & 1, nullptr) || lost;
         if (kFp8) {
             // quantise the row once (every copy carries the same bytes)
             const int xvec = p.H / 8;
             for (int v0 = 0; v0 < xvec; v0 += kThreads) {   // same trip count for every thread (the quantiser shuffles)
                 const int v = v0 + tid;
                 const bool in = v < xvec;
-                const uint4 d = in ? __ldg(xrow + v) : make_uint4(0, 0, 0, 0);
+                const uint4 d = in ? xrow[v] : make_uint4(0, 0, 0, 0);
                 uint2 q;
                 float scale;
                 quantize8(d, in, q, scale);
@@ -220,9 +265,9 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
                 const int w0 = 3 * g;
                 uint4 blk;
                 blk.x = seq;   // the flag leads the block
-                blk.y = w0 < nwords ? (kFp8 ? xw[w0] : __ldg(xw + w0)) : 0u;
-                blk.z = w0 + 1 < nwords ? (kFp8 ? xw[w0 + 1] : __ldg(xw + w0 + 1)) : 0u;
-                blk.w = w0 + 2 < nwords ? (kFp8 ? xw[w0 + 2] : __ldg(xw + w0 + 2)) : 0u;
+                blk.y = w0 < nwords ? xw[w0] : 0u;
+                blk.z = w0 + 1 < nwords ? xw[w0 + 1] : 0u;
+                blk.w = w0 + 2 < nwords ? xw[w0 + 2] : 0u;
                 for (int j = 0; j < k; ++j) {
                     const int where = ps[j];
                     if (where >= 0) st_relaxed_v4(sp.tff_wire + (size_t)where * wire_row + (size_t)g * 16, blk);
@@ -231,7 +276,7 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
         } else {
             unsigned long long mine = 0ull;
             for (int v = tid; v < nvec; v += kThreads) {
-                const uint4 d = kFp8 ? reinterpret_cast<const uint4*>(qrow)[v] : __ldg(xrow + v);
+                const uint4 d = kFp8 ? reinterpret_cast<const uint4*>(qrow)[v] : xrow[v];
                 if (kProto == kDC && v < pvec && (v % kDcBlockVecs) < kDcMarkerVecs) mine += marker_words(d);
                 for (int j = 0; j < k; ++j) {
                     const int where = ps[j];
@@ -266,8 +311,10 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
                 if (tid < k && ps[tid] >= 0) red_release_add(sp.sw_rows + par * R + ps[tid] / p.cap, 1u);
             }
         }
-        if (kFp8) __syncthreads();   // the quantised row is reused for the next token
+        if (kFp8 || tl + 2 < ntok) __syncthreads();   // the quantised row and the row's buffer are used again
+        if (tid == 32 && tl + 2 < ntok) fetch_row(tl + 2);
     }
+    if (lost) report(p.status, kErrTimeout);
     if (kProto == kDC) {
         // one fence per sender and batch, then the checksum packet of every region
         __threadfence();
@@ -278,67 +325,104 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
         }
     }
     if (tid == 0) times[2] = global_ns();
+    if (kTable) {
+        // counts and offsets nobody inside this kernel waits for (the launches before wrote them otherwise); behind the
+        // rows, which the receivers wait for
+        if (c == 0) write_totals(p, tot, eo, tid, kThreads);
+        write_own_sources(p, t0, t1, bmaps, base, cnt + 2 * (p.B + 1), tid, kThreads, 0);
+    }
+    if (kProto == kTFF) __syncthreads();   // (the strips may lie where the rows were)
 
-    // ---- receiver: region u / Q, slice u % Q of its rows
+    // ---- receiver
     Waiter wt{&abort_flag, global_ns() + kWaitLimitNs, p.status, kProto == kSP ? sp.sp_dirty : nullptr};
     const int Q = p.grid / R > 1 ? p.grid / R : 1;
     bool duty = false;
+    if (kProto == kTFF || kProto == kSP) {
+        // Every CTA takes an equal share of all rows of all regions, a warp kStrip DataBlocks of a row at a time: its
+        // lanes look at neighbouring blocks, with all loads of the strip in flight before any of them is looked at.  What a Token-Flag strip carries passes through shared
+        // memory, so that it leaves in 16-byte stores.  (Four blocks per thread in flight and three 4-byte stores
+        // per block: 12.5 us from the last row sent to the last one confirmed at 128 tokens, now MEASURED_RX.)
+        constexpr int kBatch = kStrip / 32;
+        const int per_row = kProto == kTFF ? sp.tff_blocks : nvec;
+        const int strips_per_row = (per_row + kStrip - 1) / kStrip;
+        const size_t row_stride = kProto == kTFF ? wire_row : sp_row;
+        const uint4 sentinel = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
+        uint32_t* const mine = strips + (kProto == kTFF ? warp * kStripWords : 0);
+        long long all = 0;
+        for (int r = 0; r < R; ++r) all += nrows[r] < p.cap ? nrows[r] : p.cap;
+        const long long from = all * c / p.grid, to = all * (c + 1) / p.grid;   // this CTA's share
+        duty = to > from;
+        long long first = 0;   // rows of the regions before r
+        bool ok = true;
+        for (int r = 0; r < R && first < to && ok; ++r) {
+            const int n_r = nrows[r] < p.cap ? nrows[r] : p.cap;
+            const int lo = (int)(from > first ? (from - first < n_r ? from - first : n_r) : 0);
+            const int hi = (int)(to - first < n_r ? to - first : n_r);
+            first += n_r;
+            for (int i = warp; ok && i < (hi - lo) * strips_per_row; i += kWarps) {
+                const int row = lo + i / strips_per_row, g0 = (i % strips_per_row) * kStrip;
+                const size_t grow = (size_t)r * p.cap + row;
+                uint8_t* const wire = (kProto == kTFF ? sp.tff_wire : sp.sp_wire) + grow * row_stride + (size_t)g0 * 16;
+                const int n = min(kStrip, per_row - g0);   // blocks of this strip
+                uint4 blk[kBatch];
+                unsigned missing = 0u;   // bit b: this lane's b-th block has not arrived
+#pragma unroll
+                for (int b = 0; b < kBatch; ++b) missing |= b * 32 + lane < n ? 1u << b : 0u;
+                unsigned spins = 0;
+                for (;;) {   // (all missing blocks side by side: one after the other a late strip cost eight round trips)
+#pragma unroll
+                    for (int b = 0; b < kBatch; ++b)
+                        if (missing >> b & 1u) blk[b] = ld_relaxed_v4(wire + (size_t)(b * 32 + lane) * 16);
+#pragma unroll
+                    for (int b = 0; b < kBatch; ++b)
+                        if ((missing >> b & 1u) && !(kProto == kTFF ? blk[b].x != seq : is_sentinel(blk[b]))) missing &= ~(1u << b);
+                    if (missing == 0u) break;
+                    if (!wt.keep_waiting(spins)) { ok = false; break; }
+                }
+#pragma unroll
+                for (int b = 0; b < kBatch; ++b) {
+                    const int g = b * 32 + lane;
+                    if (g >= n || (missing >> b & 1u)) continue;
+                    if (kProto == kTFF) {
+                        mine[3 * g] = blk[b].y;
+                        mine[3 * g + 1] = blk[b].z;
+                        mine[3 * g + 2] = blk[b].w;
+                    } else {
+                        const int v = g0 + g;
+                        if (!kFp8 || v < pvec) {
+                            *reinterpret_cast<uint4*>(p.recv_x + grow * p.rowB + (size_t)v * 16) = blk[b];
+                        } else {
+                            const uint32_t dw[4] = {blk[b].x, blk[b].y, blk[b].z, blk[b].w};
+                            for (int q = 0; q < 4; ++q)
+                                if (4 * v + q < nwords) put_word(grow, 4 * v + q, dw[q]);
+                        }
+                        st_relaxed_v4(wire + (size_t)g * 16, sentinel);   // consumed: ready for the next call
+                    }
+                }
+                ok = __all_sync(0xffffffffu, ok);
+                if (kProto == kTFF) {
+                    // words [3 * g0, 3 * g0 + 3 * n) of the wire row (a strip begins on a multiple of four words)
+                    for (int q = lane; ok && q < kStripWords / 4; q += 32) {
+                        const int w = 3 * g0 + 4 * q;
+                        if (4 * q >= 3 * n || w >= nwords) break;
+                        const uint4 d = *reinterpret_cast<const uint4*>(mine + 4 * q);
+                        if (w + 4 <= pwords) {
+                            *reinterpret_cast<uint4*>(p.recv_x + grow * p.rowB + (size_t)w * 4) = d;
+                        } else {   // (scales; the words behind the row's last block are not written)
+                            const uint32_t dw[4] = {d.x, d.y, d.z, d.w};
+                            for (int z = 0; z < 4; ++z)
+                                if (w + z < nwords) put_word(grow, w + z, dw[z]);
+                        }
+                    }
+                    __syncwarp();   // the strip's buffer is used again
+                }
+            }
+        }
+    }
     for (int u = c; u < R * Q; u += p.grid) {
         const int r = u / Q, q = u % Q;
         const int n_r = nrows[r] < p.cap ? nrows[r] : p.cap;
-        if (kProto == kTFF || kProto == kSP) {
-            const int lo = (int)((long long)n_r * q / Q), hi = (int)((long long)n_r * (q + 1) / Q);
-            duty = duty || hi > lo;
-            // The slice's DataBlocks as one index space; every thread keeps kBatch loads in
-            // flight and only then looks at what they brought (a block that has not arrived
-            // is polled on its own).
-            constexpr int kBatch = 4;
-            const int per_row = kProto == kTFF ? sp.tff_blocks : nvec;
-            const size_t row_stride = kProto == kTFF ? wire_row : sp_row;
-            uint8_t* const wire = (kProto == kTFF ? sp.tff_wire : sp.sp_wire) + ((size_t)r * p.cap + lo) * row_stride;
-            const size_t row0 = (size_t)r * p.cap + lo;   // global row of the slice's first row
-            const int items = (hi - lo) * per_row;
-            const uint4 sentinel = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
-            bool ok = true;
-            for (int i0 = tid; ok && i0 < items && !*wt.abort; i0 += kBatch * kThreads) {
-                uint4 blk[kBatch];
-                int row[kBatch], g[kBatch];
-#pragma unroll
-                for (int b = 0; b < kBatch; ++b) {
-                    const int i = i0 + b * kThreads;
-                    row[b] = i / per_row;
-                    g[b] = i - row[b] * per_row;
-                    if (i < items) blk[b] = ld_relaxed_v4(wire + row[b] * row_stride + (size_t)g[b] * 16);
-                }
-#pragma unroll
-                for (int b = 0; b < kBatch; ++b) {
-                    if (i0 + b * kThreads >= items) break;
-                    uint8_t* const src = wire + row[b] * row_stride + (size_t)g[b] * 16;
-                    unsigned spins = 0;
-                    while (kProto == kTFF ? blk[b].x != seq : is_sentinel(blk[b])) {
-                        if (!wt.keep_waiting(spins)) { ok = false; break; }
-                        blk[b] = ld_relaxed_v4(src);
-                    }
-                    if (!ok) break;
-                    const size_t grow = row0 + row[b];
-                    if (kProto == kTFF) {
-                        const int w0 = 3 * g[b];
-                        if (w0 < nwords) put_word(grow, w0, blk[b].y);
-                        if (w0 + 1 < nwords) put_word(grow, w0 + 1, blk[b].z);
-                        if (w0 + 2 < nwords) put_word(grow, w0 + 2, blk[b].w);
-                    } else {
-                        if (!kFp8 || g[b] < pvec) {
-                            *reinterpret_cast<uint4*>(p.recv_x + grow * p.rowB + (size_t)g[b] * 16) = blk[b];
-                        } else {
-                            const uint32_t dw[4] = {blk[b].x, blk[b].y, blk[b].z, blk[b].w};
-                            for (int i = 0; i < 4; ++i)
-                                if (4 * g[b] + i < nwords) put_word(grow, 4 * g[b] + i, dw[i]);
-                        }
-                        st_relaxed_v4(src, sentinel);   // consumed: ready for the next call
-                    }
-                }
-            }
-        } else if (q == 0) {
+        if (kProto != kTFF && kProto != kSP && q == 0) {
             duty = true;
             if (kProto == kSW) {
                 if (tid == 0) (void)wait_count(sp.sw_rows + par * R + r, (unsigned)n_r, wt);
@@ -416,8 +500,7 @@ cudaError_t launch_one(const Params& p, const SmemPlan& pl, const SyncParams& sp
 }  // namespace
 
 int sync_extra_smem(const Params& p) {
-    const int qrow = p.payload ? ((p.H + 4 * p.G + 15) / 16) * 16 : 0;   // FP8: the quantised row of the token being sent
-    return p.R * 8 + 128 + qrow + 16;
+    return p.R * 8 + 128 + qrow_bytes(p) + 16 + (strips_in_ring(p) ? 0 : kWarps * kStripWords * 4);
 }
 
 cudaError_t launch_sync_dispatch(const Params& p, const SmemPlan& pl, const SyncParams& sp, bool whole_table,
