@@ -60,8 +60,9 @@ __device__ __forceinline__ int counted_expert(const CountArgs& p, int t, int raw
 // Written for few instructions: this runs once per launch, so what it costs first of all is fetching its code (a
 // first form, which collected a token's slots in 32-bit words of bins and transposed them, was 600 instructions
 // and took 5 us for its first 32 tokens).  The adds are cheap: 3.6 cycles per warp for random bins.
+// Tokens of [lo2, hi2) are counted into cnt2[] as well (all << 16, experts only).
 static __device__ __noinline__ void count_tokens(const CountArgs p, int lo, int hi, int split, bool ranks, unsigned* cnt,
-                                                 int tid, int n) {
+                                                 int tid, int n, int lo2 = 0, int hi2 = 0, unsigned* cnt2 = nullptr) {
     const int k = p.k;
     const bool words = k == 8 || k == 4;   // a token's ids are whole 16-byte words (topk_idx is 16-byte aligned)
     const int none = p.E + p.R;
@@ -118,6 +119,11 @@ static __device__ __noinline__ void count_tokens(const CountArgs p, int lo, int 
             }
 #pragma unroll
             for (int j = 0; j < 8; ++j) atomicAdd(cnt + (e[j] >= 0 ? e[j] : none), inc);
+            if (t >= lo2 && t < hi2) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (e[j] >= 0) atomicAdd(cnt2 + e[j], 0x10000u);
+            }
             if (ranks) {   // a rank counts a token once: with the first of the slots that name it
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
@@ -141,6 +147,7 @@ static __device__ __noinline__ void count_tokens(const CountArgs p, int lo, int 
                 e[j] = v;
                 if (v < 0) continue;
                 atomicAdd(cnt + v, inc);
+                if (t >= lo2 && t < hi2) atomicAdd(cnt2 + v, 0x10000u);
                 if (!ranks) continue;
                 const int r = p.L == 1 ? v : fast_div(v, p.L_magic);
                 bool first = true;
@@ -189,7 +196,11 @@ __device__ __forceinline__ int own_below(const BinMaps& m, int bin, int tl) {
 
 // What the source ranks whose tokens begin among [t0, t1) report (cnt, src_offset).  base[e]: rows before the CTA's
 // tokens in expert e's segment.  Tokens of the last such rank beyond the CTA's own are counted from the table into
-// cnt (E + R + 1 words).  Run by n threads that share barrier `bar`.
+// cnt (E + R + 1 words), unless that has been done.  Run by n threads that share barrier `bar`.
+__device__ __forceinline__ int own_sources_end(const Params& p, int t1) {   // first token beyond the source ranks that begin below t1
+    return src_begin(min(p.S, (int)(((int64_t)t1 * p.S + p.T - 1) / p.T)), p.T, p.S);
+}
+template <bool kCounted>
 static __device__ void write_own_sources(const Params& p, int t0, int t1, const BinMaps& bmaps, const int* base, unsigned* cnt,
                                          int tid, int n, int bar) {
     // source ranks s_lo .. s_hi - 1
@@ -197,7 +208,7 @@ static __device__ void write_own_sources(const Params& p, int t0, int t1, const 
     const int s_hi = min(p.S, (int)(((int64_t)t1 * p.S + p.T - 1) / p.T));
     if (s_hi <= s_lo) return;
     const int last_end = src_begin(s_hi, p.T, p.S);
-    if (last_end > t1) {
+    if (!kCounted && last_end > t1) {
         for (int e = tid; e < p.E; e += n) cnt[e] = 0u;
         group_sync(bar, n);
         count_tokens(count_args(p), t1, last_end, 0, false, cnt, tid, n);

@@ -655,7 +655,7 @@ __device__ __forceinline__ void cluster_duty(Cta& x, int dtid, int dn, int bar) 
     x.rows_landed(0);
     if (c == 0) write_totals(p, tot, eo, dtid, dn);
     if (part != 0 || ntok == 0) return;
-    write_own_sources(p, t0, t1, bmaps, base, cnt, dtid, dn, bar);
+    write_own_sources<false>(p, t0, t1, bmaps, base, cnt, dtid, dn, bar);
 }
 
 // ---------------------------------------------------------------------- layout group

@@ -169,11 +169,11 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
     unsigned* own = cnt + p.B + 1;
     bool twice = false;
     if (kTable) {
-        for (int b = tid; b < 2 * (p.B + 1); b += kThreads) cnt[b] = 0u;
+        for (int b = tid; b < 3 * (p.B + 1); b += kThreads) cnt[b] = 0u;
         for (int b = tid; b < pl.map_groups * pl.map_bp; b += kThreads) bmaps.bm[b] = 0u;
         __syncthreads();
         twice = stage_own(p, t0, t1, ids_sm, bmaps.bm, bmaps.bp, own, kThreads - 1 - tid, kThreads);
-        count_tokens(count_args(p), 0, p.T, t0, true, cnt, tid, kThreads);
+        count_tokens(count_args(p), 0, p.T, t0, true, cnt, tid, kThreads, t1, t1 > t0 ? own_sources_end(p, t1) : t1, cnt + 2 * (p.B + 1));
     } else {
         stage_ids(p, t0, t1, ids_sm, tid, kThreads);
     }
@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
         // counts and offsets nobody inside this kernel waits for (the launches before wrote them otherwise); behind the
         // rows, which the receivers wait for
         if (c == 0) write_totals(p, tot, eo, tid, kThreads);
-        write_own_sources(p, t0, t1, bmaps, base, cnt + 2 * (p.B + 1), tid, kThreads, 0);
+        write_own_sources<true>(p, t0, t1, bmaps, base, cnt + 2 * (p.B + 1), tid, kThreads, 0);
     }
     if (kProto == kTFF) __syncthreads();   // (the strips may lie where the rows were)
 
