@@ -196,17 +196,17 @@ __device__ __forceinline__ int own_below(const BinMaps& m, int bin, int tl) {
 
 // What the source ranks whose tokens begin among [t0, t1) report (cnt, src_offset).  base[e]: rows before the CTA's
 // tokens in expert e's segment.  Tokens of the last such rank beyond the CTA's own are counted from the table into
-// cnt (E + R + 1 words), unless that has been done.  Run by n threads that share barrier `bar`.
+// cnt (E + R + 1 words), unless that has been done.  The column parts of a chunk share its source ranks.  Run by n threads that share barrier `bar`.
 __device__ __forceinline__ int own_sources_end(const Params& p, int t1) {   // first token beyond the source ranks that begin below t1
     return src_begin(min(p.S, (int)(((int64_t)t1 * p.S + p.T - 1) / p.T)), p.T, p.S);
 }
 template <bool kCounted>
-static __device__ void write_own_sources(const Params& p, int t0, int t1, const BinMaps& bmaps, const int* base, unsigned* cnt,
+static __device__ void write_own_sources(const Params& p, int t0, int t1, int part, int parts, const BinMaps& bmaps, const int* base, unsigned* cnt,
                                          int tid, int n, int bar) {
     // source ranks s_lo .. s_hi - 1
     const int s_lo = (int)(((int64_t)t0 * p.S + p.T - 1) / p.T);
     const int s_hi = min(p.S, (int)(((int64_t)t1 * p.S + p.T - 1) / p.T));
-    if (s_hi <= s_lo) return;
+    if (s_hi - s_lo <= part) return;
     const int last_end = src_begin(s_hi, p.T, p.S);
     if (!kCounted && last_end > t1) {
         for (int e = tid; e < p.E; e += n) cnt[e] = 0u;
@@ -215,12 +215,14 @@ static __device__ void write_own_sources(const Params& p, int t0, int t1, const 
         group_sync(bar, n);
     }
 #pragma unroll 1
-    for (int i = tid; i < (s_hi - s_lo) * p.E; i += n) {
-        const int d = i / p.E, e = i - d * p.E, s = s_lo + d;
+    for (int s = s_lo + part; s < s_hi; s += parts) {
         const int b0 = src_begin(s, p.T, p.S), b1 = src_begin(s + 1, p.T, p.S);
-        const int before = own_below(bmaps, e, b0 - t0);
-        p.cnt[(size_t)s * p.E + e] = own_below(bmaps, e, min(b1, t1) - t0) - before + (b1 > t1 ? (int)(cnt[e] >> 16) : 0);
-        p.src_offset[(size_t)s * p.E + e] = base[e] + before;
+#pragma unroll 1
+        for (int e = tid; e < p.E; e += n) {
+            const int before = own_below(bmaps, e, b0 - t0);
+            p.cnt[(size_t)s * p.E + e] = own_below(bmaps, e, min(b1, t1) - t0) - before + (b1 > t1 ? (int)(cnt[e] >> 16) : 0);
+            p.src_offset[(size_t)s * p.E + e] = base[e] + before;
+        }
     }
 }
 

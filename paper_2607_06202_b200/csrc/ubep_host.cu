@@ -25,25 +25,27 @@ constexpr int kStealMinTokensPerChunk = 40;  // shorter slices: the hand-out cos
 constexpr int kDefaultCountWarps = 8;            // FP8: warps of the count group while the others quantise (measured sweep;
                                                  // -1 in the buffer = this default, and none with token stealing)
 constexpr int64_t kLocalMaxSlots = 8192;        // small-T limit of the combine launch mode and of the protocol / sharded paths
-// AUTO: up to which size every CTA derives the layout alone; larger tables are counted by clusters of CTAs.  Measured on
-// seven shape families; the figures are dispatches alone, every CTA alone against clusters of two.
-// One row per (token, rank): the work per CTA grows with the tokens; the more bytes a token has, the more of it is
-// hidden behind the copies (7168 channels: 1536 tokens 34.5 and 35.8 us, 2048 tokens 48.8 and 47.0; 4096 channels: 512
-// tokens 11.1 and 11.6, 1024 tokens 16.7 and 16.1; 1024 channels: 512 tokens 9.2 and 9.4, 1024 tokens 12.2 and 10.7).
-// FP8 rows have fewer (7168 channels: 512 tokens 13.1 and 13.4, 768 tokens 18.2 and 16.2).  More than 32 ranks take
-// more words per token (72 ranks, bf16 512 tokens 15.8 and 15.6, FP8 128 tokens 9.7 and 10.1, 512 tokens 16.5 and 14.0).
+// AUTO: up to which size every CTA derives the layout alone (one row per (token, rank)); larger tables are counted by
+// clusters of CTAs.  Measured on six shape families; the figures are dispatches alone, every CTA alone against the better of
+// clusters of one and two.  bf16 rows: 1536 tokens of 7168 channels 35.1 and 35.8 us, of 4096 20.1 and 21.0, of 1024 10.0 and
+// 12.4, but 2048 tokens of 7168 channels 48.8 and 47.0; rows below 1 KB: 1024 tokens 7.7 and 8.4, 1536 9.4 and 8.7.  More than
+// 32 ranks take more words per token (72 ranks: 512 tokens 15.4 and 16.3, 768 21.7 and 21.5).  FP8 rows: long ones are quantised by
+// fewer warps here (7168 channels: 64 tokens 7.9 and 8.7, 200 tokens 10.7 and 9.9); short ones 1024 tokens 10.5 and 11.7, 72
+// ranks 64 tokens 10.7 and 9.2.
 int local_fast_max_tokens(const Params& p) {
-    if (p.payload) return p.R > 32 ? 224 : 544;
-    const int by_bytes = p.H * 2 / 9;
-    return p.R > 32 || by_bytes < 448 ? 448 : by_bytes;
+    if (p.payload) return p.R > 32 ? 32 : p.k * p.H >= 40 * 1024 ? 128 : 1152;
+    return p.R > 32 ? 640 : p.H < 512 ? 1152 : 1600;
 }
-// One row per (token, expert), bf16 rows, in tokens * bins (8 tokens, 288 bins: 7.5 and 7.9 us, 32 tokens: 7.7 and 7.4;
-// 64 tokens, 136 bins: 7.2 and 7.6, 256 tokens: 10.1 and 8.2; 512 tokens, 20 bins: 7.9 and 8.2, 1024 tokens: 10.5
-// and 8.5).  FP8 rows: by clusters throughout.
-constexpr int64_t kLocalAllBinsMax = 9000;
-// Cluster sizes: two up to 32 K slots, eight from 64 K on (dispatch + combine, sizes 2 / 4 / 8: 24576 slots 88.2 / 88.8 /
-// 90.2 us, 32768 slots 150 / 151 / 152, 65536 slots 213 / 212 / 209, 131072 slots 555 / 555 / 544).
-constexpr int64_t kCluster2MaxSlots = 32768, kCluster8MinSlots = 65536;
+// CTAs per cluster.  Larger clusters count their share of the table sooner and cost a cluster barrier and CTAs (of a B200's
+// 148 SMs 132 can be used in clusters of four, 120 in clusters of eight).  Short rows are over soon, so that the counting
+// shows (1024 channels, top-4, sizes 1 / 2 / 4: 333 tokens 7.4 / 7.5 / 7.7 us, 512 tokens 8.5 / 7.9 / 7.7, 1536 tokens 14.4 / 11.3 / 9.9);
+// with long ones it hides behind the copies (7168 channels: 512 tokens 14.7 / 15.3 / 16.6, 1536 tokens 37.6 / 37.8 / 37.6; dispatch +
+// combine, sizes 2 / 4 / 8: 4096 tokens 150 / 151 / 152, 8192 tokens of 4096 channels 213 / 212 / 209, 16384 tokens 555 / 555 / 544).
+int cluster_size(const Params& p) {
+    const int64_t slots = (int64_t)p.T * p.k;
+    if (p.H * 2 < 8192) return p.T <= 448 ? 1 : 4;
+    return p.T <= 1280 ? 1 : slots <= 32768 ? 2 : slots < 65536 ? 4 : 8;
+}
 inline size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
 struct ArenaLayout {
@@ -446,34 +448,32 @@ int ubep_dispatch(ubep_buffer_t* buf, const void* x, const int32_t* topk_idx, co
     p.parts = 1;
     p.grid = p.nchunks;
     const int n = buf->lay.nchunks;
-    const int64_t slots = (int64_t)T * p.k;
-    if (mode == UBEP_PIPELINE_AUTO) {
-        // With the rank-level fast path, and for the smallest tables, every CTA derives what it needs alone; beyond
-        // that clusters of CTAs count the table between them (larger clusters cost CTAs: of a B200's 148 SMs 132
-        // can be used in clusters of four, 120 in clusters of eight).
-        mode = UBEP_PIPELINE_FUSED;
-        const bool alone = p.local_fast ? T <= local_fast_max_tokens(p) : !p.payload && (int64_t)T * p.B <= kLocalAllBinsMax;
-        if (alone) {
-            mode = UBEP_PIPELINE_LOCAL;
-        } else {
-            const int cs = slots <= kCluster2MaxSlots ? 2 : slots < kCluster8MinSlots ? 4 : 8;
-            int ctas = ubep::cluster_ctas(cs, buf->max_smem);
-            ctas = (ctas < n ? ctas : n) / cs * cs;
-            if (ctas > 0 && T <= 65535) {   // (counts are 16 bits wide)
-                p.cluster = cs;
-                p.steal = T >= kStealMinTokensPerChunk * ctas ? 1 : 0;
-                if (p.steal) p.nchunks = p.grid = ctas;   // whole rows are handed out
-                else split_work(p, ctas);
-                if (ubep::plan_dispatch(p, ubep::kModeCluster, buf->max_smem, &pl) == 0) mode = ubep::kModeCluster;
-                else p.cluster = 1;
-            }
-        }
-    }
-    if (mode == UBEP_PIPELINE_LOCAL) {
+    // by clusters of cs CTAs, if that fits
+    auto by_cluster = [&](int cs) {
+        int ctas = cs > 1 ? ubep::cluster_ctas(cs, buf->max_smem) : n;
+        ctas = (ctas < n ? ctas : n) / cs * cs;
+        if (ctas <= 0 || T > 65535) return false;   // (counts are 16 bits wide)
+        p.cluster = cs;
+        p.steal = T >= kStealMinTokensPerChunk * ctas ? 1 : 0;
+        if (p.steal) { p.parts = 1; p.nchunks = p.grid = ctas; }   // whole rows are handed out
+        else split_work(p, ctas);
+        if (ubep::plan_dispatch(p, ubep::kModeCluster, buf->max_smem, &pl) == 0) return true;
+        p.cluster = 1;
+        p.steal = 0;
+        return false;
+    };
+    auto alone = [&]() {   // rank-level rows, every CTA from the whole table
         split_work(p, n);
-        if (ubep::plan_dispatch(p, mode, buf->max_smem, &pl) != 0) {
-            if (buf->cfg.pipeline == UBEP_PIPELINE_LOCAL) return UBEP_ERR_ARG;
-            mode = UBEP_PIPELINE_FUSED;   // table too large for shared memory
+        return ubep::plan_dispatch(p, UBEP_PIPELINE_LOCAL, buf->max_smem, &pl) == 0;
+    };
+    if (mode == UBEP_PIPELINE_AUTO) {
+        if (p.local_fast && T <= local_fast_max_tokens(p) && alone()) mode = UBEP_PIPELINE_LOCAL;
+        else mode = by_cluster(cluster_size(p)) ? ubep::kModeCluster : UBEP_PIPELINE_FUSED;
+    } else if (mode == UBEP_PIPELINE_LOCAL) {
+        if (!alone()) return UBEP_ERR_ARG;   // table too large for shared memory
+        if (!p.local_fast) {   // every bin has to be counted: a cluster of one (which keeps the table nowhere)
+            if (!by_cluster(1)) return UBEP_ERR_ARG;
+            mode = ubep::kModeCluster;
         }
     }
     if (mode == UBEP_PIPELINE_FUSED || mode == UBEP_PIPELINE_PHASED) {

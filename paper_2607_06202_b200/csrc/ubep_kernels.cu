@@ -7,7 +7,10 @@
 //                                     layout steps of different CTAs are ordered by
 //                                     release/acquire flags instead of launches (kernel
 //                                     decomposition).  LOCAL: every CTA derives its offsets
-//                                     from the whole routing table (small T*k, no flags).
+//                                     from the whole routing table (small T*k, no flags), rank-level
+//                                     rows.  Clusters (ubep_cluster.cuh): the CTAs of a cluster
+//                                     count the table between them; a cluster of one for small
+//                                     tables with one row per (token, expert).
 //   combine_kernel<K>                 gather + fp32 weighted sum + one bf16 rounding
 //   layout_kernel<K, W>               counts only (ubep_get_dispatch_layout)
 #include <atomic>
@@ -62,7 +65,6 @@ struct Cta {
     unsigned epoch, in_bytes, out_bytes;   // (epoch: 0 until the role that needs it has learnt it from *epoch_late)
     unsigned* epoch_late;
     size_t in_off, out_off;
-    bool fast_local;
     bool early0;  // flag-free kernel: the copies of the CTA's first row are issued by the warp that assigns the rows
     int issued;   // rows whose load the mover has started (thread 0's copy is used when leaving early)
     bool early_arrival;   // the mover warp publishes the arrival counters
@@ -100,7 +102,6 @@ struct Cta {
     [[maybe_unused]] int* const order_sm = (x).order_sm;                                                     \
     [[maybe_unused]] const unsigned epoch = (x).epoch, in_bytes = (x).in_bytes, out_bytes = (x).out_bytes;   \
     [[maybe_unused]] const size_t in_off = (x).in_off, out_off = (x).out_off;                                \
-    [[maybe_unused]] const bool fast_local = (x).fast_local;                                                 \
     [[maybe_unused]] int& issued = (x).issued;                                                               \
     /* layout group: warps 1 .. nw; a compile-time constant where it is always all 15 */                    \
     [[maybe_unused]] const int nw = (all15) ? kWarps - 1 : (x).nw;                                           \
@@ -266,7 +267,7 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
         // Flag-free kernel: the routing table first, the rows after it.  The table is the one load the
         // whole layout waits for; the rows of 148 CTAs queued in front of it cost about a microsecond.
         const RankMaps rm{bmaps.bm, bmaps.mask_t, (p.R + 31) / 32, ((p.R + 31) / 32) * 32, (p.T + 31) / 32};
-        if (fast_local) {
+        if (kMode == kModeLocal) {
             // Two rows are asked for at once, so that the first copies find their row in shared memory when
             // the movers are released; then this warp lends a hand with the routing table and asks for the
             // rest of the ring.  (More than two rows in front of the table delay it, 148 CTAs' worth of them
@@ -289,9 +290,6 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
             issued = head;
             cluster_wait();
             cluster_arrive();    // (this warp reads nothing of the others)
-            ok = mbar_wait(x.staged_bar, 0, abortp);
-            ok = __all_sync(0xffffffffu, ok);
-        } else if (kMode == kModeLocal) {
             ok = mbar_wait(x.staged_bar, 0, abortp);
             ok = __all_sync(0xffffffffu, ok);
         }
@@ -373,7 +371,7 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
             }
         }
     } else {
-        if (fast_local) {
+        if (kMode == kModeLocal) {
             const RankMaps rm{bmaps.bm, bmaps.mask_t, (p.R + 31) / 32, ((p.R + 31) / 32) * 32, (p.T + 31) / 32};
             local_stage_and_rank_maps(p, ids_sm, rm, rm.groups, 0, kWarps, lane);   // the table first, the rows after it
             group_sync(2, kThreads);
@@ -386,7 +384,7 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
             cluster_arrive();
             ok = mbar_wait(x.staged_bar, 0, abortp);
             ok = __all_sync(0xffffffffu, ok);
-        } else if (kMode == kModeLocal || x.beside) {
+        } else if (x.beside) {
             // the routing table first: it is the one load the layout waits for
             ok = mbar_wait(x.staged_bar, 0, abortp);
             ok = __all_sync(0xffffffffu, ok);
@@ -461,7 +459,7 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
             }
         }
     }
-    if (kFp8 && fast_local && ok) {
+    if (kFp8 && kMode == kModeLocal && ok) {
         // metadata of the CTA's own tokens (see the row group): one warp, no barrier but its own
         ok = mbar_wait(&ready_bar, 0, abortp);
         ok = __all_sync(0xffffffffu, ok);
@@ -654,8 +652,7 @@ __device__ __forceinline__ void cluster_duty(Cta& x, int dtid, int dn, int bar) 
     }
     x.rows_landed(0);
     if (c == 0) write_totals(p, tot, eo, dtid, dn);
-    if (part != 0 || ntok == 0) return;
-    write_own_sources<false>(p, t0, t1, bmaps, base, cnt, dtid, dn, bar);
+    if (ntok != 0) write_own_sources<false>(p, t0, t1, part, p.parts, bmaps, base, cnt, dtid, dn, bar);
 }
 
 // ---------------------------------------------------------------------- layout group
@@ -670,7 +667,7 @@ __device__ __forceinline__ int layout_group(Cta& x) {
     // Small global reads whose values are needed only after the first barriers: issue the
     // loads now (first trip of each loop), store to shared memory after the ids are staged.
     const int order_r = kMode != kModeCluster && gtid < p.R ? __ldg(p.order_pos + gtid) : 0;
-    const bool stage_w = kMode != kModeCluster && !(kMode == kModeLocal && p.local_fast);
+    const bool stage_w = kMode != kModeCluster && kMode != kModeLocal;
     const float w_first = (stage_w && gtid < ntok * p.k) ? __ldg(p.topk_w + (size_t)t0 * p.k + gtid) : 0.0f;
     auto stage_small = [&](int n) {   // by n threads
         if (gtid < p.R) order_sm[gtid] = order_r;
@@ -680,7 +677,7 @@ __device__ __forceinline__ int layout_group(Cta& x) {
             for (int i = gtid + n; i < ntok * p.k; i += n) w_sm[i] = __ldg(p.topk_w + (size_t)t0 * p.k + i);
         }
     };
-    if (kMode == kModeLocal && p.local_fast) {
+    if (kMode == kModeLocal) {
         // rank-level rows first, movers released, expert-level outputs afterwards
         const RankMaps rm{bmaps.bm, bmaps.mask_t, (p.R + 31) / 32, ((p.R + 31) / 32) * 32, (p.T + 31) / 32};
         int* row_sm = reinterpret_cast<int*>(w_sm);
@@ -764,48 +761,13 @@ __device__ __forceinline__ int layout_group(Cta& x) {
             const int Q = p.grid / p.R > 1 ? p.grid / p.R : 1;
             // ... once the movers are released: started earlier, these warps take issue slots and
             // shared-memory bandwidth from the few threads every copy of this CTA is waiting for.  (Small tables: the
-            // copies end long before these outputs, which start at once.)
-            const bool go = p.T <= kEarlyDutyTokens || mbar_wait_idle(&ready_bar, 0, abortp);
+            // copies end long before these outputs, which start at once; not with FP8 rows, which have to be quantised.)
+            const bool go = (!kFp8 && p.T <= kEarlyDutyTokens) || mbar_wait_idle(&ready_bar, 0, abortp);
             for (int u = c; go && u < p.R * Q; u += p.grid)
                 local_rank_duty(p, u / Q, u % Q, Q, ids_sm, rm, hist, gw - dgw0, dw, lane, gtid - dgw0 * 32, dn, 3);
             if (gtid == dgw0 * 32) trace(p, c, kTrScanned);   // deferred outputs written
             if (kFp8) return go ? 3 : 0;   // (these warps do not quantise: the row group's warps do)
         }
-    } else if (kMode == kModeLocal) {
-        // every CTA: bitmaps over the whole routing table -> totals, the rows before its
-        // own tokens, and (CTAs with a source-rank duty) that rank's counts
-        int* tot = hist;
-        int* pre = hist + p.B;
-        int* eo = hist + 2 * p.B;
-        stage_ids(p, 0, p.T, ids_sm, gtid, gn);
-        stage_small(gn);
-        group_sync(1, gn);
-        if (gtid == 0) {
-            mbar_arrive(x.staged_bar);   // the mover may fetch rows now
-            trace(p, c, kTrCounted);
-        }
-        local_counts_all_bins(p, ids_sm, bmaps, t0, tot, pre, eo, gtid, gn, gw, nw, lane, 1);
-        if (gtid == 0) trace(p, c, kTrScanSeen);
-        ids = ids_sm + (size_t)t0 * p.k;
-        finalize_chunk(p, t0, t1, ids, w_sm,
-                       [&](int e, int tl) { return eo[e] + pre[e] + bits_in_range(bmaps, e, t0, t0 + tl); },
-                       [&](int r, int tl) { return pre[p.E + r] + bits_in_range(bmaps, p.E + r, t0, t0 + tl); },
-                       part == 0, c, order_sm, pos_raw, key, arr, gtid, gn);
-        group_sync(1, gn);
-        if (gtid == 0) trace(p, c, kTrFinalized);
-        if (p.ordered) {   // a destination table is set: the copies of a token in its order (else pos_raw is pos)
-            order_destinations(p, pos_raw, key, pos, ntok * p.k, gtid, gn);
-            group_sync(1, gn);
-        }
-        if (gtid == 0) {
-            mbar_arrive(&ready_bar);
-            trace(p, c, kTrReady);
-            *x.epoch_late = read_epoch_and_check_in(p);   // nothing needs it before the kernel's last lines
-        }
-        // outputs nobody inside this kernel waits for
-        if (c == 0) write_totals(p, tot, eo, gtid, gn);
-        if (part == 0)
-            for (int s = ch; s < p.S; s += p.nchunks) write_source_from_maps(p, s, bmaps, eo, gtid, gn);   // source ranks this CTA reports
     } else if (kMode == kModeCluster) {
         cluster_layout<kFp8, kSteal>(x);
         if (kFp8 && gw >= nw) return 2;   // off to quantise
@@ -1282,11 +1244,10 @@ __global__ void __launch_bounds__(kThreads, 1) dispatch_kernel(const Params p, c
                   pl.map_wb, pl.map_bp, pl.map_groups},
           reinterpret_cast<int*>(smem + pl.off_hist), arr, reinterpret_cast<int*>(smem + pl.off_order),
           epoch, in_bytes, out_bytes, &epoch_sm, (size_t)part * in_bytes, (size_t)part * out_bytes,
-          kMode == kModeLocal && p.local_fast != 0,
           // (its stage is never loaded a second time, no order of destinations is asked for, a lane per copy)
-          kMode == kModeLocal && p.local_fast != 0 && !kFp8 && !kSteal && !p.ordered && p.k <= 32 && t1 > t0 &&
+          kMode == kModeLocal && !kFp8 && !kSteal && !p.ordered && p.k <= 32 && t1 > t0 &&
               t1 - t0 <= stages,
-          0, kMode == kModeCluster || (kMode == kModeLocal && p.local_fast != 0),
+          0, kMode == kModeCluster || kMode == kModeLocal,
           // the mover; the row group (rank-level rows, bf16) or the duty group (clusters); who issues FP8 copies
           1 + (kMode == kModeCluster ? nw - (kFp8 && pl.q_long ? 1 : 0) : kFp8 ? 0 : kRowWarps) +
               (kFp8 ? (pl.q_long ? 1 : pl.q_warps) : 0)};

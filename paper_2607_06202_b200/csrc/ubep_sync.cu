@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
         // counts and offsets nobody inside this kernel waits for (the launches before wrote them otherwise); behind the
         // rows, which the receivers wait for
         if (c == 0) write_totals(p, tot, eo, tid, kThreads);
-        write_own_sources<true>(p, t0, t1, bmaps, base, cnt + 2 * (p.B + 1), tid, kThreads, 0);
+        write_own_sources<true>(p, t0, t1, 0, 1, bmaps, base, cnt + 2 * (p.B + 1), tid, kThreads, 0);
     }
     if (kProto == kTFF) __syncthreads();   // (the strips may lie where the rows were)
 
