@@ -47,8 +47,10 @@ enum { UBEP_PAYLOAD_BF16 = 0, UBEP_PAYLOAD_FP8_E4M3 = 1 };
 
 /* How ubep_dispatch schedules its steps. */
 enum {
-    UBEP_PIPELINE_AUTO = 0,   /* LOCAL for small routing tables (how small depends on whether */
-                              /* the one-row-per-rank fast path applies), else FUSED          */
+    UBEP_PIPELINE_AUTO = 0,   /* LOCAL for small routing tables with one row per (token, rank), */
+                              /* otherwise one kernel in which clusters of CTAs count the table */
+                              /* between them (no waits between clusters); FUSED where neither  */
+                              /* fits                                                         */
     UBEP_PIPELINE_PHASED = 1, /* count -> prefix sums -> scatter as three launches; the        */
                               /* kernel boundaries play the role of the global barriers of    */
                               /* the bulk-synchronous dispatch (Sec. 2.3, phases 2-5)         */
@@ -283,8 +285,7 @@ int ubep_map_workers(const int32_t *order /*[dev]*/, const int32_t *counts /*[de
  * Table 3); Token-Flag blocks and Sentinel blocks are cut from that, the checksum markers from the
  * payload.  What arrives goes to the region's payload and scale arrays.
  *
- * Routing tables of any size: up to 8192 slots (T * k), and while the table with the bitmaps of all its
- * bins (T x (E + R) bits) fits in a CTA's shared memory, every CTA derives the layout from the whole
+ * Routing tables of any size: up to 8192 slots (T * k) every CTA derives the layout from the whole
  * table, as UBEP_PIPELINE_LOCAL does (one launch); for a larger table the counting and prefix-sum
  * kernels of UBEP_PIPELINE_PHASED run in front of the protocol kernel (three launches).  One CTA per SM at most, launched
  * cooperatively (receivers wait for senders of the same grid, so the grid must be resident at once:
