@@ -21,7 +21,8 @@ namespace {
 std::atomic<uint64_t> g_launches{0};
 
 constexpr size_t kAlign = 256;
-constexpr int kStealMinTokensPerChunk = 40;  // shorter slices: the hand-out costs more than the tail it removes (measured)
+constexpr int kStealMinTokensPerChunk = 40;  // shorter slices: the hand-out costs more than the tail it removes (measured);
+                                             // so it does for short rows (8192 tokens of 1024 channels, top-4: 73 us, without 27)
 constexpr int kDefaultCountWarps = 8;            // FP8: warps of the count group while the others quantise (measured sweep;
                                                  // -1 in the buffer = this default, and none with token stealing)
 constexpr int64_t kLocalMaxSlots = 8192;        // small-T limit of the combine launch mode and of the protocol / sharded paths
@@ -43,7 +44,7 @@ int local_fast_max_tokens(const Params& p) {
 // combine, sizes 2 / 4 / 8: 4096 tokens 150 / 151 / 152, 8192 tokens of 4096 channels 213 / 212 / 209, 16384 tokens 555 / 555 / 544).
 int cluster_size(const Params& p) {
     const int64_t slots = (int64_t)p.T * p.k;
-    if (p.H * 2 < 8192) return p.T <= 448 ? 1 : 4;
+    if (p.H * 2 < 8192) return p.T <= 448 ? 1 : p.T <= 1536 ? 4 : 8;
     return p.T <= 1280 ? 1 : slots <= 32768 ? 2 : slots < 65536 ? 4 : 8;
 }
 inline size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
@@ -454,8 +455,9 @@ int ubep_dispatch(ubep_buffer_t* buf, const void* x, const int32_t* topk_idx, co
         ctas = (ctas < n ? ctas : n) / cs * cs;
         if (ctas <= 0 || T > 65535) return false;   // (counts are 16 bits wide)
         p.cluster = cs;
-        p.steal = T >= kStealMinTokensPerChunk * ctas ? 1 : 0;
-        if (p.steal) { p.parts = 1; p.nchunks = p.grid = ctas; }   // whole rows are handed out
+        p.parts = 1;
+        p.steal = T >= kStealMinTokensPerChunk * ctas && !ubep::short_rows(p) ? 1 : 0;
+        if (p.steal) p.nchunks = p.grid = ctas;   // whole rows are handed out
         else split_work(p, ctas);
         if (ubep::plan_dispatch(p, ubep::kModeCluster, buf->max_smem, &pl) == 0) return true;
         p.cluster = 1;
@@ -481,7 +483,7 @@ int ubep_dispatch(ubep_buffer_t* buf, const void* x, const int32_t* topk_idx, co
         p.nchunks = n;
         p.grid = n;
         // slices that are long enough are handed out in blocks so that faster SMs can take over the tail of slower ones
-        p.steal = T >= kStealMinTokensPerChunk * p.nchunks ? 1 : 0;
+        p.steal = T >= kStealMinTokensPerChunk * p.nchunks && !ubep::short_rows(p) ? 1 : 0;
         // With token stealing the count group is not used unless asked for: measured equal at top-8 and slower at
         // top-4 (16384 tokens: 161 against 174 us) -- every hand-out is a round trip that idle quantising warps do not hide.
         if (p.steal && buf->count_warps < 0) p.count_warps = 0;

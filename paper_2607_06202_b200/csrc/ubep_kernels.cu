@@ -117,22 +117,36 @@ __device__ __forceinline__ void publish_arrivals(const Params& p, const int* arr
         if (arr[r]) red_release_add(p.arrival + half * p.R + r, (unsigned)(arr[r] * (8 / p.parts)));
 }
 
-// Short rows, all of them in the ring (row n in stage n): `rows` of them at once, a lane per copy.  (A trip costs 0.4 us
-// however few bytes it sends; rows with 32 KB of copies take longer than that by themselves.  Dispatch of 1536
-// tokens, 1024 channels, top-4: 11.4 us, one row at a time 14.3.)  Out of line: the code of long rows stays short.
-static __device__ __noinline__ bool send_short_rows(int n0, int ntok, int rows, int k, uint64_t* full_bar, const int* pos,
-                                                    const uint8_t* smem, int stage_bytes, uint8_t* dst, int rowB,
-                                                    unsigned bytes, volatile int* abort) {
+// Short rows (row n in ring stage n % stages; the first `head` of them are on their way): `rows` of them at once, a lane
+// per copy.  (A trip costs 0.4 us however few bytes it sends; rows with 32 KB of copies take longer than that by
+// themselves.  Dispatch of 1536 tokens, 1024 channels, top-4: 11.4 us, one row at a time 14.3.)  Out of line: the code
+// of long rows stays short.  Returns how many loads were issued, negative if a wait gave up.
+static __device__ __noinline__ int send_short_rows(int n0, int ntok, int head, int rows, int stages, int k, uint64_t* full_bar,
+                                                   const int* pos, uint8_t* smem, int stage_bytes, uint8_t* dst, int rowB,
+                                                   unsigned bytes, const uint8_t* src, size_t src_stride, unsigned in_bytes,
+                                                   volatile int* abort) {
     const int lane = threadIdx.x & 31, sub = lane / k, j = lane - sub * k;
     for (int n = n0; n < ntok; n += rows) {
         const int row = n + sub;
         const bool mine = sub < rows && row < ntok;
-        if (!__all_sync(0xffffffffu, !mine || mbar_wait(&full_bar[mine ? row : 0], 0, abort))) return false;
+        const int s = mine ? row % stages : 0;
+        if (!__all_sync(0xffffffffu, !mine || mbar_wait(&full_bar[s], (row / stages) & 1, abort))) return -1 - head;
         const int where = mine ? pos[row * k + j] : -1;
-        if (where >= 0) bulk_store(dst + (size_t)where * rowB, smem + (size_t)row * stage_bytes, bytes);
+        if (where >= 0) bulk_store(dst + (size_t)where * rowB, smem + (size_t)s * stage_bytes, bytes);
         bulk_commit();
+        if (head < ntok) {
+            bulk_wait_read<1>();   // every lane: its copies of the trips before this one have read their stages
+            __syncwarp();
+            const int more = min(min(ntok, n + stages) - head, 32);   // rows that go where rows before n were
+            if (lane < more) {
+                const int r = head + lane, rs = r % stages;
+                mbar_arrive_expect_tx(&full_bar[rs], in_bytes);
+                bulk_load(smem + (size_t)rs * stage_bytes, src + (size_t)r * src_stride, in_bytes, &full_bar[rs]);
+            }
+            head += max(more, 0);
+        }
     }
-    return true;
+    return head;
 }
 
 // ------------------------------------------------------------------------ mover warp
@@ -262,7 +276,7 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
     const int early = (kMode == kModeLocal || kMode == kModeCluster || kSteal) ? kMaxStages : 3;
     if (!kFp8) {
         // loads run (stages - 3) rows ahead; up to 3 rows' stores stay in flight (all rows at once where they fit)
-        const int ahead = !kSteal && ntok <= stages ? ntok : stages - 3;
+        const int ahead = !kSteal && ntok <= stages ? ntok : pl.trip_rows > 1 ? stages : stages - 3;
         int tl = 0;
         // Flag-free kernel: the routing table first, the rows after it.  The table is the one load the
         // whole layout waits for; the rows of 148 CTAs queued in front of it cost about a microsecond.
@@ -315,8 +329,14 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
             const int n0 = x.early0 ? 1 : 0;   // (the first row's copies may have been issued by the row group)
             if (pl.trip_rows > 1) {
                 if (lane == 0) trace(p, c, kTrFirstRow);
-                if (ok) ok = send_short_rows(n0, ntok, pl.trip_rows, p.k, full_bar, pos, smem, pl.stage_bytes, p.recv_x + out_off, p.rowB,
-                                     out_bytes, x.abort_flag);
+                if (ok) {
+                    const int sent = send_short_rows(n0, ntok, head, pl.trip_rows, stages, p.k, full_bar, pos, smem, pl.stage_bytes,
+                                                     p.recv_x + out_off, p.rowB, out_bytes,
+                                                     reinterpret_cast<const uint8_t*>(p.x) + (size_t)t0 * p.H * 2 + in_off,
+                                                     (size_t)p.H * 2, in_bytes, x.abort_flag);
+                    ok = sent >= 0;
+                    issued = head = ok ? sent : -1 - sent;
+                }
             } else
             for (int n = n0; ok && n < ntok; ++n) {
                 const int s = n % stages;
@@ -1491,6 +1511,12 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(const Params p, 
 
 static int round_up_i(int v, int m) { return (v + m - 1) / m * m; }
 
+// Rows (pieces of rows) that the kernel sends several at a time: see send_short_rows and the comment above Fp8Ring.
+bool short_rows(const Params& p) {
+    const int64_t copies = (int64_t)p.k * (p.rowB / p.parts);
+    return p.payload ? copies < 40 * 1024 : p.k <= 16 && copies <= 16384;
+}
+
 // Shared-memory plan of the dispatch kernel for one call; -1 if it cannot fit.
 int plan_dispatch(const Params& p, int mode, int max_smem, SmemPlan* out) {
     SmemPlan pl{};
@@ -1510,7 +1536,7 @@ int plan_dispatch(const Params& p, int mode, int max_smem, SmemPlan* out) {
     const int64_t bm_ints = (int64_t)pl.map_groups * pl.map_bp;
     const bool beside = p.payload && (mode == kModeCluster || (mode != kModeLocal && p.count_warps > 0));
     if (p.payload) {   // who quantises, and how (see Fp8Ring)
-        pl.q_long = (int64_t)p.k * (p.rowB / p.parts) >= 40 * 1024 ? 1 : 0;
+        pl.q_long = short_rows(p) ? 0 : 1;
         pl.q_warp0 = beside ? (mode == kModeCluster ? kClusterCountWarps : p.count_warps) + 1 : pl.q_long ? 2 : 1;
         const int most = fast ? kFastQuantWarps + (pl.q_long ? 0 : 1) : kWarps - pl.q_warp0;
         pl.q_warps = p.quant_warps < most ? p.quant_warps : most;
@@ -1554,8 +1580,10 @@ int plan_dispatch(const Params& p, int mode, int max_smem, SmemPlan* out) {
     int at = pl.stages * pl.stage_bytes;
     const int copies = p.k * (p.rowB / p.parts);
     pl.trip_rows = 1;
-    if (!p.payload && !p.steal && p.k <= 16 && chunk_tokens > 2 && chunk_tokens <= pl.stages && copies <= 16384)
+    if (!p.payload && !p.steal && chunk_tokens > 2 && short_rows(p)) {
         pl.trip_rows = 32 / p.k < 32768 / copies ? 32 / p.k : 32768 / copies;
+        if (chunk_tokens > pl.stages && pl.trip_rows > pl.stages / 3) pl.trip_rows = pl.stages / 3 > 1 ? pl.stages / 3 : 1;
+    }
     pl.off_out = at; at += pl.out_stages * pl.out_stage_bytes;
     pl.off_ids = at; at += (int)ids_ints * 4;
     pl.off_mask = at; at += (int)mask_ints * 4;

@@ -12,6 +12,7 @@ namespace ubep {
 int plan_dispatch(const Params& p, int mode, int max_smem, SmemPlan* out);
 
 int cluster_ctas(int cluster, int max_smem);
+bool short_rows(const Params& p);
 cudaError_t launch_count_scan(const Params& p, const SmemPlan& pl, cudaStream_t st);
 cudaError_t launch_dispatch(const Params& p, int mode, const SmemPlan& pl, cudaStream_t st, int* launches);
 cudaError_t launch_combine(const uint16_t* y, const int32_t* slot_pos, const float* topk_w, int T, int H, int k,
