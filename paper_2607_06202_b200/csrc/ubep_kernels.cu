@@ -1177,8 +1177,16 @@ __device__ __forceinline__ void fp8_worker(Cta& x, int qw) {
 // computed by earlier launches), or all 15 warps compute the layout and warps 2..15 quantise
 // afterwards (the flag-free kernel, whose layout is pure computation); warp 1 issues the copies of long rows
 // once the layout is done.
+//
+// The flag-free instance needs so few registers that two combine CTAs would fit beside it.  Then every combine CTA of a
+// small batch is placed during the dispatch, the dispatch after it is let in as soon as this one leaves, and the combine
+// runs with the registers that are left (sixteen layers of 128 tokens: 208 us; with one combine CTA beside it 179).
+// A warp that leaves at once holds the registers in question.
+template <int kMode, bool kFp8>
+constexpr int kDispatchThreads = kThreads + (kMode == kModeLocal && !kFp8 ? 32 : 0);
 template <int kMode, bool kFp8, bool kSteal>
-__global__ void __launch_bounds__(kThreads, 1) dispatch_kernel(const Params p, const SmemPlan pl) {
+__global__ void __launch_bounds__((kDispatchThreads<kMode, kFp8>), 1) dispatch_kernel(const Params p, const SmemPlan pl) {
+    if ((kDispatchThreads<kMode, kFp8>) > kThreads && threadIdx.x >= kThreads) return;
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) uint64_t full_bar[kMaxStages];    // input row landed
     __shared__ __align__(8) uint64_t empty_bar[kMaxStages];   // FP8: input row consumed
@@ -1661,7 +1669,7 @@ static cudaError_t launch_dispatch_s(const Params& p, const SmemPlan& pl, cudaSt
     auto kern = dispatch_kernel<kMode, kFp8, kSteal>;
     cudaError_t e = allow_dispatch_smem<kMode, kFp8, kSteal>(pl.total);
     if (e != cudaSuccess) return e;
-    return launch_overlapped(kern, p.grid, kThreads, (size_t)pl.total, st, kMode == kModeFused,
+    return launch_overlapped(kern, p.grid, kDispatchThreads<kMode, kFp8>, (size_t)pl.total, st, kMode == kModeFused,
                              kMode == kModeCluster ? p.cluster : 1, p, pl);
 }
 
