@@ -564,7 +564,7 @@ int ubep_dispatch_sync(ubep_buffer_t* buf, int protocol, const void* x, const in
     p.parts = 1;
     p.grid = p.nchunks;
     ubep::SmemPlan pl{};
-    const int extra = ubep::sync_extra_smem(p);
+    const int extra = ubep::sync_extra_smem(p, protocol);
     // Small tables are recounted by every CTA; for larger ones TokenCnt and CalCumSum run as launches of their
     // own in front of the kernel, over the same chunks (as the phased schedule of ubep_dispatch does).
     const bool whole_table = (int64_t)T * buf->cfg.topk <= kLocalMaxSlots &&

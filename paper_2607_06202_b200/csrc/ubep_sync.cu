@@ -325,13 +325,14 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
         }
     }
     if (tid == 0) times[2] = global_ns();
-    if (kTable) {
-        // counts and offsets nobody inside this kernel waits for (the launches before wrote them otherwise); behind the
-        // rows, which the receivers wait for
-        if (c == 0) write_totals(p, tot, eo, tid, kThreads);
-        write_own_sources<true>(p, t0, t1, 0, 1, bmaps, base, cnt + 2 * (p.B + 1), tid, kThreads, 0);
-    }
     if (kProto == kTFF) __syncthreads();   // (the strips may lie where the rows were)
+    if (kTable && warp >= kWarps / 2) {
+        // counts and offsets nobody inside this kernel waits for (the launches before wrote them otherwise); behind the
+        // rows, which the receivers wait for, and by half of the warps: the others turn to receiving at once
+        constexpr int n = kThreads / 2;
+        if (c == 0) write_totals(p, tot, eo, tid - n, n);
+        write_own_sources<true>(p, t0, t1, 0, 1, bmaps, base, cnt + 2 * (p.B + 1), tid - n, n, 0);
+    }
 
     // ---- receiver
     Waiter wt{&abort_flag, global_ns() + kWaitLimitNs, p.status, kProto == kSP ? sp.sp_dirty : nullptr};
@@ -479,7 +480,7 @@ template <int kProto>
 cudaError_t launch_one(const Params& p, const SmemPlan& pl, const SyncParams& sp, bool whole_table, cudaStream_t st) {
     auto kern = whole_table ? (p.payload ? sync_dispatch_kernel<kProto, true, true> : sync_dispatch_kernel<kProto, false, true>)
                             : (p.payload ? sync_dispatch_kernel<kProto, true, false> : sync_dispatch_kernel<kProto, false, false>);
-    const int smem = pl.total + sync_extra_smem(p);
+    const int smem = pl.total + sync_extra_smem(p, kProto);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     // Receivers wait for senders that are other CTAs of this grid: a cooperative launch, which the
@@ -499,8 +500,8 @@ cudaError_t launch_one(const Params& p, const SmemPlan& pl, const SyncParams& sp
 
 }  // namespace
 
-int sync_extra_smem(const Params& p) {
-    return p.R * 8 + 128 + qrow_bytes(p) + 16 + (strips_in_ring(p) ? 0 : kWarps * kStripWords * 4);
+int sync_extra_smem(const Params& p, int protocol) {
+    return p.R * 8 + 128 + qrow_bytes(p) + 16 + (protocol != kTFF || strips_in_ring(p) ? 0 : kWarps * kStripWords * 4);
 }
 
 cudaError_t launch_sync_dispatch(const Params& p, const SmemPlan& pl, const SyncParams& sp, bool whole_table,

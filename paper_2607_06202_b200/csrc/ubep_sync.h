@@ -26,7 +26,7 @@ struct SyncParams {
 };
 
 // Dynamic shared memory the kernel needs beyond the dispatch plan's total.
-int sync_extra_smem(const Params& p);
+int sync_extra_smem(const Params& p, int protocol);
 
 // whole_table: every CTA derives the layout from the whole routing table in shared memory; otherwise the
 // count / prefix-sum launches (launch_count_scan) have run before over the same p.nchunks chunks.
