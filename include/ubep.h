@@ -465,6 +465,29 @@ int ubep_debug_set_count_warps(ubep_buffer_t *buf, int32_t n);
 int ubep_debug_set_prefetch_rows(ubep_buffer_t *buf, int32_t n);
 
 /*
+ * How ubep_dispatch would schedule T tokens of a buffer with this configuration, worked out on the host alone (no
+ * device is asked, nothing is launched).  max_smem: shared memory a CTA may use; ctas [host]: CTAs of the persistent
+ * kernel that can run at once, alone and in clusters of 2, 4 and 8; count_warps, quant_warps as the two hooks above set
+ * them (-1 and 14 by default).  plan [host] gets the values below.  For tests of the kernel's ring sizes.
+ */
+enum {
+    UBEP_DEBUG_PLAN_MODE = 0,      /* UBEP_PIPELINE_*; 4 = layout by clusters                   */
+    UBEP_DEBUG_PLAN_CHUNKS,        /* token chunks ...                                          */
+    UBEP_DEBUG_PLAN_PARTS,         /* ... times column parts = CTAs                             */
+    UBEP_DEBUG_PLAN_CLUSTER,       /* CTAs per cluster                                          */
+    UBEP_DEBUG_PLAN_STEAL,         /* 1 = tokens are handed out to CTAs that run out of work    */
+    UBEP_DEBUG_PLAN_STAGES,        /* rows in the ring of fetched rows                          */
+    UBEP_DEBUG_PLAN_OUT_STAGES,    /* FP8: quantised rows in shared memory                      */
+    UBEP_DEBUG_PLAN_LONG_ROWS,     /* FP8: 1 = a ring of quantised rows, 0 = teams of warps     */
+    UBEP_DEBUG_PLAN_TEAMS,         /* FP8 with teams: how many                                  */
+    UBEP_DEBUG_PLAN_TEAM_WARPS,    /* ... and warps in each                                     */
+    UBEP_DEBUG_PLAN_SMEM,          /* dynamic shared memory of the kernel                       */
+    UBEP_DEBUG_PLAN_COUNT_
+};
+int ubep_debug_plan(const ubep_config_t *cfg, int32_t T, int32_t max_smem, const int32_t ctas[4], int32_t count_warps,
+                    int32_t quant_warps, int32_t plan[UBEP_DEBUG_PLAN_COUNT_]);
+
+/*
  * Measurement aid: launches a kernel that does nothing (one small CTA per SM) on `cuda_stream`,
  * the ordinary way or, with ahead != 0, with programmatic stream serialization like the dispatch
  * and the small-batch combine kernels.  Timed in a chain it gives the floor that every kernel

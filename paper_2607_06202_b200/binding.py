@@ -44,7 +44,7 @@ _VIEW_DTYPES = [torch.uint8, torch.float32, torch.int32, torch.float32, torch.in
 EXPORTS = ["ubep_buffer_bytes", "ubep_buffer_create", "ubep_buffer_destroy", "ubep_set_replicas",
            "ubep_set_dest_order", "ubep_get_dispatch_layout", "ubep_get_dispatch_layout_static", "ubep_dispatch", "ubep_combine", "ubep_view",
            "ubep_status", "ubep_epoch", "ubep_launch_count", "ubep_debug_withhold_flag", "ubep_debug_trace",
-           "ubep_debug_set_quant_warps", "ubep_debug_set_count_warps", "ubep_debug_set_prefetch_rows", "ubep_debug_empty_launch",
+           "ubep_debug_set_quant_warps", "ubep_debug_set_count_warps", "ubep_debug_set_prefetch_rows", "ubep_debug_empty_launch", "ubep_debug_plan",
            "ubep_last_cuda_error", "ubep_strerror", "ubep_map_workers",
            "ubep_sync_wire_bytes", "ubep_sync_attach", "ubep_dispatch_sync", "ubep_sync_view",
            "ubep_sync_scan_sentinel",
@@ -92,6 +92,8 @@ def load() -> ctypes.CDLL:
     lib.ubep_debug_set_quant_warps.restype, lib.ubep_debug_set_quant_warps.argtypes = ctypes.c_int, [vp, i32]
     lib.ubep_debug_set_count_warps.restype, lib.ubep_debug_set_count_warps.argtypes = ctypes.c_int, [vp, i32]
     lib.ubep_debug_set_prefetch_rows.restype, lib.ubep_debug_set_prefetch_rows.argtypes = ctypes.c_int, [vp, i32]
+    lib.ubep_debug_plan.restype = ctypes.c_int
+    lib.ubep_debug_plan.argtypes = [ctypes.POINTER(ubep_config_t), i32, i32, ctypes.POINTER(i32), i32, i32, ctypes.POINTER(i32)]
     lib.ubep_debug_empty_launch.restype, lib.ubep_debug_empty_launch.argtypes = ctypes.c_int, [vp, i32, vp]
     lib.ubep_last_cuda_error.restype, lib.ubep_last_cuda_error.argtypes = ctypes.c_char_p, [vp]
     lib.ubep_strerror.restype, lib.ubep_strerror.argtypes = ctypes.c_char_p, [ctypes.c_int]
@@ -274,6 +276,17 @@ def ubep_debug_set_count_warps(buf, n: int) -> None:
 
 def ubep_debug_set_prefetch_rows(buf, n: int) -> None:
     _check(load().ubep_debug_set_prefetch_rows(buf, n), "ubep_debug_set_prefetch_rows", buf)
+
+
+PLAN_NAMES = ("mode", "chunks", "parts", "cluster", "steal", "stages", "out_stages", "long_rows", "teams", "team_warps", "smem")
+
+
+def ubep_debug_plan(cfg: ubep_config_t, T: int, max_smem: int, ctas, count_warps: int = -1, quant_warps: int = 14) -> dict:
+    """How ubep_dispatch would schedule T tokens; ctas: CTAs that can run at once, alone and in clusters of 2, 4, 8."""
+    plan = (ctypes.c_int32 * len(PLAN_NAMES))()
+    _check(load().ubep_debug_plan(ctypes.byref(cfg), T, max_smem, (ctypes.c_int32 * 4)(*ctas), count_warps, quant_warps,
+                                  plan), "ubep_debug_plan")
+    return dict(zip(PLAN_NAMES, plan))
 
 
 def ubep_debug_empty_launch(buf, ahead: bool, stream=None) -> None:

@@ -287,6 +287,58 @@ void split_work(Params& p, int ctas) {
     p.grid = p.nchunks * best;
 }
 
+// How a dispatch is scheduled: fills in what the schedule says of p, and the kernel's plan.  Returns the mode, or an
+// error code.  n: the buffer's CTAs; count_warps as set for the buffer; cluster_ctas(cs): CTAs that can run in clusters of cs.
+template <typename ClusterCtas>
+int choose_schedule(Params& p, int pipeline, int n, int count_warps, int max_smem, ClusterCtas cluster_ctas,
+                    ubep::SmemPlan* pl) {
+    int mode = pipeline;
+    p.parts = 1;
+    p.grid = p.nchunks;
+    // by clusters of cs CTAs, if that fits
+    auto by_cluster = [&](int cs) {
+        int ctas = cs > 1 ? cluster_ctas(cs) : n;
+        ctas = (ctas < n ? ctas : n) / cs * cs;
+        if (ctas <= 0 || p.T > 65535) return false;   // (counts are 16 bits wide)
+        p.cluster = cs;
+        p.parts = 1;
+        p.steal = p.T >= kStealMinTokensPerChunk * ctas && !ubep::short_rows(p) ? 1 : 0;
+        if (p.steal) p.nchunks = p.grid = ctas;   // whole rows are handed out
+        else split_work(p, ctas);
+        if (ubep::plan_dispatch(p, ubep::kModeCluster, max_smem, pl) == 0) return true;
+        p.cluster = 1;
+        p.steal = 0;
+        return false;
+    };
+    auto alone = [&]() {   // rank-level rows, every CTA from the whole table
+        split_work(p, n);
+        return ubep::plan_dispatch(p, UBEP_PIPELINE_LOCAL, max_smem, pl) == 0;
+    };
+    if (mode == UBEP_PIPELINE_AUTO) {
+        if (p.local_fast && p.T <= local_fast_max_tokens(p) && alone()) mode = UBEP_PIPELINE_LOCAL;
+        else mode = by_cluster(cluster_size(p)) ? ubep::kModeCluster : UBEP_PIPELINE_FUSED;
+    } else if (mode == UBEP_PIPELINE_LOCAL) {
+        if (!alone()) return UBEP_ERR_ARG;   // table too large for shared memory
+        if (!p.local_fast) {   // every bin has to be counted: a cluster of one (which keeps the table nowhere)
+            if (!by_cluster(1)) return UBEP_ERR_ARG;
+            mode = ubep::kModeCluster;
+        }
+    }
+    if (mode == UBEP_PIPELINE_FUSED || mode == UBEP_PIPELINE_PHASED) {
+        p.parts = 1;
+        p.nchunks = n;
+        p.grid = n;
+        // slices that are long enough are handed out in blocks so that faster SMs can take over the tail of slower ones
+        p.steal = p.T >= kStealMinTokensPerChunk * p.nchunks && !ubep::short_rows(p) ? 1 : 0;
+        // With token stealing the count group is not used unless asked for: measured equal at top-8 and slower at
+        // top-4 (16384 tokens: 161 against 174 us) -- every hand-out is a round trip that idle quantising warps do not hide.
+        if (p.steal && count_warps < 0) p.count_warps = 0;
+        if (p.steal && ubep::plan_dispatch(p, mode, max_smem, pl) != 0) p.steal = 0;   // (rows too long for the ring it needs)
+        if (!p.steal && ubep::plan_dispatch(p, mode, max_smem, pl) != 0) return UBEP_ERR_ARG;
+    }
+    return mode;
+}
+
 // Makes the buffer's device current for the scope of one call.
 struct DeviceGuard {
     int prev = -1;
@@ -443,53 +495,11 @@ int ubep_dispatch(ubep_buffer_t* buf, const void* x, const int32_t* topk_idx, co
     p.topk_w = topk_w;
     p.withhold = buf->withhold;
     buf->withhold = -1;
-    int mode = buf->cfg.pipeline;
     ubep::SmemPlan pl{};
     int launches = 0;
-    p.parts = 1;
-    p.grid = p.nchunks;
-    const int n = buf->lay.nchunks;
-    // by clusters of cs CTAs, if that fits
-    auto by_cluster = [&](int cs) {
-        int ctas = cs > 1 ? ubep::cluster_ctas(cs, buf->max_smem) : n;
-        ctas = (ctas < n ? ctas : n) / cs * cs;
-        if (ctas <= 0 || T > 65535) return false;   // (counts are 16 bits wide)
-        p.cluster = cs;
-        p.parts = 1;
-        p.steal = T >= kStealMinTokensPerChunk * ctas && !ubep::short_rows(p) ? 1 : 0;
-        if (p.steal) p.nchunks = p.grid = ctas;   // whole rows are handed out
-        else split_work(p, ctas);
-        if (ubep::plan_dispatch(p, ubep::kModeCluster, buf->max_smem, &pl) == 0) return true;
-        p.cluster = 1;
-        p.steal = 0;
-        return false;
-    };
-    auto alone = [&]() {   // rank-level rows, every CTA from the whole table
-        split_work(p, n);
-        return ubep::plan_dispatch(p, UBEP_PIPELINE_LOCAL, buf->max_smem, &pl) == 0;
-    };
-    if (mode == UBEP_PIPELINE_AUTO) {
-        if (p.local_fast && T <= local_fast_max_tokens(p) && alone()) mode = UBEP_PIPELINE_LOCAL;
-        else mode = by_cluster(cluster_size(p)) ? ubep::kModeCluster : UBEP_PIPELINE_FUSED;
-    } else if (mode == UBEP_PIPELINE_LOCAL) {
-        if (!alone()) return UBEP_ERR_ARG;   // table too large for shared memory
-        if (!p.local_fast) {   // every bin has to be counted: a cluster of one (which keeps the table nowhere)
-            if (!by_cluster(1)) return UBEP_ERR_ARG;
-            mode = ubep::kModeCluster;
-        }
-    }
-    if (mode == UBEP_PIPELINE_FUSED || mode == UBEP_PIPELINE_PHASED) {
-        p.parts = 1;
-        p.nchunks = n;
-        p.grid = n;
-        // slices that are long enough are handed out in blocks so that faster SMs can take over the tail of slower ones
-        p.steal = T >= kStealMinTokensPerChunk * p.nchunks && !ubep::short_rows(p) ? 1 : 0;
-        // With token stealing the count group is not used unless asked for: measured equal at top-8 and slower at
-        // top-4 (16384 tokens: 161 against 174 us) -- every hand-out is a round trip that idle quantising warps do not hide.
-        if (p.steal && buf->count_warps < 0) p.count_warps = 0;
-        if (p.steal && ubep::plan_dispatch(p, mode, buf->max_smem, &pl) != 0) p.steal = 0;   // (rows too long for the ring it needs)
-        if (!p.steal && ubep::plan_dispatch(p, mode, buf->max_smem, &pl) != 0) return UBEP_ERR_ARG;
-    }
+    const int mode = choose_schedule(p, buf->cfg.pipeline, buf->lay.nchunks, buf->count_warps, buf->max_smem,
+                                     [&](int cs) { return ubep::cluster_ctas(cs, buf->max_smem); }, &pl);
+    if (mode < 0) return mode;
     cudaError_t e = ubep::launch_dispatch(p, mode, pl, st, &launches);
     if (e != cudaSuccess) return cuda_fail(buf, e);
     g_launches += launches;
@@ -845,6 +855,41 @@ int ubep_debug_set_count_warps(ubep_buffer_t* buf, int32_t n) {
 int ubep_debug_set_prefetch_rows(ubep_buffer_t* buf, int32_t n) {
     if (!buf || n < 1) return UBEP_ERR_ARG;
     buf->prefetch_rows = n;
+    return UBEP_OK;
+}
+
+int ubep_debug_plan(const ubep_config_t* cfg, int32_t T, int32_t max_smem, const int32_t ctas[4], int32_t count_warps,
+                    int32_t quant_warps, int32_t plan[UBEP_DEBUG_PLAN_COUNT_]) {
+    if (!cfg || !valid_config(*cfg) || !ctas || !plan || T < 1 || T > cfg->max_tokens) return UBEP_ERR_ARG;
+    if (count_warps < -1 || count_warps > ubep::kWarps - 3 || quant_warps < 1 || quant_warps > ubep::kWarps - 2) return UBEP_ERR_ARG;
+    int n = cfg->num_ctas > 0 && cfg->num_ctas < ctas[0] ? cfg->num_ctas : ctas[0];
+    if (n > ubep::kMaxChunks) n = ubep::kMaxChunks;
+    if (n < 1) return UBEP_ERR_ARG;
+    ubep_buffer b{};   // (no device behind it: only sizes are looked at)
+    b.cfg = *cfg;
+    b.lay = make_layout(*cfg, n);
+    b.arena = reinterpret_cast<uint8_t*>(kAlign);
+    b.sm_khz = 1;
+    b.quant_warps = quant_warps;
+    b.count_warps = count_warps;
+    b.prefetch_rows = INT32_MAX;
+    b.my_rank = -1;
+    Params p = make_params(&b, T);
+    ubep::SmemPlan pl{};
+    const int mode = choose_schedule(p, cfg->pipeline, n, count_warps, max_smem,
+                                     [&](int cs) { return ctas[cs == 2 ? 1 : cs == 4 ? 2 : 3]; }, &pl);
+    if (mode < 0) return mode;
+    plan[UBEP_DEBUG_PLAN_MODE] = mode;
+    plan[UBEP_DEBUG_PLAN_CHUNKS] = p.nchunks;
+    plan[UBEP_DEBUG_PLAN_PARTS] = p.parts;
+    plan[UBEP_DEBUG_PLAN_CLUSTER] = p.cluster;
+    plan[UBEP_DEBUG_PLAN_STEAL] = p.steal;
+    plan[UBEP_DEBUG_PLAN_STAGES] = pl.stages;
+    plan[UBEP_DEBUG_PLAN_OUT_STAGES] = pl.out_stages;
+    plan[UBEP_DEBUG_PLAN_LONG_ROWS] = pl.q_long;
+    plan[UBEP_DEBUG_PLAN_TEAMS] = pl.q_teams;
+    plan[UBEP_DEBUG_PLAN_TEAM_WARPS] = pl.q_team_warps;
+    plan[UBEP_DEBUG_PLAN_SMEM] = pl.total;
     return UBEP_OK;
 }
 

@@ -1591,8 +1591,6 @@ int plan_dispatch(const Params& p, int mode, int max_smem, SmemPlan* out) {
     const int64_t in = pl.stage_bytes, out_b = pl.out_stage_bytes;
     if (p.payload && !pl.q_long) {
         // Two quantised rows per team, the rest for rows that have been fetched: as many as there are teams at least.
-        // (Then the row a team waits for is at most one round of the ring behind the row it had before, and the
-        // parity of the stage's barrier tells them apart.)
         while (pl.q_teams > 1 && room < pl.q_teams * (in + 2 * out_b)) --pl.q_teams;
         pl.q_team_warps = pl.q_warps / pl.q_teams;
         pl.out_stages = 2 * pl.q_teams;
@@ -1612,6 +1610,11 @@ int plan_dispatch(const Params& p, int mode, int max_smem, SmemPlan* out) {
     if (room < least * in) return -1;
     pl.stages = room / in > max_stages ? max_stages : (int)(room / in);
     if (pl.stages > want) pl.stages = want;
+    // Teams: where the ring is used more than once, every stage belongs to one team (row n is in stage n % stages and
+    // goes to team n % teams).  A team waits by the parity of the stage's barrier, which only tells the row it waits for
+    // from the row that had the stage before: that one must have landed, and loads land in any order, so it must have been
+    // this team's own.  (A team needs one stage: rows leave an SM at 0.9 us each at 32 KB of copies, a load takes about as long.)
+    if (p.payload && !pl.q_long && pl.stages < chunk_tokens) pl.stages -= pl.stages % pl.q_teams;
     int at = pl.stages * pl.stage_bytes;
     const int copies = p.k * (p.rowB / p.parts);
     pl.trip_rows = 1;
