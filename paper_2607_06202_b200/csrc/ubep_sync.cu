@@ -402,6 +402,7 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
                 }
                 ok = __all_sync(0xffffffffu, ok);
                 if (kProto == kTFF) {
+                    __syncwarp();   // the lanes' words are in the strip (the vote orders no memory)
                     // words [3 * g0, 3 * g0 + 3 * n) of the wire row (a strip begins on a multiple of four words)
                     for (int q = lane; ok && q < kStripWords / 4; q += 32) {
                         const int w = 3 * g0 + 4 * q;
