@@ -160,6 +160,8 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
         // urgent to do yet, so it fetches it while the layout group already stages the routing table.
         unsigned ep = 0;
         if (x.lane == 0) {
+            // (before anybody can claim from this chunk: pos_flag is released behind a wait for epoch_bar)
+            if (kSteal) x.p.cursor[x.ch] = 0;
             ep = read_epoch_and_check_in(x.p);
             *x.epoch_late = ep;
             mbar_arrive(x.epoch_bar);
@@ -267,7 +269,6 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
         }
         head += n;
     };
-    if (kSteal && lane == 0) p.cursor[ch] = 0;   // before anybody can claim from this chunk
     // Rows fetched before the layout is done.  With flags the layout takes many microseconds in which a
     // few small loads and stores of every CTA wait on one another; a ring-full of rows per CTA fetched
     // meanwhile fills the memory system's queues in front of them.  Three rows start the copies, the

@@ -21,3 +21,12 @@ def _in_order(text, *marks):
 def test_a_token_flag_strip_is_complete_before_other_lanes_read_it():
     # (a warp vote brings lanes together but orders no memory)
     _in_order(_source("ubep_sync.cu"), "mine[3 * g + 2] = ", "__syncwarp()", "reinterpret_cast<const uint4*>(mine")
+
+
+def test_a_chunks_cursor_is_reset_before_its_destinations_are_released():
+    # (the layout group waits for epoch_bar before it releases pos_flag: what the mover warp stored before it arrived there
+    # is ordered in front of that release, what it stores later is not)
+    mover = _source("ubep_kernels.cu")
+    mover = mover[mover.index("void mover_warp("):mover.index("constexpr int kClusterCountWarps")]
+    _in_order(mover, "cursor[x.ch] = 0", "mbar_arrive(x.epoch_bar)")
+    assert mover.count("cursor[ch] = 0") + mover.count("cursor[x.ch] = 0") == 1
