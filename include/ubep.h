@@ -168,7 +168,9 @@ int ubep_set_dest_order(ubep_buffer_t *buf, const int32_t *order /*[host] [R]*/)
  * slot; the ids of one token are distinct -- a repeated id is reported as UBEP_ERR_BAD_INDEX
  * and the later slot counts as empty).  Outputs [dev], caller-owned:
  * num_tokens_per_rank [R], num_tokens_per_expert [E], is_token_in_rank u8 [T, R]
- * (any of them may be NULL).  One launch on `cuda_stream`.
+ * (any of them may be NULL).  One launch on `cuda_stream`; calls on one buffer must be
+ * stream-ordered: the counts of calls that overlap on the GPU are undefined (calls after them
+ * are not affected).
  */
 int ubep_get_dispatch_layout(ubep_buffer_t *buf, const int32_t *topk_idx /*[dev]*/, int32_t T,
                              int32_t *num_tokens_per_rank /*[dev]*/,
@@ -194,8 +196,8 @@ int ubep_get_dispatch_layout(ubep_buffer_t *buf, const int32_t *topk_idx /*[dev]
  * current) and keeps it; make that first call before any stream capture begins.  The call
  * itself calls no cudaMalloc, cudaFree or other allocating routine.  All calls on a device
  * share the one array: calls whose kernels may overlap on the GPU (different streams) race
- * on it -- keep them on one stream or otherwise ordered.  The array is zero between calls;
- * the kernel leaves it so.
+ * on it -- keep them on one stream or otherwise ordered (their counts are undefined; calls
+ * after them are not affected).  The array is zero between calls; the kernel leaves it so.
  */
 #define UBEP_STATIC_MAX_BINS 1024
 int ubep_get_dispatch_layout_static(const int32_t *topk_idx /*[dev]*/, int32_t T, int32_t topk,

@@ -467,7 +467,7 @@ int ubep_get_dispatch_layout(ubep_buffer_t* buf, const int32_t* topk_idx, int32_
     Params p = make_params(buf, T);
     p.topk_idx = topk_idx;
     cudaError_t e = ubep::launch_layout(p, num_tokens_per_rank, num_tokens_per_expert, is_token_in_rank,
-                                        at<int32_t>(buf, buf->lay.layout_acc), at<unsigned>(buf, buf->lay.ticket), st);
+                                        at<int32_t>(buf, buf->lay.layout_acc), p.B, at<unsigned>(buf, buf->lay.ticket), st);
     if (e != cudaSuccess) return cuda_fail(buf, e);
     g_launches += 1;
     return UBEP_OK;

@@ -1423,7 +1423,7 @@ __global__ void __launch_bounds__(256) combine_kernel(const uint16_t* __restrict
 // side (16 bytes each where the table allows it), the experts are counted in shared memory, the ranks it visits
 // become a bit mask per lane, which the warp transposes so that every rank's count is one population count.
 // A CTA adds its counts to the totals in `acc`, the last one to finish (ticket) hands them out and leaves `acc`
-// zero for the next call.
+// and the ticket zero for the next call.
 //
 // Bound by latency: table (cold, 1.2 us) -> counts -> adds -> ticket -> totals.  One group of 32 tokens per warp
 // and four warps per CTA keep every step one trip deep.  Measured at 4096 tokens, top-8 of 256 experts: 6.4 us per call
@@ -1438,7 +1438,7 @@ template <int kK, int kW>
 __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(const Params p, int32_t* num_tokens_per_rank,
                                                                int32_t* num_tokens_per_expert,
                                                                uint8_t* is_token_in_rank, int32_t* acc,
-                                                               unsigned* ticket) {
+                                                               int acc_words, unsigned* ticket) {
     extern __shared__ int hist[];   // [B]
     __shared__ bool last;
     const int B = p.B, R = p.R, T = p.T, k = kK ? kK : p.k, lane = threadIdx.x & 31;
@@ -1527,20 +1527,23 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(const Params p, 
         if (hist[b]) atomicAdd(acc + b, hist[b]);
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1u;
+    // The shares of a grid's CTAs add up to 2^32, so the ticket is zero again when all have come, whatever else is under
+    // way: calls that overlap on the GPU (which share the totals, so that their answers are undefined) leave nothing behind.
+    const unsigned share = 0xffffffffu / gridDim.x;
+    const unsigned mine = blockIdx.x == 0 ? 0u - share * (gridDim.x - 1u) : share;
+    if (threadIdx.x == 0) last = atomicAdd(ticket, mine) + mine == 0u;
     __syncthreads();
     if (!last) return;
     __threadfence();
     for (int b = threadIdx.x; b < B; b += kLayoutThreads) {
-        const int sum = __ldcg(acc + b);
-        acc[b] = 0;
+        const int sum = atomicExch(acc + b, 0);   // (zero for the next call)
         if (b < p.E) {
             if (num_tokens_per_expert) num_tokens_per_expert[b] = sum;
         } else if (num_tokens_per_rank) {
             num_tokens_per_rank[b - p.E] = sum;
         }
     }
-    if (threadIdx.x == 0) *ticket = 0u;  // ready for the next call
+    for (int b = B + threadIdx.x; b < acc_words; b += kLayoutThreads) acc[b] = 0;   // (an overlapping call may have had more bins)
 }
 
 // ------------------------------------------------------------------------- launchers
@@ -1823,7 +1826,7 @@ cudaError_t launch_empty(int num_sms, bool ahead, cudaStream_t st) {
 }
 
 cudaError_t launch_layout(const Params& p, int32_t* num_tokens_per_rank, int32_t* num_tokens_per_expert,
-                          uint8_t* is_token_in_rank, int32_t* acc, unsigned* ticket, cudaStream_t st) {
+                          uint8_t* is_token_in_rank, int32_t* acc, int acc_words, unsigned* ticket, cudaStream_t st) {
     // a group of 32 tokens per warp; beyond two CTAs per SM a warp takes several
     const int64_t groups = ((int64_t)p.T + 31) / 32, per_cta = kLayoutThreads / 32;
     int64_t blocks = (groups + per_cta - 1) / per_cta;
@@ -1832,7 +1835,7 @@ cudaError_t launch_layout(const Params& p, int32_t* num_tokens_per_rank, int32_t
     const size_t smem = sizeof(int) * (size_t)p.B;
     auto go = [&](auto kern) {
         return launch_overlapped(kern, (int)blocks, kLayoutThreads, smem, st, false, 1, p, num_tokens_per_rank,
-                                 num_tokens_per_expert, is_token_in_rank, acc, ticket);
+                                 num_tokens_per_expert, is_token_in_rank, acc, acc_words, ticket);
     };
     if (p.R > 32 * kLayoutMaskWords) return go(layout_kernel<0, 0>);
     const bool narrow = p.R <= 32;

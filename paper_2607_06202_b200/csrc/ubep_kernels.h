@@ -18,8 +18,9 @@ cudaError_t launch_dispatch(const Params& p, int mode, const SmemPlan& pl, cudaS
 cudaError_t launch_combine(const uint16_t* y, const int32_t* slot_pos, const float* topk_w, int T, int H, int k,
                            uint16_t* out, int num_sms, bool ahead, cudaStream_t st);
 cudaError_t launch_empty(int num_sms, bool ahead, cudaStream_t st);
-// acc: p.B words and the ticket word, all zero between calls (the kernel leaves them so).
+// acc: acc_words words (p.B at least) and the ticket word, all zero between calls (the kernel leaves them so, also where
+// calls that share them overlapped).
 cudaError_t launch_layout(const Params& p, int32_t* num_tokens_per_rank, int32_t* num_tokens_per_expert,
-                          uint8_t* is_token_in_rank, int32_t* acc, unsigned* ticket, cudaStream_t st);
+                          uint8_t* is_token_in_rank, int32_t* acc, int acc_words, unsigned* ticket, cudaStream_t st);
 
 }  // namespace ubep

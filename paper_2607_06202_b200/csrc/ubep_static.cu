@@ -1,6 +1,7 @@
 // ubep_get_dispatch_layout_static: the counts-only step for callers that cannot give the
 // library any device memory of their own beyond inputs and outputs -- no arena, no buffer
-// handle.  The totals that the counting kernel adds up and its completion ticket live in a fixed array inside this library's device image instead.
+// handle.  The totals that the counting kernel adds up and its completion ticket live in a fixed array inside this
+// library's device image instead.
 #include <cstdint>
 
 #include "../../include/ubep.h"
@@ -55,6 +56,6 @@ extern "C" int ubep_get_dispatch_layout_static(const int32_t* topk_idx, int32_t 
     unsigned* ticket = reinterpret_cast<unsigned*>(scratch + kStaticBins);
     // The kernel's last CTA leaves the totals and the ticket at zero, so nothing has to be cleared between calls.
     const cudaError_t e = ubep::launch_layout(p, num_tokens_per_rank, num_tokens_per_expert, is_token_in_rank, scratch,
-                                              ticket, static_cast<cudaStream_t>(cuda_stream));
+                                              kStaticBins, ticket, static_cast<cudaStream_t>(cuda_stream));
     return e == cudaSuccess ? UBEP_OK : UBEP_ERR_CUDA;
 }

@@ -39,3 +39,33 @@ def test_counts_match_the_oracle(T, E, R, k):
     only = torch.full((E,), -1, dtype=torch.int32, device="cuda")
     B.ubep_get_dispatch_layout(buf.handle, torch.from_numpy(idx).cuda(), T, None, only, None)
     assert np.array_equal(only.cpu().numpy(), lay.num_tokens_per_expert)
+
+
+@pytest.mark.parametrize("static", [False, True])
+def test_overlapping_calls_do_not_spoil_later_ones(static):
+    """Calls on two streams share the totals and the ticket: their counts are undefined, those of a later call are not."""
+    E, R, k, most = 64, 8, 4, 9000
+    rng = np.random.Generator(np.random.PCG64(3))
+    tables = [np.argsort(rng.random((T, E)), axis=1)[:, :k].astype(np.int32) for T in (most, 130, 2500, 31)]
+    dev = [torch.from_numpy(t).cuda() for t in tables]
+    buf = B.Buffer(num_ranks=R, num_experts=E, hidden=8, topk=k, max_tokens=most, rows_per_rank_cap=1)
+    outs = [(torch.empty(R, dtype=torch.int32, device="cuda"), torch.empty(E, dtype=torch.int32, device="cuda")) for _ in range(2)]
+
+    def call(table, out, stream=None):
+        if static:
+            B.ubep_get_dispatch_layout_static(table, table.shape[0], k, E, R, *out, None, stream)
+        else:
+            B.ubep_get_dispatch_layout(buf.handle, table, table.shape[0], *out, None, stream)
+
+    call(dev[0], outs[0])   # (the static one's first call looks up its array)
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    torch.cuda.synchronize()
+    for rounds in range(40):
+        for i in range(6):
+            call(dev[(rounds + i) % 4], outs[i % 2], streams[i % 2])
+        torch.cuda.synchronize()
+        n = rounds % 4
+        call(dev[n], outs[0])
+        lay = oracle.layout(tables[n], E, R, R, 0)
+        assert np.array_equal(outs[0][0].cpu().numpy(), lay.num_tokens_per_rank)
+        assert np.array_equal(outs[0][1].cpu().numpy(), lay.num_tokens_per_expert)
