@@ -217,8 +217,8 @@ PyObject* py_layout(PyObject*, PyObject* const* a, Py_ssize_t n) {
 }
 
 // layout_new(handle, topk_idx, num_ranks, num_experts, device, stream): the tuple (tokens_per_rank [R] int32,
-// tokens_per_expert [E] int32, is_token_in_rank [T, R] uint8), or the code.  One block of memory serves all
-// three (three calls of torch.empty were 7 of the call's 13 us on the host).
+// tokens_per_expert [E] int32, is_token_in_rank [T, R] uint8), or the code.  Three allocations: each result is a tensor of
+// its own, which a caller may keep, save or resize without the others.
 PyObject* py_layout_new(PyObject*, PyObject* const* a, Py_ssize_t n) {
     try {
         if (!want_args(n, 6)) return nullptr;
@@ -229,31 +229,20 @@ PyObject* py_layout_new(PyObject*, PyObject* const* a, Py_ssize_t n) {
         if (!handle_arg(a[0], &buf) || !tensor_arg(a[1], &idx) || !rows_of(a[1], &T) || !int_arg(a[2], &R) ||
             !int_arg(a[3], &E) || !int_arg(a[4], &device) || !stream_arg(a[5], &st))
             return nullptr;
-        constexpr int64_t kAlign = 256;
-        const int64_t off_e = (R * 4 + kAlign - 1) / kAlign * kAlign;
-        const int64_t off_t = off_e + (E * 4 + kAlign - 1) / kAlign * kAlign;
         const c10::Device dev(c10::kCUDA, (c10::DeviceIndex)device);
-        const at::Tensor block = at::detail::empty_cuda({off_t + (int64_t)T * R}, at::kByte, dev, c10::nullopt);
-        auto part = [&](at::ScalarType type, int64_t byte_off, c10::IntArrayRef size) {
-            at::Tensor t = at::detail::make_tensor<c10::TensorImpl>(c10::Storage(block.storage()), block.key_set(),
-                                                                    c10::scalarTypeToTypeMeta(type));
-            t.unsafeGetTensorImpl()->set_storage_offset(byte_off / (int64_t)c10::elementSize(type));
-            t.unsafeGetTensorImpl()->set_sizes_contiguous(size);
-            return t;
-        };
-        at::Tensor npr = part(at::kInt, 0, {(int64_t)R});
-        at::Tensor npe = part(at::kInt, off_e, {(int64_t)E});
-        at::Tensor itr = part(at::kByte, off_t, {(int64_t)T, (int64_t)R});
-        uint8_t* base = static_cast<uint8_t*>(block.data_ptr());
+        at::Tensor parts[3] = {at::detail::empty_cuda({(int64_t)R}, at::kInt, dev, c10::nullopt),
+                               at::detail::empty_cuda({(int64_t)E}, at::kInt, dev, c10::nullopt),
+                               at::detail::empty_cuda({(int64_t)T, (int64_t)R}, at::kByte, dev, c10::nullopt)};
+        void* po[3] = {parts[0].data_ptr(), parts[1].data_ptr(), parts[2].data_ptr()};
         const int rc = without_gil([&] {
-            return f_layout(buf, static_cast<const int32_t*>(idx), T, reinterpret_cast<int32_t*>(base), reinterpret_cast<int32_t*>(base + off_e), base + off_t, st);
+            return f_layout(buf, static_cast<const int32_t*>(idx), T, static_cast<int32_t*>(po[0]),
+                            static_cast<int32_t*>(po[1]), static_cast<uint8_t*>(po[2]), st);
         });
         if (rc != UBEP_OK) return PyLong_FromLong(rc);
         PyObject* out = PyTuple_New(3);
         if (!out) return nullptr;
-        at::Tensor* parts[3] = {&npr, &npe, &itr};
         for (int i = 0; i < 3; ++i) {
-            PyObject* o = THPVariable_Wrap(std::move(*parts[i]));
+            PyObject* o = THPVariable_Wrap(std::move(parts[i]));
             if (!o) {
                 Py_DECREF(out);
                 return nullptr;

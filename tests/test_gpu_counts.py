@@ -69,3 +69,14 @@ def test_overlapping_calls_do_not_spoil_later_ones(static):
         lay = oracle.layout(tables[n], E, R, R, 0)
         assert np.array_equal(outs[0][0].cpu().numpy(), lay.num_tokens_per_rank)
         assert np.array_equal(outs[0][1].cpu().numpy(), lay.num_tokens_per_expert)
+
+
+def test_the_results_are_tensors_of_their_own():
+    """Each has its own storage: keeping or saving the small ones does not keep or save the mask."""
+    buf = B.Buffer(num_ranks=4, num_experts=16, hidden=8, topk=2, max_tokens=500, rows_per_rank_cap=1)
+    idx = torch.zeros((500, 2), dtype=torch.int32, device="cuda")
+    idx[:, 1] = 5
+    out = buf.get_dispatch_layout(idx)
+    assert [t.untyped_storage().nbytes() for t in out] == [4 * 4, 4 * 16, 500 * 4]
+    assert [t.storage_offset() for t in out] == [0, 0, 0]
+    assert len({t.untyped_storage().data_ptr() for t in out}) == 3
