@@ -80,13 +80,20 @@ bool handle_arg(PyObject* o, ubep_buffer_t** buf) {
     return !PyErr_Occurred();
 }
 
-// None = torch's current stream; otherwise an object with a `cuda_stream` handle, or the handle.
+// None = torch's current stream; otherwise an object with a `cuda_stream` handle, or the handle as anything int() takes.
 bool stream_arg(PyObject* o, void** st) {
     if (o == Py_None) {
         *st = c10::cuda::getCurrentCUDAStream().stream();
         return true;
     }
-    PyObject* h = PyLong_Check(o) ? Py_NewRef(o) : PyObject_GetAttrString(o, "cuda_stream");
+    PyObject* h = nullptr;
+    if (PyLong_Check(o)) {
+        h = Py_NewRef(o);
+    } else if (PyObject_HasAttrString(o, "cuda_stream")) {
+        h = PyObject_GetAttrString(o, "cuda_stream");
+    } else {
+        h = PyNumber_Long(o);
+    }
     if (!h) return false;
     *st = PyLong_AsVoidPtr(h);
     Py_DECREF(h);

@@ -112,3 +112,24 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(B, "LIB_PATH", str(tmp_path / "libubep.so"))
     with pytest.raises(RuntimeError, match="missing"):
         B.load()
+
+
+def test_stream_handles_of_any_integer_type(lib):
+    # (a null buffer is refused by the library itself: the arguments in front of it were taken)
+    import ctypes
+
+    import numpy as np
+
+    class Handle:
+        cuda_stream = 0
+
+    class Convertible:
+        def __int__(self):
+            return 0
+
+    for stream in (0, True, np.int64(0), np.uint64(0), Handle(), Convertible()):
+        with pytest.raises(B.UbepError) as e:
+            B.ubep_dispatch(None, None, None, None, 0, stream)
+        assert e.value.code == B.UBEP_ERR_ARG
+    with pytest.raises((TypeError, ValueError)):   # (what int() of it raises)
+        B.ubep_dispatch(None, None, None, None, 0, ctypes.c_void_p(0))
