@@ -66,7 +66,9 @@ enum {
     UBEP_PIPELINE_LOCAL = 3   /* one persistent kernel in which every CTA derives its offsets */
                               /* from the whole routing table itself (no flags; small T*k:    */
                               /* asked for explicitly with a table that does not fit in       */
-                              /* shared memory, ubep_dispatch returns UBEP_ERR_ARG)           */
+                              /* shared memory, ubep_dispatch returns UBEP_ERR_ARG; with so   */
+                              /* many experts that a CTA has no room for their counts beside  */
+                              /* its rows, it runs as PHASED)                                 */
 };
 
 typedef struct {

@@ -255,6 +255,19 @@ Params make_params(ubep_buffer* b, int T) {
     return p;
 }
 
+// Rows can be cut into `parts` pieces: whole 16-byte vectors, of FP8 rows whole scale groups.
+// FP8 rows: a piece's scales must still be a bulk copy (a multiple of 16 bytes); with plain stores for
+// the scales and payload pieces under 2 KB a dispatch of 384 tokens took 33 us against 21 us for 512
+bool can_cut(const Params& p, int ctas, int parts) {
+    if (ctas / parts < 1 || (p.H * 2 / parts) % 16 != 0 || (p.H * 2) % parts != 0) return false;
+    if (p.payload && ((p.H / parts) % 128 != 0 || p.H % parts != 0)) return false;
+    return !p.payload || parts == 1 || ((p.G / parts) * 4) % 16 == 0;
+}
+void cut(Params& p, int ctas, int parts) {
+    p.parts = parts;
+    p.nchunks = ctas / parts;
+    p.grid = p.nchunks * parts;
+}
 // Cuts the work of a flag-free kernel over `ctas` CTAs: token chunks, and column parts of a row so that the slices
 // are balanced to about 5 %.  The CTA with the most work sets the pace: ceil(T / chunks) tokens of 1 / parts of a
 // row each.  Smaller pieces cost more per byte (measured on the decode shape, layout by every CTA alone: 4 parts + 8 to
@@ -267,13 +280,8 @@ void split_work(Params& p, int ctas) {
     double best_cost = 0.0;
     const bool by_cluster = p.cluster > 1;
     const double piece_penalty[4] = {1.0, by_cluster ? 1.05 : 1.0, by_cluster ? 1.1 : 1.15, by_cluster ? 1.15 : 1.6};
-    for (int parts = 1, i = 0; parts <= 8; parts *= 2, ++i) {
+    for (int parts = 1, i = 0; parts <= 8 && can_cut(p, ctas, parts); parts *= 2, ++i) {
         const int chunks = ctas / parts;
-        if (chunks < 1 || (p.H * 2 / parts) % 16 != 0 || (p.H * 2) % parts != 0) break;
-        if (p.payload && ((p.H / parts) % 128 != 0 || p.H % parts != 0)) break;
-        // FP8 rows: a piece's scales must still be a bulk copy (a multiple of 16 bytes); with plain stores for
-        // the scales and payload pieces under 2 KB a dispatch of 384 tokens took 33 us against 21 us for 512
-        if (p.payload && parts > 1 && ((p.G / parts) * 4) % 16 != 0) break;
         const int most = (p.T + chunks - 1) / chunks, piece = p.H * 2 / parts;
         if (parts > 1 && (piece < (most > 1 ? 4096 : 1536) || (most > 1 && p.payload))) break;
         const double cost = (double)most / parts * piece_penalty[i];
@@ -282,9 +290,16 @@ void split_work(Params& p, int ctas) {
             best_cost = cost;
         }
     }
-    p.parts = best;
-    p.nchunks = ctas / best;
-    p.grid = p.nchunks * best;
+    cut(p, ctas, best);
+}
+// ... and in finer pieces where the ring cannot hold those (rows beyond 50 KB).
+bool split_to_fit(Params& p, int ctas, int mode, int max_smem, ubep::SmemPlan* pl) {
+    split_work(p, ctas);
+    for (;;) {
+        if (ubep::plan_dispatch(p, mode, max_smem, pl) == 0) return true;
+        if (p.parts >= 8 || !can_cut(p, ctas, 2 * p.parts)) return false;
+        cut(p, ctas, 2 * p.parts);
+    }
 }
 
 // How a dispatch is scheduled: fills in what the schedule says of p, and the kernel's plan.  Returns the mode, or an
@@ -310,18 +325,31 @@ int choose_schedule(Params& p, int pipeline, int n, int count_warps, int max_sme
         p.steal = 0;
         return false;
     };
-    auto alone = [&]() {   // rank-level rows, every CTA from the whole table
+    auto alone = [&](bool finer) {   // rank-level rows, every CTA from the whole table
+        if (finer) return split_to_fit(p, n, UBEP_PIPELINE_LOCAL, max_smem, pl);
         split_work(p, n);
         return ubep::plan_dispatch(p, UBEP_PIPELINE_LOCAL, max_smem, pl) == 0;
     };
+    // The last resort: counted by launches of their own, a CTA holds its own tokens only, in column parts where whole
+    // rows would not fit in the ring.  (Every CTA of such a chunk writes the same metadata.)  Tables of many thousand
+    // experts, whose three arrays of counts leave a cluster no room.
+    auto phased_in_parts = [&]() {
+        p.cluster = 1;
+        p.steal = 0;
+        return split_to_fit(p, n, UBEP_PIPELINE_PHASED, max_smem, pl);
+    };
     if (mode == UBEP_PIPELINE_AUTO) {
-        if (p.local_fast && p.T <= local_fast_max_tokens(p) && alone()) mode = UBEP_PIPELINE_LOCAL;
+        if (p.local_fast && p.T <= local_fast_max_tokens(p) && alone(false)) mode = UBEP_PIPELINE_LOCAL;
         else mode = by_cluster(cluster_size(p)) ? ubep::kModeCluster : UBEP_PIPELINE_FUSED;
     } else if (mode == UBEP_PIPELINE_LOCAL) {
-        if (!alone()) return UBEP_ERR_ARG;   // table too large for shared memory
-        if (!p.local_fast) {   // every bin has to be counted: a cluster of one (which keeps the table nowhere)
-            if (!by_cluster(1)) return UBEP_ERR_ARG;
-            mode = ubep::kModeCluster;
+        const bool fast = p.local_fast && alone(true);
+        if (!fast) {
+            p.local_fast = 0;
+            if (!alone(true)) return UBEP_ERR_ARG;   // table too large for shared memory
+            // every bin has to be counted: a cluster of one (which keeps the table nowhere)
+            if (by_cluster(1)) mode = ubep::kModeCluster;
+            else if (phased_in_parts()) return UBEP_PIPELINE_PHASED;
+            else return UBEP_ERR_ARG;
         }
     }
     if (mode == UBEP_PIPELINE_FUSED || mode == UBEP_PIPELINE_PHASED) {
@@ -334,7 +362,10 @@ int choose_schedule(Params& p, int pipeline, int n, int count_warps, int max_sme
         // top-4 (16384 tokens: 161 against 174 us) -- every hand-out is a round trip that idle quantising warps do not hide.
         if (p.steal && count_warps < 0) p.count_warps = 0;
         if (p.steal && ubep::plan_dispatch(p, mode, max_smem, pl) != 0) p.steal = 0;   // (rows too long for the ring it needs)
-        if (!p.steal && ubep::plan_dispatch(p, mode, max_smem, pl) != 0) return UBEP_ERR_ARG;
+        if (!p.steal && ubep::plan_dispatch(p, mode, max_smem, pl) != 0) {
+            if (pipeline != UBEP_PIPELINE_AUTO || !phased_in_parts()) return UBEP_ERR_ARG;
+            mode = UBEP_PIPELINE_PHASED;
+        }
     }
     return mode;
 }

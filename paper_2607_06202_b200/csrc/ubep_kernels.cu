@@ -1723,7 +1723,12 @@ cudaError_t launch_count_scan(const Params& p, const SmemPlan& pl, cudaStream_t 
         return e;
     count_kernel<<<p.nchunks, 256, count_smem, st>>>(p, pl);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    scan_kernel<<<p.R, 256, sizeof(int) * (p.L + 1), st>>>(p);
+    const int scan_smem = (int)sizeof(int) * (p.L + 1);
+    static std::atomic<int> scan_granted[kAttrDevices];
+    if (scan_smem > 48 * 1024 &&
+        (e = allow_dynamic_smem(reinterpret_cast<const void*>(scan_kernel), scan_smem, scan_granted)) != cudaSuccess)
+        return e;
+    scan_kernel<<<p.R, 256, scan_smem, st>>>(p);
     return cudaGetLastError();
 }
 

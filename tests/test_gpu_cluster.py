@@ -69,3 +69,14 @@ def test_an_expert_named_twice(k, dedup):
     buf.dispatch(x, Hn.to_dev(dup), w)
     assert buf.status() == B.UBEP_ERR_BAD_INDEX
     Hn.check_dispatch(buf, wl_clean, lay, cap, recv)
+
+
+@pytest.mark.parametrize("cfg,pipeline", [
+    (dict(T=22, H=64, E=9360, R=39, k=8), B.UBEP_PIPELINE_LOCAL),
+    (dict(T=20, H=64, E=13000, R=1, k=4), B.UBEP_PIPELINE_LOCAL),
+    (dict(T=229, H=30816, E=18, R=6, k=4, dedup=1), B.UBEP_PIPELINE_LOCAL),
+    (dict(T=238, H=34816, E=231, R=33, k=4, payload=1, dedup=1), 0),
+    (dict(T=260, H=38112, E=144, R=4, k=1), 0),
+])
+def test_where_the_counts_or_whole_rows_do_not_fit(cfg, pipeline):
+    _run(W.Config("w", seed=cfg["T"], **cfg), pipeline=pipeline)

@@ -42,3 +42,26 @@ def test_a_stage_of_short_fp8_rows_belongs_to_one_team(k):
                 wraps += 1
                 assert pl["stages"] % pl["teams"] == 0, (T, H, E, R, k, dedup, pipeline, count, quant, pl)
     assert seen > 100 and (k > 8 or wraps > 100)
+
+
+@pytest.mark.parametrize("pipeline,cfg", [
+    # (the layout by clusters needs more words per bin than the kernel that held every bin's bitmaps did)
+    (LOCAL, dict(T=22, H=64, E=9360, R=39, k=8)),
+    (LOCAL, dict(T=15, H=640, E=10215, R=15, k=20, payload=1)),
+    (LOCAL, dict(T=4, H=1128, E=9965, R=5, k=11, dedup=1, num_ctas=4)),
+    (AUTO, dict(T=3, H=24656, E=6066, R=1011, k=27)),
+    (AUTO, dict(T=179, H=36864, E=988, R=52, k=1, payload=1, dedup=1)),
+    (AUTO, dict(T=6, H=18880, E=6714, R=746, k=7, num_ctas=8)),
+    # (rank-level rows: the table fits, the maps of the expert-level outputs no longer do)
+    (LOCAL, dict(T=5622, H=512, E=12, R=1, k=7, payload=1, dedup=1)),
+])
+def test_calls_that_were_taken_before_clusters_are_still_taken(pipeline, cfg):
+    pl = plan(pipeline=pipeline, **cfg)
+    assert pl is not None and pl["smem"] <= SMEM
+    assert pl["chunks"] * pl["parts"] <= (cfg.get("num_ctas") or CTAS[0])
+
+
+def test_a_table_that_does_not_fit_is_refused_by_the_flag_free_schedule():
+    for dedup in (0, 1):
+        assert plan(T=40000, H=256, E=64, R=8, k=8, dedup=dedup, pipeline=LOCAL) is None
+        assert plan(T=40000, H=256, E=64, R=8, k=8, dedup=dedup) is not None
