@@ -732,6 +732,7 @@ int ubep_dispatch_sharded(ubep_buffer_t* buf, const void* x_local, const int32_t
     p.trace = nullptr;
     p.parts = 1;
     p.grid = p.nchunks;
+    p.local_fast = 0;   // (every bin's bitmaps, no maps of expert-level outputs)
     ubep::SmemPlan pl{};
     const bool whole_table = (int64_t)T * buf->cfg.topk <= kLocalMaxSlots &&
                              ubep::plan_dispatch(p, UBEP_PIPELINE_LOCAL, buf->max_smem - ubep::sharded_extra_smem(p), &pl) == 0;

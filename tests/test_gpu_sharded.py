@@ -38,8 +38,8 @@ def token_range(s, T, R):
     return s * T // R, (s + 1) * T // R
 
 
-def make_ranks(cfg, cap, wl_phys):
-    bufs = [Hn.make_buffer(cfg, cap) for _ in range(cfg.R)]
+def make_ranks(cfg, cap, wl_phys, num_ctas=0):
+    bufs = [Hn.make_buffer(cfg, cap, num_ctas=num_ctas) for _ in range(cfg.R)]
     ptrs = [b.arena.data_ptr() for b in bufs]
     for r, b in enumerate(bufs):
         if wl_phys is not None:
@@ -115,6 +115,19 @@ def test_sharded_dispatch_and_combine_match_the_oracle(case):
         if b1 > b0:
             Hn.check_combine(out, want[b0:b1])
         assert bufs[s].status() == 0
+
+
+def test_a_table_that_just_fits_beside_the_rows():
+    """Fewer CTAs than ranks, so that no chunks aligned with the ranks stand in for the whole table; one row per
+    (token, rank), whose maps of the expert-level outputs are no part of this path."""
+    cfg = W.Config("fits", T=6123, H=7400, E=55, R=5, k=1, dedup=1, seed=5112)
+    wl = W.make_workload(cfg)
+    _, lay, cap, recv = Hn.oracle_reference(wl, num_threads=8)
+    x, idx, w, _, _ = Hn.device_inputs(wl)
+    bufs = make_ranks(cfg, cap, None, num_ctas=2)
+    dispatch_all(bufs, cfg, x, idx, w)
+    for r in range(cfg.R):
+        check_rank(bufs, r, cfg, lay, recv)
 
 
 def test_a_receiver_whose_senders_have_not_run_gives_up_and_recovers():
