@@ -605,17 +605,22 @@ int ubep_dispatch_sync(ubep_buffer_t* buf, int protocol, const void* x, const in
     p.parts = 1;
     p.grid = p.nchunks;
     ubep::SmemPlan pl{};
-    const int extra = ubep::sync_extra_smem(p, protocol);
     // Small tables are recounted by every CTA; for larger ones TokenCnt and CalCumSum run as launches of their
     // own in front of the kernel, over the same chunks (as the phased schedule of ubep_dispatch does).
-    const bool whole_table = (int64_t)T * buf->cfg.topk <= kLocalMaxSlots &&
-                             ubep::plan_dispatch(p, ubep::kModeCluster, buf->max_smem - extra, &pl) == 0;   // (a cluster of one)
-    if (!whole_table && ubep::plan_dispatch(p, UBEP_PIPELINE_PHASED, buf->max_smem - extra, &pl) != 0)
-        return UBEP_ERR_ARG;
+    bool whole_table = false;
+    auto fits = [&](bool strips) {
+        const int room = buf->max_smem - ubep::sync_extra_smem(p, protocol, strips);
+        whole_table = (int64_t)T * buf->cfg.topk <= kLocalMaxSlots &&
+                      ubep::plan_dispatch(p, ubep::kModeCluster, room, &pl) == 0;   // (a cluster of one)
+        return whole_table || ubep::plan_dispatch(p, UBEP_PIPELINE_PHASED, room, &pl) == 0;
+    };
+    const bool strips = fits(true);
+    if (!strips && !fits(false)) return UBEP_ERR_ARG;   // (tables of ten thousand experts leave no 48 KB for the strips)
     const WireLayout& w = buf->wlay;
     ubep::SyncParams sp{};
     sp.protocol = protocol;
     sp.tff_blocks = w.tff_blocks;
+    sp.tff_strips = strips;
     sp.tff_wire = buf->wire + w.off[UBEP_SYNC_VIEW_TFF_WIRE];
     sp.sp_wire = buf->wire + w.off[UBEP_SYNC_VIEW_SP_WIRE];
     sp.checksum = reinterpret_cast<unsigned long long*>(buf->wire + w.off[UBEP_SYNC_VIEW_CHECKSUM]);

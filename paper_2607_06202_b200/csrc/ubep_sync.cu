@@ -384,7 +384,11 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
                 for (int b = 0; b < kBatch; ++b) {
                     const int g = b * 32 + lane;
                     if (g >= n || (missing >> b & 1u)) continue;
-                    if (kProto == kTFF) {
+                    if (kProto == kTFF && !sp.tff_strips) {
+                        const uint32_t dw[3] = {blk[b].y, blk[b].z, blk[b].w};
+                        for (int q = 0; q < 3; ++q)
+                            if (3 * (g0 + g) + q < nwords) put_word(grow, 3 * (g0 + g) + q, dw[q]);
+                    } else if (kProto == kTFF) {
                         mine[3 * g] = blk[b].y;
                         mine[3 * g + 1] = blk[b].z;
                         mine[3 * g + 2] = blk[b].w;
@@ -401,7 +405,7 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
                     }
                 }
                 ok = __all_sync(0xffffffffu, ok);
-                if (kProto == kTFF) {
+                if (kProto == kTFF && sp.tff_strips) {
                     __syncwarp();   // the lanes' words are in the strip (the vote orders no memory)
                     // words [3 * g0, 3 * g0 + 3 * n) of the wire row (a strip begins on a multiple of four words)
                     for (int q = lane; ok && q < kStripWords / 4; q += 32) {
@@ -481,7 +485,7 @@ template <int kProto>
 cudaError_t launch_one(const Params& p, const SmemPlan& pl, const SyncParams& sp, bool whole_table, cudaStream_t st) {
     auto kern = whole_table ? (p.payload ? sync_dispatch_kernel<kProto, true, true> : sync_dispatch_kernel<kProto, false, true>)
                             : (p.payload ? sync_dispatch_kernel<kProto, true, false> : sync_dispatch_kernel<kProto, false, false>);
-    const int smem = pl.total + sync_extra_smem(p, kProto);
+    const int smem = pl.total + sync_extra_smem(p, kProto, sp.tff_strips != 0);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     // Receivers wait for senders that are other CTAs of this grid: a cooperative launch, which the
@@ -501,8 +505,9 @@ cudaError_t launch_one(const Params& p, const SmemPlan& pl, const SyncParams& sp
 
 }  // namespace
 
-int sync_extra_smem(const Params& p, int protocol) {
-    return p.R * 8 + 128 + qrow_bytes(p) + 16 + (protocol != kTFF || strips_in_ring(p) ? 0 : kWarps * kStripWords * 4);
+int sync_extra_smem(const Params& p, int protocol, bool strips) {
+    const bool room = protocol == kTFF && strips && !strips_in_ring(p);
+    return p.R * 8 + 128 + qrow_bytes(p) + 16 + (room ? kWarps * kStripWords * 4 : 0);
 }
 
 cudaError_t launch_sync_dispatch(const Params& p, const SmemPlan& pl, const SyncParams& sp, bool whole_table,

@@ -14,6 +14,7 @@ constexpr int kSyncTimeSlots = 8;    // per-CTA time stamps of the last call
 struct SyncParams {
     int protocol;                   // UBEP_SYNC_*
     int tff_blocks;                 // 16-byte DataBlocks per row: ceil(rowB / 12)
+    int tff_strips;                 // Token-Flag payload passes through shared memory (else in single words)
     uint8_t* tff_wire;              // [R * cap][16 * tff_blocks]
     uint8_t* sp_wire;               // [R * cap][rowB]
     unsigned long long* checksum;   // [2][R]
@@ -25,8 +26,8 @@ struct SyncParams {
     unsigned long long* times;      // [grid][kSyncTimeSlots]
 };
 
-// Dynamic shared memory the kernel needs beyond the dispatch plan's total.
-int sync_extra_smem(const Params& p, int protocol);
+// Dynamic shared memory the kernel needs beyond the dispatch plan's total; with Token-Flag strips or without.
+int sync_extra_smem(const Params& p, int protocol, bool strips);
 
 // whole_table: every CTA derives the layout from the whole routing table in shared memory; otherwise the
 // count / prefix-sum launches (launch_count_scan) have run before over the same p.nchunks chunks.

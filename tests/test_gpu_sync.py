@@ -37,6 +37,9 @@ CASES = {
     "large": W.Config("large", T=1500, H=256, E=32, R=8, k=8, seed=4108),
     "large_fp8_dedup": W.Config("large_fp8_dedup", T=2100, H=256, E=64, R=16, k=8, payload=1, dedup=1, seed=4109),
     "large_replicas": W.Config("large_replicas", T=3000, H=128, E=36, R=4, k=4, seed=4110, E_logical=32),
+    # so many experts that no room is left for the strips through which Token-Flag payload leaves otherwise
+    "many_experts": W.Config("many_experts", T=24, H=64, E=16000, R=2, k=2, seed=4111),
+    "many_experts_fp8": W.Config("many_experts_fp8", T=30, H=256, E=15000, R=10, k=4, payload=1, dedup=1, seed=4112),
 }
 
 
