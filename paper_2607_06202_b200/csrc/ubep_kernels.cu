@@ -238,6 +238,7 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
     int* item_src = reinterpret_cast<int*>(smem + pl.off_item);           // [stages] (chunk << 16 | index), -1 = end
     int* item_pos = item_src + kStealStages;                              // [stages, k] destinations of stolen tokens
     int head = 0, tail = 0;   // rows whose load was issued / whose copies were issued
+    unsigned ticket = 0u, epoch_mine = 0u;   // (flag-free kernel, FP8 rows)
     // load of the feeder's next token into ring stage head % stages
     auto issue_item = [&](int tl) {
         const int s = head % stages;
@@ -392,10 +393,12 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
             }
         }
     } else {
+        unsigned epoch_ctr = 0u;
         if (kMode == kModeLocal) {
             const RankMaps rm{bmaps.bm, bmaps.mask_t, (p.R + 31) / 32, ((p.R + 31) / 32) * 32, (p.T + 31) / 32};
             local_stage_and_rank_maps(p, ids_sm, rm, rm.groups, 0, kWarps, lane);   // the table first, the rows after it
             group_sync(2, kThreads);
+            if (lane == 0) epoch_ctr = ld_relaxed(p.epoch_ctr);
         } else if (kMode == kModeCluster) {
             if (!kSteal) {   // (see above)
                 issue_first(min(min(2, p.prefetch_rows), min(stages, ntok)));
@@ -479,6 +482,14 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
                 break;
             }
         }
+        if (kMode == kModeLocal && lane == 0) {
+            // The epoch (see the row group): asked for in front of the rows, and the ticket taken here, whatever became of
+            // the loads; its answer is looked at further down.  (By the first warp of the row group, which quantises, the two
+            // round trips to L2 held the first row up: 0.2 us of a layer of 1 to 128 tokens.)
+            epoch_mine = epoch_from_counter(epoch_ctr);
+            *x.epoch_late = epoch_mine;
+            ticket = atomicAdd(p.done_ticket, 1u);
+        }
     }
     if (kFp8 && kMode == kModeLocal && ok) {
         // metadata of the CTA's own tokens (see the row group): one warp, no barrier but its own
@@ -493,6 +504,7 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
             if (part == 0) local_meta_dedup(p, t0, t1, ids_sm, pos_raw, reinterpret_cast<int*>(w_sm), w_own, lane, 32);
         }
     }
+    if (kFp8 && kMode == kModeLocal && lane == 0) epoch_finish_check_in(p, ticket, epoch_mine);
     if (!ok && lane == 0) {
         report(p.status, kErrTimeout);  // a wait gave up: record it and let everybody leave
         abort_flag = 1;
@@ -739,24 +751,23 @@ __device__ __forceinline__ int layout_group(Cta& x) {
                 order_destinations(p, pos_raw, key, pos, ntok * p.k, gtid, rn);
                 group_sync(1, rn);
             }
-            unsigned ticket = 0u, ep_mine = 0u;
             if (gtid == 0) {
                 mbar_arrive(&ready_bar);
                 trace(p, c, kTrReady);
+            }
+            // FP8 rows: every copy waits for a quantised row, so this group goes straight on to quantise
+            // (its first warp to issue the copies of long rows; the warps of the duty group take no part, a CTA of
+            // this kernel has few rows).  The epoch, and the metadata of the own tokens, are left to the loader warp,
+            // which is idle once the CTA's few rows are asked for.
+            if (kFp8) return 1;
+            unsigned ticket = 0u, ep_mine = 0u;
+            if (gtid == 0) {
                 // The epoch: nothing needs it before the kernel's last lines.  A relaxed load (nothing
                 // is ordered against it); its value is in hand before the ticket is taken -- the store
                 // to shared memory needs it -- and the ticket's answer is looked at at the end.
                 ep_mine = epoch_from_counter(ld_relaxed(p.epoch_ctr));
                 *x.epoch_late = ep_mine;
                 ticket = atomicAdd(p.done_ticket, 1u);
-            }
-            if (kFp8) {
-                // FP8 rows: every copy waits for a quantised row, so this group goes straight on to quantise
-                // (its first warp to issue the copies; the warps of the duty group take no part, a CTA of
-                // this kernel has few rows).  The metadata of the own tokens is written by the loader warp,
-                // which is idle once the CTA's few rows are asked for.
-                if (gtid == 0) epoch_finish_check_in(p, ticket, ep_mine);
-                return 1;
             }
             if (part == 0) {
                 float* w_own = reinterpret_cast<float*>(key);   // the ordering keys are no longer needed
@@ -1116,8 +1127,7 @@ __device__ __forceinline__ void fp8_worker(Cta& x, int qw) {
             }
         }
         good = good && __all_sync(0xffffffffu, mbar_wait_idle(&full_bar[s], par, abortp));
-        if (tw > 1) good = !group_or(5 + team, tw * 32, !good);   // (the warps of a team leave together)
-        if (!good) break;
+        if (tw == 1 && !good) break;
         const int from = kSteal ? q.item_src[s] : ((ch << 16) | n);
         if (from < 0) break;   // the loader's closing item
         if (i >= 2) {          // the copies of the row before the last one have read its slot
@@ -1133,7 +1143,7 @@ __device__ __forceinline__ void fp8_worker(Cta& x, int qw) {
         uint8_t* dst = q.out_ring + (size_t)os * pl.out_stage_bytes;
         float* dst_scale = reinterpret_cast<float*>(dst + out_bytes);
         // four vectors per thread and trip, independent of each other
-        for (int vb = m * 32; vb < nvec; vb += 4 * tw * 32) {
+        for (int vb = m * 32; good && vb < nvec; vb += 4 * tw * 32) {
             uint4 in[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -1153,7 +1163,10 @@ __device__ __forceinline__ void fp8_worker(Cta& x, int qw) {
             }
         }
         fence_proxy_async_smem();   // the bulk stores read what we just wrote
-        team_sync();
+        // (each warp of a team begins as soon as the row is there, some of them before the rows are assigned; they leave together)
+        if (tw > 1) good = !group_or(5 + team, tw * 32, !good);
+        else __syncwarp();
+        if (!good) break;
         if (lane == 0) mbar_arrive(&empty_bar[s]);
         if (m != 0) continue;
         if (tw == 1 && i == 0 && !ready && !__any_sync(0xffffffffu, mbar_test_wait(&ready_bar, 0))) continue;
@@ -1276,7 +1289,7 @@ __global__ void __launch_bounds__((kDispatchThreads<kMode, kFp8>), 1) dispatch_k
           // (its stage is never loaded a second time, no order of destinations is asked for, a lane per copy)
           kMode == kModeLocal && !kFp8 && !kSteal && !p.ordered && p.k <= 32 && t1 > t0 &&
               t1 - t0 <= stages,
-          0, kMode == kModeCluster || kMode == kModeLocal,
+          0, kMode == kModeCluster || (kMode == kModeLocal && !kFp8),
           // the mover; the row group (rank-level rows, bf16) or the duty group (clusters); who issues FP8 copies
           1 + (kMode == kModeCluster ? nw - (kFp8 && pl.q_long ? 1 : 0) : kFp8 ? 0 : kRowWarps) +
               (kFp8 ? (pl.q_long ? 1 : pl.q_warps) : 0)};
