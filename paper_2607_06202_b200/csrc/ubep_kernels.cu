@@ -46,6 +46,11 @@ __global__ void __launch_bounds__(256) scan_kernel(const Params p) {
     scan_rank_sources(p, blockIdx.x, sm_i, threadIdx.x, 256);
 }
 
+// What a kernel instance moves: bf16 rows, or FP8 rows in one of the two arrangements of the comment above Fp8Ring.  An instance
+// holds the code of one of them: what a CTA runs once arrives cold, and with both in one instance a layer of 1 to 128 tokens
+// took 0.3 to 0.5 us more.  Token stealing goes with long rows.
+enum RowKind { kBf16Rows = 0, kShortFp8Rows = 1, kLongFp8Rows = 2 };
+
 constexpr int kRowWarps = 4;   // flag-free kernel, rank-level rows: warps 1 .. 4 assign the rows of the CTA's tokens
 
 // Everything the roles of one dispatch CTA share.
@@ -152,8 +157,9 @@ static __device__ __noinline__ int send_short_rows(int n0, int ntok, int head, i
 // ------------------------------------------------------------------------ mover warp
 // Warp 0.  Lane 0 issues the TMA loads; for bf16 rows lane j issues the TMA store of slot j,
 // so the k copies of a row are issued side by side; for FP8 rows the warp only loads.
-template <int kMode, bool kFp8, bool kSteal>
+template <int kMode, int kRows, bool kSteal>
 __device__ __forceinline__ void mover_warp(Cta& x) {
+    constexpr bool kFp8 = kRows != kBf16Rows;
     if (kMode == kModeCluster) cluster_arrive();   // (this warp counts nothing)
     if (kMode != kModeLocal) {
         // The epoch: one acquire load and one ticket, two round trips to L2.  This warp has nothing
@@ -467,17 +473,9 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
                 issue_item(tl);
                 issued = head;
             } else {
-                // closing items, one for each team of quantising warps (without stealing they know the row count)
-                for (int q = 0; ok && q < (pl.q_long ? 1 : pl.q_teams); ++q) {
-                    const int cs = (head + q) % stages;
-                    if (head + q >= stages) {
-                        ok = mbar_wait(&empty_bar[cs], (((head + q) / stages) - 1) & 1, abortp);
-                        ok = __all_sync(0xffffffffu, ok);
-                    }
-                    if (ok && lane == 0) {
-                        item_src[cs] = -1;
-                        mbar_arrive(&full_bar[cs]);
-                    }
+                if (lane == 0) {   // the closing item
+                    item_src[s] = -1;
+                    mbar_arrive(&full_bar[s]);
                 }
                 break;
             }
@@ -692,8 +690,9 @@ __device__ __forceinline__ void cluster_duty(Cta& x, int dtid, int dn, int bar) 
 // Warps 1..15: TokenCnt, CalCumSum (by exchange or alone), slot -> row assignment; releases
 // the movers and then writes what nobody inside the kernel waits for.  Returns 1, 0 if a wait ran
 // out, or 2 for a warp that has done its share of the counting and now leaves to quantise.
-template <int kMode, bool kFp8, bool kSteal>
+template <int kMode, int kRows, bool kSteal>
 __device__ __forceinline__ int layout_group(Cta& x) {
+    constexpr bool kFp8 = kRows != kBf16Rows;
     UBEP_CTA_LOCALS(x, !kFp8);
     bool ok = true;
     const int* ids = ids_sm;  // staged slots of this CTA's tokens
@@ -803,7 +802,7 @@ __device__ __forceinline__ int layout_group(Cta& x) {
     } else if (kMode == kModeCluster) {
         cluster_layout<kFp8, kSteal>(x);
         if (kFp8 && gw >= nw) return 2;   // off to quantise
-        const int d0 = kFp8 && pl.q_long ? 1 : 0;
+        constexpr int d0 = kRows == kLongFp8Rows ? 1 : 0;
         if (gw < d0) return 1;            // off to issue the copies
         // the others write what nobody waits for
         cluster_duty<kFp8>(x, gtid - d0 * 32, gn - d0 * 32, kFp8 ? 3 : 1);
@@ -1084,7 +1083,6 @@ __device__ __forceinline__ void fp8_store_issuer(Cta& x) {
 }
 
 // Short rows (see Fp8Ring): quantising warp qw, in teams that send what they have quantised themselves.
-template <bool kSteal>
 __device__ __forceinline__ void fp8_worker(Cta& x, int qw) {
     UBEP_CTA_LOCALS(x, false);
     const Fp8Ring q = fp8_ring(x);
@@ -1096,7 +1094,7 @@ __device__ __forceinline__ void fp8_worker(Cta& x, int qw) {
     };
     const int nvec = (int)in_bytes / 16;   // 8-channel vectors in this CTA's piece
     bool ready = false, good = true;
-    int sent = 0, from0 = 0, from1 = 0;    // rows of this team on their way; origins of the rows in its two slots
+    int sent = 0;   // rows of this team on their way
     auto layout_done = [&]() {
         if (!ready) {
             good = __all_sync(0xffffffffu, mbar_wait_idle(&ready_bar, 0, abortp) && !*abortp);   // no rows without a layout
@@ -1105,13 +1103,13 @@ __device__ __forceinline__ void fp8_worker(Cta& x, int qw) {
     };
     auto send = [&]() {
         const int os = team * 2 + (sent & 1);
-        fp8_issue<kSteal>(x, q, q.out_ring + (size_t)os * pl.out_stage_bytes, (sent & 1) ? from1 : from0, os);
+        fp8_issue<false>(x, q, q.out_ring + (size_t)os * pl.out_stage_bytes, (ch << 16) | (team + sent * teams), os);
         ++sent;
     };
     int i = 0;
     for (;; ++i) {
         const int n = team + i * teams;
-        if (!kSteal && n >= ntok) break;
+        if (n >= ntok) break;
         const int s = n % stages;
         const unsigned par = (n / stages) & 1;
         if (tw == 1 && sent < i) {   // the first row still waits for the layout: whichever comes first
@@ -1128,17 +1126,11 @@ __device__ __forceinline__ void fp8_worker(Cta& x, int qw) {
         }
         good = good && __all_sync(0xffffffffu, mbar_wait_idle(&full_bar[s], par, abortp));
         if (tw == 1 && !good) break;
-        const int from = kSteal ? q.item_src[s] : ((ch << 16) | n);
-        if (from < 0) break;   // the loader's closing item
         if (i >= 2) {          // the copies of the row before the last one have read its slot
             if (m == 0) bulk_wait_read<1>();
             team_sync();
         }
         const int os = team * 2 + (i & 1);
-        if (i & 1) from1 = from;
-        else from0 = from;
-        if (kSteal && m == 0 && (from >> 16) != ch)   // a row of another chunk: its destinations travel with it
-            for (int j = lane; j < p.k; j += 32) q.out_pos[os * p.k + j] = q.item_pos[s * p.k + j];
         const uint8_t* src = smem + (size_t)s * pl.stage_bytes;
         uint8_t* dst = q.out_ring + (size_t)os * pl.out_stage_bytes;
         float* dst_scale = reinterpret_cast<float*>(dst + out_bytes);
@@ -1196,11 +1188,12 @@ __device__ __forceinline__ void fp8_worker(Cta& x, int qw) {
 // small batch is placed during the dispatch, the dispatch after it is let in as soon as this one leaves, and the combine
 // runs with the registers that are left (sixteen layers of 128 tokens: 208 us; with one combine CTA beside it 179).
 // A warp that leaves at once holds the registers in question.
-template <int kMode, bool kFp8>
-constexpr int kDispatchThreads = kThreads + (kMode == kModeLocal && !kFp8 ? 32 : 0);
-template <int kMode, bool kFp8, bool kSteal>
-__global__ void __launch_bounds__((kDispatchThreads<kMode, kFp8>), 1) dispatch_kernel(const Params p, const SmemPlan pl) {
-    if ((kDispatchThreads<kMode, kFp8>) > kThreads && threadIdx.x >= kThreads) return;
+template <int kMode, int kRows>
+constexpr int kDispatchThreads = kThreads + (kMode == kModeLocal && kRows == kBf16Rows ? 32 : 0);
+template <int kMode, int kRows, bool kSteal>
+__global__ void __launch_bounds__((kDispatchThreads<kMode, kRows>), 1) dispatch_kernel(const Params p, const SmemPlan pl) {
+    constexpr bool kFp8 = kRows != kBf16Rows, kLong = kRows == kLongFp8Rows;
+    if ((kDispatchThreads<kMode, kRows>) > kThreads && threadIdx.x >= kThreads) return;
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) uint64_t full_bar[kMaxStages];    // input row landed
     __shared__ __align__(8) uint64_t empty_bar[kMaxStages];   // FP8: input row consumed
@@ -1225,9 +1218,9 @@ __global__ void __launch_bounds__((kDispatchThreads<kMode, kFp8>), 1) dispatch_k
     if (tid == 0) {
         for (int s = 0; s < stages; ++s) {
             mbar_init(&full_bar[s], 1);
-            mbar_init(&empty_bar[s], !kFp8 ? 1 : pl.q_long ? pl.q_warps : pl.q_team_warps);
+            mbar_init(&empty_bar[s], !kFp8 ? 1 : kLong ? pl.q_warps : pl.q_team_warps);
         }
-        for (int s = 0; kFp8 && pl.q_long && s < pl.out_stages; ++s) {
+        for (int s = 0; kLong && s < pl.out_stages; ++s) {
             mbar_init(&out_full[s], pl.q_warps);
             mbar_init(&out_empty[s], 1);
         }
@@ -1291,22 +1284,25 @@ __global__ void __launch_bounds__((kDispatchThreads<kMode, kFp8>), 1) dispatch_k
               t1 - t0 <= stages,
           0, kMode == kModeCluster || (kMode == kModeLocal && !kFp8),
           // the mover; the row group (rank-level rows, bf16) or the duty group (clusters); who issues FP8 copies
-          1 + (kMode == kModeCluster ? nw - (kFp8 && pl.q_long ? 1 : 0) : kFp8 ? 0 : kRowWarps) +
-              (kFp8 ? (pl.q_long ? 1 : pl.q_warps) : 0)};
+          1 + (kMode == kModeCluster ? nw - (kLong ? 1 : 0) : kFp8 ? 0 : kRowWarps) +
+              (kLong ? 1 : kFp8 ? pl.q_warps : 0)};
 
     if (x.warp == 0) {
-        mover_warp<kMode, kFp8, kSteal>(x);
+        mover_warp<kMode, kRows, kSteal>(x);
     } else {
-        const int lg = layout_group<kMode, kFp8, kSteal>(x);   // 0 = a wait ran out, 1 = done, 2 = left to quantise
+        const int lg = layout_group<kMode, kRows, kSteal>(x);   // 0 = a wait ran out, 1 = done, 2 = left to quantise
         // (2: beside the rest of the layout; 1: after it, unless the quantising warps are others)
         const int qw = x.warp - pl.q_warp0;
-        if (kFp8 && pl.q_long && lg == 1 && x.warp == 1) {
-            fp8_store_issuer<kSteal>(x);
+        if (kLong && lg == 1 && x.warp == 1) {
+            if constexpr (kLong) fp8_store_issuer<kSteal>(x);
             if (x.early_arrival) x.rows_landed(0);
         } else if (kFp8 && (lg == 2 || (lg == 1 && !beside)) && qw >= 0 && qw < pl.q_warps) {
-            if (pl.q_long) fp8_quantiser<kSteal>(x, qw);
-            else fp8_worker<kSteal>(x, qw);
-            if (x.early_arrival && !pl.q_long) x.rows_landed(0);
+            if constexpr (kLong) {
+                fp8_quantiser<kSteal>(x, qw);
+            } else if constexpr (kFp8) {
+                fp8_worker(x, qw);
+                if (x.early_arrival) x.rows_landed(0);
+            }
         }
     }
     if (kMode == kModeCluster) cluster_wait();   // the others have read what this CTA counted
@@ -1593,7 +1589,7 @@ int plan_dispatch(const Params& p, int mode, int max_smem, SmemPlan* out) {
         const int most = fast ? kFastQuantWarps + (pl.q_long ? 0 : 1) : kWarps - pl.q_warp0;
         pl.q_warps = p.quant_warps < most ? p.quant_warps : most;
         pl.q_teams = pl.q_warps;
-        if (!p.steal && pl.q_teams > chunk_tokens) pl.q_teams = chunk_tokens < 1 ? 1 : chunk_tokens;
+        if (pl.q_teams > chunk_tokens) pl.q_teams = chunk_tokens < 1 ? 1 : chunk_tokens;
         pl.out_stages = !pl.q_long ? 2 * pl.q_teams : beside ? kMaxOutStages : kOutStages;   // at most
     }
     const int item_ints = p.steal ? (kStealStages + pl.out_stages) * (p.k + 1) : 0;
@@ -1705,25 +1701,30 @@ static cudaError_t allow_dynamic_smem(const void* kern, int bytes, std::atomic<i
     return e;
 }
 
-template <int kMode, bool kFp8, bool kSteal>
+template <int kMode, int kRows, bool kSteal>
 static cudaError_t allow_dispatch_smem(int bytes) {
     static std::atomic<int> granted[kAttrDevices];
-    return allow_dynamic_smem(reinterpret_cast<const void*>(dispatch_kernel<kMode, kFp8, kSteal>), bytes, granted);
+    return allow_dynamic_smem(reinterpret_cast<const void*>(dispatch_kernel<kMode, kRows, kSteal>), bytes, granted);
 }
 
-template <int kMode, bool kFp8, bool kSteal>
+template <int kMode, int kRows, bool kSteal>
 static cudaError_t launch_dispatch_s(const Params& p, const SmemPlan& pl, cudaStream_t st) {
-    auto kern = dispatch_kernel<kMode, kFp8, kSteal>;
-    cudaError_t e = allow_dispatch_smem<kMode, kFp8, kSteal>(pl.total);
+    auto kern = dispatch_kernel<kMode, kRows, kSteal>;
+    cudaError_t e = allow_dispatch_smem<kMode, kRows, kSteal>(pl.total);
     if (e != cudaSuccess) return e;
-    return launch_overlapped(kern, p.grid, kDispatchThreads<kMode, kFp8>, (size_t)pl.total, st, kMode == kModeFused,
+    return launch_overlapped(kern, p.grid, kDispatchThreads<kMode, kRows>, (size_t)pl.total, st, kMode == kModeFused,
                              kMode == kModeCluster ? p.cluster : 1, p, pl);
 }
 
-template <int kMode, bool kFp8>
+template <int kMode>
 static cudaError_t launch_dispatch_t(const Params& p, const SmemPlan& pl, cudaStream_t st) {
-    if (kMode != kModeLocal && p.steal) return launch_dispatch_s<kMode, kFp8, true>(p, pl, st);
-    return launch_dispatch_s<kMode, kFp8, false>(p, pl, st);
+    if constexpr (kMode != kModeLocal) {
+        if (p.steal) return p.payload ? launch_dispatch_s<kMode, kLongFp8Rows, true>(p, pl, st)
+                                      : launch_dispatch_s<kMode, kBf16Rows, true>(p, pl, st);
+    }
+    if (!p.payload) return launch_dispatch_s<kMode, kBf16Rows, false>(p, pl, st);
+    return pl.q_long ? launch_dispatch_s<kMode, kLongFp8Rows, false>(p, pl, st)
+                     : launch_dispatch_s<kMode, kShortFp8Rows, false>(p, pl, st);
 }
 
 // TokenCnt and CalCumSum as two launches over the whole routing table (chunk histograms, then per rank
@@ -1769,8 +1770,8 @@ int cluster_ctas(int cluster, int max_smem) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (allow_dispatch_smem<kModeCluster, false, false>(smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&n, reinterpret_cast<const void*>(dispatch_kernel<kModeCluster, false, false>), &cfg) != cudaSuccess)
+    if (allow_dispatch_smem<kModeCluster, kBf16Rows, false>(smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, reinterpret_cast<const void*>(dispatch_kernel<kModeCluster, kBf16Rows, false>), &cfg) != cudaSuccess)
         n = 0;
     (void)cudaGetLastError();
     if (cached) known[dev][slot].store(n * cluster + 1, std::memory_order_relaxed);
@@ -1783,17 +1784,11 @@ cudaError_t launch_dispatch(const Params& p, int mode, const SmemPlan& pl, cudaS
     if (mode == kModePhased) {
         if ((e = launch_count_scan(p, pl, st)) != cudaSuccess) return e;
         *launches = 3;
-        return p.payload ? launch_dispatch_t<kModePhased, true>(p, pl, st)
-                         : launch_dispatch_t<kModePhased, false>(p, pl, st);
+        return launch_dispatch_t<kModePhased>(p, pl, st);
     }
-    if (mode == kModeCluster)
-        return p.payload ? launch_dispatch_t<kModeCluster, true>(p, pl, st)
-                         : launch_dispatch_t<kModeCluster, false>(p, pl, st);
-    if (mode == kModeLocal)
-        return p.payload ? launch_dispatch_t<kModeLocal, true>(p, pl, st)
-                         : launch_dispatch_t<kModeLocal, false>(p, pl, st);
-    return p.payload ? launch_dispatch_t<kModeFused, true>(p, pl, st)
-                     : launch_dispatch_t<kModeFused, false>(p, pl, st);
+    if (mode == kModeCluster) return launch_dispatch_t<kModeCluster>(p, pl, st);
+    if (mode == kModeLocal) return launch_dispatch_t<kModeLocal>(p, pl, st);
+    return launch_dispatch_t<kModeFused>(p, pl, st);
 }
 
 template <int K, bool kStream>
