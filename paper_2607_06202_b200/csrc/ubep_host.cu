@@ -926,7 +926,7 @@ int ubep_debug_plan(const ubep_config_t* cfg, int32_t T, int32_t max_smem, const
     plan[UBEP_DEBUG_PLAN_LONG_ROWS] = pl.q_long;
     plan[UBEP_DEBUG_PLAN_TEAMS] = pl.q_teams;
     plan[UBEP_DEBUG_PLAN_TEAM_WARPS] = pl.q_team_warps;
-    plan[UBEP_DEBUG_PLAN_SMEM] = pl.total;
+    plan[UBEP_DEBUG_PLAN_SMEM] = ubep::with_room_beside(pl.total);
     return UBEP_OK;
 }
 

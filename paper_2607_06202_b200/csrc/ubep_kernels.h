@@ -12,6 +12,7 @@ namespace ubep {
 int plan_dispatch(const Params& p, int mode, int max_smem, SmemPlan* out);
 
 int cluster_ctas(int cluster, int max_smem);
+int with_room_beside(int dynamic);   // the dynamic shared memory a dispatch with a plan of this size asks for
 bool short_rows(const Params& p);
 cudaError_t launch_count_scan(const Params& p, const SmemPlan& pl, cudaStream_t st);
 cudaError_t launch_dispatch(const Params& p, int mode, const SmemPlan& pl, cudaStream_t st, int* launches);

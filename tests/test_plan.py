@@ -65,3 +65,17 @@ def test_a_table_that_does_not_fit_is_refused_by_the_flag_free_schedule():
     for dedup in (0, 1):
         assert plan(T=40000, H=256, E=64, R=8, k=8, dedup=dedup, pipeline=LOCAL) is None
         assert plan(T=40000, H=256, E=64, R=8, k=8, dedup=dedup) is not None
+
+
+@pytest.mark.parametrize("payload", [0, 1])
+def test_a_combine_cta_fits_beside_a_small_dispatch(payload):
+    """An SM's shared memory is cut to the smallest size that holds the dispatch's CTA (with its static memory and the 1 KB
+    every CTA takes): 1 KB of it must be left, or the combine is placed only when the dispatch has ended."""
+    sizes = [kb * 1024 for kb in (8, 16, 32, 64, 100, 132, 164, 196, 228)]
+    for H, T, (E, R, k) in itertools.product((256, 512, 1024, 2048, 4096, 5120, 7168), (1, 13, 40, 74, 90, 128, 200, 256, 512),
+                                             ((16, 4, 2), (32, 8, 4), (128, 8, 4), (256, 32, 8))):
+        pl = plan(T, H, E, R, k, payload=payload, dedup=1)
+        for static in (768, 1024, 1280):
+            need = pl["smem"] + static + 1024
+            size = next(s for s in sizes if s >= need)
+            assert size - need >= 1024 or size == sizes[-1], (H, T, E, R, k, pl, static)
