@@ -458,7 +458,8 @@ int ubep_debug_trace(ubep_buffer_t *buf, int32_t enable);
  * warps first; the count group is what goes on through the flag exchange.  n = 0: all 15 warps
  * compute the layout and up to 14 of them quantise afterwards.  n = -1 (default): 8, or 0 when slices
  * are long enough for token stealing.  Applies to the PHASED and FUSED schedules; the flag-free
- * LOCAL schedule, whose layout waits for nobody, always runs as n = 0.
+ * LOCAL schedule, whose layout waits for nobody, always runs as n = 0, and where clusters count the table
+ * it is always 5 warps.
  * ubep_debug_set_quant_warps: at most n warps quantise (1 <= n <= 14, default 14), the rest idle.
  * ubep_debug_set_prefetch_rows: the loader fetches at most n rows before the layout is done
  * (default: as many as the rings hold).

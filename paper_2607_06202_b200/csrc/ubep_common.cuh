@@ -307,7 +307,7 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 // Where the dispatch kernel keeps things in dynamic shared memory (byte offsets).
 struct SmemPlan {
     int stages, stage_bytes;          // input row ring
-    int trip_rows;                    // bf16 rows whose copies leave side by side (short rows that all fit in the ring)
+    int trip_rows;                    // bf16: short rows whose copies leave side by side (any number of tokens)
     int out_stages, out_stage_bytes;  // FP8: quantised rows in shared memory (long rows: a ring; short ones: two per team)
     int q_long;                       // ... 1 = long rows
     int q_warps, q_warp0;             // ... quantising warps, the first of them

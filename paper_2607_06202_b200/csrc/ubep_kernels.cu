@@ -1177,17 +1177,20 @@ __device__ __forceinline__ void fp8_worker(Cta& x, int qw) {
 }
 
 // --------------------------------------------------------------------- dispatch kernel
-// Warp roles: warp 0 = mover; warps 1..15 = layout group (count, prefix sums, row
-// assignment).  FP8 rows: warp 0 only loads; either the layout group is warps 1 .. count_warps and
-// the warps behind them quantise beside it (the kernels whose layout waits for other CTAs or was
-// computed by earlier launches), or all 15 warps compute the layout and warps 2..15 quantise
-// afterwards (the flag-free kernel, whose layout is pure computation); warp 1 issues the copies of long rows
-// once the layout is done.
+// Warp roles: warp 0 = mover; warps 1..15 = layout group (count, prefix sums, row assignment).  FP8 rows: warp 0 only loads,
+// and some of the others quantise (plan_dispatch: q_warp0, q_warps):
+//   clusters    all 15 warps count, then warps 6..15 quantise beside the rest of the layout, which warps 1..5 do;
+//   FUSED, PHASED with a count group   the same with warps 1..count_warps; without one all 15 compute the layout and
+//               warps 2..15 (short rows: 1..15, at most 14) quantise afterwards;
+//   LOCAL       warps 1..4 assign the rows and then quantise with the next warps, five or six in all (warp 1 not with long
+//               rows); the others write the expert-level outputs.
+// Warp 1 issues the copies of long rows once the layout is done; short rows are sent by who quantised them.
 //
-// The flag-free instance needs so few registers that two combine CTAs would fit beside it.  Then every combine CTA of a
-// small batch is placed during the dispatch, the dispatch after it is let in as soon as this one leaves, and the combine
-// runs with the registers that are left (sixteen layers of 128 tokens: 208 us; with one combine CTA beside it 179).
-// A warp that leaves at once holds the registers in question.
+// The flag-free instance for bf16 rows needs so few registers that two combine CTAs of top-8 (64 registers) would fit beside it.
+// Then every combine CTA of a small batch is placed during the dispatch, the dispatch after it is let in as soon as this one
+// leaves, and the combine runs with the registers that are left (sixteen layers of 128 tokens, top-8: 208 us; with one combine CTA
+// beside it 179).  A warp that leaves at once holds the registers in question.  (The combines of top-4 and top-2 take 40 and 32
+// registers, of which two and three CTAs still fit: no harm was seen there, 1 to 512 tokens of 256 to 2048 channels.)
 template <int kMode, int kRows>
 constexpr int kDispatchThreads = kThreads + (kMode == kModeLocal && kRows == kBf16Rows ? 32 : 0);
 template <int kMode, int kRows, bool kSteal>

@@ -7,8 +7,8 @@
 
 namespace ubep {
 
-// Shared-memory plan of the dispatch kernel (ring depth, offsets, total); -1 if the
-// bookkeeping of this call does not fit beside a four-row ring.
+// Shared-memory plan of the dispatch kernel (ring depth, offsets, total); -1 if the bookkeeping of this call does not
+// fit beside a ring of four rows (FP8 rows without stealing: two, and the quantised rows).
 int plan_dispatch(const Params& p, int mode, int max_smem, SmemPlan* out);
 
 int cluster_ctas(int cluster, int max_smem);
