@@ -80,3 +80,26 @@ def test_an_expert_named_twice(k, dedup):
 ])
 def test_where_the_counts_or_whole_rows_do_not_fit(cfg, pipeline):
     _run(W.Config("w", seed=cfg["T"], **cfg), pipeline=pipeline)
+
+
+@pytest.mark.parametrize("cfg", [
+    dict(T=4096, H=4096, E=128, R=16, k=8),   # 28 rows per CTA, ten teams of one warp
+    dict(T=4097, H=4096, E=128, R=16, k=8, dedup=1),
+    dict(T=8192, H=7168, E=64, R=8, k=4),     # 56 rows per CTA, seven teams
+])
+def test_short_fp8_rows_whose_ring_is_used_more_than_once(cfg):
+    wl = W.make_workload(W.Config("ring", payload=1, seed=cfg["T"], **cfg))
+    _, lay, cap, recv = Hn.oracle_reference(wl, num_threads=8)
+    buf = Hn.make_buffer(wl.cfg, cap)
+    x, idx, w, _, _ = Hn.device_inputs(wl)
+    for _ in range(4):
+        buf.recv_x.fill_(Hn.FILL)
+        buf.dispatch(x, idx, w)
+        Hn.check_dispatch(buf, wl, lay, cap, recv)
+
+
+@pytest.mark.parametrize("H", [4992, 5120, 5248])
+@pytest.mark.parametrize("T", [90, 700])
+def test_around_the_line_between_short_and_long_fp8_rows(H, T):
+    for dedup in (0, 1):
+        _run(W.Config("l", T=T, H=H, E=64, R=8, k=8, payload=1, dedup=dedup, seed=H + T))

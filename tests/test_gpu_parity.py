@@ -341,9 +341,11 @@ def test_fp8_special_values_match_the_oracle():
 ])
 @pytest.mark.parametrize("shape", [
     dict(T=600, H=1024, E=32, R=8, k=4),                 # 4 tokens per CTA: fewer rows than ring stages
-    dict(T=7000, H=512, E=64, R=8, k=6),                 # 47 tokens per CTA: token stealing, ring wraps many times
-    dict(T=6100, H=7168, E=72, R=18, k=4),               # stealing with rows so large that the input ring is short
+    dict(T=7000, H=512, E=64, R=8, k=6),                 # 47 short rows per CTA: teams of warps, the ring is used more than once
+    dict(T=6100, H=7168, E=72, R=18, k=4),               # short rows (28 KB of copies) so large that the input ring is short
     dict(T=1500, H=384, E=24, R=3, k=3, dedup=1),        # scales of a row are 12 bytes: no bulk copy carries them
+    dict(T=6100, H=7168, E=72, R=18, k=6),               # long rows (42 KB of copies), token stealing
+    dict(T=900, H=5120, E=32, R=8, k=8),                 # long rows, just: 40 KB of copies; no stealing
 ])
 def test_warp_role_split_does_not_change_results(shape, count_warps, quant_warps, prefetch, pipeline):
     """How many warps count, how many quantise, and how far the loader runs ahead of the layout
