@@ -476,7 +476,7 @@ int ubep_debug_set_prefetch_rows(ubep_buffer_t *buf, int32_t n);
  * them (-1 and 14 by default).  plan [host] gets the values below.  For tests of the kernel's ring sizes.
  */
 enum {
-    UBEP_DEBUG_PLAN_MODE = 0,      /* UBEP_PIPELINE_*; 4 = layout by clusters                   */
+    UBEP_DEBUG_PLAN_MODE = 0,      /* UBEP_PIPELINE_*; 4 = layout by clusters, 5 = small batch  */
     UBEP_DEBUG_PLAN_CHUNKS,        /* token chunks ...                                          */
     UBEP_DEBUG_PLAN_PARTS,         /* ... times column parts = CTAs                             */
     UBEP_DEBUG_PLAN_CLUSTER,       /* CTAs per cluster                                          */

@@ -26,7 +26,8 @@ constexpr int kFastQuantWarps = 5;     // FP8, long rows, in the flag-free kerne
                                        // 512 / 1024 tokens: 15.5 / 24.3 us with 4, 15.5 / 25.3 with 6, 15.7 / 30.7 with 8, 18.0 / 38.2 with 10)
 constexpr int kStorePending = 3;       // FP8, long rows: rows whose bulk stores may still be reading shared memory
 constexpr int kTraceSlots = 16;        // per-CTA phase time stamps (optional tracing)
-constexpr int kModePhased = 1, kModeFused = 2, kModeLocal = 3, kModeCluster = 4;
+constexpr int kLeastStatic = 768;      // static shared memory of the persistent dispatch kernels, at least
+constexpr int kModePhased = 1, kModeFused = 2, kModeLocal = 3, kModeCluster = 4, kModeFew = 5;
 // Every wait in the kernels gives up after this many nanoseconds of wall time.
 constexpr unsigned long long kWaitLimitNs = 1500000000ull;
 
@@ -316,6 +317,7 @@ struct SmemPlan {
     int off_out, off_ids, off_mask, off_bm, off_pos, off_key, off_ord, off_w, off_hist, off_arr, off_order;
     int off_item;                     // per ring stage: where its token comes from, positions of stolen tokens
     int off_cnt;                      // layout by clusters: three arrays of counts
+    int duty_units;                   // small batches: warps that share the counts and offsets of a rank
     int total;
 };
 

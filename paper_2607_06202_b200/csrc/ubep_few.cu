@@ -1,0 +1,414 @@
+// Dispatch of small batches: a CTA has no more slots of the routing table than warps (plan_few below).
+//
+// What bounds it is latency, not bytes: 13 tokens are 1.4 MB.  The kernels for larger batches spend most of such a call on
+// control flow that is worth its while only with many rows -- rings, roles that release one another through barriers, counting
+// and prefix sums through shared memory, and every jump to a piece of code that has not run yet costs 0.1 us (64 functions 2 KB
+// apart, called once: 300 cycles each, 190 the second time; code that runs straight on: 3.5 cycles per instruction).  Here the
+// table is staged once; then every slot of the CTA's own tokens is a warp's, which counts the table for its own expert and rank
+// alone, sends its copy, writes its metadata and adds to the arrival counter by itself.  There is no barrier after the
+// one behind the staging (FP8 rows: one more, between quantising and sending).
+#include "ubep_kernels.h"
+#include "ubep_launch.cuh"
+#include "ubep_layout.cuh"
+#include "ubep_quant.cuh"
+
+namespace ubep {
+
+namespace {
+
+constexpr unsigned kAll = 0xffffffffu;
+constexpr int kFewSmem = 120 * 1024;   // more than half of an SM's shared memory
+
+// 1 << n, and 0 from 32 on (also for the large values that negative numbers are).
+__device__ __forceinline__ unsigned bit_or_none(unsigned n) {
+    unsigned v;
+    asm("shl.b32 %0, 1, %1;" : "=r"(v) : "r"(n));
+    return v;
+}
+// The n lowest bits; all of them from 32 on, none up to 0.
+__device__ __forceinline__ unsigned low_bits(int n) { return bit_or_none((unsigned)max(n, 0)) - 1u; }
+
+// The staged table: 16-bit physical expert ids, kNone for a slot that is empty or bad.
+constexpr unsigned kNone = 0xffffu;
+
+// The experts first .. first + 31 that token t selects, one bit each.  (An expert named twice is one bit.)
+template <int K>
+__device__ __forceinline__ unsigned experts_of(const uint16_t* ids, int t, unsigned first) {
+    unsigned w[4] = {0u, 0u, 0u, 0u};
+    if (K == 8) {
+        const uint4 v = *reinterpret_cast<const uint4*>(ids + t * 8);
+        w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
+    } else if (K == 4) {
+        const uint2 v = *reinterpret_cast<const uint2*>(ids + t * 4);
+        w[0] = v.x; w[1] = v.y;
+    } else if (K == 1) {
+        w[0] = ids[t] | kNone << 16;
+    } else {
+#pragma unroll
+        for (int i = 0; i < K / 2; ++i) w[i] = reinterpret_cast<const unsigned*>(ids + t * K)[i];
+    }
+    unsigned m = 0u;
+#pragma unroll
+    for (int i = 0; i < (K + 1) / 2; ++i) m |= bit_or_none((w[i] & 0xffffu) - first) | bit_or_none((w[i] >> 16) - first);
+    return m;
+}
+
+// kN slots of token t: raw ids in, physical experts out, kNone where there is none; `bad` if an id is out of range.  (All
+// look-ups of a step side by side.)
+template <int kN>
+__device__ __forceinline__ void resolve_slots(const Params& p, int t, int (&e)[kN], bool& bad) {
+    if (p.phys != nullptr) {
+        int nc[kN];
+#pragma unroll
+        for (int i = 0; i < kN; ++i) {
+            const bool in = (unsigned)e[i] < (unsigned)p.E_log;
+            bad |= !in && e[i] != -1;
+            nc[i] = in ? __ldg(p.ncopies + e[i]) : 0;
+        }
+#pragma unroll
+        for (int i = 0; i < kN; ++i) {
+            const bool in = (unsigned)e[i] < (unsigned)p.E_log, ok = nc[i] >= 1 && nc[i] <= p.C;
+            bad |= in && !ok;
+            const int copy = nc[i] > 2 ? t % nc[i] : nc[i] == 2 ? t & 1 : 0;
+            e[i] = ok ? __ldg(p.phys + (size_t)e[i] * p.C + copy) : -1;
+            bad |= ok && e[i] < 0;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < kN; ++i) {
+        const bool valid = (unsigned)e[i] < (unsigned)p.E;
+        bad |= !valid && e[i] != -1;
+        e[i] = valid ? e[i] : (int)kNone;
+    }
+}
+
+template <int K, bool kFp8, bool kDedup>
+__global__ void __launch_bounds__(kThreads, 1) few_kernel(const Params p, const SmemPlan pl) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    __shared__ __align__(8) uint64_t row_bar[kWarps];   // per own token: its row has landed
+    __shared__ unsigned epoch_sm;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, c = blockIdx.x;
+    const int part = c % p.parts, ch = c / p.parts;
+    const int t0 = (int)chunk_begin(ch, p.T, p.nchunks), ntok = (int)chunk_begin(ch + 1, p.T, p.nchunks) - t0;
+    const unsigned in_bytes = (unsigned)(p.H * 2 / p.parts), out_bytes = (unsigned)(p.rowB / p.parts);
+    const size_t out_off = (size_t)part * out_bytes;
+    const uint8_t* xs = reinterpret_cast<const uint8_t*>(p.x) + (size_t)t0 * p.H * 2 + (size_t)part * in_bytes;
+    uint16_t* ids = reinterpret_cast<uint16_t*>(smem + pl.off_ids);
+    griddep_launch();
+    if (warp == 0) {
+        if (lane < ntok) mbar_init(&row_bar[lane], 1);
+        mbar_fence_init();
+    }
+    {   // (prefetches into L2 read no value, so they may run ahead of the wait: see dispatch_kernel)
+        const char* tab = reinterpret_cast<const char*>(p.topk_idx);
+        if (tid * 128 < p.T * K * 4) asm volatile("prefetch.global.L2 [%0];" ::"l"(tab + tid * 128));
+        if (p.phys != nullptr) {
+            if (tid * 32 < p.E_log) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.ncopies + tid * 32));
+            if (tid * 32 < (int64_t)p.E_log * p.C) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.phys + tid * 32));
+        }
+        const int lines = (int)((in_bytes + 127u) / 128u);
+        for (int tl = 0; tl < ntok; ++tl)
+            for (int i = tid; i < lines; i += kThreads) asm volatile("prefetch.global.L2 [%0];" ::"l"(xs + (size_t)tl * p.H * 2 + (size_t)i * 128));
+    }
+    griddep_wait();
+    if (tid == 0) trace_begin(p, c);
+
+    // ---- the routing table, by warps 1 .. 15; warp 0 asks for the own rows and for the epoch
+    bool bad = false;
+    if (warp == 0) {
+        const unsigned ctr = lane == 0 ? ld_relaxed(p.epoch_ctr) : 0u;
+        if (lane < ntok) {
+            mbar_arrive_expect_tx(&row_bar[lane], in_bytes);
+            bulk_load(smem + (size_t)lane * pl.stage_bytes, xs + (size_t)lane * p.H * 2, in_bytes, &row_bar[lane]);
+        }
+        if (lane == 0) epoch_sm = epoch_from_counter(ctr);
+    } else {
+        constexpr int kV = K % 4 == 0 ? 4 : K % 2 == 0 ? 2 : 1;   // slots per load
+#pragma unroll 1
+        for (int i = tid - 32; i < p.T * (K / kV); i += kThreads - 32) {
+            const int t = i / (K / kV);
+            if (kV == 4) {
+                const int4 v = __ldg(reinterpret_cast<const int4*>(p.topk_idx) + i);
+                int e[4] = {v.x, v.y, v.z, v.w};
+                resolve_slots(p, t, e, bad);
+                reinterpret_cast<uint2*>(ids)[i] = make_uint2((unsigned)(e[0] | e[1] << 16), (unsigned)(e[2] | e[3] << 16));
+            } else if (kV == 2) {
+                const int2 v = __ldg(reinterpret_cast<const int2*>(p.topk_idx) + i);
+                int e[2] = {v.x, v.y};
+                resolve_slots(p, t, e, bad);
+                reinterpret_cast<unsigned*>(ids)[i] = (unsigned)(e[0] | e[1] << 16);
+            } else {
+                int e[1] = {__ldg(p.topk_idx + i)};
+                resolve_slots(p, t, e, bad);
+                ids[i] = (uint16_t)e[0];
+            }
+        }
+    }
+    // this warp's slot, if it has one: slot j of own token tl
+    const int tl = warp / K, j = warp % K, t = t0 + tl;
+    const bool slot = tl < ntok;
+    const float w_i = slot && lane < K ? __ldg(p.topk_w + (size_t)t * K + lane) : 0.0f;   // the token's gate weights, a lane each
+    __syncthreads();
+    if (tid == 0) trace(p, c, kTrCounted);
+    unsigned ticket = 0u;
+    if (tid == 0) ticket = atomicAdd(p.done_ticket, 1u);   // (every CTA has read the epoch when the last ticket is taken)
+    const unsigned half = epoch_sm & 1u;
+
+    // ---- the slot's row: tokens before t that chose the expert, behind the experts of the rank in front of it; with one
+    // row per (token, rank): tokens before t that visit the rank
+    const unsigned lbits = low_bits(p.L);
+    bool send = false, sent = false;
+    int r = 0, gpos = -1;
+    auto copy = [&]() {   // bf16: the row, which has landed
+        if (lane == 0) bulk_store(p.recv_x + (size_t)gpos * p.rowB + out_off, smem + (size_t)tl * pl.stage_bytes, out_bytes);
+        bulk_commit();
+        sent = true;
+    };
+    if (slot) {
+        const unsigned e_i = lane < K ? ids[t * K + lane] : kNone;
+        const unsigned e = __shfl_sync(kAll, e_i, j);
+        const bool valid = e != kNone && !__any_sync(kAll, lane < j && e_i == e);   // (of an expert named twice the first slot counts)
+        if (e != kNone && !valid) bad = true;
+        int row = -1;
+        if (valid) {
+            r = p.L == 1 ? (int)e : fast_div((int)e, p.L_magic);
+            const unsigned f = (unsigned)(r * p.L), d = e - f, below = (1u << d) - 1u;
+            unsigned acc = 0u;
+#pragma unroll 2
+            for (int tt = lane; tt < p.T; tt += 32) {
+                const unsigned m = experts_of<K>(ids, tt, f) & lbits;
+                acc += (unsigned)__popc(m & below) << 16;
+                if (tt < t) acc += ((m >> d) & 1u) << 16 | (m != 0u ? 1u : 0u);
+            }
+            acc = __reduce_add_sync(kAll, acc);
+            const int at = (int)(acc >> 16);
+            row = kDedup ? (int)(acc & 0xffffu) : at;
+            const bool here = e_i - f < (unsigned)p.L;   // (this lane's slot names the same rank)
+            const bool first = !kDedup || !__any_sync(kAll, here && lane < j);
+            const bool fits = row < p.cap;
+            gpos = fits ? r * p.cap + row : -1;
+            send = first && fits;
+            if (!kFp8 && send && __all_sync(kAll, mbar_test_wait(&row_bar[tl], 0))) copy();   // (the metadata while it is on its way)
+            bool full = !fits;
+            if (part == 0) {
+                if (kDedup) {
+                    if (at < p.er_cap) {
+                        if (lane == 0) p.expert_rows[(size_t)r * p.er_cap + at] = row;
+                    } else {
+                        full = true;
+                    }
+                    if (send) {
+                        bool again = false;   // a slot of the token in front of this lane's names the same expert
+#pragma unroll
+                        for (int i = 1; i < K; ++i) {
+                            const unsigned other = __shfl_up_sync(kAll, e_i, i);
+                            again = again || (lane >= i && other == e_i);
+                        }
+                        if (lane < K) {
+                            p.recv_topk_idx[(size_t)gpos * K + lane] = here && !again ? (int)(e_i - f) : -1;
+                            p.recv_topk_w[(size_t)gpos * K + lane] = here && !again ? w_i : 0.0f;
+                        }
+                    }
+                } else if (send && lane == j) {
+                    p.recv_weight[gpos] = w_i;
+                }
+                if (send && lane == 0) p.recv_src_idx[gpos] = t;
+            }
+            if (full) report(p.status, kErrCapacity);
+        }
+        if (part == 0 && lane == 0) {
+            p.slot_row[(size_t)t * K + j] = row;
+            p.slot_pos[(size_t)t * K + j] = gpos;
+        }
+    }
+    if (bad) report(p.status, kErrBadIndex);
+    if (tid == 0) trace(p, c, kTrFinalized);
+
+    // ---- the copy
+    if (kFp8) {
+        // every warp quantises: eight channels per lane
+        const int nvec = (int)in_bytes / 16;
+        const int gp = p.G / p.parts;   // scale groups of this CTA's piece
+        const int strips = (nvec + 31) / 32;   // of a row, a warp's vectors at a time
+        bool got = true;
+#pragma unroll 1
+        for (int u = warp; u < ntok * strips; u += 2 * kWarps) {   // two strips side by side
+            uint4 d[2];
+            int i[2], v[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int uh = u + h * kWarps;
+                i[h] = uh / strips;
+                v[h] = (uh - i[h] * strips) * 32 + lane;
+                if (uh >= ntok * strips) v[h] = nvec;   // nothing
+                d[h] = make_uint4(0, 0, 0, 0);
+                if (v[h] < nvec) {
+                    got = mbar_wait(&row_bar[i[h]], 0, nullptr) && got;
+                    d[h] = *reinterpret_cast<const uint4*>(smem + (size_t)i[h] * pl.stage_bytes + (size_t)v[h] * 16);
+                }
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (h == 1 && u + kWarps >= ntok * strips) break;   // (the whole warp)
+                uint8_t* out = smem + pl.off_out + (size_t)i[h] * pl.out_stage_bytes;
+                uint2 q;
+                float sc;
+                quantize8(d[h], v[h] < nvec, q, sc);
+                if (v[h] < nvec) {
+                    *reinterpret_cast<uint2*>(out + (size_t)v[h] * 8) = q;
+                    if ((lane & 15) == 0) reinterpret_cast<float*>(out + out_bytes)[v[h] >> 4] = sc;
+                }
+            }
+        }
+        if (!got) report(p.status, kErrTimeout);
+        fence_proxy_async_smem();   // the bulk stores read what has just been written
+        if (__syncthreads_or(!got)) send = false;
+        if (send) {
+            const uint8_t* src = smem + pl.off_out + (size_t)tl * pl.out_stage_bytes;
+            float* scales = p.recv_scale + (size_t)gpos * p.G + part * gp;
+            if ((gp & 3) == 0) {
+                if (lane == 1) bulk_store(scales, src + out_bytes, (unsigned)gp * 4u);
+            } else {   // (a piece of scales that no bulk copy can carry)
+                for (int i = lane; i < gp; i += 32) scales[i] = reinterpret_cast<const float*>(src + out_bytes)[i];
+            }
+            if (lane == 0) bulk_store(p.recv_x + (size_t)gpos * p.rowB + out_off, src, out_bytes);
+            bulk_commit();
+        }
+    } else if (send && !sent) {
+        send = __all_sync(kAll, mbar_wait(&row_bar[tl], 0, nullptr));
+        if (send) copy();
+        else report(p.status, kErrTimeout);
+    }
+    if (tid == 0) trace(p, c, kTrIssued);
+
+    // ---- what no row waits for: per rank the totals and the expert offsets, per source rank counts and offsets.  A unit is
+    // a rank and as many source ranks as there are lanes for, a lane per (source rank, expert); the warps without a slot, the
+    // last ones of every CTA, come first.  (One loop of few instructions that keeps nothing per group of tokens: with the
+    // groups unrolled and their bitmaps in registers the call of 1 to 13 tokens took 0.6 us more.)
+    const int lsh = 32 - __clz(p.L - 1);   // experts of a rank, rounded up to a power of two
+#pragma unroll 1
+    for (int u = (kWarps - 1 - warp) * p.grid + c; u < p.R * pl.duty_units; u += kWarps * p.grid) {
+        const int ur = u / pl.duty_units, uq = u - ur * pl.duty_units, f = ur * p.L;
+        const int l = lane & ((1 << lsh) - 1), s = (uq << (5 - lsh)) + (lane >> lsh);
+        const bool mine = s < p.S && l < p.L;
+        const int b0 = src_begin(min(s, p.S), p.T, p.S), b1 = src_begin(min(s + 1, p.S), p.T, p.S);
+        int tot = 0, visits = 0;         // tokens that chose expert `lane` of the rank / that visit it
+        int before = 0, after = 0;       // tokens before the source rank's first and behind its last one that chose expert l
+#pragma unroll 1
+        for (int g = 0; g < p.T; g += 32) {
+            const unsigned m = g + lane < p.T ? experts_of<K>(ids, g + lane, (unsigned)f) & lbits : 0u;
+            visits += m != 0u ? 1 : 0;
+            const unsigned bm = transpose32(m, lane);   // lane = expert, bit = token
+            tot += __popc(bm);
+            const unsigned of_l = __shfl_sync(kAll, bm, l);
+            before += __popc(of_l & low_bits(b0 - g));
+            after += __popc(of_l & low_bits(b1 - g));
+        }
+        const int incl = warp_incl_scan(tot, lane), eo = incl - tot, eo_l = __shfl_sync(kAll, eo, l);
+        if (mine) {
+            p.cnt[(size_t)s * p.E + f + l] = after - before;
+            p.src_offset[(size_t)s * p.E + f + l] = eo_l + before;
+        }
+        if (uq == 0) {
+            if (lane < p.L) {
+                p.expert_offset[f + lane] = eo;
+                p.num_tokens_per_expert[f + lane] = tot;
+            }
+            visits = __reduce_add_sync(kAll, visits);
+            const int rows = __shfl_sync(kAll, incl, 31);
+            if (lane == 0) {
+                p.num_tokens_per_rank[ur] = visits;
+                p.num_rows_per_rank[ur] = kDedup ? visits : rows;
+            }
+        }
+    }
+    if (tid == 0) trace(p, c, kTrScanned);
+
+    // ---- the arrival counters (eighths of a row: see publish_arrivals): every warp for its own row
+    if (send) {
+        bulk_wait_all<0>();
+        __syncwarp();
+        if (lane == 0) {
+            if (tid == 0) trace(p, c, kTrStored);
+            red_release_add(p.arrival + half * p.R + r, (unsigned)(8 / p.parts));
+        }
+    }
+    if (c == p.grid - 1 && warp == kWarps - 1) {   // those of the next call live in the other half
+        for (int i = lane; i < p.R; i += 32) p.arrival[(half ^ 1u) * p.R + i] = 0;
+        if (lane == 0) p.claimed[half ^ 1u] = 0;
+    }
+    if (warp == 0) {
+        if (lane == 0) epoch_finish_check_in(p, ticket, epoch_sm);
+        if (lane < ntok) (void)mbar_wait(&row_bar[lane], 0, nullptr);   // (a row that no slot sends may still be landing)
+    }
+    if (tid == 0) trace(p, c, kTrEnd);
+}
+
+template <int K, bool kFp8, bool kDedup>
+cudaError_t launch_few_t(const Params& p, const SmemPlan& pl, cudaStream_t st) {
+    auto kern = few_kernel<K, kFp8, kDedup>;
+    const int smem = with_room_beside(pl.total, 0);
+    static std::atomic<int> granted[kAttrDevices];
+    cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void*>(kern), smem, granted);
+    if (e != cudaSuccess) return e;
+    return launch_overlapped(kern, p.grid, kThreads, (size_t)smem, st, false, 1, p, pl);
+}
+template <int K>
+cudaError_t launch_few_k(const Params& p, const SmemPlan& pl, cudaStream_t st) {
+    if (p.payload) return p.dedup ? launch_few_t<K, true, true>(p, pl, st) : launch_few_t<K, true, false>(p, pl, st);
+    return p.dedup ? launch_few_t<K, false, true>(p, pl, st) : launch_few_t<K, false, false>(p, pl, st);
+}
+
+}  // namespace
+
+// Small batches: every slot of the CTA's tokens has a warp.  A slot's warp reads the whole table (T tokens of k slots and some
+// 8 more instructions' worth each) and an SM's four schedulers share the warps of up to `most` tokens, so the line lies at a
+// product of these.  Dispatch + combine in one graph, as before and this way: 1 token of 7168 channels, top-8, bf16 8.4 and 5.3 us,
+// 16 tokens of 4096 channels 8.6 and 5.5, 128 of 256 channels, top-2 7.9 and 4.6; near the line 256 tokens of 4096 channels,
+// top-8 12.0 and 12.0 (FP8 rows 13.3 and 12.9), 444 of 1024, top-4 9.8 and 8.3 (10.2 and 9.9), 592 of 256, top-2 9.6 and 9.6
+// (FP8); beyond it 296 tokens of 4096 channels, top-8 12.4 and 13.3, 512 of 1024, top-4 10.1 and 10.5, 740 of 256, top-2, FP8
+// 9.9 and 11.1.
+constexpr int kFewWork = 65536;
+bool plan_few(const Params& p, int max_smem, SmemPlan* out) {
+    const int most = (p.T + p.nchunks - 1) / p.nchunks;   // tokens of a CTA
+    if (most * p.k > kWarps || (int64_t)most * p.k * p.T * (p.k + 8) > kFewWork || p.L > 32 || p.ordered) return false;
+    if (p.k != 1 && p.k != 2 && p.k != 4 && p.k != 6 && p.k != 8) return false;
+    if (p.payload && p.quant_warps < kWarps - 2) return false;   // (fewer quantising warps were asked for)
+    SmemPlan pl{};
+    auto round_up = [](int64_t v, int m) { return (v + m - 1) / m * m; };
+    const int64_t stage = round_up((int64_t)p.H * 2 / p.parts, 128);
+    const int64_t out_stage = p.payload ? round_up((int64_t)p.rowB / p.parts + (p.G / p.parts) * 4, 128) : 0;
+    const int64_t total = most * (stage + out_stage) + round_up((int64_t)p.T * p.k * 2, 128);
+    if (total + 1536 > max_smem) return false;   // (1.5 KB: static shared memory)
+    pl.stages = most;
+    pl.stage_bytes = (int)stage;
+    pl.trip_rows = 1;
+    pl.out_stages = p.payload ? most : 0;
+    pl.out_stage_bytes = (int)out_stage;
+    pl.q_warps = p.payload ? kWarps : 0;   // one team of all of them
+    pl.q_teams = p.payload ? 1 : 0;
+    pl.q_team_warps = pl.q_warps;
+    pl.off_out = (int)(most * stage);
+    pl.off_ids = pl.off_out + (int)(most * out_stage);
+    // One CTA per SM.  Two of them fit in an SM's registers, and where a call may be placed while the combine before it runs
+    // (programmatic launches), SMs without combine CTAs took two and others none: sixteen layers of 128 tokens of 7168 channels,
+    // top-8, in one graph 12.6 us per layer, this way 10.4.  (Warps that leave at once do not hold their registers: no change.)
+    pl.total = (int)(total < kFewSmem ? kFewSmem : total);
+    int at_once = 32;   // source ranks a warp looks at together
+    for (int l = 1; l < p.L; l *= 2) at_once /= 2;
+    pl.duty_units = (p.S + at_once - 1) / at_once;
+    *out = pl;
+    return true;
+}
+
+cudaError_t launch_few(const Params& p, const SmemPlan& pl, cudaStream_t st) {
+    switch (p.k) {
+        case 1: return launch_few_k<1>(p, pl, st);
+        case 2: return launch_few_k<2>(p, pl, st);
+        case 4: return launch_few_k<4>(p, pl, st);
+        case 6: return launch_few_k<6>(p, pl, st);
+        default: return launch_few_k<8>(p, pl, st);
+    }
+}
+
+}  // namespace ubep

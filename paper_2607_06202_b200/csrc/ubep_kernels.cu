@@ -13,10 +13,9 @@
 //                                     tables with one row per (token, expert).
 //   combine_kernel<K>                 gather + fp32 weighted sum + one bf16 rounding
 //   layout_kernel<K, W>               counts only (ubep_get_dispatch_layout)
-#include <atomic>
-
 #include "ubep_cluster.cuh"
 #include "ubep_kernels.h"
+#include "ubep_launch.cuh"
 #include "ubep_layout.cuh"
 #include "ubep_quant.cuh"
 
@@ -1656,54 +1655,6 @@ int plan_dispatch(const Params& p, int mode, int max_smem, SmemPlan* out) {
     return 0;
 }
 
-// Launch that lets the kernel be placed while its predecessor in the stream drains (the
-// kernels above call griddep_wait() before they read anything).  `together`: a cooperative
-// launch -- the kernel's CTAs wait for flags that other CTAs of the same grid publish, so they
-// must all be resident at once; the runtime then refuses a grid that cannot be (a synchronous
-// error instead of CTAs spinning until their bounded waits run out) and starts the grid only
-// when every CTA has a place.  Such a kernel is not launched ahead of its predecessor's end.
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_overlapped(void (*kern)(KArgs...), int grid, int block, size_t smem, cudaStream_t st,
-                                     bool together, int cluster, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    if (together) {
-        attr[0].id = cudaLaunchAttributeCooperative;
-        attr[0].val.cooperative = 1;
-    } else {
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-    }
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cluster > 1) {
-        attr[1].id = cudaLaunchAttributeClusterDimension;
-        attr[1].val.clusterDim.x = (unsigned)cluster;
-        attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
-        cfg.numAttrs = 2;
-    }
-    return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
-// The dynamic shared-memory limit of a kernel is a sticky attribute: per kernel instance and
-// device only a larger request has to reach the runtime (the call costs host time that an
-// enqueue-bound caller sees on every dispatch).  `granted` belongs to one kernel instance.
-constexpr int kAttrDevices = 64;
-static cudaError_t allow_dynamic_smem(const void* kern, int bytes, std::atomic<int>* granted) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    const bool cached = dev >= 0 && dev < kAttrDevices;
-    if (cached && granted[dev].load(std::memory_order_relaxed) >= bytes) return cudaSuccess;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess && cached) granted[dev].store(bytes, std::memory_order_relaxed);
-    return e;
-}
-
 template <int kMode, int kRows, bool kSteal>
 static cudaError_t allow_dispatch_smem(int bytes) {
     static std::atomic<int> granted[kAttrDevices];
@@ -1715,8 +1666,8 @@ static cudaError_t allow_dispatch_smem(int bytes) {
 // layers of 74 tokens of 1024 channels, FP8, in one graph, 15.4 of 16 KB, 10.6 us, with the next size 9.9; 128 tokens of 256
 // channels, 7.5 of 8 KB, 10.2 and 9.5; 74 tokens of 2048 channels, bf16, 9.1 and 8.5.  So such a call asks for a little more.
 // (The largest size for every call: 512 tokens of 7168 channels 24.3 -> 25.6, more combine CTAs beside the dispatch.)
-int with_room_beside(int dynamic) {
-    constexpr int kLeast = 768 + 1024, kMost = 1280 + 1024;   // static memory of the dispatch kernels, reserved
+int with_room_beside(int dynamic, int least_static) {
+    const int kLeast = least_static + 1024, kMost = 1280 + 1024;   // static memory of the dispatch kernels, reserved
     for (int kb : {8, 16, 32, 64, 100, 132, 164, 196}) {
         const int size = kb * 1024;
         if (dynamic + kLeast <= size && dynamic + kMost + 1024 > size) return size - kLeast + 128;
@@ -1727,7 +1678,7 @@ int with_room_beside(int dynamic) {
 template <int kMode, int kRows, bool kSteal>
 static cudaError_t launch_dispatch_s(const Params& p, const SmemPlan& pl, cudaStream_t st) {
     auto kern = dispatch_kernel<kMode, kRows, kSteal>;
-    const int smem = with_room_beside(pl.total);
+    const int smem = with_room_beside(pl.total, kLeastStatic);
     cudaError_t e = allow_dispatch_smem<kMode, kRows, kSteal>(smem);
     if (e != cudaSuccess) return e;
     return launch_overlapped(kern, p.grid, kDispatchThreads<kMode, kRows>, (size_t)smem, st, kMode == kModeFused,
@@ -1804,6 +1755,7 @@ cudaError_t launch_dispatch(const Params& p, int mode, const SmemPlan& pl, cudaS
         *launches = 3;
         return launch_dispatch_t<kModePhased>(p, pl, st);
     }
+    if (mode == kModeFew) return launch_few(p, pl, st);
     if (mode == kModeCluster) return launch_dispatch_t<kModeCluster>(p, pl, st);
     if (mode == kModeLocal) return launch_dispatch_t<kModeLocal>(p, pl, st);
     return launch_dispatch_t<kModeFused>(p, pl, st);

@@ -12,8 +12,12 @@ namespace ubep {
 int plan_dispatch(const Params& p, int mode, int max_smem, SmemPlan* out);
 
 int cluster_ctas(int cluster, int max_smem);
-int with_room_beside(int dynamic);   // the dynamic shared memory a dispatch with a plan of this size asks for
+// The dynamic shared memory a dispatch with a plan of this size asks for, at least `least_static` of static memory beside it.
+int with_room_beside(int dynamic, int least_static);
 bool short_rows(const Params& p);
+// Small batches (ubep_few.cu): the plan, if the call -- cut into chunks and column parts -- is one of them.
+bool plan_few(const Params& p, int max_smem, SmemPlan* out);
+cudaError_t launch_few(const Params& p, const SmemPlan& pl, cudaStream_t st);
 cudaError_t launch_count_scan(const Params& p, const SmemPlan& pl, cudaStream_t st);
 cudaError_t launch_dispatch(const Params& p, int mode, const SmemPlan& pl, cudaStream_t st, int* launches);
 cudaError_t launch_combine(const uint16_t* y, const int32_t* slot_pos, const float* topk_w, int T, int H, int k,

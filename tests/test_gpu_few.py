@@ -1,0 +1,108 @@
+"""Small batches (a warp per slot of the CTA's own tokens): the edges of what is taken that way, against the oracle."""
+import numpy as np
+import pytest
+
+from paper_2607_06202_b200 import binding as B
+from paper_2607_06202_b200 import workload as W
+from tests import harness as Hn
+
+FEW = 5
+SHAPES = [(7168, 256, 32, 8), (4096, 128, 16, 8), (2048, 128, 8, 4), (256, 16, 4, 2)]
+
+
+def mode(T, H, E, R, k, payload=0, dedup=0, **kw):
+    cfg = B.ubep_config_t(R, E, H, k, T, 128, 0, payload, dedup, 0, kw.get("pipeline", 0), kw.get("num_ctas", 0))
+    return B.ubep_debug_plan(cfg, T, 232448, (148, 148, 132, 120), **{n: v for n, v in kw.items() if n == "quant_warps"})
+
+
+def test_which_calls_are_small_batches():
+    for (H, E, R, k), last in zip(SHAPES, (256, 256, 444, 655)):
+        for payload, dedup in ((0, 0), (1, 0), (0, 1), (1, 1)):
+            small = [T for T in range(1, 800) if mode(T, H, E, R, k, payload, dedup)["mode"] == FEW]
+            assert set(range(1, 149)) <= set(small) and max(small) == last, (H, k, payload, dedup, max(small))
+            for T in (1, 148, max(small)):
+                pl = mode(T, H, E, R, k, payload, dedup)
+                assert -(-T // pl["chunks"]) * k <= 16 and pl["stages"] >= -(-T // pl["chunks"])
+                assert 118 * 1024 < pl["smem"] <= 232448   # (one CTA per SM)
+    assert mode(100, 256, 64, 1, 8)["mode"] != FEW                              # 64 experts on one rank
+    assert mode(100, 256, 64, 8, 5)["mode"] != FEW                              # slots that are no vector
+    assert mode(100, 256, 64, 8, 8, num_ctas=40)["mode"] != FEW                 # more slots than warps
+    assert mode(100, 256, 64, 8, 8, payload=1, quant_warps=3)["mode"] != FEW
+    assert mode(8, 16384, 64, 8, 1, num_ctas=1)["mode"] != FEW                  # the rows do not fit
+    for pipeline in (1, 2, 3):
+        assert mode(16, 256, 64, 8, 8, pipeline=pipeline)["mode"] != FEW
+
+
+def _run(T, H, E, R, k, payload, dedup, empty=0.0, **kw):
+    cfg = W.Config("few", T=T, H=H, E=E, R=R, k=k, payload=payload, dedup=dedup, seed=T + H + k, **kw)
+    wl = W.make_workload(cfg)
+    if empty:
+        wl = W.with_empty_slots(wl, empty, seed=T)
+    Hn.run_case(wl, threads=8)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("payload,dedup", [(0, 0), (1, 0), (0, 1), (1, 1)])
+@pytest.mark.parametrize("H,E,R,k,tokens", [
+    (7168, 256, 32, 8, (1, 2, 19, 37, 75, 148, 149, 256)),   # eight, four, two column parts, whole rows, two tokens per CTA
+    (128, 32, 1, 8, (1, 31, 32, 33, 256, 257)),              # every expert on one rank: all bits of a word
+    (640, 96, 96, 6, (5, 148, 296)),                         # one expert per rank; scales that no bulk copy can carry
+    (1024, 32, 8, 4, (3, 149, 444, 445)),
+    (256, 16, 4, 2, (64, 148, 297, 655, 656)),
+    (384, 24, 8, 1, (1, 33, 700)),
+])
+def test_sizes(H, E, R, k, tokens, payload, dedup):
+    for T in tokens:
+        _run(T, H, E, R, k, payload, dedup, empty=0.15 if T % 2 else 0.0)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("T", [1, 40, 200])
+def test_source_ranks_replicas_and_narrow_rows(T):
+    for S in (1, 7, 40, 900):
+        _run(T, 8, 60, 20, 4, 0, T % 2, num_src_ranks=S)
+    for payload in (0, 1):
+        _run(T, 256, 288, 72, 8, payload, 1, E_logical=256)
+        _run(T, 256, 288, 72, 8, payload, 0, E_logical=256)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dedup", [0, 1])
+def test_bad_ids_experts_named_twice_and_capacity(dedup):
+    cfg = W.Config("few", T=90, H=128, E=32, R=4, k=8, dedup=dedup, seed=3)
+    wl = W.make_workload(cfg)
+    given, clean = wl.topk_idx.copy(), wl.topk_idx.copy()
+    clean[::3, 7] = -1
+    given[::3, 7] = given[::3, 0]
+    clean[1, 2] = clean[4, 0] = -1
+    given[1, 2], given[4, 0] = 32, -2
+    want = W.Workload(cfg, wl.x, clean, wl.topk_w)
+    _, lay, cap, recv = Hn.oracle_reference(want)
+    buf = Hn.make_buffer(cfg, cap)
+    x, _, w, _, _ = Hn.device_inputs(wl)
+    buf.dispatch(x, Hn.to_dev(given), w)
+    assert buf.status() == B.UBEP_ERR_BAD_INDEX
+    Hn.check_dispatch(buf, want, lay, cap, recv)
+    small = int(lay.num_rows_per_rank.max()) - 2
+    buf = Hn.make_buffer(cfg, small)
+    buf.dispatch(x, Hn.to_dev(clean), w)
+    assert buf.status() == B.UBEP_ERR_CAPACITY
+    assert np.array_equal(buf.cnt.cpu().numpy(), lay.cnt) and np.array_equal(buf.slot_row[:cfg.T].cpu().numpy(), lay.slot_row)
+    for r in range(cfg.R):
+        n = min(int(lay.num_rows_per_rank[r]), small)
+        assert np.array_equal(buf.recv_src_idx[r, :n].cpu().numpy(), recv.recv_src_idx[r, :n])
+        assert np.array_equal(buf.recv_x[r, :n].cpu().numpy(), recv.recv_x[r, :n])
+
+
+@pytest.mark.gpu
+def test_between_calls_of_other_sizes():
+    """The arrival counters and the count of tokens handed out of a call are cleared by the call before it."""
+    cfgs = [W.Config("mix", T=T, H=2048, E=64, R=8, k=8, seed=T) for T in (13, 6000, 200)]
+    refs = [Hn.oracle_reference(W.make_workload(c), cap=8192, num_threads=8) for c in cfgs]
+    buf = Hn.make_buffer(cfgs[1], 8192)
+    wls = [W.make_workload(c) for c in cfgs]
+    dev = [Hn.device_inputs(wl) for wl in wls]
+    for i in (0, 1, 2, 1, 1, 0, 0, 1):
+        buf.recv_x.fill_(Hn.FILL)
+        buf.dispatch(*dev[i][:3])
+        Hn.check_dispatch(buf, wls[i], refs[i][1], 8192, refs[i][3], check_tails=False)
