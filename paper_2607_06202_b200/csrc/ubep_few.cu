@@ -30,6 +30,7 @@ __device__ __forceinline__ unsigned low_bits(int n) { return bit_or_none((unsign
 
 // The staged table: 16-bit physical expert ids, kNone for a slot that is empty or bad.
 constexpr unsigned kNone = 0xffffu;
+__device__ __forceinline__ unsigned pack16(int a, int b) { return ((unsigned)a & 0xffffu) | (unsigned)b << 16; }
 
 // The experts first .. first + 31 that token t selects, one bit each.  (An expert named twice is one bit.)
 template <int K>
@@ -51,35 +52,6 @@ __device__ __forceinline__ unsigned experts_of(const uint16_t* ids, int t, unsig
 #pragma unroll
     for (int i = 0; i < (K + 1) / 2; ++i) m |= bit_or_none((w[i] & 0xffffu) - first) | bit_or_none((w[i] >> 16) - first);
     return m;
-}
-
-// kN slots of token t: raw ids in, physical experts out, kNone where there is none; `bad` if an id is out of range.  (All
-// look-ups of a step side by side.)
-template <int kN>
-__device__ __forceinline__ void resolve_slots(const Params& p, int t, int (&e)[kN], bool& bad) {
-    if (p.phys != nullptr) {
-        int nc[kN];
-#pragma unroll
-        for (int i = 0; i < kN; ++i) {
-            const bool in = (unsigned)e[i] < (unsigned)p.E_log;
-            bad |= !in && e[i] != -1;
-            nc[i] = in ? __ldg(p.ncopies + e[i]) : 0;
-        }
-#pragma unroll
-        for (int i = 0; i < kN; ++i) {
-            const bool in = (unsigned)e[i] < (unsigned)p.E_log, ok = nc[i] >= 1 && nc[i] <= p.C;
-            bad |= in && !ok;
-            const int copy = nc[i] > 2 ? t % nc[i] : nc[i] == 2 ? t & 1 : 0;
-            e[i] = ok ? __ldg(p.phys + (size_t)e[i] * p.C + copy) : -1;
-            bad |= ok && e[i] < 0;
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < kN; ++i) {
-        const bool valid = (unsigned)e[i] < (unsigned)p.E;
-        bad |= !valid && e[i] != -1;
-        e[i] = valid ? e[i] : (int)kNone;
-    }
 }
 
 template <int K, bool kFp8, bool kDedup>
@@ -131,12 +103,12 @@ __global__ void __launch_bounds__(kThreads, 1) few_kernel(const Params p, const 
                 const int4 v = __ldg(reinterpret_cast<const int4*>(p.topk_idx) + i);
                 int e[4] = {v.x, v.y, v.z, v.w};
                 resolve_slots(p, t, e, bad);
-                reinterpret_cast<uint2*>(ids)[i] = make_uint2((unsigned)(e[0] | e[1] << 16), (unsigned)(e[2] | e[3] << 16));
+                reinterpret_cast<uint2*>(ids)[i] = make_uint2(pack16(e[0], e[1]), pack16(e[2], e[3]));
             } else if (kV == 2) {
                 const int2 v = __ldg(reinterpret_cast<const int2*>(p.topk_idx) + i);
                 int e[2] = {v.x, v.y};
                 resolve_slots(p, t, e, bad);
-                reinterpret_cast<unsigned*>(ids)[i] = (unsigned)(e[0] | e[1] << 16);
+                reinterpret_cast<unsigned*>(ids)[i] = pack16(e[0], e[1]);
             } else {
                 int e[1] = {__ldg(p.topk_idx + i)};
                 resolve_slots(p, t, e, bad);

@@ -12,7 +12,9 @@
 //                                     count the table between them; a cluster of one for small
 //                                     tables with one row per (token, expert).
 //   combine_kernel<K>                 gather + fp32 weighted sum + one bf16 rounding
-//   layout_kernel<K, W>               counts only (ubep_get_dispatch_layout)
+//   layout_kernel<K>                  counts only (ubep_get_dispatch_layout)
+#include <type_traits>
+
 #include "ubep_cluster.cuh"
 #include "ubep_kernels.h"
 #include "ubep_launch.cuh"
@@ -1430,44 +1432,47 @@ __global__ void __launch_bounds__(256) combine_kernel(const uint16_t* __restrict
 }
 
 // ---------------------------------------------------------------- counts-only layout
-// ubep_get_dispatch_layout.  One warp takes 32 tokens, a lane per token: the lane's slots are fetched side by
-// side (16 bytes each where the table allows it), the experts are counted in shared memory, the ranks it visits
-// become a bit mask per lane, which the warp transposes so that every rank's count is one population count.
-// A CTA adds its counts to the totals in `acc`, the last one to finish (ticket) hands them out and leaves `acc`
-// and the ticket zero for the next call.
+// ubep_get_dispatch_layout.  A lane per token: its slots are fetched side by side (16 bytes each where the table allows it), the
+// experts and the ranks it visits are counted in shared memory, and which ranks those are becomes a tile of 32 tokens' bytes in
+// shared memory that leaves in 16-byte stores.
 //
-// Bound by latency: table (cold, 1.2 us) -> counts -> adds -> ticket -> totals.  One group of 32 tokens per warp
-// and four warps per CTA keep every step one trip deep.  Measured at 4096 tokens, top-8 of 256 experts: 6.4 us per call
-// in a stream of calls; before (a thread per token walking its slots through local memory, 148 chunk histograms
-// in global memory summed by one CTA) 29.7 us.
+// Bound by latency: table (cold, 1.2 us) -> counts -> sums over the CTAs.  kCluster: the CTAs are one cluster and read one
+// another's counts; nothing outside shared memory is needed, and one CTA needs not even that.  Otherwise a CTA adds its
+// counts to the totals in `acc`, and the last one to finish (ticket) hands them out and leaves `acc` and the ticket zero for
+// the next call: a fence and two round trips to L2 more, but as many SMs as there are tokens for.
+// Captured calls, top-8 of 256 experts on 32 ranks, one cluster / totals in global memory: 1 token 2.6 / 4.6 us, 512 tokens 3.2 / 4.9, 4096
+// tokens 4.4 / 5.3, 8192 tokens 6.2 / 5.4; top-4 of 32 experts on 8 ranks 1 token 2.0 / 3.3, 4096 tokens 3.1 / 4.0, 8192 tokens 4.4 / 4.1.  (Rank
+// masks per lane, transposed by the warp, and no cluster: 4.8, 5.2, 5.7 and 5.8 us on 32 ranks; with four words of masks, 72 ranks,
+// 4096 tokens 7.0, now 4.8.)
 constexpr int kLayoutThreads = 128;
-constexpr int kLayoutMaskWords = 4;   // ranks as bit masks: up to 128 of them
+constexpr int kLayoutClusterTokens = 8 * kThreads;   // eight CTAs, a token per thread
+constexpr int kLayoutTileRanks = 128;   // most ranks whose bytes go through shared memory
 
-// kK: slots per token if fixed (0: p.k, at most kMaxTopk); kW: words of the rank mask (0: more than 128 ranks,
-// counted slot by slot)
-template <int kK, int kW>
-__global__ void __launch_bounds__(kLayoutThreads) layout_kernel(const Params p, int32_t* num_tokens_per_rank,
+// kK: slots per token if fixed (0: p.k, at most kMaxTopk); kTile: no more ranks than kLayoutTileRanks
+template <int kK, bool kTile, bool kCluster>
+__global__ void __launch_bounds__(kCluster ? kThreads : kLayoutThreads) layout_kernel(const Params p, int32_t* num_tokens_per_rank,
                                                                int32_t* num_tokens_per_expert,
                                                                uint8_t* is_token_in_rank, int32_t* acc,
                                                                int acc_words, unsigned* ticket) {
-    extern __shared__ int hist[];   // [B]
+    extern __shared__ __align__(16) int hist[];   // [B], then a tile per warp
     __shared__ bool last;
+    constexpr int kN = kCluster ? kThreads : kLayoutThreads, kSlots = kK ? kK : kMaxTopk, kUnroll = kK ? kK : 1;
     const int B = p.B, R = p.R, T = p.T, k = kK ? kK : p.k, lane = threadIdx.x & 31;
-    for (int b = threadIdx.x; b < B; b += kLayoutThreads) hist[b] = 0;
+    uint8_t* tile = reinterpret_cast<uint8_t*>(hist + (B + 3) / 4 * 4) + (threadIdx.x >> 5) * 32 * R;   // [32, R]
+    for (int b = threadIdx.x; b < B; b += kN) hist[b] = 0;
     griddep_launch();
     griddep_wait();
     __syncthreads();
-    constexpr int kWords = kW ? kW : 1;
-    constexpr int kSlots = kK ? kK : kMaxTopk;
-    constexpr int kUnroll = kK ? kK : 1;
-    const bool by_word = (R & 3) == 0 && (reinterpret_cast<uintptr_t>(is_token_in_rank) & 3) == 0;
-    const int warps = gridDim.x * (kLayoutThreads / 32);
+    const int warps = gridDim.x * (kN / 32);
     bool bad = false;
-    for (int g = blockIdx.x * (kLayoutThreads / 32) + (threadIdx.x >> 5); g * 32 < T; g += warps) {
+    for (int g = blockIdx.x * (kN / 32) + (threadIdx.x >> 5); g * 32 < T; g += warps) {
         const int t = g * 32 + lane;
-        unsigned m[kWords];
-#pragma unroll
-        for (int w = 0; w < kWords; ++w) m[w] = 0u;
+        const bool flags = is_token_in_rank != nullptr;
+        uint8_t* out = flags ? is_token_in_rank + (size_t)g * 32 * R : nullptr;
+        if (kTile && flags) {
+            for (int i = lane; i < 2 * R; i += 32) reinterpret_cast<uint4*>(tile)[i] = make_uint4(0, 0, 0, 0);
+            __syncwarp();
+        }
         if (t < T) {
             const int32_t* src = p.topk_idx + (size_t)t * k;
             int e[kSlots];
@@ -1481,60 +1486,94 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(const Params p, 
 #pragma unroll kUnroll
                 for (int j = 0; j < k; ++j) e[j] = __ldg(src + j);
             }
-            uint8_t* flags = is_token_in_rank ? is_token_in_rank + (size_t)t * R : nullptr;
-            if (kW == 0 && flags)
-                for (int r = 0; r < R; ++r) flags[r] = 0;
-#pragma unroll kUnroll
-            for (int j = 0; j < k; ++j) {
-                e[j] = resolve_expert(p, t, e[j], bad);
-#pragma unroll kUnroll
-                for (int jj = 0; jj < j; ++jj)
-                    if (e[j] >= 0 && e[jj] == e[j]) {   // an expert named twice: reported, the later slot counts as empty
-                        bad = true;
-                        e[j] = -1;
-                    }
-                if (e[j] < 0) continue;
-                atomicAdd(&hist[e[j]], 1);
-                const int r = p.L == 1 ? e[j] : fast_div(e[j], p.L_magic);
-                if (kW) {
+            uint8_t* mine = !flags ? nullptr : kTile ? tile + lane * R : out + (size_t)lane * R;
+            if (!kTile && flags)
+                for (int r = 0; r < R; ++r) mine[r] = 0;
+            if (kK) {
+                resolve_slots(p, t, e, bad);
+                bool twice = false;
 #pragma unroll
-                    for (int w = 0; w < kWords; ++w) m[w] |= (kW == 1 || w == (r >> 5)) ? 1u << (r & 31) : 0u;
-                } else {
-                    bool first = true;
-#pragma unroll kUnroll
-                    for (int jj = 0; jj < j; ++jj) first = first && !(e[jj] >= r * p.L && e[jj] < (r + 1) * p.L);
+                for (int j = 0; j < kSlots; ++j) {
+                    e[j] = e[j] >= 0 ? e[j] : -1 - j;   // (no two empty slots are equal)
+#pragma unroll
+                    for (int i = 0; i < j; ++i) twice = twice || e[i] == e[j];
+                }
+                if (twice) {   // an expert named twice: reported, the later slot counts as empty
+                    bad = true;
+#pragma unroll
+                    for (int j = 1; j < kSlots; ++j)
+#pragma unroll
+                        for (int i = 0; i < j; ++i)
+                            if (e[i] == e[j]) e[j] = -1 - j;
+                }
+#pragma unroll
+                for (int j = 0; j < kSlots; ++j) {
+                    if (e[j] >= 0) atomicAdd(&hist[e[j]], 1);
+                    e[j] = e[j] < 0 ? e[j] : p.L == 1 ? e[j] : fast_div(e[j], p.L_magic);
+                    bool first = e[j] >= 0;   // a rank counts a token once: with the first of the slots that name it
+#pragma unroll
+                    for (int i = 0; i < j; ++i) first = first && e[i] != e[j];
                     if (first) {
-                        atomicAdd(&hist[p.E + r], 1);
-                        if (flags) flags[r] = 1;
+                        atomicAdd(&hist[p.E + e[j]], 1);
+                        if (flags) mine[e[j]] = 1;
                     }
                 }
-            }
-            if (kW && flags) {
-                if (by_word) {   // four ranks per store: bit i of the nibble into byte i of a word
-                    uint32_t* out = reinterpret_cast<uint32_t*>(flags);
-#pragma unroll
-                    for (int w = 0; w < kWords; ++w)
-#pragma unroll
-                        for (int q = 0; q < 8; ++q)
-                            if (w * 8 + q < R / 4) out[w * 8 + q] = (((m[w] >> (4 * q)) & 15u) * 0x00204081u) & 0x01010101u;
-                } else {
-#pragma unroll
-                    for (int w = 0; w < kWords; ++w)
-                        for (int r = w * 32; r < min(R, w * 32 + 32); ++r) flags[r] = (uint8_t)((m[w] >> (r & 31)) & 1u);
+            } else {
+#pragma unroll 1
+                for (int j = 0; j < k; ++j) {
+                    e[j] = resolve_expert(p, t, e[j], bad);
+#pragma unroll 1
+                    for (int i = 0; i < j; ++i)
+                        if (e[j] >= 0 && e[i] == e[j]) {
+                            bad = true;
+                            e[j] = -1;
+                        }
+                    if (e[j] < 0) continue;
+                    atomicAdd(&hist[e[j]], 1);
+                    const int r = p.L == 1 ? e[j] : fast_div(e[j], p.L_magic);
+                    bool first = true;
+#pragma unroll 1
+                    for (int i = 0; i < j; ++i) first = first && !(e[i] >= r * p.L && e[i] < (r + 1) * p.L);
+                    if (first) {
+                        atomicAdd(&hist[p.E + r], 1);
+                        if (flags) mine[r] = 1;
+                    }
                 }
             }
         }
-        if (kW) {
-#pragma unroll
-            for (int w = 0; w < kWords; ++w) {
-                const int c = __popc(transpose32(m[w], lane));
-                if (c) atomicAdd(&hist[p.E + w * 32 + lane], c);
+        if (kTile && flags) {
+            __syncwarp();
+            const int bytes = min(32, T - g * 32) * R;
+            if ((reinterpret_cast<uintptr_t>(is_token_in_rank) & 15) == 0) {   // (32 tokens' bytes start on a 32-byte boundary)
+                for (int i = lane; i < bytes / 16; i += 32) reinterpret_cast<uint4*>(out)[i] = reinterpret_cast<const uint4*>(tile)[i];
+                for (int i = bytes / 16 * 16 + lane; i < bytes; i += 32) out[i] = tile[i];
+            } else {
+                for (int i = lane; i < bytes; i += 32) out[i] = tile[i];
             }
+            __syncwarp();   // (the tile is used again)
         }
     }
     if (bad) report(p.status, kErrBadIndex);
+    if (kCluster) {
+        const int cs = gridDim.x;
+        cluster_arrive();
+        cluster_wait();
+        for (int b = (int)threadIdx.x * cs + (int)blockIdx.x; b < B; b += kN * cs) {
+            unsigned sum = 0u;
+#pragma unroll 8
+            for (int q = 0; q < cs; ++q) sum += ld_cluster(reinterpret_cast<const unsigned*>(hist) + b, (unsigned)q);
+            if (b < p.E) {
+                if (num_tokens_per_expert) num_tokens_per_expert[b] = (int)sum;
+            } else if (num_tokens_per_rank) {
+                num_tokens_per_rank[b - p.E] = (int)sum;
+            }
+        }
+        cluster_arrive();   // (a CTA's counts stay until all have read them)
+        cluster_wait();
+        return;
+    }
     __syncthreads();
-    for (int b = threadIdx.x; b < B; b += kLayoutThreads)
+    for (int b = threadIdx.x; b < B; b += kN)
         if (hist[b]) atomicAdd(acc + b, hist[b]);
     __threadfence();
     __syncthreads();
@@ -1546,7 +1585,7 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(const Params p, 
     __syncthreads();
     if (!last) return;
     __threadfence();
-    for (int b = threadIdx.x; b < B; b += kLayoutThreads) {
+    for (int b = threadIdx.x; b < B; b += kN) {
         const int sum = atomicExch(acc + b, 0);   // (zero for the next call)
         if (b < p.E) {
             if (num_tokens_per_expert) num_tokens_per_expert[b] = sum;
@@ -1554,7 +1593,7 @@ __global__ void __launch_bounds__(kLayoutThreads) layout_kernel(const Params p, 
             num_tokens_per_rank[b - p.E] = sum;
         }
     }
-    for (int b = B + threadIdx.x; b < acc_words; b += kLayoutThreads) acc[b] = 0;   // (an overlapping call may have had more bins)
+    for (int b = B + threadIdx.x; b < acc_words; b += kN) acc[b] = 0;   // (an overlapping call may have had more bins)
 }
 
 // ------------------------------------------------------------------------- launchers
@@ -1808,26 +1847,46 @@ cudaError_t launch_empty(int num_sms, bool ahead, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+template <int kK, bool kTile, bool kCluster>
+static cudaError_t launch_layout_t(const Params& p, int blocks, int smem, int32_t* per_rank, int32_t* per_expert, uint8_t* in_rank,
+                                   int32_t* acc, int acc_words, unsigned* ticket, cudaStream_t st) {
+    auto kern = layout_kernel<kK, kTile, kCluster>;
+    if (smem > 48 * 1024) {
+        static std::atomic<int> granted[kAttrDevices];
+        const cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void*>(kern), smem, granted);
+        if (e != cudaSuccess) return e;
+    }
+    return launch_overlapped(kern, blocks, kCluster ? kThreads : kLayoutThreads, (size_t)smem, st, false, kCluster ? blocks : 1, p,
+                             per_rank, per_expert, in_rank, acc, acc_words, ticket);
+}
+
 cudaError_t launch_layout(const Params& p, int32_t* num_tokens_per_rank, int32_t* num_tokens_per_expert,
                           uint8_t* is_token_in_rank, int32_t* acc, int acc_words, unsigned* ticket, cudaStream_t st) {
-    // a group of 32 tokens per warp; beyond two CTAs per SM a warp takes several
-    const int64_t groups = ((int64_t)p.T + 31) / 32, per_cta = kLayoutThreads / 32;
-    int64_t blocks = (groups + per_cta - 1) / per_cta;
-    if (blocks > 296) blocks = 296;
+    const bool tile = p.R <= kLayoutTileRanks;
+    const int counts = (p.B + 3) / 4 * 16;
+    const bool cluster = p.T <= kLayoutClusterTokens && counts <= 48 * 1024;
+    const int threads = cluster ? kThreads : kLayoutThreads;
+    // a token per thread; beyond one cluster (two CTAs per SM) a thread takes several
+    int64_t blocks = ((int64_t)p.T + threads - 1) / threads;
+    const int64_t most = cluster ? kLayoutClusterTokens / kThreads : 296;
+    if (blocks > most) blocks = most;
     if (blocks < 1) blocks = 1;
-    const size_t smem = sizeof(int) * (size_t)p.B;
-    auto go = [&](auto kern) {
-        return launch_overlapped(kern, (int)blocks, kLayoutThreads, smem, st, false, 1, p, num_tokens_per_rank,
-                                 num_tokens_per_expert, is_token_in_rank, acc, acc_words, ticket);
+    while (cluster && (blocks & (blocks - 1)) != 0) ++blocks;   // a power of two
+    const int smem = counts + (tile ? threads * p.R : 0);
+    auto go = [&](auto kk, auto tl) {
+        if (cluster) return launch_layout_t<kk(), tl(), true>(p, (int)blocks, smem, num_tokens_per_rank, num_tokens_per_expert, is_token_in_rank, acc, acc_words, ticket, st);
+        return launch_layout_t<kk(), tl(), false>(p, (int)blocks, smem, num_tokens_per_rank, num_tokens_per_expert, is_token_in_rank, acc, acc_words, ticket, st);
     };
-    if (p.R > 32 * kLayoutMaskWords) return go(layout_kernel<0, 0>);
-    const bool narrow = p.R <= 32;
-    switch (p.k) {
-        case 2: return narrow ? go(layout_kernel<2, 1>) : go(layout_kernel<2, kLayoutMaskWords>);
-        case 4: return narrow ? go(layout_kernel<4, 1>) : go(layout_kernel<4, kLayoutMaskWords>);
-        case 8: return narrow ? go(layout_kernel<8, 1>) : go(layout_kernel<8, kLayoutMaskWords>);
-        default: return narrow ? go(layout_kernel<0, 1>) : go(layout_kernel<0, kLayoutMaskWords>);
-    }
+    auto by_k = [&](auto tl) {
+        switch (p.k) {
+            case 2: return go(std::integral_constant<int, 2>{}, tl);
+            case 4: return go(std::integral_constant<int, 4>{}, tl);
+            case 6: return go(std::integral_constant<int, 6>{}, tl);
+            case 8: return go(std::integral_constant<int, 8>{}, tl);
+            default: return go(std::integral_constant<int, 0>{}, tl);
+        }
+    };
+    return tile ? by_k(std::true_type{}) : by_k(std::false_type{});
 }
 
 }  // namespace ubep

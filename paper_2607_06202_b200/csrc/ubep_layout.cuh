@@ -39,6 +39,35 @@ __device__ __forceinline__ int resolve_expert(const Params& p, int t, int raw) {
     return e;
 }
 
+// kN slots of token t: raw ids in, physical experts out, -1 where there is none; `bad` if an id is out of range.  (All
+// look-ups of a step side by side.)
+template <int kN>
+__device__ __forceinline__ void resolve_slots(const Params& p, int t, int (&e)[kN], bool& bad) {
+    if (p.phys != nullptr) {
+        int nc[kN];
+#pragma unroll
+        for (int i = 0; i < kN; ++i) {
+            const bool in = (unsigned)e[i] < (unsigned)p.E_log;
+            bad |= !in && e[i] != -1;
+            nc[i] = in ? __ldg(p.ncopies + e[i]) : 0;
+        }
+#pragma unroll
+        for (int i = 0; i < kN; ++i) {
+            const bool in = (unsigned)e[i] < (unsigned)p.E_log, ok = nc[i] >= 1 && nc[i] <= p.C;
+            bad |= in && !ok;
+            const int copy = nc[i] > 2 ? t % nc[i] : nc[i] == 2 ? t & 1 : 0;
+            e[i] = ok ? __ldg(p.phys + (size_t)e[i] * p.C + copy) : -1;
+            bad |= ok && e[i] < 0;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < kN; ++i) {
+        const bool valid = (unsigned)e[i] < (unsigned)p.E;
+        bad |= !valid && e[i] != -1;
+        e[i] = valid ? e[i] : -1;
+    }
+}
+
 __device__ __forceinline__ int warp_sum(int v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

@@ -80,3 +80,24 @@ def test_the_results_are_tensors_of_their_own():
     assert [t.untyped_storage().nbytes() for t in out] == [4 * 4, 4 * 16, 500 * 4]
     assert [t.storage_offset() for t in out] == [0, 0, 0]
     assert len({t.untyped_storage().data_ptr() for t in out}) == 3
+
+
+@pytest.mark.parametrize("T", [512, 513, 1025, 4096, 4097])
+@pytest.mark.parametrize("E,R,k", [(72, 9, 6), (128, 128, 8), (129, 129, 1), (8, 2, 4), (12, 3, 2)])
+def test_one_cluster_and_beyond(T, E, R, k):
+    """One CTA, clusters of two to eight, and totals in global memory; masks that start on no 16-byte boundary."""
+    rng = np.random.Generator(np.random.PCG64(T + E))
+    idx = np.argsort(rng.random((T, E)), axis=1)[:, :k].astype(np.int32)
+    idx[rng.random(idx.shape) < 0.2] = -1
+    lay = oracle.layout(idx, E, R, R, 0)
+    buf = B.Buffer(num_ranks=R, num_experts=E, hidden=8, topk=k, max_tokens=T, rows_per_rank_cap=1)
+    npr, npe = (torch.full((n,), -1, dtype=torch.int32, device="cuda") for n in (R, E))
+    for off in (0, 4, 1):
+        raw = torch.full((T * R + 32,), 7, dtype=torch.uint8, device="cuda")
+        B.ubep_get_dispatch_layout(buf.handle, torch.from_numpy(idx).cuda(), T, npr, npe, raw[off:off + T * R])
+        assert buf.status() == 0
+        assert np.array_equal(npr.cpu().numpy(), lay.num_tokens_per_rank)
+        assert np.array_equal(npe.cpu().numpy(), lay.num_tokens_per_expert)
+        got = raw.cpu().numpy()
+        assert np.array_equal(got[off:off + T * R].reshape(T, R), lay.is_token_in_rank)
+        assert (got[:off] == 7).all() and (got[off + T * R:] == 7).all()
