@@ -10,7 +10,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libubep.so")
 SOURCES = ["ubep_kernels.cu", "ubep_few.cu", "ubep_host.cu", "ubep_static.cu", "ubep_mapper.cu", "ubep_sync.cu", "ubep_sharded.cu"]
-DEPENDS = SOURCES + ["ubep_common.cuh", "ubep_cluster.cuh", "ubep_launch.cuh", "ubep_layout.cuh", "ubep_quant.cuh", "ubep_kernels.h", "ubep_sync.h", "ubep_sharded.h", "../../include/ubep.h"]
+DEPENDS = SOURCES + ["ubep_common.cuh", "ubep_cluster.cuh", "ubep_launch.cuh", "ubep_few.cuh", "ubep_layout.cuh", "ubep_quant.cuh", "ubep_kernels.h", "ubep_sync.h", "ubep_sharded.h", "../../include/ubep.h"]
 NATIVE = os.path.join(HERE, "_native.so")             # CPython module of the calls a layer makes every step
 NATIVE_DEPENDS = ["ubep_py.cpp", "../../include/ubep.h"]
 

@@ -7,52 +7,16 @@
 // table is staged once; then every slot of the CTA's own tokens is a warp's, which counts the table for its own expert and rank
 // alone, sends its copy, writes its metadata and adds to the arrival counter by itself.  There is no barrier after the
 // one behind the staging (FP8 rows: one more, between quantising and sending).
+#include "ubep_few.cuh"
 #include "ubep_kernels.h"
 #include "ubep_launch.cuh"
-#include "ubep_layout.cuh"
 #include "ubep_quant.cuh"
 
 namespace ubep {
 
 namespace {
 
-constexpr unsigned kAll = 0xffffffffu;
 constexpr int kFewSmem = 120 * 1024;   // more than half of an SM's shared memory
-
-// 1 << n, and 0 from 32 on (also for the large values that negative numbers are).
-__device__ __forceinline__ unsigned bit_or_none(unsigned n) {
-    unsigned v;
-    asm("shl.b32 %0, 1, %1;" : "=r"(v) : "r"(n));
-    return v;
-}
-// The n lowest bits; all of them from 32 on, none up to 0.
-__device__ __forceinline__ unsigned low_bits(int n) { return bit_or_none((unsigned)max(n, 0)) - 1u; }
-
-// The staged table: 16-bit physical expert ids, kNone for a slot that is empty or bad.
-constexpr unsigned kNone = 0xffffu;
-__device__ __forceinline__ unsigned pack16(int a, int b) { return ((unsigned)a & 0xffffu) | (unsigned)b << 16; }
-
-// The experts first .. first + 31 that token t selects, one bit each.  (An expert named twice is one bit.)
-template <int K>
-__device__ __forceinline__ unsigned experts_of(const uint16_t* ids, int t, unsigned first) {
-    unsigned w[4] = {0u, 0u, 0u, 0u};
-    if (K == 8) {
-        const uint4 v = *reinterpret_cast<const uint4*>(ids + t * 8);
-        w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
-    } else if (K == 4) {
-        const uint2 v = *reinterpret_cast<const uint2*>(ids + t * 4);
-        w[0] = v.x; w[1] = v.y;
-    } else if (K == 1) {
-        w[0] = ids[t] | kNone << 16;
-    } else {
-#pragma unroll
-        for (int i = 0; i < K / 2; ++i) w[i] = reinterpret_cast<const unsigned*>(ids + t * K)[i];
-    }
-    unsigned m = 0u;
-#pragma unroll
-    for (int i = 0; i < (K + 1) / 2; ++i) m |= bit_or_none((w[i] & 0xffffu) - first) | bit_or_none((w[i] >> 16) - first);
-    return m;
-}
 
 template <int K, bool kFp8, bool kDedup>
 __global__ void __launch_bounds__(kThreads, 1) few_kernel(const Params p, const SmemPlan pl) {
@@ -95,26 +59,7 @@ __global__ void __launch_bounds__(kThreads, 1) few_kernel(const Params p, const 
         }
         if (lane == 0) epoch_sm = epoch_from_counter(ctr);
     } else {
-        constexpr int kV = K % 4 == 0 ? 4 : K % 2 == 0 ? 2 : 1;   // slots per load
-#pragma unroll 1
-        for (int i = tid - 32; i < p.T * (K / kV); i += kThreads - 32) {
-            const int t = i / (K / kV);
-            if (kV == 4) {
-                const int4 v = __ldg(reinterpret_cast<const int4*>(p.topk_idx) + i);
-                int e[4] = {v.x, v.y, v.z, v.w};
-                resolve_slots(p, t, e, bad);
-                reinterpret_cast<uint2*>(ids)[i] = make_uint2(pack16(e[0], e[1]), pack16(e[2], e[3]));
-            } else if (kV == 2) {
-                const int2 v = __ldg(reinterpret_cast<const int2*>(p.topk_idx) + i);
-                int e[2] = {v.x, v.y};
-                resolve_slots(p, t, e, bad);
-                reinterpret_cast<unsigned*>(ids)[i] = pack16(e[0], e[1]);
-            } else {
-                int e[1] = {__ldg(p.topk_idx + i)};
-                resolve_slots(p, t, e, bad);
-                ids[i] = (uint16_t)e[0];
-            }
-        }
+        bad = stage_table<K>(p, ids, tid - 32, kThreads - 32);
     }
     // this warp's slot, if it has one: slot j of own token tl
     const int tl = warp / K, j = warp % K, t = t0 + tl;
@@ -126,72 +71,23 @@ __global__ void __launch_bounds__(kThreads, 1) few_kernel(const Params p, const 
     if (tid == 0) ticket = atomicAdd(p.done_ticket, 1u);   // (every CTA has read the epoch when the last ticket is taken)
     const unsigned half = epoch_sm & 1u;
 
-    // ---- the slot's row: tokens before t that chose the expert, behind the experts of the rank in front of it; with one
-    // row per (token, rank): tokens before t that visit the rank
-    const unsigned lbits = low_bits(p.L);
+    // ---- the slot's row, its copy if the row has landed, its metadata
     bool send = false, sent = false;
     int r = 0, gpos = -1;
-    auto copy = [&]() {   // bf16: the row, which has landed
+    auto copy = [&]() {   // bf16
         if (lane == 0) bulk_store(p.recv_x + (size_t)gpos * p.rowB + out_off, smem + (size_t)tl * pl.stage_bytes, out_bytes);
         bulk_commit();
         sent = true;
     };
     if (slot) {
-        const unsigned e_i = lane < K ? ids[t * K + lane] : kNone;
-        const unsigned e = __shfl_sync(kAll, e_i, j);
-        const bool valid = e != kNone && !__any_sync(kAll, lane < j && e_i == e);   // (of an expert named twice the first slot counts)
-        if (e != kNone && !valid) bad = true;
-        int row = -1;
-        if (valid) {
-            r = p.L == 1 ? (int)e : fast_div((int)e, p.L_magic);
-            const unsigned f = (unsigned)(r * p.L), d = e - f, below = (1u << d) - 1u;
-            unsigned acc = 0u;
-#pragma unroll 2
-            for (int tt = lane; tt < p.T; tt += 32) {
-                const unsigned m = experts_of<K>(ids, tt, f) & lbits;
-                acc += (unsigned)__popc(m & below) << 16;
-                if (tt < t) acc += ((m >> d) & 1u) << 16 | (m != 0u ? 1u : 0u);
-            }
-            acc = __reduce_add_sync(kAll, acc);
-            const int at = (int)(acc >> 16);
-            row = kDedup ? (int)(acc & 0xffffu) : at;
-            const bool here = e_i - f < (unsigned)p.L;   // (this lane's slot names the same rank)
-            const bool first = !kDedup || !__any_sync(kAll, here && lane < j);
-            const bool fits = row < p.cap;
-            gpos = fits ? r * p.cap + row : -1;
-            send = first && fits;
-            if (!kFp8 && send && __all_sync(kAll, mbar_test_wait(&row_bar[tl], 0))) copy();   // (the metadata while it is on its way)
-            bool full = !fits;
-            if (part == 0) {
-                if (kDedup) {
-                    if (at < p.er_cap) {
-                        if (lane == 0) p.expert_rows[(size_t)r * p.er_cap + at] = row;
-                    } else {
-                        full = true;
-                    }
-                    if (send) {
-                        bool again = false;   // a slot of the token in front of this lane's names the same expert
-#pragma unroll
-                        for (int i = 1; i < K; ++i) {
-                            const unsigned other = __shfl_up_sync(kAll, e_i, i);
-                            again = again || (lane >= i && other == e_i);
-                        }
-                        if (lane < K) {
-                            p.recv_topk_idx[(size_t)gpos * K + lane] = here && !again ? (int)(e_i - f) : -1;
-                            p.recv_topk_w[(size_t)gpos * K + lane] = here && !again ? w_i : 0.0f;
-                        }
-                    }
-                } else if (send && lane == j) {
-                    p.recv_weight[gpos] = w_i;
-                }
-                if (send && lane == 0) p.recv_src_idx[gpos] = t;
-            }
-            if (full) report(p.status, kErrCapacity);
-        }
-        if (part == 0 && lane == 0) {
-            p.slot_row[(size_t)t * K + j] = row;
-            p.slot_pos[(size_t)t * K + j] = gpos;
-        }
+        const SlotRow s = slot_row<K>(p, ids, t, j, kDedup, lane);
+        bad = bad || s.twice;
+        r = s.r;
+        gpos = s.valid && s.row < p.cap ? r * p.cap + s.row : -1;
+        send = s.first && gpos >= 0;
+        if (!kFp8 && send && __all_sync(kAll, mbar_test_wait(&row_bar[tl], 0))) copy();   // (the metadata while it is on its way)
+        if (part == 0) slot_meta<K>(p, s, t, j, gpos, w_i, kDedup, lane);
+        else if (s.valid && gpos < 0) report(p.status, kErrCapacity);
     }
     if (bad) report(p.status, kErrBadIndex);
     if (tid == 0) trace(p, c, kTrFinalized);
@@ -253,47 +149,10 @@ __global__ void __launch_bounds__(kThreads, 1) few_kernel(const Params p, const 
     }
     if (tid == 0) trace(p, c, kTrIssued);
 
-    // ---- what no row waits for: per rank the totals and the expert offsets, per source rank counts and offsets.  A unit is
-    // a rank and as many source ranks as there are lanes for, a lane per (source rank, expert); the warps without a slot, the
-    // last ones of every CTA, come first.  (One loop of few instructions that keeps nothing per group of tokens: with the
-    // groups unrolled and their bitmaps in registers the call of 1 to 13 tokens took 0.6 us more.)
-    const int lsh = 32 - __clz(p.L - 1);   // experts of a rank, rounded up to a power of two
+    // ---- what no row waits for; the warps without a slot, the last ones of every CTA, come first
 #pragma unroll 1
-    for (int u = (kWarps - 1 - warp) * p.grid + c; u < p.R * pl.duty_units; u += kWarps * p.grid) {
-        const int ur = u / pl.duty_units, uq = u - ur * pl.duty_units, f = ur * p.L;
-        const int l = lane & ((1 << lsh) - 1), s = (uq << (5 - lsh)) + (lane >> lsh);
-        const bool mine = s < p.S && l < p.L;
-        const int b0 = src_begin(min(s, p.S), p.T, p.S), b1 = src_begin(min(s + 1, p.S), p.T, p.S);
-        int tot = 0, visits = 0;         // tokens that chose expert `lane` of the rank / that visit it
-        int before = 0, after = 0;       // tokens before the source rank's first and behind its last one that chose expert l
-#pragma unroll 1
-        for (int g = 0; g < p.T; g += 32) {
-            const unsigned m = g + lane < p.T ? experts_of<K>(ids, g + lane, (unsigned)f) & lbits : 0u;
-            visits += m != 0u ? 1 : 0;
-            const unsigned bm = transpose32(m, lane);   // lane = expert, bit = token
-            tot += __popc(bm);
-            const unsigned of_l = __shfl_sync(kAll, bm, l);
-            before += __popc(of_l & low_bits(b0 - g));
-            after += __popc(of_l & low_bits(b1 - g));
-        }
-        const int incl = warp_incl_scan(tot, lane), eo = incl - tot, eo_l = __shfl_sync(kAll, eo, l);
-        if (mine) {
-            p.cnt[(size_t)s * p.E + f + l] = after - before;
-            p.src_offset[(size_t)s * p.E + f + l] = eo_l + before;
-        }
-        if (uq == 0) {
-            if (lane < p.L) {
-                p.expert_offset[f + lane] = eo;
-                p.num_tokens_per_expert[f + lane] = tot;
-            }
-            visits = __reduce_add_sync(kAll, visits);
-            const int rows = __shfl_sync(kAll, incl, 31);
-            if (lane == 0) {
-                p.num_tokens_per_rank[ur] = visits;
-                p.num_rows_per_rank[ur] = kDedup ? visits : rows;
-            }
-        }
-    }
+    for (int u = (kWarps - 1 - warp) * p.grid + c; u < p.R * pl.duty_units; u += kWarps * p.grid)
+        write_table_unit<K>(p, ids, u, pl.duty_units, kDedup, lane);
     if (tid == 0) trace(p, c, kTrScanned);
 
     // ---- the arrival counters (eighths of a row: see publish_arrivals): every warp for its own row
@@ -333,14 +192,6 @@ cudaError_t launch_few_k(const Params& p, const SmemPlan& pl, cudaStream_t st) {
 
 }  // namespace
 
-// Small batches: every slot of the CTA's tokens has a warp.  A slot's warp reads the whole table (T tokens of k slots and some
-// 8 more instructions' worth each) and an SM's four schedulers share the warps of up to `most` tokens, so the line lies at a
-// product of these.  Dispatch + combine in one graph, as before and this way: 1 token of 7168 channels, top-8, bf16 8.4 and 5.3 us,
-// 16 tokens of 4096 channels 8.6 and 5.5, 128 of 256 channels, top-2 7.9 and 4.6; near the line 256 tokens of 4096 channels,
-// top-8 12.0 and 12.0 (FP8 rows 13.3 and 12.9), 444 of 1024, top-4 9.8 and 8.3 (10.2 and 9.9), 592 of 256, top-2 9.6 and 9.6
-// (FP8); beyond it 296 tokens of 4096 channels, top-8 12.4 and 13.3, 512 of 1024, top-4 10.1 and 10.5, 740 of 256, top-2, FP8
-// 9.9 and 11.1.
-constexpr int kFewWork = 65536;
 bool plan_few(const Params& p, int max_smem, SmemPlan* out) {
     const int most = (p.T + p.nchunks - 1) / p.nchunks;   // tokens of a CTA
     if (most * p.k > kWarps || (int64_t)most * p.k * p.T * (p.k + 8) > kFewWork || p.L > 32 || p.ordered) return false;
@@ -366,9 +217,7 @@ bool plan_few(const Params& p, int max_smem, SmemPlan* out) {
     // (programmatic launches), SMs without combine CTAs took two and others none: sixteen layers of 128 tokens of 7168 channels,
     // top-8, in one graph 12.6 us per layer, this way 10.4.  (Warps that leave at once do not hold their registers: no change.)
     pl.total = (int)(total < kFewSmem ? kFewSmem : total);
-    int at_once = 32;   // source ranks a warp looks at together
-    for (int l = 1; l < p.L; l *= 2) at_once /= 2;
-    pl.duty_units = (p.S + at_once - 1) / at_once;
+    pl.duty_units = table_units(p);
     *out = pl;
     return true;
 }

@@ -623,7 +623,8 @@ int ubep_dispatch_sync(ubep_buffer_t* buf, int protocol, const void* x, const in
                       ubep::plan_dispatch(p, ubep::kModeCluster, room, &pl) == 0;   // (a cluster of one)
         return whole_table || ubep::plan_dispatch(p, UBEP_PIPELINE_PHASED, room, &pl) == 0;
     };
-    const bool strips = fits(true);
+    const bool few = ubep::plan_sync_few(p, protocol, buf->max_smem, &pl);
+    const bool strips = few || fits(true);
     if (!strips && !fits(false)) return UBEP_ERR_ARG;   // (tables of ten thousand experts leave no 48 KB for the strips)
     const WireLayout& w = buf->wlay;
     ubep::SyncParams sp{};
@@ -650,12 +651,12 @@ int ubep_dispatch_sync(ubep_buffer_t* buf, int protocol, const void* x, const in
         if (e != cudaSuccess) return cuda_fail(buf, e);
         buf->sp_dirty = false;
     }
-    if (!whole_table) {
+    if (!few && !whole_table) {
         e = ubep::launch_count_scan(p, pl, st);
         if (e != cudaSuccess) return cuda_fail(buf, e);
         g_launches += 2;
     }
-    e = ubep::launch_sync_dispatch(p, pl, sp, whole_table, st);
+    e = ubep::launch_sync_dispatch(p, pl, sp, few ? ubep::kSyncFew : whole_table ? ubep::kSyncWhole : ubep::kSyncLaunched, st);
     if (e != cudaSuccess) return cuda_fail(buf, e);
     g_launches += 1;
     return UBEP_OK;

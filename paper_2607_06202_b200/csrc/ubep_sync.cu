@@ -12,6 +12,7 @@
 //
 // A DataBlock is the 16 bytes one thread stores with a single 128-bit access.
 #include "ubep_cluster.cuh"
+#include "ubep_few.cuh"
 #include "ubep_quant.cuh"
 #include "ubep_sync.h"
 
@@ -94,6 +95,9 @@ __device__ __forceinline__ bool wait_count(const unsigned* ctr, unsigned want, W
     return true;
 }
 
+// Behind the plan: checksums [R] of 8 bytes, the regions' first rows [R + 1], the quantised row.
+__host__ __device__ inline int sync_first(const Params& p) { return p.R * 8; }
+__host__ __device__ inline int sync_qrow(const Params& p) { return (sync_first(p) + (p.R + 1) * 4 + 15) / 16 * 16; }
 __host__ __device__ inline int qrow_bytes(const Params& p) { return p.payload ? ((p.H + 4 * p.G + 15) / 16) * 16 : 0; }
 __host__ __device__ inline bool strips_in_ring(const Params& p) {   // (a plan has four rows at least, two for FP8 rows)
     return (p.payload ? 2 : 4) * 2 * p.H >= kWarps * kStripWords * 4;
@@ -103,12 +107,16 @@ __host__ __device__ inline bool strips_in_ring(const Params& p) {   // (a plan h
 // wire row of H + 4 * H / 128 bytes); the sender quantises a row once into shared memory and sends from
 // there; what arrives goes to the payload and the scale array of the receive region.  The checksum
 // markers of Data-for-Checksum are taken from the payload bytes.
-// kTable: the layout is derived here from the whole routing table in shared memory (small tables).
-// Otherwise it comes from count_kernel / scan_kernel, launched before over the same chunks: the CTA stages
-// only its own tokens and reads the rows of earlier chunks, the expert offsets and the region sizes.
-template <int kProto, bool kFp8, bool kTable>
+// kLayout: kLaunched, from count_kernel / scan_kernel, launched before over the same chunks: the CTA stages only its own tokens
+// and reads the rows of earlier chunks, the expert offsets and the region sizes.  kWhole: every CTA counts the whole routing table.
+// K > 0, small tables of K slots per token: a warp per slot (ubep_few.cuh); the CTAs of a chunk share its rows, a range of their
+// blocks each.
+constexpr int kLaunched = 0, kWhole = -1;
+template <int kProto, bool kFp8, int kLayout>
 __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params p, const SmemPlan pl,
                                                                    const SyncParams sp) {
+    constexpr bool kTable = kLayout == kWhole, kFew = kLayout > 0;
+    constexpr int K = kFew ? kLayout : 1;
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ unsigned seq_sm;
     __shared__ int abort_flag;
@@ -124,17 +132,36 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
     float* w_sm = reinterpret_cast<float*>(smem + pl.off_w);
     int* hist = reinterpret_cast<int*>(smem + pl.off_hist);
     int* nrows = reinterpret_cast<int*>(smem + pl.off_arr);     // rows every region receives
+    int* first = reinterpret_cast<int*>(smem + pl.total + sync_first(p));   // [R + 1] (Token-Flag and Sentinel receivers)
     int* order_sm = reinterpret_cast<int*>(smem + pl.off_order);
     unsigned long long* chk_sm = reinterpret_cast<unsigned long long*>(smem + pl.total);   // DC: [R]
-    uint8_t* qrow = smem + pl.total + (((size_t)p.R * 8 + 15) & ~(size_t)15);              // FP8: the quantised row
+    uint8_t* qrow = smem + pl.total + sync_qrow(p);                                         // FP8: the quantised row
     // TFF: [kWarps, kStripWords]; in the ring of rows, which the receiver no longer needs, where that is large enough
-    uint32_t* strips = reinterpret_cast<uint32_t*>(strips_in_ring(p) ? smem : qrow + qrow_bytes(p));
+    uint32_t* strips = reinterpret_cast<uint32_t*>(kFew || strips_in_ring(p) ? smem : qrow + qrow_bytes(p));
     __shared__ __align__(8) uint64_t row_bar[2];   // the row of an even / odd token has landed in ring stage 0 / 1
     const BinMaps bmaps{reinterpret_cast<unsigned*>(smem + pl.off_mask), reinterpret_cast<unsigned*>(smem + pl.off_bm),
                         pl.map_wb, pl.map_bp, pl.map_groups};
-    const int t0 = (int)chunk_begin(c, p.T, p.nchunks), t1 = (int)chunk_begin(c + 1, p.T, p.nchunks);
+    const int parts = kFew ? p.parts : 1, part = kFew ? c % parts : 0, ch = kFew ? c / parts : c;
+    const int t0 = (int)chunk_begin(ch, p.T, p.nchunks), t1 = (int)chunk_begin(ch + 1, p.T, p.nchunks);
     const int ntok = t1 - t0;
+    uint16_t* ids16 = reinterpret_cast<uint16_t*>(smem + pl.off_ids);   // (kFew)
+    auto fetch_row = [&](int tl) {   // one thread; the row before the last one has been sent
+        mbar_arrive_expect_tx(&row_bar[tl & 1], (unsigned)p.H * 2u);
+        bulk_load(smem + (size_t)(tl & 1) * pl.stage_bytes, p.x + (size_t)(t0 + tl) * p.H, (unsigned)p.H * 2u, &row_bar[tl & 1]);
+    };
+    constexpr int kFetcher = kFew ? 0 : 32;   // (kFew: warp 0 has no part in staging the table)
+    if (tid == kFetcher) {
+        mbar_init(&row_bar[0], 1);
+        mbar_init(&row_bar[1], 1);
+        mbar_fence_init();
+        if (ntok > 0) fetch_row(0);   // on its way while the layout is computed
+        if (ntok > 1) fetch_row(1);
+    }
 
+    if (kFew) {
+        for (int r = tid; r < R; r += kThreads) nrows[r] = 0;
+        __syncthreads();
+    }
     if (tid == 0) {
         seq_sm = read_seq_and_check_in(sp, p.grid);
         abort_flag = 0;
@@ -148,17 +175,6 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
     }
     if (kProto == kDC)
         for (int r = tid; r < R; r += kThreads) chk_sm[r] = 0ull;
-    auto fetch_row = [&](int tl) {   // one thread; the row before the last one has been sent
-        mbar_arrive_expect_tx(&row_bar[tl & 1], (unsigned)p.H * 2u);
-        bulk_load(smem + (size_t)(tl & 1) * pl.stage_bytes, p.x + (size_t)(t0 + tl) * p.H, (unsigned)p.H * 2u, &row_bar[tl & 1]);
-    };
-    if (tid == 32) {
-        mbar_init(&row_bar[0], 1);
-        mbar_init(&row_bar[1], 1);
-        mbar_fence_init();
-        if (ntok > 0) fetch_row(0);   // on its way while the layout is computed
-        if (ntok > 1) fetch_row(1);
-    }
 
     // ---- layout: counts of every bin over the whole routing table -> totals, the rows before this CTA's tokens,
     // expert offsets, rows of this CTA's slots
@@ -168,7 +184,20 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
     unsigned* cnt = reinterpret_cast<unsigned*>(smem + pl.off_cnt);   // (kTable)
     unsigned* own = cnt + p.B + 1;
     bool twice = false;
-    if (kTable) {
+    if (kFew) {
+        bool bad = warp != 0 && stage_tokens<K>(p, ids16, nrows, p.dedup != 0, tid - 32, kThreads - 32);
+        __syncthreads();
+        for (int sl = warp; sl < ntok * K; sl += kWarps) {
+            const int t = t0 + sl / K, j = sl % K;
+            const float w_i = part == 0 && lane < K ? __ldg(p.topk_w + (size_t)t * K + lane) : 0.0f;
+            const SlotRow s = slot_row<K>(p, ids16, t, j, p.dedup != 0, lane);
+            bad = bad || s.twice;
+            const int gpos = s.valid && s.row < p.cap ? s.r * p.cap + s.row : -1;
+            if (lane == 0) pos[sl] = s.first ? gpos : -1;
+            if (part == 0) slot_meta<K>(p, s, t, j, gpos, w_i, p.dedup != 0, lane);
+        }
+        if (bad) report(p.status, kErrBadIndex);
+    } else if (kTable) {
         for (int b = tid; b < 3 * (p.B + 1); b += kThreads) cnt[b] = 0u;
         for (int b = tid; b < pl.map_groups * pl.map_bp; b += kThreads) bmaps.bm[b] = 0u;
         __syncthreads();
@@ -177,8 +206,10 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
     } else {
         stage_ids(p, t0, t1, ids_sm, tid, kThreads);
     }
-    for (int r = tid; r < R; r += kThreads) order_sm[r] = __ldg(p.order_pos + r);
-    for (int i = tid; i < ntok * k; i += kThreads) w_sm[i] = __ldg(p.topk_w + (size_t)t0 * k + i);
+    if (!kFew) {
+        for (int r = tid; r < R; r += kThreads) order_sm[r] = __ldg(p.order_pos + r);
+        for (int i = tid; i < ntok * k; i += kThreads) w_sm[i] = __ldg(p.topk_w + (size_t)t0 * k + i);
+    }
     if (__syncthreads_or(twice)) {
         local_clean_own_duplicates(p, 0, ntok, ids_sm, tid, kThreads);
         __syncthreads();
@@ -206,7 +237,8 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
                        [&](int e, int tl) { return base[e] + own_below(bmaps, e, tl); },
                        [&](int r, int tl) { return base[p.E + r] + own_below(bmaps, p.E + r, tl); },
                        true, c, order_sm, pos, key, nullptr, tid, kThreads);
-    } else {
+        __syncthreads();
+    } else if (!kFew) {
         build_bin_maps(p, ids_sm, ntok, bmaps, warp, kWarps, lane);
         int* base_sm = hist;   // per bin: rows of all earlier chunks (+ the expert's offset in its region)
         for (int b = tid; b < p.B; b += kThreads)
@@ -217,8 +249,8 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
                        [&](int e, int tl) { return base_sm[e] + bits_in_range(bmaps, e, 0, tl); },
                        [&](int r, int tl) { return base_sm[p.E + r] + bits_in_range(bmaps, p.E + r, 0, tl); },
                        true, c, order_sm, pos, key, nullptr, tid, kThreads);
+        __syncthreads();
     }
-    __syncthreads();
     if (tid == 0) times[1] = global_ns();
     // ---- sender: the rows of tokens [t0, t1), one token at a time, all threads on a row
     const int wbytes = kFp8 ? p.H + 4 * p.G : p.rowB;   // bytes of one row on the wire
@@ -261,7 +293,7 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
         }
         if (kProto == kTFF) {
             const uint32_t* xw = kFp8 ? reinterpret_cast<const uint32_t*>(qrow) : reinterpret_cast<const uint32_t*>(xrow);
-            for (int g = tid; g < sp.tff_blocks; g += kThreads) {
+            for (int g = sp.tff_blocks * part / parts + tid; g < sp.tff_blocks * (part + 1) / parts; g += kThreads) {
                 const int w0 = 3 * g;
                 uint4 blk;
                 blk.x = seq;   // the flag leads the block
@@ -275,7 +307,7 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
             }
         } else {
             unsigned long long mine = 0ull;
-            for (int v = tid; v < nvec; v += kThreads) {
+            for (int v = nvec * part / parts + tid; v < nvec * (part + 1) / parts; v += kThreads) {
                 const uint4 d = kFp8 ? reinterpret_cast<const uint4*>(qrow)[v] : xrow[v];
                 if (kProto == kDC && v < pvec && (v % kDcBlockVecs) < kDcMarkerVecs) mine += marker_words(d);
                 for (int j = 0; j < k; ++j) {
@@ -312,7 +344,7 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
             }
         }
         if (kFp8 || tl + 2 < ntok) __syncthreads();   // the quantised row and the row's buffer are used again
-        if (tid == 32 && tl + 2 < ntok) fetch_row(tl + 2);
+        if (tid == kFetcher && tl + 2 < ntok) fetch_row(tl + 2);
     }
     if (lost) report(p.status, kErrTimeout);
     if (kProto == kDC) {
@@ -325,7 +357,21 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
         }
     }
     if (tid == 0) times[2] = global_ns();
-    if (kProto == kTFF) __syncthreads();   // (the strips may lie where the rows were)
+    constexpr bool kByBlock = kProto == kTFF || kProto == kSP;   // receivers look at every block
+    if (kByBlock && warp == 0) {   // first[r]: rows of the regions before r
+        int run = 0;
+        for (int r0 = 0; r0 < R; r0 += 32) {
+            const int r = r0 + lane, n = r < R ? min(nrows[r], p.cap) : 0, incl = warp_incl_scan(n, lane);
+            if (r < R) first[r + 1] = run + incl;
+            run += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        if (lane == 0) first[0] = 0;
+    }
+    if (kByBlock) __syncthreads();   // (the strips may lie where the rows were)
+    if (kFew && warp >= kWarps / 2) {   // (see below)
+        for (int u = (warp - kWarps / 2) * p.grid + c; u < p.R * pl.duty_units; u += kWarps / 2 * p.grid)
+            write_table_unit<K>(p, ids16, u, pl.duty_units, p.dedup != 0, lane);
+    }
     if (kTable && warp >= kWarps / 2) {
         // counts and offsets nobody inside this kernel waits for (the launches before wrote them otherwise); behind the
         // rows, which the receivers wait for, and by half of the warps: the others turn to receiving at once
@@ -349,22 +395,26 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
         const size_t row_stride = kProto == kTFF ? wire_row : sp_row;
         const uint4 sentinel = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
         uint32_t* const mine = strips + (kProto == kTFF ? warp * kStripWords : 0);
-        long long all = 0;
-        for (int r = 0; r < R; ++r) all += nrows[r] < p.cap ? nrows[r] : p.cap;
-        const long long from = all * c / p.grid, to = all * (c + 1) / p.grid;   // this CTA's share
-        duty = to > from;
-        long long first = 0;   // rows of the regions before r
+        const int from = (int)((long long)first[R] * c / p.grid), to = (int)((long long)first[R] * (c + 1) / p.grid);
+        duty = to > from;   // this CTA's share
         bool ok = true;
-        for (int r = 0; r < R && first < to && ok; ++r) {
-            const int n_r = nrows[r] < p.cap ? nrows[r] : p.cap;
-            const int lo = (int)(from > first ? (from - first < n_r ? from - first : n_r) : 0);
-            const int hi = (int)(to - first < n_r ? to - first : n_r);
-            first += n_r;
-            for (int i = warp; ok && i < (hi - lo) * strips_per_row; i += kWarps) {
-                const int row = lo + i / strips_per_row, g0 = (i % strips_per_row) * kStrip;
-                const size_t grow = (size_t)r * p.cap + row;
-                uint8_t* const wire = (kProto == kTFF ? sp.tff_wire : sp.sp_wire) + grow * row_stride + (size_t)g0 * 16;
-                const int n = min(kStrip, per_row - g0);   // blocks of this strip
+        const int count = (to - from) * strips_per_row;
+        uint8_t* const wires = kProto == kTFF ? sp.tff_wire : sp.sp_wire;
+        struct Strip {
+            size_t grow;    // row of the receive regions
+            int g0, n;      // its blocks g0 .. g0 + n - 1
+        };
+        auto strip_at = [&](int i) -> Strip {
+            const int row = from + i / strips_per_row, g0 = (i % strips_per_row) * kStrip;
+            int r = -1;   // its region
+            for (int r0 = 0; r0 <= R; r0 += 32) r += __popc(__ballot_sync(0xffffffffu, r0 + lane <= R && first[r0 + lane] <= row));
+            return {(size_t)r * p.cap + (row - first[r]), g0, min(kStrip, per_row - g0)};
+        };
+        for (int i = warp; ok && i < count; i += kWarps) {
+                const Strip at = strip_at(i);
+                const size_t grow = at.grow;
+                const int g0 = at.g0, n = at.n;
+                uint8_t* const wire = wires + grow * row_stride + (size_t)g0 * 16;
                 uint4 blk[kBatch];
                 unsigned missing = 0u;   // bit b: this lane's b-th block has not arrived
 #pragma unroll
@@ -422,7 +472,6 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
                     }
                     __syncwarp();   // the strip's buffer is used again
                 }
-            }
         }
     }
     for (int u = c; u < R * Q; u += p.grid) {
@@ -481,11 +530,10 @@ __global__ void __launch_bounds__(256) sentinel_scan_kernel(const uint4* __restr
     if ((threadIdx.x & 31) == 0 && mine) atomicAdd(count, mine);
 }
 
-template <int kProto>
-cudaError_t launch_one(const Params& p, const SmemPlan& pl, const SyncParams& sp, bool whole_table, cudaStream_t st) {
-    auto kern = whole_table ? (p.payload ? sync_dispatch_kernel<kProto, true, true> : sync_dispatch_kernel<kProto, false, true>)
-                            : (p.payload ? sync_dispatch_kernel<kProto, true, false> : sync_dispatch_kernel<kProto, false, false>);
-    const int smem = pl.total + sync_extra_smem(p, kProto, sp.tff_strips != 0);
+template <int kProto, int kLayout>
+cudaError_t launch_one(const Params& p, const SmemPlan& pl, const SyncParams& sp, cudaStream_t st) {
+    auto kern = p.payload ? sync_dispatch_kernel<kProto, true, kLayout> : sync_dispatch_kernel<kProto, false, kLayout>;
+    const int smem = pl.total + sync_extra_smem(p, kProto, kLayout <= 0 && sp.tff_strips != 0);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     // Receivers wait for senders that are other CTAs of this grid: a cooperative launch, which the
@@ -503,20 +551,58 @@ cudaError_t launch_one(const Params& p, const SmemPlan& pl, const SyncParams& sp
     return cudaLaunchKernelEx(&cfg, kern, p, pl, sp);
 }
 
+template <int kProto>
+cudaError_t launch_layout(const Params& p, const SmemPlan& pl, const SyncParams& sp, int how, cudaStream_t st) {
+    if (how == kSyncLaunched) return launch_one<kProto, kLaunched>(p, pl, sp, st);
+    if (how == kSyncWhole) return launch_one<kProto, kWhole>(p, pl, sp, st);
+    if (p.k == 2) return launch_one<kProto, 2>(p, pl, sp, st);
+    if (p.k == 4) return launch_one<kProto, 4>(p, pl, sp, st);
+    return launch_one<kProto, 8>(p, pl, sp, st);
+}
+
 }  // namespace
+
+bool plan_sync_few(Params& p, int protocol, int max_smem, SmemPlan* out) {
+    if ((p.k != 2 && p.k != 4 && p.k != 8) || p.L > 32) return false;
+    // idle CTAs take a part of the rows (not with stop-and-wait, whose counters count rows)
+    while (protocol != kSW && p.T <= p.nchunks / 2 && p.nchunks % 2 == 0 && p.parts < 4) {
+        p.nchunks /= 2;
+        p.parts *= 2;
+    }
+    const int most = (p.T + p.nchunks - 1) / p.nchunks;
+    auto round_up = [](int64_t v, int m) { return (v + m - 1) / m * m; };
+    SmemPlan pl{};
+    const int64_t stage = round_up((int64_t)p.H * 2, 128), strips = protocol == kTFF ? kWarps * kStripWords * 4 : 0;
+    const int64_t ring = 2 * stage > strips ? 2 * stage : strips;   // (the Token-Flag strips lie where the rows were)
+    const int64_t at_pos = ring + round_up((int64_t)p.T * p.k * 2, 128), at_arr = at_pos + (int64_t)most * p.k * 4;
+    const int64_t total = round_up(at_arr + (int64_t)p.R * 4, 128);
+    if ((int64_t)most * p.k * p.T * (p.k + 8) > kFewWork || total + sync_extra_smem(p, protocol, false) + 1536 > max_smem) {
+        p.nchunks *= p.parts;
+        p.parts = 1;
+        return false;
+    }
+    pl.stages = 2;
+    pl.stage_bytes = (int)stage;
+    pl.off_ids = (int)ring;
+    pl.off_pos = (int)at_pos;
+    pl.off_arr = (int)at_arr;
+    pl.duty_units = table_units(p);
+    pl.total = (int)total;
+    *out = pl;
+    return true;
+}
 
 int sync_extra_smem(const Params& p, int protocol, bool strips) {
     const bool room = protocol == kTFF && strips && !strips_in_ring(p);
-    return p.R * 8 + 128 + qrow_bytes(p) + 16 + (room ? kWarps * kStripWords * 4 : 0);
+    return sync_qrow(p) + 128 + qrow_bytes(p) + 16 + (room ? kWarps * kStripWords * 4 : 0);
 }
 
-cudaError_t launch_sync_dispatch(const Params& p, const SmemPlan& pl, const SyncParams& sp, bool whole_table,
-                                 cudaStream_t st) {
+cudaError_t launch_sync_dispatch(const Params& p, const SmemPlan& pl, const SyncParams& sp, int how, cudaStream_t st) {
     switch (sp.protocol) {
-        case kSW: return launch_one<kSW>(p, pl, sp, whole_table, st);
-        case kTFF: return launch_one<kTFF>(p, pl, sp, whole_table, st);
-        case kDC: return launch_one<kDC>(p, pl, sp, whole_table, st);
-        case kSP: return launch_one<kSP>(p, pl, sp, whole_table, st);
+        case kSW: return launch_layout<kSW>(p, pl, sp, how, st);
+        case kTFF: return launch_layout<kTFF>(p, pl, sp, how, st);
+        case kDC: return launch_layout<kDC>(p, pl, sp, how, st);
+        case kSP: return launch_layout<kSP>(p, pl, sp, how, st);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -29,10 +29,12 @@ struct SyncParams {
 // Dynamic shared memory the kernel needs beyond the dispatch plan's total; with Token-Flag strips or without.
 int sync_extra_smem(const Params& p, int protocol, bool strips);
 
-// whole_table: every CTA derives the layout from the whole routing table in shared memory; otherwise the
-// count / prefix-sum launches (launch_count_scan) have run before over the same p.nchunks chunks.
-cudaError_t launch_sync_dispatch(const Params& p, const SmemPlan& pl, const SyncParams& sp, bool whole_table,
-                                 cudaStream_t st);
+// Where the layout comes from: the count / prefix-sum launches (launch_count_scan) that have run before over the same
+// p.nchunks chunks; the whole routing table, counted by every CTA; for small tables a warp per slot.
+constexpr int kSyncLaunched = 0, kSyncWhole = 1, kSyncFew = 2;
+cudaError_t launch_sync_dispatch(const Params& p, const SmemPlan& pl, const SyncParams& sp, int how, cudaStream_t st);
+// Whether the call is one of the last kind: the plan then, and p's chunks and parts (unchanged otherwise).
+bool plan_sync_few(Params& p, int protocol, int max_smem, SmemPlan* out);
 
 // Counts the 16-byte vectors of x that consist of 0xFFFF elements only.
 cudaError_t launch_sentinel_scan(const void* x, long long n_vec, unsigned long long* count, int num_sms,

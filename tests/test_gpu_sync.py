@@ -281,3 +281,19 @@ def test_one_captured_graph_of_all_protocols_replays_with_new_routing():
             Hn.check_dispatch(b, wl, lay, cap, recv, arrival=False)
             wire_checks(b, proto, cfg, lay, recv, b.sync_views["times"].shape[0])
             assert int(b.sync_views["seq"].item()) == 2 + it     # one warm-up call, then one per replay
+
+
+@pytest.mark.parametrize("proto", PROTOCOLS)
+@pytest.mark.parametrize("payload,dedup", [(0, 0), (1, 1)])
+@pytest.mark.parametrize("E,R,k,tokens", [(32, 1, 8, (1, 37, 38, 74, 256, 257)), (48, 48, 4, (75, 149, 445)), (20, 5, 2, (33, 656))])
+def test_a_warp_per_slot(E, R, k, tokens, payload, dedup, proto):
+    """Four, two and one CTAs per row, several tokens per CTA, around the line to the count of the whole table."""
+    for T in tokens:
+        cfg = W.Config("slots", T=T, H=640, E=E, R=R, k=k, payload=payload, dedup=dedup, seed=T + E, num_src_ranks=7)
+        wl = W.with_empty_slots(W.make_workload(cfg), 0.1, seed=T)
+        ids, lay, cap, recv = Hn.oracle_reference(wl)
+        buf = Hn.make_buffer(cfg, cap)
+        buf.attach_sync()
+        x, idx, w, _, _ = Hn.device_inputs(wl)
+        buf.dispatch_sync(proto, x, idx, w)
+        Hn.check_dispatch(buf, wl, lay, cap, recv, arrival=False)
