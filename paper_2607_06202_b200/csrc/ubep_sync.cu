@@ -411,67 +411,98 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
             return {(size_t)r * p.cap + (row - first[r]), g0, min(kStrip, per_row - g0)};
         };
         for (int i = warp; ok && i < count; i += kWarps) {
-                const Strip at = strip_at(i);
-                const size_t grow = at.grow;
-                const int g0 = at.g0, n = at.n;
-                uint8_t* const wire = wires + grow * row_stride + (size_t)g0 * 16;
-                uint4 blk[kBatch];
-                unsigned missing = 0u;   // bit b: this lane's b-th block has not arrived
+            const Strip at = strip_at(i);
+            const size_t grow = at.grow;
+            const int g0 = at.g0, n = at.n;
+            uint8_t* const wire = wires + grow * row_stride + (size_t)g0 * 16;
+            uint4 blk[kBatch];
+            unsigned missing = 0u;   // bit b: this lane's b-th block has not arrived
 #pragma unroll
-                for (int b = 0; b < kBatch; ++b) missing |= b * 32 + lane < n ? 1u << b : 0u;
-                unsigned spins = 0;
-                for (;;) {   // (all missing blocks side by side: one after the other a late strip cost eight round trips)
+            for (int b = 0; b < kBatch; ++b) missing |= b * 32 + lane < n ? 1u << b : 0u;
+            unsigned spins = 0;
+            for (;;) {   // (all missing blocks side by side: one after the other a late strip cost eight round trips)
 #pragma unroll
-                    for (int b = 0; b < kBatch; ++b)
-                        if (missing >> b & 1u) blk[b] = ld_relaxed_v4(wire + (size_t)(b * 32 + lane) * 16);
+                for (int b = 0; b < kBatch; ++b)
+                    if (missing >> b & 1u) blk[b] = ld_relaxed_v4(wire + (size_t)(b * 32 + lane) * 16);
 #pragma unroll
-                    for (int b = 0; b < kBatch; ++b)
-                        if ((missing >> b & 1u) && !(kProto == kTFF ? blk[b].x != seq : is_sentinel(blk[b]))) missing &= ~(1u << b);
-                    if (missing == 0u) break;
-                    if (!wt.keep_waiting(spins)) { ok = false; break; }
-                }
+                for (int b = 0; b < kBatch; ++b)
+                    if ((missing >> b & 1u) && !(kProto == kTFF ? blk[b].x != seq : is_sentinel(blk[b]))) missing &= ~(1u << b);
+                if (missing == 0u) break;
+                if (!wt.keep_waiting(spins)) { ok = false; break; }
+            }
+            ok = __all_sync(0xffffffffu, ok);
+            // Payload alone, as every strip of bf16 rows: few conditions, and what leaves leaves side by side.  (Token-Flag, 128 tokens of
+            // 7168 channels, from the last row sent to the last one confirmed 7.5 us with a condition per word, now 5.7.)
+            if (ok && (kProto != kTFF || sp.tff_strips) && (!kFp8 || (kProto == kTFF ? 3 * (g0 + n) <= pwords : g0 + n <= pvec))) {
+                uint4* const to16 = reinterpret_cast<uint4*>(p.recv_x + grow * p.rowB) + (kProto == kTFF ? g0 / 4 * 3 : g0);
+                if (kProto == kTFF) {
 #pragma unroll
-                for (int b = 0; b < kBatch; ++b) {
-                    const int g = b * 32 + lane;
-                    if (g >= n || (missing >> b & 1u)) continue;
-                    if (kProto == kTFF && !sp.tff_strips) {
-                        const uint32_t dw[3] = {blk[b].y, blk[b].z, blk[b].w};
-                        for (int q = 0; q < 3; ++q)
-                            if (3 * (g0 + g) + q < nwords) put_word(grow, 3 * (g0 + g) + q, dw[q]);
-                    } else if (kProto == kTFF) {
-                        mine[3 * g] = blk[b].y;
-                        mine[3 * g + 1] = blk[b].z;
-                        mine[3 * g + 2] = blk[b].w;
-                    } else {
-                        const int v = g0 + g;
-                        if (!kFp8 || v < pvec) {
-                            *reinterpret_cast<uint4*>(p.recv_x + grow * p.rowB + (size_t)v * 16) = blk[b];
-                        } else {
-                            const uint32_t dw[4] = {blk[b].x, blk[b].y, blk[b].z, blk[b].w};
-                            for (int q = 0; q < 4; ++q)
-                                if (4 * v + q < nwords) put_word(grow, 4 * v + q, dw[q]);
-                        }
-                        st_relaxed_v4(wire + (size_t)g * 16, sentinel);   // consumed: ready for the next call
+                    for (int b = 0; b < kBatch; ++b) {
+                        if (b * 32 + lane >= n) continue;
+                        mine[3 * (b * 32 + lane)] = blk[b].y;
+                        mine[3 * (b * 32 + lane) + 1] = blk[b].z;
+                        mine[3 * (b * 32 + lane) + 2] = blk[b].w;
                     }
-                }
-                ok = __all_sync(0xffffffffu, ok);
-                if (kProto == kTFF && sp.tff_strips) {
-                    __syncwarp();   // the lanes' words are in the strip (the vote orders no memory)
-                    // words [3 * g0, 3 * g0 + 3 * n) of the wire row (a strip begins on a multiple of four words)
-                    for (int q = lane; ok && q < kStripWords / 4; q += 32) {
-                        const int w = 3 * g0 + 4 * q;
-                        if (4 * q >= 3 * n || w >= nwords) break;
-                        const uint4 d = *reinterpret_cast<const uint4*>(mine + 4 * q);
-                        if (w + 4 <= pwords) {
-                            *reinterpret_cast<uint4*>(p.recv_x + grow * p.rowB + (size_t)w * 4) = d;
-                        } else {   // (scales; the words behind the row's last block are not written)
-                            const uint32_t dw[4] = {d.x, d.y, d.z, d.w};
-                            for (int z = 0; z < 4; ++z)
-                                if (w + z < nwords) put_word(grow, w + z, dw[z]);
-                        }
-                    }
+                    __syncwarp();
+                    const int n16 = min(3 * n, pwords - 3 * g0) / 4;   // (the words behind the row's last block are not written)
+#pragma unroll
+                    for (int q = 0; q < kBatch * 3 / 4; ++q)
+                        if (q * 32 + lane < n16) blk[q] = reinterpret_cast<const uint4*>(mine)[q * 32 + lane];
+#pragma unroll
+                    for (int q = 0; q < kBatch * 3 / 4; ++q)
+                        if (q * 32 + lane < n16) to16[q * 32 + lane] = blk[q];
                     __syncwarp();   // the strip's buffer is used again
+                } else {
+#pragma unroll
+                    for (int b = 0; b < kBatch; ++b) {
+                        if (b * 32 + lane >= n) continue;
+                        to16[b * 32 + lane] = blk[b];
+                        st_relaxed_v4(wire + (size_t)(b * 32 + lane) * 16, sentinel);   // consumed: ready for the next call
+                    }
                 }
+                continue;
+            }
+#pragma unroll
+            for (int b = 0; b < kBatch; ++b) {
+                const int g = b * 32 + lane;
+                if (g >= n || (missing >> b & 1u)) continue;
+                if (kProto == kTFF && !sp.tff_strips) {
+                    const uint32_t dw[3] = {blk[b].y, blk[b].z, blk[b].w};
+                    for (int q = 0; q < 3; ++q)
+                        if (3 * (g0 + g) + q < nwords) put_word(grow, 3 * (g0 + g) + q, dw[q]);
+                } else if (kProto == kTFF) {
+                    mine[3 * g] = blk[b].y;
+                    mine[3 * g + 1] = blk[b].z;
+                    mine[3 * g + 2] = blk[b].w;
+                } else {
+                    const int v = g0 + g;
+                    if (!kFp8 || v < pvec) {
+                        *reinterpret_cast<uint4*>(p.recv_x + grow * p.rowB + (size_t)v * 16) = blk[b];
+                    } else {
+                        const uint32_t dw[4] = {blk[b].x, blk[b].y, blk[b].z, blk[b].w};
+                        for (int q = 0; q < 4; ++q)
+                            if (4 * v + q < nwords) put_word(grow, 4 * v + q, dw[q]);
+                    }
+                    st_relaxed_v4(wire + (size_t)g * 16, sentinel);   // consumed: ready for the next call
+                }
+            }
+            if (kProto == kTFF && sp.tff_strips) {
+                __syncwarp();   // the lanes' words are in the strip (the vote orders no memory)
+                // words [3 * g0, 3 * g0 + 3 * n) of the wire row (a strip begins on a multiple of four words)
+                for (int q = lane; ok && q < kStripWords / 4; q += 32) {
+                    const int w = 3 * g0 + 4 * q;
+                    if (4 * q >= 3 * n || w >= nwords) break;
+                    const uint4 d = *reinterpret_cast<const uint4*>(mine + 4 * q);
+                    if (w + 4 <= pwords) {
+                        *reinterpret_cast<uint4*>(p.recv_x + grow * p.rowB + (size_t)w * 4) = d;
+                    } else {   // (scales; the words behind the row's last block are not written)
+                        const uint32_t dw[4] = {d.x, d.y, d.z, d.w};
+                        for (int z = 0; z < 4; ++z)
+                            if (w + z < nwords) put_word(grow, w + z, dw[z]);
+                    }
+                }
+                __syncwarp();   // the strip's buffer is used again
+            }
         }
     }
     for (int u = c; u < R * Q; u += p.grid) {
