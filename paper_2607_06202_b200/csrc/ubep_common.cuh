@@ -82,14 +82,14 @@ struct Params {
     unsigned* arrival;    // [2, R]
     // token stealing (large T): chunk c's tokens are handed out in blocks through cursor[c],
     // to its owner and, once pos_flag[c] holds the epoch, to CTAs that ran out of work
-    int steal;            // 1 = on
+    int steal;            // 1 = on: the last steal_tail(n) of a chunk's n tokens are handed out
     int quant_warps;      // FP8: warps that quantise at most (1 .. kWarps - 2)
     int count_warps;      // FP8 with flags or kernel boundaries: warps 1 .. count_warps compute the layout while the
                           // warps after them already quantise the rows the loader has fetched (0 = all 15 warps
                           // compute the layout and quantise afterwards)
     int prefetch_rows;    // FP8: rows the loader may fetch before the layout is done (the rings bound it as well)
     int32_t* copy_pos;    // [T, k] destinations in issue order (-1 = no copy), for thieves
-    unsigned* cursor;     // [nchunks] tokens of the chunk handed out so far
+    unsigned* cursor;     // [nchunks] tokens of the chunk's tail handed out so far
     unsigned* pos_flag;   // [nchunks] == epoch: copy_pos of the chunk is final
     unsigned* claimed;    // [2] tokens handed out in this dispatch (half = epoch & 1)
     int32_t* status;
@@ -108,6 +108,9 @@ __device__ __forceinline__ int src_begin(int s, int T, int S) {
     if ((int64_t)S * T < 0x7fffffffLL) return (int)((unsigned)s * (unsigned)T / (unsigned)S);  // the usual case
     return (int)((int64_t)s * T / S);
 }
+// Token stealing: how many tokens of a chunk of n are handed out through its cursor, the last ones; the ones before them are their
+// owner's, who needs no claim for them.  (CTA times differ by up to a fifth, so three eighths are more than change hands.)
+__host__ __device__ inline int steal_tail(int n) { return (3 * n + 7) / 8; }
 // Chunk that owns token b: the c with chunk_begin(c) <= b < chunk_begin(c + 1).
 __device__ __forceinline__ int chunk_of(int b, int T, int n) {
     return (int)((((int64_t)b + 1) * n - 1) / T);

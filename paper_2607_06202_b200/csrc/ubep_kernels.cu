@@ -185,19 +185,27 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
     unsigned pend = 0;                      // lane 0: answer of a claim made ahead of time
     bool pend_valid = false, feeder_done = false;
     int scanned = 0;                        // victims looked at so far
-    if (!kSteal) blk_hi = ntok;            // no stealing: the whole chunk, no atomics
+    blk_hi = kSteal ? ntok - steal_tail(ntok) : ntok;   // the chunk (without stealing), or what is handed out to nobody else: no claims
+    // (With a claim per two tokens from the first one on, a round trip to L2 each, the ring was not full when the movers were
+    // released: the first copy of 8192 tokens of 4096 channels left 4 us later.)
+    if (kSteal && ntok > 0) {
+        if (lane == 0) pend = atomicAdd(p.cursor + ch, (unsigned)kStealBlock);   // the first block of the tail, ahead of time
+        pend_valid = true;
+    }
+    const int q_tok = p.T / p.nchunks, q_more = p.T - q_tok * p.nchunks;   // (chunks have q_tok tokens, q_more of them one more)
+    const int tails = kSteal ? q_more * steal_tail(q_tok + 1) + (p.nchunks - q_more) * steal_tail(q_tok) : 0;
     auto pick_victim = [&]() -> int {
         while (scanned < p.nchunks - 1) {
             unsigned done = 0;
             if (lane == 0) done = __ldcg(p.claimed + (epoch & 1));
-            if ((int)__shfl_sync(0xffffffffu, done, 0) >= p.T) return -1;   // every token is handed out
+            if ((int)__shfl_sync(0xffffffffu, done, 0) >= tails) return -1;   // every tail is handed out
             const int idx = scanned + lane;
             int cand = ch + 1 + idx;
             if (cand >= p.nchunks) cand -= p.nchunks;
             int rem = 0;
             if (idx < p.nchunks - 1 && ld_acquire(p.pos_flag + cand) == epoch) {
                 const int nt = (int)chunk_begin(cand + 1, p.T, p.nchunks) - (int)chunk_begin(cand, p.T, p.nchunks);
-                rem = nt - (int)__ldcg(p.cursor + cand);
+                rem = steal_tail(nt) - (int)__ldcg(p.cursor + cand);
             }
             int best = rem > 0 ? (rem << 9) | cand : 0;   // most remaining tokens first (cand < 512)
 #pragma unroll
@@ -227,9 +235,10 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
             if (!pend_valid && lane == 0) pend = atomicAdd(p.cursor + v, (unsigned)kStealBlock);
             const int old = (int)__shfl_sync(0xffffffffu, pend, 0);
             pend_valid = false;
-            if (old < v_ntok) {
-                blk_lo = old;
-                blk_hi = min(old + kStealBlock, v_ntok);
+            const int v_tail = steal_tail(v_ntok);
+            if (old < v_tail) {
+                blk_lo = v_ntok - v_tail + old;
+                blk_hi = min(blk_lo + kStealBlock, v_ntok);
                 if (lane == 0) {
                     atomicAdd(p.claimed + (epoch & 1), (unsigned)(blk_hi - blk_lo));
                     pend = atomicAdd(p.cursor + v, (unsigned)kStealBlock);   // answer needed a block later
@@ -277,6 +286,19 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
         }
         head += n;
     };
+    // The same with stealing, for tokens that are handed out to nobody else.
+    auto issue_own = [&](int n) {
+        if (lane < n) {
+            const int tl = blk_lo + lane, s = (head + lane) % stages;
+            item_src[s] = (ch << 16) | tl;
+            mbar_arrive_expect_tx(&full_bar[s], in_bytes);
+            bulk_load(smem + (size_t)s * pl.stage_bytes,
+                      reinterpret_cast<const uint8_t*>(p.x) + (size_t)(t0 + tl) * p.H * 2 + in_off, in_bytes, &full_bar[s]);
+        }
+        __syncwarp();
+        head += n;
+        blk_lo += n;
+    };
     // Rows fetched before the layout is done.  With flags the layout takes many microseconds in which a
     // few small loads and stores of every CTA wait on one another; a ring-full of rows per CTA fetched
     // meanwhile fills the memory system's queues in front of them.  Three rows start the copies, the
@@ -306,7 +328,7 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
             // Two rows at once, the rest of the ring when the counts have been exchanged: a ring-full of rows per
             // CTA in flight slows the reads of the other CTAs' shared memory down (by 2 us at 1537 tokens).
             if (kSteal) {
-                while (head < 2 && next_token(tl, false) == 1) issue_item(tl);
+                issue_own(min(2, blk_hi));
             } else {
                 issue_first(max(min(2, min(ahead, ntok)), 0));
             }
@@ -317,6 +339,7 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
             ok = __all_sync(0xffffffffu, ok);
         }
         if (kSteal) {
+            issue_own(max(min(min(ahead, early) - head, min(blk_hi - blk_lo, 32)), 0));
             while (head < min(ahead, early) && next_token(tl, false) == 1) issue_item(tl);
         } else {
             issue_first(max(min(min(min(ahead, early), ntok), 32) - head, 0));
@@ -407,10 +430,9 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
             group_sync(2, kThreads);
             if (lane == 0) epoch_ctr = ld_relaxed(p.epoch_ctr);
         } else if (kMode == kModeCluster) {
-            if (!kSteal) {   // (see above)
-                issue_first(min(min(2, p.prefetch_rows), min(stages, ntok)));
-                issued = head;
-            }
+            if (kSteal) issue_own(min(min(2, p.prefetch_rows), min(stages, blk_hi)));   // (see above)
+            else issue_first(min(min(2, p.prefetch_rows), min(stages, ntok)));
+            issued = head;
             cluster_wait();
             cluster_arrive();
             ok = mbar_wait(x.staged_bar, 0, abortp);
@@ -618,11 +640,15 @@ __device__ __forceinline__ void cluster_layout(Cta& x) {
         trace(p, c, kTrReady);
     }
     if (kSteal) {
-        // this chunk's destinations, for CTAs that run out of work and take over some of its tokens
-        for (int i = gtid; i < ntok * p.k; i += gn) p.copy_pos[(size_t)t0 * p.k + i] = pos[i];
-        if (gtid == 0) (void)mbar_wait(x.epoch_bar, 0, abortp);
-        group_sync(bid, gn);
-        if (gtid == 0) st_release(p.pos_flag + ch, *reinterpret_cast<volatile unsigned*>(x.epoch_late));
+        // this chunk's destinations, for CTAs that run out of work and take over some of its tokens (FP8 rows: not by the warp
+        // that issues the copies, whose first one left 2 us later)
+        constexpr int s0 = kFp8 ? 1 : 0, sbar = kFp8 ? 3 : 1;
+        if (gw < s0) return;
+        const int st = gtid - s0 * 32, sn = gn - s0 * 32;
+        for (int i = st; i < ntok * p.k; i += sn) p.copy_pos[(size_t)t0 * p.k + i] = pos[i];
+        if (st == 0) (void)mbar_wait(x.epoch_bar, 0, abortp);
+        group_sync(sbar, sn);
+        if (st == 0) st_release(p.pos_flag + ch, *reinterpret_cast<volatile unsigned*>(x.epoch_late));
     }
 }
 

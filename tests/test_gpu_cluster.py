@@ -103,3 +103,11 @@ def test_short_fp8_rows_whose_ring_is_used_more_than_once(cfg):
 def test_around_the_line_between_short_and_long_fp8_rows(H, T):
     for dedup in (0, 1):
         _run(W.Config("l", T=T, H=H, E=64, R=8, k=8, payload=1, dedup=dedup, seed=H + T))
+
+
+@pytest.mark.parametrize("H,payload", [(2048, 0), (5120, 1)])
+@pytest.mark.parametrize("T", [4800, 4801, 5919, 6100])
+def test_where_tails_of_the_slices_are_handed_out(T, H, payload):
+    """Slices of 40 tokens and a few more, some of them one longer than others, on 120 CTAs: heads without claims, tails with."""
+    for dedup in (0, 1):
+        _run(W.Config("tail", T=T, H=H, E=32, R=4, k=8, payload=payload, dedup=dedup, seed=T), num_ctas=120)
