@@ -342,9 +342,10 @@ int choose_schedule(Params& p, int pipeline, int n, int count_warps, int max_sme
         split_work(p, n);
         if (ubep::plan_few(p, max_smem, pl)) return ubep::kModeFew;
         // (In halves of rows a CTA has more tokens than warps.  Two whole rows instead are worth it where every bin has to be
-        // counted otherwise, or more ranks than a word has bits: dispatch + combine of 185 tokens of 7168 channels, top-8, bf16
-        // 15.7 -> 14.8 us, of 4096 channels 12.5 -> 10.9; 72 ranks, one row per (token, rank) 18.6 -> 15.7.)
-        if (p.parts > 1 && (!p.dedup || p.R > 32)) {
+        // counted otherwise, or more ranks than a word has bits, or rows are short: dispatch + combine of 185 tokens of 7168
+        // channels, top-8, bf16 15.7 -> 14.8 us, of 4096 channels 12.5 -> 10.9; one row per (token, rank) with 72 ranks 18.6 -> 15.7,
+        // with 16 ranks 5120 channels 12.0 -> 11.4, 4096 11.4 -> 10.5; but 7168 channels on 32 ranks 14.1 and about 15.)
+        if (p.parts > 1 && (!p.dedup || p.R > 32 || p.H * 2 <= 10240)) {
             cut(p, n, 1);
             if (ubep::plan_few(p, max_smem, pl)) return ubep::kModeFew;
         }

@@ -45,7 +45,7 @@ def _run(T, H, E, R, k, payload, dedup, empty=0.0, **kw):
 @pytest.mark.parametrize("payload,dedup", [(0, 0), (1, 0), (0, 1), (1, 1)])
 @pytest.mark.parametrize("H,E,R,k,tokens", [
     (7168, 256, 32, 8, (1, 2, 19, 37, 75, 148, 149, 256)),   # eight, four, two column parts, whole rows, two tokens per CTA
-    (128, 32, 1, 8, (1, 31, 32, 33, 256, 257)),              # every expert on one rank: all bits of a word
+    (128, 32, 1, 8, (1, 31, 32, 33, 160, 256, 257)),              # every expert on one rank: all bits of a word
     (640, 96, 96, 6, (5, 148, 296)),                         # one expert per rank; scales that no bulk copy can carry
     (1024, 32, 8, 4, (3, 149, 444, 445)),
     (256, 16, 4, 2, (64, 148, 297, 655, 656)),
