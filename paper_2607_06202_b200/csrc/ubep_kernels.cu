@@ -1856,6 +1856,7 @@ cudaError_t launch_combine(const uint16_t* y, const int32_t* slot_pos, const flo
         case 1: return launch_combine_k<1>(ahead, g, st, y, slot_pos, topk_w, T, H, k, out);
         case 2: return launch_combine_k<2>(ahead, g, st, y, slot_pos, topk_w, T, H, k, out);
         case 4: return launch_combine_k<4>(ahead, g, st, y, slot_pos, topk_w, T, H, k, out);
+        case 6: return launch_combine_k<6>(ahead, g, st, y, slot_pos, topk_w, T, H, k, out);
         case 8: return launch_combine_k<8>(ahead, g, st, y, slot_pos, topk_w, T, H, k, out);
         default: return launch_combine_k<0>(ahead, g, st, y, slot_pos, topk_w, T, H, k, out);
     }
