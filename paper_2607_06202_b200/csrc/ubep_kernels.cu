@@ -11,6 +11,7 @@
 //                                     rows.  Clusters (ubep_cluster.cuh): the CTAs of a cluster
 //                                     count the table between them; a cluster of one for small
 //                                     tables with one row per (token, expert).
+//                                     (Small batches: ubep_few.cu.)
 //   combine_kernel<K>                 gather + fp32 weighted sum + one bf16 rounding
 //   layout_kernel<K>                  counts only (ubep_get_dispatch_layout)
 #include <type_traits>
@@ -1891,7 +1892,8 @@ cudaError_t launch_layout(const Params& p, int32_t* num_tokens_per_rank, int32_t
                           uint8_t* is_token_in_rank, int32_t* acc, int acc_words, unsigned* ticket, cudaStream_t st) {
     const bool tile = p.R <= kLayoutTileRanks;
     const int counts = (p.B + 3) / 4 * 16;
-    const bool cluster = p.T <= kLayoutClusterTokens && counts <= 48 * 1024;
+    if (p.B * 4 > 48 * 1024) return cudaErrorInvalidValue;   // (the counts of some twelve thousand bins at most)
+    const bool cluster = p.T <= kLayoutClusterTokens;
     const int threads = cluster ? kThreads : kLayoutThreads;
     // a token per thread; beyond one cluster (two CTAs per SM) a thread takes several
     int64_t blocks = ((int64_t)p.T + threads - 1) / threads;
