@@ -290,7 +290,7 @@ int ubep_map_workers(const int32_t *order /*[dev]*/, const int32_t *counts /*[de
  * payload.  What arrives goes to the region's payload and scale arrays.
  *
  * Routing tables of any size: up to 8192 slots (T * k) every CTA derives the layout from the whole
- * table, as UBEP_PIPELINE_LOCAL does (one launch); for a larger table the counting and prefix-sum
+ * table (one launch), for small ones a warp per slot of the CTA's tokens; for a larger table the counting and prefix-sum
  * kernels of UBEP_PIPELINE_PHASED run in front of the protocol kernel (three launches).  One CTA per SM at most, launched
  * cooperatively (receivers wait for senders of the same grid, so the grid must be resident at once:
  * a grid that cannot be is refused with UBEP_ERR_CUDA instead of running into its timeouts).  Everything
