@@ -1827,26 +1827,38 @@ cudaError_t launch_dispatch(const Params& p, int mode, const SmemPlan& pl, cudaS
     return launch_dispatch_t<kModeFused>(p, pl, st);
 }
 
+// Both kinds of calls are placed while their predecessor still runs (and wait for its end before they read anything).  A large
+// one asks for as much L1 as there is: its gathers land there, and beside a dispatch or behind one whose division of the SM it
+// inherits, with most of it shared memory, it takes a quarter longer (prefill 80 -> 102 us).  So it is placed only where that
+// division can be changed, SM by SM as the dispatch's CTAs leave, not behind the last of them: dispatch + combine of 1537 tokens of 4096
+// channels, top-8 43.9 -> 43.3 us against an ordinary launch, 2500 tokens of 2048 channels, top-4 26.2 -> 25.7, 4096 of 7168, FP8, 148.8 ->
+// 147.9; placed ahead without asking 46.0, 26.6 and 169.6.  Small calls don't wait for it: 128 tokens of 256 channels 4.6 us, 5.4 with it.
 template <int K, bool kStream>
-static cudaError_t launch_combine_s(bool ahead, int g, cudaStream_t st, const uint16_t* y, const int32_t* slot_pos,
+static cudaError_t launch_combine_s(bool small, int g, cudaStream_t st, const uint16_t* y, const int32_t* slot_pos,
                                     const float* topk_w, int T, int H, int k, uint16_t* out) {
-    if (ahead) return launch_overlapped(combine_kernel<K, kStream>, g, 256, 0, st, false, 1, y, slot_pos, topk_w, T, H, k, out);
-    combine_kernel<K, kStream><<<g, 256, 0, st>>>(y, slot_pos, topk_w, T, H, k, out);
-    return cudaGetLastError();
+    if (small) return launch_overlapped(combine_kernel<K, kStream>, g, 256, 0, st, false, 1, y, slot_pos, topk_w, T, H, k, out);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)g);
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[1].val.sharedMemCarveout = cudaSharedmemCarveoutMaxL1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, combine_kernel<K, kStream>, y, slot_pos, topk_w, T, H, k, out);
 }
 template <int K>
-static cudaError_t launch_combine_k(bool ahead, int g, cudaStream_t st, const uint16_t* y, const int32_t* slot_pos,
+static cudaError_t launch_combine_k(bool small, int g, cudaStream_t st, const uint16_t* y, const int32_t* slot_pos,
                                     const float* topk_w, int T, int H, int k, uint16_t* out) {
-    if ((int64_t)T * k * H * 2 <= kStreamMaxBytes) return launch_combine_s<K, true>(ahead, g, st, y, slot_pos, topk_w, T, H, k, out);
-    return launch_combine_s<K, false>(ahead, g, st, y, slot_pos, topk_w, T, H, k, out);
+    if ((int64_t)T * k * H * 2 <= kStreamMaxBytes) return launch_combine_s<K, true>(small, g, st, y, slot_pos, topk_w, T, H, k, out);
+    return launch_combine_s<K, false>(small, g, st, y, slot_pos, topk_w, T, H, k, out);
 }
 
-// `ahead`: let the kernel be placed while its predecessor in the stream still runs (it waits for the
-// predecessor's end before it reads anything).  Worth 0.4 us per layer beside the short decode-sized
-// dispatch; beside a long dispatch the parked CTAs were measured to slow it down by far more than the
-// launch latency they hide, so the caller asks for it only for small T.
 cudaError_t launch_combine(const uint16_t* y, const int32_t* slot_pos, const float* topk_w, int T, int H, int k,
-                           uint16_t* out, int num_sms, bool ahead, cudaStream_t st) {
+                           uint16_t* out, int num_sms, bool small, cudaStream_t st) {
     const int64_t total = (int64_t)T * (H / 8);
     int64_t blocks = (total + 255) / 256;
     const int64_t cap = (int64_t)num_sms * 8;
@@ -1854,12 +1866,12 @@ cudaError_t launch_combine(const uint16_t* y, const int32_t* slot_pos, const flo
     if (blocks < 1) blocks = 1;
     const int g = (int)blocks;
     switch (k) {
-        case 1: return launch_combine_k<1>(ahead, g, st, y, slot_pos, topk_w, T, H, k, out);
-        case 2: return launch_combine_k<2>(ahead, g, st, y, slot_pos, topk_w, T, H, k, out);
-        case 4: return launch_combine_k<4>(ahead, g, st, y, slot_pos, topk_w, T, H, k, out);
-        case 6: return launch_combine_k<6>(ahead, g, st, y, slot_pos, topk_w, T, H, k, out);
-        case 8: return launch_combine_k<8>(ahead, g, st, y, slot_pos, topk_w, T, H, k, out);
-        default: return launch_combine_k<0>(ahead, g, st, y, slot_pos, topk_w, T, H, k, out);
+        case 1: return launch_combine_k<1>(small, g, st, y, slot_pos, topk_w, T, H, k, out);
+        case 2: return launch_combine_k<2>(small, g, st, y, slot_pos, topk_w, T, H, k, out);
+        case 4: return launch_combine_k<4>(small, g, st, y, slot_pos, topk_w, T, H, k, out);
+        case 6: return launch_combine_k<6>(small, g, st, y, slot_pos, topk_w, T, H, k, out);
+        case 8: return launch_combine_k<8>(small, g, st, y, slot_pos, topk_w, T, H, k, out);
+        default: return launch_combine_k<0>(small, g, st, y, slot_pos, topk_w, T, H, k, out);
     }
 }
 

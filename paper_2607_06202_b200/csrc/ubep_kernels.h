@@ -21,7 +21,7 @@ cudaError_t launch_few(const Params& p, const SmemPlan& pl, cudaStream_t st);
 cudaError_t launch_count_scan(const Params& p, const SmemPlan& pl, cudaStream_t st);
 cudaError_t launch_dispatch(const Params& p, int mode, const SmemPlan& pl, cudaStream_t st, int* launches);
 cudaError_t launch_combine(const uint16_t* y, const int32_t* slot_pos, const float* topk_w, int T, int H, int k,
-                           uint16_t* out, int num_sms, bool ahead, cudaStream_t st);
+                           uint16_t* out, int num_sms, bool small, cudaStream_t st);
 cudaError_t launch_empty(int num_sms, bool ahead, cudaStream_t st);
 // acc: acc_words words (p.B at least) and the ticket word, all zero between calls (the kernel leaves them so, also where
 // calls that share them overlapped).
