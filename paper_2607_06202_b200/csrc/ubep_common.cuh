@@ -332,6 +332,12 @@ struct SmemPlan {
 // a kernel launched the ordinary way.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// What such a kernel reads of its predecessors' and the caller's memory: by plain loads behind griddep_wait(), not through
+// the read-only path (ld.global.nc: __ldg, or const __restrict__ parameters), which asks for memory that nobody writes while the
+// kernel lives.  The kernel lives while the dispatch in front of it still writes its handle, and while a caller's kernel that lets
+// its dependents start early still writes a table or an expert's output.
+template <typename T>
+__device__ __forceinline__ T ld_plain(const T* p) { return *p; }
 
 // Barrier among a subset of the CTA's warps (id 1..15), `nthreads` a multiple of 32.
 __device__ __forceinline__ void group_sync(int id, int nthreads) {

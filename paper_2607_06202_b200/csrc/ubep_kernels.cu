@@ -1372,21 +1372,22 @@ __global__ void __launch_bounds__((kDispatchThreads<kMode, kRows>), 1) dispatch_
 constexpr int64_t kStreamMaxBytes = 384ll << 20;
 template <bool kStream>
 __device__ __forceinline__ uint4 load_row16(const uint4* a) {
-    if (!kStream) return __ldg(a);
-    uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(a));
+    uint4 v;   // (plain loads: see ld_plain)
+    if (!kStream) {
+        asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(a));
+        return v;
+    }
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(a));
     return v;
 }
 template <int K, bool kStream>
-__global__ void __launch_bounds__(256) combine_kernel(const uint16_t* __restrict__ y,
-                                                     const int32_t* __restrict__ slot_pos,
-                                                     const float* __restrict__ topk_w, int T, int H, int k,
-                                                     uint16_t* __restrict__ out) {
+__global__ void __launch_bounds__(256) combine_kernel(const uint16_t* y, const int32_t* slot_pos, const float* topk_w,
+                                                     int T, int H, int k, uint16_t* __restrict__ out) {
     const int nvec = H / 8;
     const int64_t total = (int64_t)T * nvec;
     const int kk = K > 0 ? K : k;
     griddep_launch();   // lets a dispatch that follows in the stream be placed while this kernel drains
-    griddep_wait();     // (only matters when this kernel itself was launched ahead of its predecessor's end)
+    griddep_wait();
     for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < total;
          u += (int64_t)gridDim.x * blockDim.x) {
         // (small calls: no 64-bit division and no scalar loads in front of the first row; in large ones, 16384 tokens, the
@@ -1404,19 +1405,19 @@ __global__ void __launch_bounds__(256) combine_kernel(const uint16_t* __restrict
             if (kStream && KK % 4 == 0) {   // (both arrays start on 16-byte boundaries)
 #pragma unroll
                 for (int j = 0; j + 3 < KK; j += 4) {
-                    const int4 a = __ldg(reinterpret_cast<const int4*>(slot_pos + (size_t)t * KK + j));
+                    const int4 a = ld_plain(reinterpret_cast<const int4*>(slot_pos + (size_t)t * KK + j));
                     wh[j] = a.x; wh[j + 1] = a.y; wh[j + 2] = a.z; wh[j + 3] = a.w;
                 }
 #pragma unroll
                 for (int j = 0; j + 3 < KK; j += 4) {
-                    const float4 b = __ldg(reinterpret_cast<const float4*>(topk_w + (size_t)t * KK + j));
+                    const float4 b = ld_plain(reinterpret_cast<const float4*>(topk_w + (size_t)t * KK + j));
                     w[j] = b.x; w[j + 1] = b.y; w[j + 2] = b.z; w[j + 3] = b.w;
                 }
             } else {
 #pragma unroll
                 for (int j = 0; j < KK; ++j) {
-                    wh[j] = __ldg(slot_pos + (size_t)t * KK + j);
-                    w[j] = __ldg(topk_w + (size_t)t * KK + j);
+                    wh[j] = ld_plain(slot_pos + (size_t)t * KK + j);
+                    w[j] = ld_plain(topk_w + (size_t)t * KK + j);
                 }
             }
 #pragma unroll
@@ -1436,9 +1437,9 @@ __global__ void __launch_bounds__(256) combine_kernel(const uint16_t* __restrict
             }
         } else {
             for (int j = 0; j < kk; ++j) {
-                const int where = __ldg(slot_pos + (size_t)t * kk + j);
+                const int where = ld_plain(slot_pos + (size_t)t * kk + j);
                 if (where < 0) continue;
-                const float w = __ldg(topk_w + (size_t)t * kk + j);
+                const float w = ld_plain(topk_w + (size_t)t * kk + j);
                 const uint4 q = load_row16<kStream>(reinterpret_cast<const uint4*>(y + (size_t)where * H) + v);
                 const uint32_t ww[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll

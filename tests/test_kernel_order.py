@@ -30,3 +30,15 @@ def test_a_chunks_cursor_is_reset_before_its_destinations_are_released():
     mover = mover[mover.index("void mover_warp("):mover.index("constexpr int kClusterCountWarps")]
     _in_order(mover, "cursor[x.ch] = 0", "mbar_arrive(x.epoch_bar)")
     assert mover.count("cursor[ch] = 0") + mover.count("cursor[x.ch] = 0") == 1
+
+
+def test_the_combine_reads_what_its_predecessors_write_with_plain_loads():
+    # (it is launched ahead of their end; the read-only path asks for memory that nobody writes while the kernel lives, which
+    # the compiler may also assume of const pointers declared __restrict__)
+    text = _source("ubep_kernels.cu")
+    combine = text[text.index("load_row16(const uint4* a)"):text.index("constexpr int kLayoutThreads")]
+    assert "__ldg" not in combine and ".nc." not in combine
+    head = combine[combine.index("combine_kernel("):]
+    head = head[:head.index("{")]
+    assert head.count("__restrict__") == 1 and "uint16_t* __restrict__ out" in head
+    _in_order(combine, "griddep_wait();", "slot_pos + ", "load_row16<kStream>")
