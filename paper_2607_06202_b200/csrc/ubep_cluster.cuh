@@ -46,8 +46,8 @@ static __device__ __noinline__ int modulo(int a, int b) { return a % b; }   // (
 __device__ __forceinline__ int counted_expert(const CountArgs& p, int t, int raw, int slot) {
     int e = raw;
     if (p.phys != nullptr) {
-        const int nc = (unsigned)e < (unsigned)p.E_log ? __ldg(p.ncopies + e) : 0;
-        e = nc >= 1 && nc <= p.C ? __ldg(p.phys + (size_t)e * p.C + modulo(t, nc)) : -1;
+        const int nc = (unsigned)e < (unsigned)p.E_log ? ld_plain(p.ncopies + e) : 0;
+        e = nc >= 1 && nc <= p.C ? ld_plain(p.phys + (size_t)e * p.C + modulo(t, nc)) : -1;
     }
     return (unsigned)e < (unsigned)p.E ? e : -1 - slot;
 }
@@ -70,8 +70,8 @@ static __device__ __noinline__ void count_tokens(const CountArgs p, int lo, int 
         const int4* src = reinterpret_cast<const int4*>(p.topk_idx + (size_t)t * k);
         a = b = make_int4(-1, -1, -1, -1);
         if (t < hi) {
-            a = __ldg(src);
-            if (k == 8) b = __ldg(src + 1);
+            a = ld_plain(src);
+            if (k == 8) b = ld_plain(src + 1);
         }
     };
     int4 na, nb;
@@ -86,7 +86,7 @@ static __device__ __noinline__ void count_tokens(const CountArgs p, int lo, int 
                 bool many = false;
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    nc[j] = (unsigned)e[j] < (unsigned)p.E_log ? __ldg(p.ncopies + e[j]) : 0;
+                    nc[j] = (unsigned)e[j] < (unsigned)p.E_log ? ld_plain(p.ncopies + e[j]) : 0;
                     many = many || nc[j] > 2;
                 }
                 if (many) {
@@ -100,7 +100,7 @@ static __device__ __noinline__ void count_tokens(const CountArgs p, int lo, int 
                 } else {
 #pragma unroll
                     for (int j = 0; j < 8; ++j)
-                        e[j] = nc[j] >= 1 && nc[j] <= p.C ? __ldg(p.phys + (size_t)e[j] * p.C + (nc[j] == 2 ? t & 1 : 0)) : -1;
+                        e[j] = nc[j] >= 1 && nc[j] <= p.C ? ld_plain(p.phys + (size_t)e[j] * p.C + (nc[j] == 2 ? t & 1 : 0)) : -1;
                 }
             }
             bool twice = false;
@@ -140,7 +140,7 @@ static __device__ __noinline__ void count_tokens(const CountArgs p, int lo, int 
             int e[kMaxTopk];
 #pragma unroll 1
             for (int j = 0; j < k; ++j) {
-                int v = counted_expert(p, t, __ldg(src + j), j);
+                int v = counted_expert(p, t, ld_plain(src + j), j);
 #pragma unroll 1
                 for (int i = 0; i < j; ++i)
                     if (e[i] == v) v = -1 - j;
@@ -169,7 +169,7 @@ __device__ __forceinline__ bool stage_own(const Params& p, int t0, int t1, int* 
 #pragma unroll 1
     for (int i = tid; i < nslots; i += n) {
         const int tl = i / p.k;
-        const int v = pack_slot(p, (size_t)t0 * p.k + i, __ldg(p.topk_idx + (size_t)t0 * p.k + i), bad);
+        const int v = pack_slot(p, (size_t)t0 * p.k + i, ld_plain(p.topk_idx + (size_t)t0 * p.k + i), bad);
         ids[i] = v;
         if (v >= 0) {
             const unsigned bit = 1u << (tl & 31);

@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(kThreads, 1) few_kernel(const Params p, const 
     // this warp's slot, if it has one: slot j of own token tl
     const int tl = warp / K, j = warp % K, t = t0 + tl;
     const bool slot = tl < ntok;
-    const float w_i = slot && lane < K ? __ldg(p.topk_w + (size_t)t * K + lane) : 0.0f;   // the token's gate weights, a lane each
+    const float w_i = slot && lane < K ? ld_plain(p.topk_w + (size_t)t * K + lane) : 0.0f;   // the token's gate weights, a lane each
     __syncthreads();
     if (tid == 0) trace(p, c, kTrCounted);
     unsigned ticket = 0u;

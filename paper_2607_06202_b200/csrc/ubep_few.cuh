@@ -62,17 +62,17 @@ __device__ __forceinline__ bool stage_table(const Params& p, uint16_t* ids, int 
     for (int i = tid; i < p.T * (K / kV); i += n) {
         const int t = i / (K / kV);
         if (kV == 4) {
-            const int4 v = __ldg(reinterpret_cast<const int4*>(p.topk_idx) + i);
+            const int4 v = ld_plain(reinterpret_cast<const int4*>(p.topk_idx) + i);
             int e[4] = {v.x, v.y, v.z, v.w};
             resolve_slots(p, t, e, bad);
             reinterpret_cast<uint2*>(ids)[i] = make_uint2(pack16(e[0], e[1]), pack16(e[2], e[3]));
         } else if (kV == 2) {
-            const int2 v = __ldg(reinterpret_cast<const int2*>(p.topk_idx) + i);
+            const int2 v = ld_plain(reinterpret_cast<const int2*>(p.topk_idx) + i);
             int e[2] = {v.x, v.y};
             resolve_slots(p, t, e, bad);
             reinterpret_cast<unsigned*>(ids)[i] = pack16(e[0], e[1]);
         } else {
-            int e[1] = {__ldg(p.topk_idx + i)};
+            int e[1] = {ld_plain(p.topk_idx + i)};
             resolve_slots(p, t, e, bad);
             ids[i] = (uint16_t)e[0];
         }
@@ -92,12 +92,12 @@ __device__ __forceinline__ bool stage_tokens(const Params& p, uint16_t* ids, int
         if (K % 4 == 0) {
 #pragma unroll
             for (int j = 0; j < K / 4; ++j) {
-                const int4 v = __ldg(reinterpret_cast<const int4*>(p.topk_idx) + t * (K / 4) + j);
+                const int4 v = ld_plain(reinterpret_cast<const int4*>(p.topk_idx) + t * (K / 4) + j);
                 e[4 * j] = v.x; e[4 * j + 1] = v.y; e[4 * j + 2] = v.z; e[4 * j + 3] = v.w;
             }
         } else {
 #pragma unroll
-            for (int j = 0; j < K; ++j) e[j] = __ldg(p.topk_idx + t * K + j);
+            for (int j = 0; j < K; ++j) e[j] = ld_plain(p.topk_idx + t * K + j);
         }
         resolve_slots(p, t, e, bad);
 #pragma unroll

@@ -520,7 +520,7 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
         if (ok) {
             float* w_own = reinterpret_cast<float*>(key);   // the ordering keys are no longer needed
             if (part == 0)
-                for (int i = lane; i < ntok * p.k; i += 32) w_own[i] = __ldg(p.topk_w + (size_t)t0 * p.k + i);
+                for (int i = lane; i < ntok * p.k; i += 32) w_own[i] = ld_plain(p.topk_w + (size_t)t0 * p.k + i);
             local_clean_own_duplicates(p, t0, t1, ids_sm, lane, 32);
             __syncwarp();
             if (part == 0) local_meta_dedup(p, t0, t1, ids_sm, pos_raw, reinterpret_cast<int*>(w_sm), w_own, lane, 32);
@@ -569,7 +569,7 @@ __device__ __forceinline__ void cluster_layout(Cta& x) {
     const bool twice = stage_own(p, t0, t1, ids_sm, bmaps.bm, bmaps.bp, own, an - 1 - gtid, an);
     count_tokens(count_args(p), lo, hi, first, ranks, cnt, gtid, an);
     if (p.ordered)
-        for (int r = gtid; r < p.R; r += an) order_sm[r] = __ldg(p.order_pos + r);
+        for (int r = gtid; r < p.R; r += an) order_sm[r] = ld_plain(p.order_pos + r);
     if (group_or(1, an, twice)) {
         local_clean_own_duplicates(p, 0, ntok, ids_sm, gtid, an);
         group_sync(1, an);
@@ -681,11 +681,11 @@ __device__ __forceinline__ void cluster_duty(Cta& x, int dtid, int dn, int bar) 
         if (where < 0) continue;
         p.recv_src_idx[where] = t0 + tl;
         if (!p.dedup) {
-            p.recv_weight[where] = __ldg(p.topk_w + i);
+            p.recv_weight[where] = ld_plain(p.topk_w + i);
         } else if ((p.k & 3) == 0) {   // rows of the two arrays start on 16-byte boundaries: four slots per store
 #pragma unroll 1
             for (int j = 0; j < p.k; j += 4) {
-                const float4 w = __ldg(reinterpret_cast<const float4*>(p.topk_w + (size_t)(t0 + tl) * p.k + j));
+                const float4 w = ld_plain(reinterpret_cast<const float4*>(p.topk_w + (size_t)(t0 + tl) * p.k + j));
                 const float wv[4] = {w.x, w.y, w.z, w.w};
                 int e4[4];
                 float w4[4];
@@ -705,7 +705,7 @@ __device__ __forceinline__ void cluster_duty(Cta& x, int dtid, int dn, int bar) 
                 const int v = ids_sm[tl * p.k + j];
                 const bool here = v >= 0 && slot_rank(v) == r;
                 p.recv_topk_idx[(size_t)where * p.k + j] = here ? slot_expert(v) - r * p.L : -1;
-                p.recv_topk_w[(size_t)where * p.k + j] = here ? __ldg(p.topk_w + (size_t)(t0 + tl) * p.k + j) : 0.0f;
+                p.recv_topk_w[(size_t)where * p.k + j] = here ? ld_plain(p.topk_w + (size_t)(t0 + tl) * p.k + j) : 0.0f;
             }
         }
     }
@@ -726,15 +726,15 @@ __device__ __forceinline__ int layout_group(Cta& x) {
     const int* ids = ids_sm;  // staged slots of this CTA's tokens
     // Small global reads whose values are needed only after the first barriers: issue the
     // loads now (first trip of each loop), store to shared memory after the ids are staged.
-    const int order_r = kMode != kModeCluster && gtid < p.R ? __ldg(p.order_pos + gtid) : 0;
+    const int order_r = kMode != kModeCluster && gtid < p.R ? ld_plain(p.order_pos + gtid) : 0;
     const bool stage_w = kMode != kModeCluster && kMode != kModeLocal;
-    const float w_first = (stage_w && gtid < ntok * p.k) ? __ldg(p.topk_w + (size_t)t0 * p.k + gtid) : 0.0f;
+    const float w_first = (stage_w && gtid < ntok * p.k) ? ld_plain(p.topk_w + (size_t)t0 * p.k + gtid) : 0.0f;
     auto stage_small = [&](int n) {   // by n threads
         if (gtid < p.R) order_sm[gtid] = order_r;
-        for (int r = gtid + n; r < p.R; r += n) order_sm[r] = __ldg(p.order_pos + r);
+        for (int r = gtid + n; r < p.R; r += n) order_sm[r] = ld_plain(p.order_pos + r);
         if (stage_w) {
             if (gtid < ntok * p.k) w_sm[gtid] = w_first;
-            for (int i = gtid + n; i < ntok * p.k; i += n) w_sm[i] = __ldg(p.topk_w + (size_t)t0 * p.k + i);
+            for (int i = gtid + n; i < ntok * p.k; i += n) w_sm[i] = ld_plain(p.topk_w + (size_t)t0 * p.k + i);
         }
     };
     if (kMode == kModeLocal) {
@@ -742,7 +742,7 @@ __device__ __forceinline__ int layout_group(Cta& x) {
         const RankMaps rm{bmaps.bm, bmaps.mask_t, (p.R + 31) / 32, ((p.R + 31) / 32) * 32, (p.T + 31) / 32};
         int* row_sm = reinterpret_cast<int*>(w_sm);
         // (the own tokens' gate weights, asked for while the table is on its way; needed for the metadata)
-        const float w_row = !kFp8 && part == 0 && gw < kRowWarps && gtid < ntok * p.k ? __ldg(p.topk_w + (size_t)t0 * p.k + gtid) : 0.0f;
+        const float w_row = !kFp8 && part == 0 && gw < kRowWarps && gtid < ntok * p.k ? ld_plain(p.topk_w + (size_t)t0 * p.k + gtid) : 0.0f;
         local_stage_and_rank_maps(p, ids_sm, rm, rm.groups, warp, kWarps, lane);   // with the mover warp
         stage_small(gn);
         group_sync(2, kThreads);
@@ -799,7 +799,7 @@ __device__ __forceinline__ int layout_group(Cta& x) {
             if (part == 0) {
                 float* w_own = reinterpret_cast<float*>(key);   // the ordering keys are no longer needed
                 if (gtid < ntok * p.k) w_own[gtid] = w_row;
-                for (int i = gtid + rn; i < ntok * p.k; i += rn) w_own[i] = __ldg(p.topk_w + (size_t)t0 * p.k + i);
+                for (int i = gtid + rn; i < ntok * p.k; i += rn) w_own[i] = ld_plain(p.topk_w + (size_t)t0 * p.k + i);
             }
             local_clean_own_duplicates(p, t0, t1, ids_sm, gtid, rn);   // (rank-level rows do not depend on them)
             group_sync(1, rn);
@@ -1507,12 +1507,12 @@ __global__ void __launch_bounds__(kCluster ? kThreads : kLayoutThreads) layout_k
             if (kK % 4 == 0 && kK > 0) {
 #pragma unroll
                 for (int j = 0; j < kSlots; j += 4) {
-                    const int4 v = __ldg(reinterpret_cast<const int4*>(src + j));
+                    const int4 v = ld_plain(reinterpret_cast<const int4*>(src + j));
                     e[j] = v.x; e[j + 1] = v.y; e[j + 2] = v.z; e[j + 3] = v.w;
                 }
             } else {
 #pragma unroll kUnroll
-                for (int j = 0; j < k; ++j) e[j] = __ldg(src + j);
+                for (int j = 0; j < k; ++j) e[j] = ld_plain(src + j);
             }
             uint8_t* mine = !flags ? nullptr : kTile ? tile + lane * R : out + (size_t)lane * R;
             if (!kTile && flags)

@@ -25,9 +25,9 @@ __device__ __forceinline__ int resolve_expert(const Params& p, int t, int raw, b
     int e = raw;
     if (p.phys != nullptr) {
         if (raw < 0 || raw >= p.E_log) { bad = true; return -1; }
-        int nc = __ldg(p.ncopies + raw);
+        int nc = ld_plain(p.ncopies + raw);
         if (nc < 1 || nc > p.C) { bad = true; return -1; }
-        e = __ldg(p.phys + (size_t)raw * p.C + (t % nc));
+        e = ld_plain(p.phys + (size_t)raw * p.C + (t % nc));
     }
     if (e < 0 || e >= p.E) { bad = true; return -1; }
     return e;
@@ -49,14 +49,14 @@ __device__ __forceinline__ void resolve_slots(const Params& p, int t, int (&e)[k
         for (int i = 0; i < kN; ++i) {
             const bool in = (unsigned)e[i] < (unsigned)p.E_log;
             bad |= !in && e[i] != -1;
-            nc[i] = in ? __ldg(p.ncopies + e[i]) : 0;
+            nc[i] = in ? ld_plain(p.ncopies + e[i]) : 0;
         }
 #pragma unroll
         for (int i = 0; i < kN; ++i) {
             const bool in = (unsigned)e[i] < (unsigned)p.E_log, ok = nc[i] >= 1 && nc[i] <= p.C;
             bad |= in && !ok;
             const int copy = nc[i] > 2 ? t % nc[i] : nc[i] == 2 ? t & 1 : 0;
-            e[i] = ok ? __ldg(p.phys + (size_t)e[i] * p.C + copy) : -1;
+            e[i] = ok ? ld_plain(p.phys + (size_t)e[i] * p.C + copy) : -1;
             bad |= ok && e[i] < 0;
         }
     }
@@ -101,11 +101,11 @@ __device__ __forceinline__ int pack_slot(const Params& p, size_t slot, int raw, 
     if (p.phys != nullptr) {
         const bool in = (unsigned)e < (unsigned)p.E_log;
         bad |= !in && e != -1;
-        const int nc = in ? __ldg(p.ncopies + e) : 1;
+        const int nc = in ? ld_plain(p.ncopies + e) : 1;
         const bool okc = in && nc >= 1 && nc <= p.C;
         bad |= in && !okc;
         const int t = (int)((unsigned)slot / (unsigned)p.k);   // (the table has fewer than 2^31 slots)
-        e = okc ? __ldg(p.phys + (size_t)e * p.C + (t % nc)) : -1;
+        e = okc ? ld_plain(p.phys + (size_t)e * p.C + (t % nc)) : -1;
         bad |= okc && e < 0;
     }
     const bool valid = (unsigned)e < (unsigned)p.E;
@@ -130,7 +130,7 @@ __device__ __forceinline__ void stage_ids(const Params& p, int t0, int t1, int* 
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int i = i0 + u * nthreads;
-                raw[u] = i < n4 ? __ldg(src4 + i) : make_int4(-1, -1, -1, -1);
+                raw[u] = i < n4 ? ld_plain(src4 + i) : make_int4(-1, -1, -1, -1);
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -149,7 +149,7 @@ __device__ __forceinline__ void stage_ids(const Params& p, int t0, int t1, int* 
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const int i = i0 + u * nthreads;
-                raw[u] = i < n ? __ldg(src + i) : -1;
+                raw[u] = i < n ? ld_plain(src + i) : -1;
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
@@ -558,13 +558,13 @@ __device__ __forceinline__ void stage_and_rank_maps_pass(const Params& p, int* i
             for (int j0 = 0; j0 < k; j0 += 8) {       // up to eight ids in flight
                 int raw[8];
                 if (vec) {
-                    const int4 a = __ldg(reinterpret_cast<const int4*>(src + j0));
-                    const int4 b = j0 + 4 < k ? __ldg(reinterpret_cast<const int4*>(src + j0 + 4)) : make_int4(-1, -1, -1, -1);
+                    const int4 a = ld_plain(reinterpret_cast<const int4*>(src + j0));
+                    const int4 b = j0 + 4 < k ? ld_plain(reinterpret_cast<const int4*>(src + j0 + 4)) : make_int4(-1, -1, -1, -1);
                     raw[0] = a.x; raw[1] = a.y; raw[2] = a.z; raw[3] = a.w;
                     raw[4] = b.x; raw[5] = b.y; raw[6] = b.z; raw[7] = b.w;
                 } else {
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) raw[u] = j0 + u < k ? __ldg(src + j0 + u) : -1;
+                    for (int u = 0; u < 8; ++u) raw[u] = j0 + u < k ? ld_plain(src + j0 + u) : -1;
                 }
                 int pk[8];
 #pragma unroll
@@ -573,10 +573,10 @@ __device__ __forceinline__ void stage_and_rank_maps_pass(const Params& p, int* i
                     if (!kPlain && p.phys != nullptr) {
                         const bool in = (unsigned)e < (unsigned)p.E_log;
                         bad |= !in && e != -1;
-                        const int nc = in ? __ldg(p.ncopies + e) : 1;
+                        const int nc = in ? ld_plain(p.ncopies + e) : 1;
                         const bool okc = in && nc >= 1 && nc <= p.C;
                         bad |= in && !okc;
-                        e = okc ? __ldg(p.phys + (size_t)e * p.C + (t % nc)) : -1;
+                        e = okc ? ld_plain(p.phys + (size_t)e * p.C + (t % nc)) : -1;
                         bad |= okc && e < 0;
                     }
                     const bool valid = (unsigned)e < (unsigned)p.E;

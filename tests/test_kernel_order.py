@@ -42,3 +42,10 @@ def test_the_combine_reads_what_its_predecessors_write_with_plain_loads():
     head = head[:head.index("{")]
     assert head.count("__restrict__") == 1 and "uint16_t* __restrict__ out" in head
     _in_order(combine, "griddep_wait();", "slot_pos + ", "load_row16<kStream>")
+
+
+def test_kernels_launched_ahead_read_with_plain_loads():
+    # (a caller's kernel that lets its dependents start early may still be writing the routing table or the replica table)
+    for name in ("ubep_common.cuh", "ubep_layout.cuh", "ubep_cluster.cuh", "ubep_few.cuh", "ubep_few.cu", "ubep_kernels.cu"):
+        text = _source(name)
+        assert "__ldg" not in text and ".nc." not in text, name
