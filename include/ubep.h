@@ -493,6 +493,21 @@ int ubep_debug_plan(const ubep_config_t *cfg, int32_t T, int32_t max_smem, const
                     int32_t quant_warps, int32_t plan[UBEP_DEBUG_PLAN_COUNT_]);
 
 /*
+ * The same for ubep_dispatch_sync with protocol UBEP_SYNC_*; ctas: CTAs that can run at once.
+ */
+enum {
+    UBEP_DEBUG_SYNC_PLAN_LAYOUT = 0, /* 0 = counted by launches of their own, 1 = the whole table by every CTA,
+                                        2 = a warp per slot of the CTA's tokens                  */
+    UBEP_DEBUG_SYNC_PLAN_CHUNKS,     /* token chunks ...                                         */
+    UBEP_DEBUG_SYNC_PLAN_PARTS,      /* ... times CTAs that share a chunk's rows                 */
+    UBEP_DEBUG_SYNC_PLAN_STRIPS,     /* 0 = Token-Flag receivers store word by word              */
+    UBEP_DEBUG_SYNC_PLAN_SMEM,       /* dynamic shared memory of the kernel                      */
+    UBEP_DEBUG_SYNC_PLAN_COUNT_
+};
+int ubep_debug_sync_plan(const ubep_config_t *cfg, int protocol, int32_t T, int32_t max_smem, int32_t ctas,
+                         int32_t plan[UBEP_DEBUG_SYNC_PLAN_COUNT_]);
+
+/*
  * Measurement aid: launches a kernel that does nothing (one small CTA per SM) on `cuda_stream`,
  * the ordinary way or, with ahead != 0, with programmatic stream serialization like the dispatch
  * and the small-batch combine kernels.  Timed in a chain it gives the floor that every kernel

@@ -380,6 +380,43 @@ int choose_schedule(Params& p, int pipeline, int n, int count_warps, int max_sme
     return mode;
 }
 
+// Where the layout of a readiness-protocol dispatch comes from (kSync...): fills in p's chunks and parts, the plan, and whether
+// Token-Flag receivers have strips (tables of ten thousand experts leave no 48 KB for them); or an error code.  Small tables are
+// recounted by every CTA; for larger ones TokenCnt and CalCumSum run as launches of their own in front of the kernel, over the
+// same chunks (as the phased schedule of ubep_dispatch does).
+int choose_sync_layout(Params& p, int protocol, int max_smem, ubep::SmemPlan* pl, bool* strips) {
+    p.parts = 1;
+    p.grid = p.nchunks;
+    *strips = true;
+    if (ubep::plan_sync_few(p, protocol, max_smem, pl)) return ubep::kSyncFew;
+    for (;; *strips = false) {
+        const int room = max_smem - ubep::sync_extra_smem(p, protocol, *strips);
+        if ((int64_t)p.T * p.k <= kLocalMaxSlots && ubep::plan_dispatch(p, ubep::kModeCluster, room, pl) == 0)   // (a cluster of one)
+            return ubep::kSyncWhole;
+        if (ubep::plan_dispatch(p, UBEP_PIPELINE_PHASED, room, pl) == 0) return ubep::kSyncLaunched;
+        if (!*strips) return UBEP_ERR_ARG;
+    }
+}
+
+// CTAs of a buffer's kernels where `most` can run at once.
+int ctas_used(const ubep_config_t& c, int most) {
+    const int n = c.num_ctas > 0 && c.num_ctas < most ? c.num_ctas : most;
+    return n < ubep::kMaxChunks ? n : ubep::kMaxChunks;
+}
+// A buffer without a device, for plans that look at sizes only.
+ubep_buffer sizes_only(const ubep_config_t& c, int n) {
+    ubep_buffer b{};
+    b.cfg = c;
+    b.lay = make_layout(c, n);
+    b.arena = reinterpret_cast<uint8_t*>(kAlign);
+    b.sm_khz = 1;
+    b.quant_warps = ubep::kWarps - 2;
+    b.count_warps = -1;
+    b.prefetch_rows = INT32_MAX;
+    b.my_rank = -1;
+    return b;
+}
+
 // Makes the buffer's device current for the scope of one call.
 struct DeviceGuard {
     int prev = -1;
@@ -612,21 +649,10 @@ int ubep_dispatch_sync(ubep_buffer_t* buf, int protocol, const void* x, const in
     p.topk_idx = topk_idx;
     p.topk_w = topk_w;
     p.trace = nullptr;
-    p.parts = 1;
-    p.grid = p.nchunks;
     ubep::SmemPlan pl{};
-    // Small tables are recounted by every CTA; for larger ones TokenCnt and CalCumSum run as launches of their
-    // own in front of the kernel, over the same chunks (as the phased schedule of ubep_dispatch does).
-    bool whole_table = false;
-    auto fits = [&](bool strips) {
-        const int room = buf->max_smem - ubep::sync_extra_smem(p, protocol, strips);
-        whole_table = (int64_t)T * buf->cfg.topk <= kLocalMaxSlots &&
-                      ubep::plan_dispatch(p, ubep::kModeCluster, room, &pl) == 0;   // (a cluster of one)
-        return whole_table || ubep::plan_dispatch(p, UBEP_PIPELINE_PHASED, room, &pl) == 0;
-    };
-    const bool few = ubep::plan_sync_few(p, protocol, buf->max_smem, &pl);
-    const bool strips = few || fits(true);
-    if (!strips && !fits(false)) return UBEP_ERR_ARG;   // (tables of ten thousand experts leave no 48 KB for the strips)
+    bool strips = true;
+    const int how = choose_sync_layout(p, protocol, buf->max_smem, &pl, &strips);
+    if (how < 0) return how;
     const WireLayout& w = buf->wlay;
     ubep::SyncParams sp{};
     sp.protocol = protocol;
@@ -652,12 +678,12 @@ int ubep_dispatch_sync(ubep_buffer_t* buf, int protocol, const void* x, const in
         if (e != cudaSuccess) return cuda_fail(buf, e);
         buf->sp_dirty = false;
     }
-    if (!few && !whole_table) {
+    if (how == ubep::kSyncLaunched) {
         e = ubep::launch_count_scan(p, pl, st);
         if (e != cudaSuccess) return cuda_fail(buf, e);
         g_launches += 2;
     }
-    e = ubep::launch_sync_dispatch(p, pl, sp, few ? ubep::kSyncFew : whole_table ? ubep::kSyncWhole : ubep::kSyncLaunched, st);
+    e = ubep::launch_sync_dispatch(p, pl, sp, how, st);
     if (e != cudaSuccess) return cuda_fail(buf, e);
     g_launches += 1;
     return UBEP_OK;
@@ -910,18 +936,11 @@ int ubep_debug_plan(const ubep_config_t* cfg, int32_t T, int32_t max_smem, const
                     int32_t quant_warps, int32_t plan[UBEP_DEBUG_PLAN_COUNT_]) {
     if (!cfg || !valid_config(*cfg) || !ctas || !plan || T < 1 || T > cfg->max_tokens) return UBEP_ERR_ARG;
     if (count_warps < -1 || count_warps > ubep::kWarps - 3 || quant_warps < 1 || quant_warps > ubep::kWarps - 2) return UBEP_ERR_ARG;
-    int n = cfg->num_ctas > 0 && cfg->num_ctas < ctas[0] ? cfg->num_ctas : ctas[0];
-    if (n > ubep::kMaxChunks) n = ubep::kMaxChunks;
+    const int n = ctas_used(*cfg, ctas[0]);
     if (n < 1) return UBEP_ERR_ARG;
-    ubep_buffer b{};   // (no device behind it: only sizes are looked at)
-    b.cfg = *cfg;
-    b.lay = make_layout(*cfg, n);
-    b.arena = reinterpret_cast<uint8_t*>(kAlign);
-    b.sm_khz = 1;
+    ubep_buffer b = sizes_only(*cfg, n);
     b.quant_warps = quant_warps;
     b.count_warps = count_warps;
-    b.prefetch_rows = INT32_MAX;
-    b.my_rank = -1;
     Params p = make_params(&b, T);
     ubep::SmemPlan pl{};
     const int mode = choose_schedule(p, cfg->pipeline, n, count_warps, max_smem,
@@ -938,6 +957,26 @@ int ubep_debug_plan(const ubep_config_t* cfg, int32_t T, int32_t max_smem, const
     plan[UBEP_DEBUG_PLAN_TEAMS] = pl.q_teams;
     plan[UBEP_DEBUG_PLAN_TEAM_WARPS] = pl.q_team_warps;
     plan[UBEP_DEBUG_PLAN_SMEM] = ubep::with_room_beside(pl.total, mode == ubep::kModeFew ? 0 : ubep::kLeastStatic);
+    return UBEP_OK;
+}
+
+int ubep_debug_sync_plan(const ubep_config_t* cfg, int protocol, int32_t T, int32_t max_smem, int32_t ctas,
+                         int32_t plan[UBEP_DEBUG_SYNC_PLAN_COUNT_]) {
+    if (!cfg || !valid_config(*cfg) || !plan || T < 1 || T > cfg->max_tokens) return UBEP_ERR_ARG;
+    if (protocol < UBEP_SYNC_SW || protocol > UBEP_SYNC_SP) return UBEP_ERR_ARG;
+    const int n = ctas_used(*cfg, ctas);
+    if (n < 1) return UBEP_ERR_ARG;
+    ubep_buffer b = sizes_only(*cfg, n);
+    Params p = make_params(&b, T);
+    ubep::SmemPlan pl{};
+    bool strips = true;
+    const int how = choose_sync_layout(p, protocol, max_smem, &pl, &strips);
+    if (how < 0) return how;
+    plan[UBEP_DEBUG_SYNC_PLAN_LAYOUT] = how;
+    plan[UBEP_DEBUG_SYNC_PLAN_CHUNKS] = p.nchunks;
+    plan[UBEP_DEBUG_SYNC_PLAN_PARTS] = p.parts;
+    plan[UBEP_DEBUG_SYNC_PLAN_STRIPS] = strips ? 1 : 0;
+    plan[UBEP_DEBUG_SYNC_PLAN_SMEM] = pl.total + ubep::sync_extra_smem(p, protocol, how != ubep::kSyncFew && strips);
     return UBEP_OK;
 }
 

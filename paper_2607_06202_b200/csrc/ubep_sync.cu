@@ -95,9 +95,9 @@ __device__ __forceinline__ bool wait_count(const unsigned* ctr, unsigned want, W
     return true;
 }
 
-// Behind the plan: checksums [R] of 8 bytes, the regions' first rows [R + 1], the quantised row.
-__host__ __device__ inline int sync_first(const Params& p) { return p.R * 8; }
-__host__ __device__ inline int sync_qrow(const Params& p) { return (sync_first(p) + (p.R + 1) * 4 + 15) / 16 * 16; }
+// Behind the plan: checksums [R] of 8 bytes or, with the protocols that have none, the regions' first rows [R + 1] (one or the
+// other: with both there was no room for tables that had been taken, of 5200 ranks for instance); the quantised row.
+__host__ __device__ inline int sync_qrow(const Params& p) { return (p.R * 8 + 15) / 16 * 16; }
 __host__ __device__ inline int qrow_bytes(const Params& p) { return p.payload ? ((p.H + 4 * p.G + 15) / 16) * 16 : 0; }
 __host__ __device__ inline bool strips_in_ring(const Params& p) {   // (a plan has four rows at least, two for FP8 rows)
     return (p.payload ? 2 : 4) * 2 * p.H >= kWarps * kStripWords * 4;
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(kThreads, 1) sync_dispatch_kernel(const Params
     float* w_sm = reinterpret_cast<float*>(smem + pl.off_w);
     int* hist = reinterpret_cast<int*>(smem + pl.off_hist);
     int* nrows = reinterpret_cast<int*>(smem + pl.off_arr);     // rows every region receives
-    int* first = reinterpret_cast<int*>(smem + pl.total + sync_first(p));   // [R + 1] (Token-Flag and Sentinel receivers)
+    int* first = reinterpret_cast<int*>(smem + pl.total);   // Token-Flag and Sentinel receivers: [R + 1]
     int* order_sm = reinterpret_cast<int*>(smem + pl.off_order);
     unsigned long long* chk_sm = reinterpret_cast<unsigned long long*>(smem + pl.total);   // DC: [R]
     uint8_t* qrow = smem + pl.total + sync_qrow(p);                                         // FP8: the quantised row
@@ -625,7 +625,7 @@ bool plan_sync_few(Params& p, int protocol, int max_smem, SmemPlan* out) {
 
 int sync_extra_smem(const Params& p, int protocol, bool strips) {
     const bool room = protocol == kTFF && strips && !strips_in_ring(p);
-    return sync_qrow(p) + 128 + qrow_bytes(p) + 16 + (room ? kWarps * kStripWords * 4 : 0);
+    return p.R * 8 + 128 + qrow_bytes(p) + 16 + (room ? kWarps * kStripWords * 4 : 0);
 }
 
 cudaError_t launch_sync_dispatch(const Params& p, const SmemPlan& pl, const SyncParams& sp, int how, cudaStream_t st) {

@@ -297,3 +297,18 @@ def test_a_warp_per_slot(E, R, k, tokens, payload, dedup, proto):
         x, idx, w, _, _ = Hn.device_inputs(wl)
         buf.dispatch_sync(proto, x, idx, w)
         Hn.check_dispatch(buf, wl, lay, cap, recv, arrival=False)
+
+
+@pytest.mark.parametrize("proto", PROTOCOLS)
+def test_the_most_ranks_whose_counts_fit(proto):
+    cfg = W.Config("many_ranks", T=3000, H=256, E=5600, R=5600, k=4, seed=21, num_src_ranks=3)
+    wl = W.make_workload(cfg)
+    _, lay, cap, recv = Hn.oracle_reference(wl, cap=16)
+    assert lay.num_rows_per_rank.max() <= cap
+    buf = Hn.make_buffer(cfg, cap)
+    buf.attach_sync()
+    x, idx, w, _, _ = Hn.device_inputs(wl)
+    for _ in range(2):
+        buf.recv_x.fill_(Hn.FILL)
+        buf.dispatch_sync(proto, x, idx, w)
+        Hn.check_dispatch(buf, wl, lay, cap, recv, arrival=False)

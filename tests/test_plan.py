@@ -79,3 +79,12 @@ def test_a_combine_cta_fits_beside_a_small_dispatch(payload):
             need = pl["smem"] + static + 1024
             size = next(s for s in sizes if s >= need)
             assert size - need >= 1024 or size == sizes[-1], (H, T, E, R, k, pl, static)
+
+
+@pytest.mark.parametrize("protocol", ["sw", "tff", "dc", "sp"])
+def test_protocol_calls_that_were_taken_before_the_receivers_prefix_sums_are_still_taken(protocol):
+    """The regions' first rows, which two of the protocols need, take no room from the plan."""
+    for E in (5200, 5600):   # the largest tables of one expert per rank that had fitted
+        cfg = B.ubep_config_t(E, E, 256, 4, 3000, 128, 0, 0, 0, 0, 0, 0)
+        pl = B.ubep_debug_sync_plan(cfg, protocol, 3000, SMEM, CTAS[0])
+        assert pl["smem"] <= SMEM and pl["layout"] == B.UBEP_SYNC_LAYOUT_LAUNCHED
