@@ -491,6 +491,8 @@ enum {
 };
 int ubep_debug_plan(const ubep_config_t *cfg, int32_t T, int32_t max_smem, const int32_t ctas[4], int32_t count_warps,
                     int32_t quant_warps, int32_t plan[UBEP_DEBUG_PLAN_COUNT_]);
+/* The same for an existing buffer, on its device and with everything that has been set for it. */
+int ubep_debug_buffer_plan(ubep_buffer_t *buf, int32_t T, int32_t plan[UBEP_DEBUG_PLAN_COUNT_]);
 
 /*
  * The same for ubep_dispatch_sync with protocol UBEP_SYNC_*; ctas: CTAs that can run at once.

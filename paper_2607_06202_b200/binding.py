@@ -45,7 +45,7 @@ EXPORTS = ["ubep_buffer_bytes", "ubep_buffer_create", "ubep_buffer_destroy", "ub
            "ubep_set_dest_order", "ubep_get_dispatch_layout", "ubep_get_dispatch_layout_static", "ubep_dispatch", "ubep_combine", "ubep_view",
            "ubep_status", "ubep_epoch", "ubep_launch_count", "ubep_debug_withhold_flag", "ubep_debug_trace",
            "ubep_debug_set_quant_warps", "ubep_debug_set_count_warps", "ubep_debug_set_prefetch_rows", "ubep_debug_empty_launch", "ubep_debug_plan",
-           "ubep_debug_sync_plan",
+           "ubep_debug_buffer_plan", "ubep_debug_sync_plan",
            "ubep_last_cuda_error", "ubep_strerror", "ubep_map_workers",
            "ubep_sync_wire_bytes", "ubep_sync_attach", "ubep_dispatch_sync", "ubep_sync_view",
            "ubep_sync_scan_sentinel",
@@ -95,6 +95,7 @@ def load() -> ctypes.CDLL:
     lib.ubep_debug_set_prefetch_rows.restype, lib.ubep_debug_set_prefetch_rows.argtypes = ctypes.c_int, [vp, i32]
     lib.ubep_debug_plan.restype = ctypes.c_int
     lib.ubep_debug_plan.argtypes = [ctypes.POINTER(ubep_config_t), i32, i32, ctypes.POINTER(i32), i32, i32, ctypes.POINTER(i32)]
+    lib.ubep_debug_buffer_plan.restype, lib.ubep_debug_buffer_plan.argtypes = ctypes.c_int, [vp, i32, ctypes.POINTER(i32)]
     lib.ubep_debug_sync_plan.restype = ctypes.c_int
     lib.ubep_debug_sync_plan.argtypes = [ctypes.POINTER(ubep_config_t), ctypes.c_int, i32, i32, i32, ctypes.POINTER(i32)]
     lib.ubep_debug_empty_launch.restype, lib.ubep_debug_empty_launch.argtypes = ctypes.c_int, [vp, i32, vp]
@@ -289,6 +290,13 @@ def ubep_debug_plan(cfg: ubep_config_t, T: int, max_smem: int, ctas, count_warps
     plan = (ctypes.c_int32 * len(PLAN_NAMES))()
     _check(load().ubep_debug_plan(ctypes.byref(cfg), T, max_smem, (ctypes.c_int32 * 4)(*ctas), count_warps, quant_warps,
                                   plan), "ubep_debug_plan")
+    return dict(zip(PLAN_NAMES, plan))
+
+
+def ubep_debug_buffer_plan(buf, T: int) -> dict:
+    """The same for an existing buffer, with everything that has been set for it."""
+    plan = (ctypes.c_int32 * len(PLAN_NAMES))()
+    _check(load().ubep_debug_buffer_plan(buf, T, plan), "ubep_debug_buffer_plan", buf)
     return dict(zip(PLAN_NAMES, plan))
 
 

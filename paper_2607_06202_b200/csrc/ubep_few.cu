@@ -197,6 +197,7 @@ bool plan_few(const Params& p, int max_smem, SmemPlan* out) {
     if (most * p.k > kWarps || (int64_t)most * p.k * p.T * (p.k + 8) > kFewWork || p.L > 32 || p.ordered) return false;
     if (p.k != 1 && p.k != 2 && p.k != 4 && p.k != 6 && p.k != 8) return false;
     if (p.payload && p.quant_warps < kWarps - 2) return false;   // (fewer quantising warps were asked for)
+    if (p.payload && p.prefetch_rows < most) return false;       // (rows to be fetched behind the layout; here all are at once)
     SmemPlan pl{};
     auto round_up = [](int64_t v, int m) { return (v + m - 1) / m * m; };
     const int64_t stage = round_up((int64_t)p.H * 2 / p.parts, 128);

@@ -417,6 +417,20 @@ ubep_buffer sizes_only(const ubep_config_t& c, int n) {
     return b;
 }
 
+void fill_plan(const Params& p, const ubep::SmemPlan& pl, int mode, int32_t* plan) {
+    plan[UBEP_DEBUG_PLAN_MODE] = mode;
+    plan[UBEP_DEBUG_PLAN_CHUNKS] = p.nchunks;
+    plan[UBEP_DEBUG_PLAN_PARTS] = p.parts;
+    plan[UBEP_DEBUG_PLAN_CLUSTER] = p.cluster;
+    plan[UBEP_DEBUG_PLAN_STEAL] = p.steal;
+    plan[UBEP_DEBUG_PLAN_STAGES] = pl.stages;
+    plan[UBEP_DEBUG_PLAN_OUT_STAGES] = pl.out_stages;
+    plan[UBEP_DEBUG_PLAN_LONG_ROWS] = pl.q_long;
+    plan[UBEP_DEBUG_PLAN_TEAMS] = pl.q_teams;
+    plan[UBEP_DEBUG_PLAN_TEAM_WARPS] = pl.q_team_warps;
+    plan[UBEP_DEBUG_PLAN_SMEM] = ubep::with_room_beside(pl.total, mode == ubep::kModeFew ? 0 : ubep::kLeastStatic);
+}
+
 // Makes the buffer's device current for the scope of one call.
 struct DeviceGuard {
     int prev = -1;
@@ -946,17 +960,20 @@ int ubep_debug_plan(const ubep_config_t* cfg, int32_t T, int32_t max_smem, const
     const int mode = choose_schedule(p, cfg->pipeline, n, count_warps, max_smem,
                                      [&](int cs) { return ctas[cs == 2 ? 1 : cs == 4 ? 2 : 3]; }, &pl);
     if (mode < 0) return mode;
-    plan[UBEP_DEBUG_PLAN_MODE] = mode;
-    plan[UBEP_DEBUG_PLAN_CHUNKS] = p.nchunks;
-    plan[UBEP_DEBUG_PLAN_PARTS] = p.parts;
-    plan[UBEP_DEBUG_PLAN_CLUSTER] = p.cluster;
-    plan[UBEP_DEBUG_PLAN_STEAL] = p.steal;
-    plan[UBEP_DEBUG_PLAN_STAGES] = pl.stages;
-    plan[UBEP_DEBUG_PLAN_OUT_STAGES] = pl.out_stages;
-    plan[UBEP_DEBUG_PLAN_LONG_ROWS] = pl.q_long;
-    plan[UBEP_DEBUG_PLAN_TEAMS] = pl.q_teams;
-    plan[UBEP_DEBUG_PLAN_TEAM_WARPS] = pl.q_team_warps;
-    plan[UBEP_DEBUG_PLAN_SMEM] = ubep::with_room_beside(pl.total, mode == ubep::kModeFew ? 0 : ubep::kLeastStatic);
+    fill_plan(p, pl, mode, plan);
+    return UBEP_OK;
+}
+
+int ubep_debug_buffer_plan(ubep_buffer_t* buf, int32_t T, int32_t plan[UBEP_DEBUG_PLAN_COUNT_]) {
+    if (!buf || !plan || T < 1 || T > buf->cfg.max_tokens) return UBEP_ERR_ARG;
+    DeviceGuard guard(buf->cfg.device);
+    if (guard.err != cudaSuccess) return cuda_fail(buf, guard.err);
+    Params p = make_params(buf, T);
+    ubep::SmemPlan pl{};
+    const int mode = choose_schedule(p, buf->cfg.pipeline, buf->lay.nchunks, buf->count_warps, buf->max_smem,
+                                     [&](int cs) { return ubep::cluster_ctas(cs, buf->max_smem); }, &pl);
+    if (mode < 0) return mode;
+    fill_plan(p, pl, mode, plan);
     return UBEP_OK;
 }
 

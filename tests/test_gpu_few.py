@@ -106,3 +106,19 @@ def test_between_calls_of_other_sizes():
         buf.recv_x.fill_(Hn.FILL)
         buf.dispatch(*dev[i][:3])
         Hn.check_dispatch(buf, wls[i], refs[i][1], 8192, refs[i][3], check_tails=False)
+
+
+@pytest.mark.gpu
+def test_rows_are_fetched_behind_the_layout_where_that_is_asked_for():
+    """The kernel asks for all rows of a CTA at once, so a call that may not do so goes another way."""
+    cfg = W.Config("few", T=200, H=512, E=32, R=4, k=8, payload=1, dedup=1, seed=11)
+    wl = W.make_workload(cfg)
+    _, lay, cap, recv = Hn.oracle_reference(wl)
+    buf = Hn.make_buffer(cfg, cap)
+    x, idx, w, _, _ = Hn.device_inputs(wl)
+    for n, few in ((1 << 30, True), (2, True), (1, False)):   # (two tokens per CTA)
+        B.ubep_debug_set_prefetch_rows(buf.handle, n)
+        assert (B.ubep_debug_buffer_plan(buf.handle, cfg.T)["mode"] == FEW) == few
+        buf.recv_x.fill_(Hn.FILL)
+        buf.dispatch(x, idx, w)
+        Hn.check_dispatch(buf, wl, lay, cap, recv)
