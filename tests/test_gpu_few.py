@@ -122,3 +122,33 @@ def test_rows_are_fetched_behind_the_layout_where_that_is_asked_for():
         buf.recv_x.fill_(Hn.FILL)
         buf.dispatch(x, idx, w)
         Hn.check_dispatch(buf, wl, lay, cap, recv)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("payload,dedup", [(0, 0), (1, 1)])
+@pytest.mark.parametrize("T", [3, 19, 60, 148, 200])
+def test_every_cta_stamps_its_phases(T, payload, dedup):
+    """Rows that the first warp does not send, CTAs without tokens, several column parts and several tokens per CTA."""
+    cfg = W.Config("few", T=T, H=1024, E=64, R=4, k=8, payload=payload, dedup=dedup, seed=T)
+    wl = W.with_empty_slots(W.make_workload(cfg), 0.4, seed=T)
+    wl.topk_idx[::2, 0] = -1
+    _, lay, cap, recv = Hn.oracle_reference(wl)
+    buf = Hn.make_buffer(cfg, cap)
+    x, idx, w, _, _ = Hn.device_inputs(wl)
+    B.ubep_debug_trace(buf.handle, True)
+    pl = B.ubep_debug_buffer_plan(buf.handle, T)
+    ctas = pl["chunks"] * pl["parts"]
+    assert pl["mode"] == FEW
+    buf.trace.zero_()
+    for _ in range(2):
+        before = buf.trace[:ctas, 10].cpu().numpy().copy()
+        buf.dispatch(x, idx, w)
+        Hn.check_dispatch(buf, wl, lay, cap, recv)
+        tr = buf.trace.cpu().numpy()[:ctas]
+        assert (tr[:, 0] > before).all()
+        # start, table staged, rows assigned, copies may leave, last copy issued, (counts written,) copies complete, end
+        for a, b in ((0, 1), (1, 5), (5, 6), (6, 8), (8, 9), (8, 3), (9, 10), (3, 10)):
+            assert (tr[:, a] <= tr[:, b]).all(), (a, b)
+        own = [c for c in range(ctas) if (c // pl["parts"]) * T // pl["chunks"] < (c // pl["parts"] + 1) * T // pl["chunks"]]
+        assert (tr[own, 6] <= tr[own, 7]).all() and (tr[own, 7] <= tr[own, 8]).all()
+        assert (tr[:, 10] - tr[:, 0]).max() < 5e6
