@@ -152,3 +152,39 @@ def test_every_cta_stamps_its_phases(T, payload, dedup):
         own = [c for c in range(ctas) if (c // pl["parts"]) * T // pl["chunks"] < (c // pl["parts"] + 1) * T // pl["chunks"]]
         assert (tr[own, 6] <= tr[own, 7]).all() and (tr[own, 7] <= tr[own, 8]).all()
         assert (tr[:, 10] - tr[:, 0]).max() < 5e6
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("T,k", [(16, 2), (200, 8)])
+def test_fp8_special_values(T, k):
+    """Zeros, groups below the floor of their maximum, infinities, values beyond the format and NaNs."""
+    cfg = W.Config("few", T=T, H=512, E=8 * k, R=4, k=k, payload=1, dedup=1, seed=12)
+    wl = W.make_workload(cfg)
+    xf = W.bf16_bits_to_f32(wl.x)
+    xf[0, :128] = 0.0
+    xf[1, 128:256] = 3e-6
+    xf[2, :] *= 1e30
+    xf[4, :128] = np.linspace(-1, 1, 128)
+    xf[5, 7], xf[6, 200] = np.inf, -np.inf
+    wl.x = W.f32_to_bf16_bits(xf)
+    wl.x[3, 5], wl.x[3, 6] = 0x7FC0, 0xFFC0
+    buf = Hn.run_case(wl)[0]
+    assert B.ubep_debug_buffer_plan(buf.handle, T)["mode"] == FEW
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("E,R", [(65504, 2047), (65535, 65535), (11200, 5600)])
+@pytest.mark.parametrize("dedup", [0, 1])
+def test_tables_of_many_experts(E, R, dedup):
+    """Ids up to the largest that 16 bits hold beside the mark of an empty slot."""
+    cfg = W.Config("few", T=40, H=128, E=E, R=R, k=8, payload=dedup, dedup=dedup, seed=31, num_src_ranks=3)
+    wl = W.with_empty_slots(W.make_workload(cfg), 0.1, seed=5)
+    wl.topk_idx[7, :3] = (E - 1, E - 2, 0)
+    _, lay, cap, recv = Hn.oracle_reference(wl, cap=8)
+    buf = Hn.make_buffer(cfg, cap)
+    assert B.ubep_debug_buffer_plan(buf.handle, cfg.T)["mode"] == FEW
+    x, idx, w, _, _ = Hn.device_inputs(wl)
+    for _ in range(2):
+        buf.recv_x.fill_(Hn.FILL)
+        buf.dispatch(x, idx, w)
+        Hn.check_dispatch(buf, wl, lay, cap, recv)

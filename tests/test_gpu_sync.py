@@ -312,3 +312,50 @@ def test_the_most_ranks_whose_counts_fit(proto):
         buf.recv_x.fill_(Hn.FILL)
         buf.dispatch_sync(proto, x, idx, w)
         Hn.check_dispatch(buf, wl, lay, cap, recv, arrival=False)
+
+
+@pytest.mark.parametrize("proto", PROTOCOLS)
+@pytest.mark.parametrize("payload,dedup", [(0, 0), (0, 1), (1, 0), (1, 1)])
+@pytest.mark.parametrize("case", [
+    # (layout, CTAs that share a row, configuration): a warp per slot; the whole table by every CTA
+    (B.UBEP_SYNC_LAYOUT_FEW, 4, dict(T=37, E=32, R=1, k=8)),
+    (B.UBEP_SYNC_LAYOUT_FEW, 2, dict(T=74, E=48, R=48, k=4)),
+    (B.UBEP_SYNC_LAYOUT_FEW, 1, dict(T=149, E=36, R=4, k=8, E_logical=32)),
+    (B.UBEP_SYNC_LAYOUT_WHOLE, 1, dict(T=257, E=32, R=1, k=8)),
+    (B.UBEP_SYNC_LAYOUT_WHOLE, 1, dict(T=445, E=48, R=48, k=4)),
+    (B.UBEP_SYNC_LAYOUT_WHOLE, 1, dict(T=90, E=36, R=4, k=3, E_logical=32)),
+    (B.UBEP_SYNC_LAYOUT_WHOLE, 1, dict(T=33, E=64, R=8, k=6)),
+    (B.UBEP_SYNC_LAYOUT_LAUNCHED, 1, dict(T=1400, E=36, R=4, k=6, E_logical=32)),
+], ids=lambda c: f"{c[0]}-{c[2]['T']}-{c[2]['k']}")
+def test_two_calls_of_every_layout(case, payload, dedup, proto):
+    """Different routing in each on one buffer, an expert named twice in some tokens; results, wire and status after each."""
+    layout, parts, kw = case
+    cfg = W.Config("twice", H=640, payload=payload, dedup=dedup, seed=kw["T"], num_src_ranks=7, **kw)
+    wls = [W.with_empty_slots(W.make_workload(dataclasses.replace(cfg, seed=s)), 0.1, seed=s) for s in (kw["T"], 77)]
+    for wl in wls:   # (one replica table: it belongs to the buffer)
+        wl.phys, wl.ncopies = wls[0].phys, wls[0].ncopies
+    given = [wl.topk_idx.copy() for wl in wls]
+    for g, wl in zip(given, wls):
+        dup = (np.arange(cfg.T) % 5 == 0) & (g[:, 0] >= 0)
+        if cfg.E_logical:   # (a replicated expert named twice may be two physical ones)
+            dup &= False
+        g[dup, cfg.k - 1] = g[dup, 0]
+        wl.topk_idx[dup, cfg.k - 1] = -1
+    cap = max(Hn.oracle_reference(wl)[2] for wl in wls)
+    buf = Hn.make_buffer(cfg, cap)
+    grid = buf.trace.shape[0]
+    pl = B.ubep_debug_sync_plan(buf.cfg, proto, cfg.T, 232448, grid)
+    assert pl["layout"] == layout and pl["parts"] == (1 if proto == "sw" else parts), pl
+    buf.attach_sync()
+    for wl, g in zip(wls, given):
+        _, lay, _, recv = Hn.oracle_reference(wl, cap=cap)
+        x, _, w, phys, ncopies = Hn.device_inputs(wl)
+        if phys is not None:
+            buf.set_replicas(phys, ncopies)
+        for view in [buf.recv_x, buf.recv_src_idx] + [buf.recv_scale] * payload + ([buf.recv_topk_idx, buf.recv_topk_w] if dedup else [buf.recv_weight]):
+            view.view(torch.uint8).fill_(Hn.FILL)
+        buf.dispatch_sync(proto, x, Hn.to_dev(g), w)
+        if not np.array_equal(g, wl.topk_idx):
+            assert buf.status() == B.UBEP_ERR_BAD_INDEX
+        Hn.check_dispatch(buf, wl, lay, cap, recv, arrival=False)
+        wire_checks(buf, proto, cfg, lay, recv, grid)

@@ -20,7 +20,11 @@ def _in_order(text, *marks):
 
 def test_a_token_flag_strip_is_complete_before_other_lanes_read_it():
     # (a warp vote brings lanes together but orders no memory)
-    _in_order(_source("ubep_sync.cu"), "mine[3 * g + 2] = ", "__syncwarp()", "reinterpret_cast<const uint4*>(mine")
+    text = _source("ubep_sync.cu")
+    # strips of payload alone, then those with conditions per word; behind either the buffer may be used again
+    _in_order(text, "mine[3 * (b * 32 + lane) + 2] = ", "__syncwarp()", "reinterpret_cast<const uint4*>(mine)[", "__syncwarp()",
+              "mine[3 * g + 2] = ", "__syncwarp()", "reinterpret_cast<const uint4*>(mine + ", "__syncwarp()")
+    assert text.count("reinterpret_cast<const uint4*>(mine") == 2
 
 
 def test_a_chunks_cursor_is_reset_before_its_destinations_are_released():
