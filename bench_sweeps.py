@@ -85,6 +85,8 @@ def spread(cfg: W.Config, order, repeats: int = 5):
         buf.set_replicas(phys, ncopies)
     buf.set_dest_order(order)
     B.ubep_debug_trace(buf.handle, True)
+    plan = B.ubep_debug_buffer_plan(buf.handle, cfg.T)
+    ctas = plan["chunks"] * plan["parts"]   # (in clusters not every SM has one; the others' stamps are of no call)
     flush = torch.empty(512 << 20, dtype=torch.uint8, device=dev)
     runs = []
     for it in range(repeats + 1):
@@ -93,7 +95,7 @@ def spread(cfg: W.Config, order, repeats: int = 5):
         torch.cuda.synchronize()
         if it == 0:
             continue                       # first run: warm-up
-        tr = buf.trace.cpu().numpy().astype(np.int64)
+        tr = buf.trace.cpu().numpy().astype(np.int64)[:ctas]
         t0 = tr[:, 0].min()
         runs.append(np.stack([(tr[:, s] - t0) / 1e3 for s in (READY, ISSUED, STORED, END)], axis=1))
     status = buf.status()
