@@ -442,7 +442,8 @@ int ubep_debug_withhold_flag(ubep_buffer_t *buf, int32_t chunk);
  * boundaries into UBEP_VIEW_TRACE: 0 start, 1 counted, 2 all counts seen, 3 prefix sums
  * published, 4 all offsets seen, 5 rows assigned, 6 movers released, 7 first row in shared
  * memory, 8 last copy issued, 9 copies complete, 10 end.  Slots a CTA does not pass keep
- * their old value.
+ * their old value.  (Small batches, where every warp sends rows of its own: the time at which the last
+ * warp of the CTA got there; 5 and 6 coincide, 7 needs a token of the CTA's, 3 = counts written.)
  */
 int ubep_debug_trace(ubep_buffer_t *buf, int32_t enable);
 

@@ -2,7 +2,7 @@
 //
 // What bounds it is latency, not bytes: 13 tokens are 1.4 MB.  The kernels for larger batches spend most of such a call on
 // control flow that is worth its while only with many rows -- rings, roles that release one another through barriers, counting
-// and prefix sums through shared memory, and every jump to a piece of code that has not run yet costs 0.1 us (64 functions 2 KB
+// and prefix sums through shared memory, and every jump to a piece of code that has not run yet costs 0.15 us (64 functions 2 KB
 // apart, called once: 300 cycles each, 190 the second time; code that runs straight on: 3.5 cycles per instruction).  Here the
 // table is staged once; then every slot of the CTA's own tokens is a warp's, which counts the table for its own expert and rank
 // alone, sends its copy, writes its metadata and adds to the arrival counter by itself.  There is no barrier after the
@@ -230,7 +230,7 @@ bool plan_few(const Params& p, int max_smem, SmemPlan* out) {
     pl.off_ids = pl.off_out + (int)(most * out_stage);
     // One CTA per SM.  Two of them fit in an SM's registers, and where a call may be placed while the combine before it runs
     // (programmatic launches), SMs without combine CTAs took two and others none: sixteen layers of 128 tokens of 7168 channels,
-    // top-8, in one graph 12.6 us per layer, this way 10.4.  (Warps that leave at once do not hold their registers: no change.)
+    // top-8, in one graph 12.6 us per layer, this way 10.4 (both at the time; 9.5 now).  (Warps that leave at once do not hold their registers: no change.)
     pl.total = (int)(total < kFewSmem ? kFewSmem : total);
     pl.duty_units = table_units(p);
     *out = pl;

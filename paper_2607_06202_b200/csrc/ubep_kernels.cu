@@ -303,8 +303,9 @@ __device__ __forceinline__ void mover_warp(Cta& x) {
     // Rows fetched before the layout is done.  With flags the layout takes many microseconds in which a
     // few small loads and stores of every CTA wait on one another; a ring-full of rows per CTA fetched
     // meanwhile fills the memory system's queues in front of them.  Three rows start the copies, the
-    // rest follows once the movers are released.  (Not with stealing: there every block of rows costs a
-    // claim, a round trip each, and those are best paid while the layout runs.)
+    // rest follows once the movers are released.  (With stealing the whole ring: so it was settled when every block of
+    // rows cost a claim, a round trip each, best paid while the layout ran.  The head of a slice costs none now; FUSED and PHASED,
+    // which AUTO takes only where the plan of the layout by clusters does not fit, have not been timed again since.)
     const int early = (kMode == kModeLocal || kMode == kModeCluster || kSteal) ? kMaxStages : 3;
     if (!kFp8) {
         // loads run (stages - 3) rows ahead; up to 3 rows' stores stay in flight (all rows at once where they fit)

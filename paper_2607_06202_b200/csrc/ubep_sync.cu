@@ -594,6 +594,8 @@ cudaError_t launch_layout(const Params& p, const SmemPlan& pl, const SyncParams&
 }  // namespace
 
 bool plan_sync_few(Params& p, int protocol, int max_smem, SmemPlan* out) {
+    // (Two, four and eight slots: every further number would be eight more kernels.  The dispatch of small batches has instances for
+    // one and six as well; here those take the whole table's count, which they always took: nobody's main path, not timed.)
     if ((p.k != 2 && p.k != 4 && p.k != 8) || p.L > 32) return false;
     // idle CTAs take a part of the rows (not with stop-and-wait, whose counters count rows)
     while (protocol != kSW && p.T <= p.nchunks / 2 && p.nchunks % 2 == 0 && p.parts < 4) {
